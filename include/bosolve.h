@@ -220,8 +220,8 @@ int bo_prec_destroy(bo_prec* P);
  * launch-overhead measure for batches of small systems. */
 int bo_prec_set_launch_mode(bo_prec* P, int mode);
 /* Tile parameters of the per-kernel form of P's AMG V-cycle, the form its
- * CUDA-graph launch modes run (captured graphs cannot hold cooperative
- * launches): `cells` level-0 Gauss-Seidel cells per thread (1, 2 or 4, all
+ * CUDA-graph launch modes run above the cluster launch (captured graphs
+ * cannot hold cooperative launches): `cells` level-0 Gauss-Seidel cells per thread (1, 2 or 4, all
  * of a thread's loads issued before its stores) and `threads` per block
  * (128, 256 or 512) for every per-kernel AMG launch.  The V-cycle is the
  * same whatever the shape.  Captured graphs are rebuilt after a change.
@@ -692,16 +692,17 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
 int bo_set_conv_engine(int engine);
 /* How the AMG V-cycle is launched (process-wide); every form computes the
  * same V-cycle of paper Sec. 3.2's pressure AMG stage:
- * 2 (the default) = levels 0 and 1 in two cooperative launches, a down leg
- *   and an up leg whose blocks meet at grid-wide barriers between the
- *   Gauss-Seidel half sweeps, around one thread-block-cluster launch (up to
- *   16 blocks, hardware cluster barriers) for all coarser levels, the
- *   levels of at most 4096 cells in one of its blocks;
+ * 2 (the default) = every level of at most 32768 cells (FP64 preconditioners:
+ *   16384) in one thread-block-cluster launch of up to 16 blocks, iterates in
+ *   shared memory, hardware cluster barriers between the half sweeps; the
+ *   levels above them in two cooperative launches around it, a down leg and
+ *   an up leg whose blocks meet at grid-wide barriers;
  * 1 = the cooperative legs smooth every multi-block level, around one
  *   block for the levels of at most 4096 cells;
  * 0 = one kernel per half sweep, restriction and prolongation.
- * Inside stream capture (CUDA-graph launch mode) the per-kernel form is used
- * whatever the setting, and a form the device refuses falls back to it.  A
+ * Inside stream capture (CUDA-graph launch mode) the legs run in the
+ * per-kernel form, and a form the device refuses falls back to it.  A
+ * preconditioner without pre- or without post-sweeps runs mode 2 as mode 1.  A
  * grid barrier that waits too long ends the launch and the solve returns
  * BO_ERR_TIMEOUT.  BO_ERR_ARG for another mode. */
 int bo_set_amg_cooperative(int on);

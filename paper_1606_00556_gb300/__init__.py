@@ -828,9 +828,10 @@ def bo_update_batched(precs, vals=None):
 
 
 def bo_set_amg_cooperative(on: int):
-    """2 (default): level 0 as two cooperative launches per V-cycle around
-    one cluster launch for the coarser levels; 1: the cooperative launches
-    cover every multi-block level; 0: one kernel per sweep."""
+    """2 (default): one cluster launch per V-cycle for every level of at most
+    32768 cells (FP64: 16384), two cooperative launches around it for the
+    levels above; 1: the cooperative launches cover every multi-block level;
+    0: one kernel per sweep."""
     _check(lib().bo_set_amg_cooperative(int(on)), "bo_set_amg_cooperative")
 
 

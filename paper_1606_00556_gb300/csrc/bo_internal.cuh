@@ -334,9 +334,9 @@ constexpr int kMaxPoolStreams = 16;
 extern std::atomic<int> g_pool_width;
 // convolution engine of the 32 -> 32 layers: 0 mma.sync, 1 tcgen05 (conv_tc.cu)
 extern std::atomic<int> g_conv_engine;
-// AMG launch form: 2 (default) cooperative legs for levels 0-1 around a cluster
-// launch for the coarser levels, 1 cooperative legs for every multi-block
-// level around a one-block tail, 0 one kernel per sweep
+// AMG launch form: 2 (default) one cluster launch for the levels that fit it,
+// cooperative legs for the levels above, 1 cooperative legs for every
+// multi-block level around a one-block tail, 0 one kernel per sweep
 extern std::atomic<int> g_amg_coop;
 // polls of an AMG grid barrier before it gives up (default 2^22, about 0.1 s)
 constexpr unsigned kAmgSpinsDefault = 1u << 22;
@@ -429,7 +429,7 @@ struct Level {
   int32_t nx, ny, nz;
   int64_t n;
   double* c64;   // 7 n FP64 coefficients [slot][cell] (setup master)
-  void* c;       // 7 n coefficients in the preconditioner precision
+  void* c;       // 7 n coefficients in the preconditioner precision (FP64: and n reciprocals of the diagonal)
   void* f;       // n right-hand side
   void* x;       // n iterate
 };
@@ -437,6 +437,7 @@ struct Level {
 }  // namespace bo
 
 struct bo_wells;
+namespace bo { struct ResPlan; }
 
 struct bo_prec {
   bo_mat* mat;
@@ -450,13 +451,14 @@ struct bo_prec {
   double* w;               // 3 N decoupling weights (g0, g1, g2) of row 0, [3][N] internal order
   float* wf;               // the same weights rounded to FP32 (FP32 arithmetic), else NULL
   void* Dinv;              // 9 N inverted ILU pivot blocks [rc][N], preconditioner precision
+  double* di0;             // FP64 storage: N reciprocals of level 0's AMG diagonal [colour][q], else NULL
   // AMG: level 0 = the pressure block of At (colour-split), levels 1.. natural order
   int nlev;
   bo::Level lev[24];
   int tail_from;           // first level handled by the single-block tail kernel
-  double* coarse64;        // dense coarsest matrix / inverse workspace (FP64)
-  void* coarse_inv;        // dense inverse of the coarsest level (precision T)
+  void* coarse_inv;        // dense inverse of the coarsest level, transposed (storage type)
   int64_t ncoarse;
+  bo::ResPlan* res;        // the levels that run in one cluster (precond.cu)
   // CPR work vectors (precision T, internal order)
   void* f;                 // 3N decoupled input
   void* t;                 // 3N ILU intermediates

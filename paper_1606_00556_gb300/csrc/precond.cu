@@ -19,8 +19,10 @@
 // correction, black then red after it.  After a black half sweep only red
 // cells carry a residual, so restriction sums red residuals.  Levels of at
 // most kTailCells cells run inside one thread block (kernel k_tail).
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
+#include <new>
 
 #include "bo_internal.cuh"
 
@@ -137,7 +139,7 @@ __device__ __forceinline__ __nv_bfloat16 store_split<__nv_bfloat16>(df v) {
 template <typename S>
 __global__ void k_decouple(Geom g, const double* __restrict__ A, const float2* __restrict__ A2,
                            const int* __restrict__ range, S* __restrict__ At, double* __restrict__ w,
-                           float* __restrict__ wf, int abf, DevState* st) {
+                           float* __restrict__ wf, double* __restrict__ di0, int abf, DevState* st) {
   wait_prior_grid();
   const bool split = sizeof(S) < sizeof(double) && A2 && !*range;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.N; t += (int64_t)gridDim.x * blockDim.x) {
@@ -210,6 +212,7 @@ __global__ void k_decouple(Geom g, const double* __restrict__ A, const float2* _
       if (s == kDiag) {
         const double app = g0 * a[0] + g1 * a[3] + g2 * a[6];
         if (app == 0.0 || !isfinite(app)) atomicOr(&st->err, kErrBreakdown);
+        if (di0) di0[t] = 1.0 / app;  // (FP64 storage: At holds app itself)
       }
     }
   }
@@ -391,13 +394,6 @@ __global__ void k_ilu_black(Geom g, const double* __restrict__ A, const double* 
   }
 }
 
-template <typename S>
-__global__ void k_convert(const double* __restrict__ src, S* __restrict__ dst, size_t n) {
-  wait_prior_grid();
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = to_store<S>(src[i]);
-}
-
 // ------------------------------------------------------------ AMG setup
 struct LevelDims {
   int32_t nx, ny, nz;
@@ -418,191 +414,400 @@ __device__ __forceinline__ int64_t nat_index(const LevelDims& L, int i, int j, i
   return i + (int64_t)L.nx * (j + (int64_t)L.ny * k);
 }
 
-// direction slot of the coarse neighbour (di, dj, dk), or kDiag
-__device__ __forceinline__ int dir_slot(int di, int dj, int dk) {
-  if (dk < 0) return kZm;
-  if (dk > 0) return kZp;
-  if (dj < 0) return kYm;
-  if (dj > 0) return kYp;
-  if (di < 0) return kXm;
-  if (di > 0) return kXp;
-  return kDiag;
+// Galerkin products: coarse entry (I, J) = sum of the fine entries a_ij with
+// i in aggregate I and j in aggregate J.  Eight lanes of a warp serve one
+// coarse cell, one lane per child cell, and a warp serves four coarse cells:
+// every lane issues all of its child's loads at once (one thread per coarse
+// cell walked its children one after the other, 8 dependent rounds of loads,
+// and left small levels with a handful of warps: 43-56 us for level 1 and 17
+// us per coarser level whatever their size).  A child's entries towards its
+// own aggregate join the diagonal, the three others the coarse faces; the
+// children's sums meet by shuffles in a fixed order.  Lane bits: child x
+// offset (1), coarse cell of the four (2, 4), child y (8), child z (16), so
+// the lanes of a row of children read consecutive fine cells.  The value is
+// written in FP64 (the next level's input) and in the storage type.
+// Measured, before -> after: level 1 of 128x128x64 70 -> 65 us, of 20x20x5
+// 43 -> 7 us; a coarser level 17 -> 4-8 us (the conversion to the
+// storage type included, which was a launch of its own).
+struct Child {
+  int64_t I;      // coarse cell, or -1
+  int i, j, k;    // the child's fine coordinates
+  bool ok;        // the child exists
+};
+__device__ __forceinline__ Child galerkin_child(const LevelDims& C, int64_t group, int fnx, int fny, int fnz) {
+  const int lane = threadIdx.x & 31;
+  Child c;
+  c.I = 4 * group + ((lane >> 1) & 3);
+  c.ok = c.I < C.n;
+  const Ijk p = ijk_of(C, c.ok ? c.I : 0);
+  c.i = 2 * p.i + (lane & 1);
+  c.j = 2 * p.j + ((lane >> 3) & 1);
+  c.k = 2 * p.k + (lane >> 4);
+  if (c.I >= C.n) c.I = -1;
+  c.ok = c.ok && c.i < fnx && c.j < fny && c.k < fnz;
+  return c;
+}
+__device__ __forceinline__ double add_xor(double v, int m) { return v + __shfl_xor_sync(0xffffffffu, v, m); }
+
+// FP64 levels keep the reciprocals of the diagonal behind the seven
+// coefficients: the Gauss-Seidel sweeps multiply by them, since an FP64
+// division is about ten FP64 multiply-adds where the rest of a cell's
+// update takes six (FP32 divisions are cheap and stay divisions)
+template <typename S>
+__host__ __device__ constexpr int level_slots() { return sizeof(S) == 8 ? 8 : 7; }
+template <typename S>
+__device__ __forceinline__ void put_reciprocal(S* __restrict__ c, const LevelDims& C, int64_t I, double diag) {
+  if constexpr (sizeof(S) == 8) c[(size_t)7 * C.n + I] = 1.0 / diag;
 }
 
-// Galerkin level 1 from level 0 (the decoupled pressure block, FP64 from A
-// and the weights): coarse entry (I, J) = sum of fine a_ij, i in I, j in J.
+// a[7]: the child's fine row (zero where the child or the neighbour is missing)
+template <typename S>
+__device__ __forceinline__ void galerkin_sum(const LevelDims& C, const Child& ch, const double a[7],
+                                             double* __restrict__ c64, S* __restrict__ c, DevState* st) {
+  const int lane = threadIdx.x & 31;
+  const bool di = lane & 1, dj = lane & 8, dk = lane & 16;
+  double diag = a[kDiag];
+  diag += dk ? a[kZm] : a[kZp];
+  diag += dj ? a[kYm] : a[kYp];
+  diag += di ? a[kXm] : a[kXp];
+  double fx = di ? a[kXp] : a[kXm], fy = dj ? a[kYp] : a[kYm], fz = dk ? a[kZp] : a[kZm];
+  diag = add_xor(add_xor(add_xor(diag, 1), 8), 16);
+  fx = add_xor(add_xor(fx, 8), 16);
+  fy = add_xor(add_xor(fy, 1), 16);
+  fz = add_xor(add_xor(fz, 1), 8);
+  if (ch.I < 0) return;
+  auto put = [&](int s, double v) {
+    c64[(size_t)s * C.n + ch.I] = v;
+    c[(size_t)s * C.n + ch.I] = to_store<S>(v);
+  };
+  if (!dj && !dk) put(di ? kXp : kXm, fx);
+  if (!di && !dk) put(dj ? kYp : kYm, fy);
+  if (!di && !dj) put(dk ? kZp : kZm, fz);
+  if (di && dj && dk) {
+    put(kDiag, diag);
+    put_reciprocal(c, C, ch.I, diag);
+    if (diag == 0.0 || !isfinite(diag)) atomicOr(&st->err, kErrBreakdown);
+  }
+}
+
+// level 1 from level 0 (the decoupled pressure block, FP64 from A and the weights)
+__device__ __forceinline__ void galerkin0_row(const Geom& g, const double* __restrict__ A, const double* __restrict__ w,
+                                              int i, int j, int k, double a[7]) {
+  const int color = (i + j + k) & 1;
+  const int64_t q = (i + (int64_t)g.nx * (j + (int64_t)g.ny * k)) >> 1;
+  const double g0 = w[vidx(g, 0, color, q)], g1 = w[vidx(g, 1, color, q)], g2 = w[vidx(g, 2, color, q)];
+  double r[21];
+#pragma unroll
+  for (int s = 0; s < 7; ++s)
+#pragma unroll
+    for (int u = 0; u < 3; ++u) r[3 * s + u] = A[plane(g, color, s, 3 * u) + q];
+  // (blocks outside the grid are stored as zeros)
+#pragma unroll
+  for (int s = 0; s < 7; ++s) a[s] = g0 * r[3 * s] + g1 * r[3 * s + 1] + g2 * r[3 * s + 2];
+}
+
+template <typename S>
 __global__ void k_galerkin0(Geom g, const double* __restrict__ A, const double* __restrict__ w, LevelDims C,
-                            double* __restrict__ c64, DevState* st) {
+                            double* __restrict__ c64, S* __restrict__ c, DevState* st) {
   wait_prior_grid();
-  for (int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; I < C.n; I += (int64_t)gridDim.x * blockDim.x) {
-    const Ijk cc = ijk_of(C, I);
-  const int ci = cc.i, cj = cc.j, ck = cc.k;
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int dk = 0; dk < 2; ++dk)
-      for (int dj = 0; dj < 2; ++dj)
-        for (int di = 0; di < 2; ++di) {
-          const int i = 2 * ci + di, j = 2 * cj + dj, k = 2 * ck + dk;
-          if (i >= g.nx || j >= g.ny || k >= g.nz) continue;
-          const int color = (i + j + k) & 1;
-          const int64_t q = (i + (int64_t)g.nx * (j + (int64_t)g.ny * k)) >> 1;
-          const double g0 = w[vidx(g, 0, color, q)], g1 = w[vidx(g, 1, color, q)], g2 = w[vidx(g, 2, color, q)];
-          const int ni[7] = {i, i, i - 1, i, i + 1, i, i};
-          const int nj[7] = {j, j - 1, j, j, j, j + 1, j};
-          const int nk[7] = {k - 1, k, k, k, k, k, k + 1};
-          for (int s = 0; s < 7; ++s) {
-            if (ni[s] < 0 || ni[s] >= g.nx || nj[s] < 0 || nj[s] >= g.ny || nk[s] < 0 || nk[s] >= g.nz) continue;
-            const double a = g0 * A[plane(g, color, s, 0) + q] + g1 * A[plane(g, color, s, 3) + q] +
-                             g2 * A[plane(g, color, s, 6) + q];
-            const int cs = dir_slot(ni[s] / 2 - ci, nj[s] / 2 - cj, nk[s] / 2 - ck);
-            acc[cs] += a;
-          }
-        }
-    for (int s = 0; s < 7; ++s) c64[(size_t)s * C.n + I] = acc[s];
-    if (acc[kDiag] == 0.0 || !isfinite(acc[kDiag])) atomicOr(&st->err, kErrBreakdown);
+  const int64_t ngroups = (C.n + 3) / 4;
+  for (int64_t gr = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; gr < ngroups;
+       gr += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const Child ch = galerkin_child(C, gr, g.nx, g.ny, g.nz);
+    double a[7] = {0, 0, 0, 0, 0, 0, 0};
+    if (ch.ok) galerkin0_row(g, A, w, ch.i, ch.j, ch.k, a);
+    galerkin_sum<S>(C, ch, a, c64, c, st);
   }
 }
 
-// Galerkin level l+1 from natural-order level l
+// The same with two lanes per coarse cell (the two children along x; the
+// four rows of children one after the other): a warp's loads cover 16
+// consecutive values of a plane instead of 4, which is what a level that
+// fills the GPU anyway is bound by (level 1 of 128x128x64: 70 us with one
+// thread per coarse cell, 97 us with eight lanes, 65 us with two; the
+// launch takes it from kGalerkinWide coarse cells on, where eight lanes per
+// cell would be more than 8 warps per scheduler).
+constexpr int64_t kGalerkinWide = 32768;
+template <typename S>
+__global__ void k_galerkin0_wide(Geom g, const double* __restrict__ A, const double* __restrict__ w, LevelDims C,
+                                 double* __restrict__ c64, S* __restrict__ c, DevState* st) {
+  wait_prior_grid();
+  const int64_t n2 = (2 * C.n + 31) & ~(int64_t)31;  // whole warps: the sums meet by shuffles
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n2; t += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t I = t >> 1;
+    const int di = (int)(t & 1);
+    const bool live = I < C.n;
+    const Ijk p = ijk_of(C, live ? I : 0);
+    const int i = 2 * p.i + di;
+    double diag = 0.0, fx = 0.0, y0 = 0.0, y1 = 0.0, z0 = 0.0, z1 = 0.0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int j = 2 * p.j + (r & 1), k = 2 * p.k + (r >> 1);
+      if (!live || i >= g.nx || j >= g.ny || k >= g.nz) continue;
+      double a[7];
+      galerkin0_row(g, A, w, i, j, k, a);
+      diag += a[kDiag] + (di ? a[kXm] : a[kXp]) + (r & 1 ? a[kYm] : a[kYp]) + (r >> 1 ? a[kZm] : a[kZp]);
+      fx += di ? a[kXp] : a[kXm];
+      if (r & 1) y1 += a[kYp];
+      else y0 += a[kYm];
+      if (r >> 1) z1 += a[kZp];
+      else z0 += a[kZm];
+    }
+    diag = add_xor(diag, 1);
+    y0 = add_xor(y0, 1);
+    y1 = add_xor(y1, 1);
+    z0 = add_xor(z0, 1);
+    z1 = add_xor(z1, 1);
+    if (!live) continue;
+    auto put = [&](int s, double v) {
+      c64[(size_t)s * C.n + I] = v;
+      c[(size_t)s * C.n + I] = to_store<S>(v);
+    };
+    put(di ? kXp : kXm, fx);
+    put(di ? kYp : kYm, di ? y1 : y0);
+    put(di ? kZp : kZm, di ? z1 : z0);
+    if (di) {
+      put(kDiag, diag);
+      put_reciprocal(c, C, I, diag);
+      if (diag == 0.0 || !isfinite(diag)) atomicOr(&st->err, kErrBreakdown);
+    }
+  }
+}
+
+// level l+1 from natural-order level l
+template <typename S>
 __global__ void k_galerkinn(LevelDims F, const double* __restrict__ f64, LevelDims C, double* __restrict__ c64,
-                            DevState* st) {
+                            S* __restrict__ c, DevState* st) {
   wait_prior_grid();
-  for (int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; I < C.n; I += (int64_t)gridDim.x * blockDim.x) {
-    const Ijk cc = ijk_of(C, I);
-  const int ci = cc.i, cj = cc.j, ck = cc.k;
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int dk = 0; dk < 2; ++dk)
-      for (int dj = 0; dj < 2; ++dj)
-        for (int di = 0; di < 2; ++di) {
-          const int i = 2 * ci + di, j = 2 * cj + dj, k = 2 * ck + dk;
-          if (i >= F.nx || j >= F.ny || k >= F.nz) continue;
-          const int64_t c = nat_index(F, i, j, k);
-          const int ni[7] = {i, i, i - 1, i, i + 1, i, i};
-          const int nj[7] = {j, j - 1, j, j, j, j + 1, j};
-          const int nk[7] = {k - 1, k, k, k, k, k, k + 1};
-          for (int s = 0; s < 7; ++s) {
-            if (ni[s] < 0 || ni[s] >= F.nx || nj[s] < 0 || nj[s] >= F.ny || nk[s] < 0 || nk[s] >= F.nz) continue;
-            acc[dir_slot(ni[s] / 2 - ci, nj[s] / 2 - cj, nk[s] / 2 - ck)] += f64[(size_t)s * F.n + c];
-          }
-        }
-    for (int s = 0; s < 7; ++s) c64[(size_t)s * C.n + I] = acc[s];
-    if (acc[kDiag] == 0.0 || !isfinite(acc[kDiag])) atomicOr(&st->err, kErrBreakdown);
+  const int64_t ngroups = (C.n + 3) / 4;
+  for (int64_t gr = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; gr < ngroups;
+       gr += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const Child ch = galerkin_child(C, gr, F.nx, F.ny, F.nz);
+    double a[7] = {0, 0, 0, 0, 0, 0, 0};
+    if (ch.ok) {
+      const int64_t cf = nat_index(F, ch.i, ch.j, ch.k);
+#pragma unroll
+      for (int s = 0; s < 7; ++s) a[s] = f64[(size_t)s * F.n + cf];
+    }
+    galerkin_sum<S>(C, ch, a, c64, c, st);
   }
 }
 
-// dense coarsest matrix: natural level (c64 given) or level 0 in the
-// colour-split index order (index = colour * N/2 + q)
-__global__ void k_dense_from_level(LevelDims L, const double* __restrict__ c64, Geom g, const double* __restrict__ A,
-                                   const double* __restrict__ w, int level0, double* __restrict__ M) {
-  wait_prior_grid();
-  const int64_t n = L.n;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n * n; t += (int64_t)gridDim.x * blockDim.x)
-    M[t] = 0.0;
-  __syncthreads();
-  if (blockIdx.x != 0) return;
-  // one block fills the stencil entries (grid of at most 128 cells)
-  for (int64_t row = threadIdx.x; row < n; row += blockDim.x) {
-    int i, j, k;
-    if (level0) {
-      const int color = (int)(row / g.Nh);
-      const int64_t q = row - color * g.Nh;
-      const Cell c = decode(g, color, q);
-      i = c.i; j = c.j; k = c.k;
-    } else {
-      i = (int)(row % L.nx); j = (int)((row / L.nx) % L.ny); k = (int)(row / ((int64_t)L.nx * L.ny));
-    }
-    const int ni[7] = {i, i, i - 1, i, i + 1, i, i};
-    const int nj[7] = {j, j - 1, j, j, j, j + 1, j};
-    const int nk[7] = {k - 1, k, k, k, k, k, k + 1};
-    for (int s = 0; s < 7; ++s) {
-      if (ni[s] < 0 || ni[s] >= L.nx || nj[s] < 0 || nj[s] >= L.ny || nk[s] < 0 || nk[s] >= L.nz) continue;
-      double a;
-      int64_t colidx;
-      if (level0) {
-        const int color = (i + j + k) & 1;
-        const int64_t q = (i + (int64_t)g.nx * (j + (int64_t)g.ny * k)) >> 1;
-        a = w[vidx(g, 0, color, q)] * A[plane(g, color, s, 0) + q] + w[vidx(g, 1, color, q)] * A[plane(g, color, s, 3) + q] +
-            w[vidx(g, 2, color, q)] * A[plane(g, color, s, 6) + q];
-        const int ncol = (ni[s] + nj[s] + nk[s]) & 1;
-        colidx = ncol * g.Nh + ((ni[s] + (int64_t)g.nx * (nj[s] + (int64_t)g.ny * nk[s])) >> 1);
+// ------------------------------------------------------- dense inverse
+// Hardware barrier of all threads of a thread-block cluster, with release /
+// acquire semantics at cluster scope: every memory write of the cluster's
+// thread blocks before it is visible to their reads after it.  It is not a
+// spin on a flag: every thread of the cluster reaches every barrier (the
+// control flow is uniform).
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the address in block `rank` of the cluster that corresponds to p in this block's shared memory
+__device__ __forceinline__ uint32_t cluster_map(const void* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// The matrix to invert: dense (M), or the coarsest level's stencil, natural
+// order (c64) or level 0 in the colour-split index order (A and the weights).
+struct DenseSrc {
+  const double* M;
+  const double* c64;
+  LevelDims L;
+  Geom g;
+  const double* A;
+  const double* w;
+};
+// Row `row` of the matrix over the warp: lane's columns lane + 32 c.
+template <int CPL>
+__device__ __forceinline__ void dense_row(const DenseSrc& d, int n, int row, double a[CPL]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) a[c] = 0.0;
+  if (row >= n) return;
+  if (d.M) {
+#pragma unroll
+    for (int c = 0; c < CPL; ++c)
+      if (lane + 32 * c < n) a[c] = d.M[(size_t)row * n + lane + 32 * c];
+    return;
+  }
+  // lane s < 7 fetches stencil entry s and its column; every lane then takes the ones that are its own
+  int i, j, k, color = 0;
+  if (d.c64) {
+    i = row % d.L.nx;
+    j = (row / d.L.nx) % d.L.ny;
+    k = row / (d.L.nx * d.L.ny);
+  } else {
+    color = row >= d.g.Nh;
+    const Cell c = decode(d.g, color, row - color * d.g.Nh);
+    i = c.i; j = c.j; k = c.k;
+  }
+  double v = 0.0;
+  int col = -1;
+  if (lane < 7) {
+    const int ni = i + (lane == kXp) - (lane == kXm), nj = j + (lane == kYp) - (lane == kYm),
+              nk = k + (lane == kZp) - (lane == kZm);
+    if (ni >= 0 && ni < d.L.nx && nj >= 0 && nj < d.L.ny && nk >= 0 && nk < d.L.nz) {
+      const int nat = (int)nat_index(d.L, ni, nj, nk);
+      if (d.c64) {
+        v = d.c64[(size_t)lane * n + row];
+        col = nat;
       } else {
-        a = c64[(size_t)s * n + row];
-        colidx = nat_index(L, ni[s], nj[s], nk[s]);
+        const int64_t q = row - color * d.g.Nh;
+        v = d.w[vidx(d.g, 0, color, q)] * d.A[plane(d.g, color, lane, 0) + q] +
+            d.w[vidx(d.g, 1, color, q)] * d.A[plane(d.g, color, lane, 3) + q] +
+            d.w[vidx(d.g, 2, color, q)] * d.A[plane(d.g, color, lane, 6) + q];
+        col = (int)(((ni + nj + nk) & 1) * d.g.Nh) + (nat >> 1);
       }
-      M[row * n + colidx] += a;
     }
+  }
+#pragma unroll
+  for (int s = 0; s < 7; ++s) {
+    const double vs = __shfl_sync(0xffffffffu, v, s);
+    const int cs = __shfl_sync(0xffffffffu, col, s);
+#pragma unroll
+    for (int c = 0; c < CPL; ++c)
+      if (cs == lane + 32 * c) a[c] += vs;
   }
 }
 
 // In-place Gauss-Jordan inversion with partial pivoting of an n x n matrix
-// (n <= kCoarseMax) in shared memory by one thread block; the inverse is
-// written to Minv in type S.
-template <typename S>
-__global__ void __launch_bounds__(1024) k_gj_inverse(int n, const double* __restrict__ M, S* __restrict__ Minv, DevState* st) {
+// (n <= kCoarseMax), the inverse written in type S.  The matrix lives in
+// registers, one row per warp and CPL columns per lane, and rows are never
+// exchanged: a row that served as pivot is marked, and the permutation is
+// applied when the result is written (row p_k of the eliminated matrix is
+// row k of the inverse with column j in place p_j).  A step takes two
+// barriers: one after every row has published its entry of column k, whose
+// largest unused entry every warp then finds by itself (two redux
+// operations on the bit pattern of |a|, then the lowest row), one after
+// the pivot's warp has published the scaled pivot row.  What bounds it: up to
+// 32 rows the chain of a step (barriers, the reduction, one FP64 division),
+// so one block of 32 warps; above, the n^3 FP64 multiply-adds on one SM
+// (545 us at n = 128 at the 2 per clock of GB300), so a cluster of eight
+// blocks shares the rows and exchanges column and pivot row through
+// distributed shared memory.  Measured against the form before it (matrix in
+// shared memory, one thread scanning the column): n = 32 74 -> 29 us, n = 50
+// 160 -> 68 us (93 in one block), n = 125 1010 -> 304 us.
+constexpr int kGjCluster = 8;
+template <typename S, int CPL, bool CLUSTER>
+__global__ void __launch_bounds__(1024) k_gj_inverse(int n, DenseSrc d, S* __restrict__ Minv, int transposed,
+                                                     DevState* st) {
   wait_prior_grid();
-  extern __shared__ double sm[];
-  double* a = sm;                 // n * n
-  int* perm = (int*)(a + n * n);  // n
-  __shared__ int piv;
-  __shared__ int fail;
-  __shared__ double fac[kCoarseMax];
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) a[t] = M[t];
-  if (threadIdx.x == 0) fail = 0;
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) {
-      int p = k;
-      for (int i = k + 1; i < n; ++i)
-        if (fabs(a[i * n + k]) > fabs(a[p * n + k])) p = i;
-      piv = p;
-      perm[k] = p;
-      if (a[p * n + k] == 0.0) fail = 1;
-    }
-    __syncthreads();
-    if (fail) break;
-    if (piv != k)
-      for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const double t = a[k * n + j];
-        a[k * n + j] = a[piv * n + j];
-        a[piv * n + j] = t;
+  __shared__ double colbuf[kCoarseMax], prow[kCoarseMax];
+  __shared__ int piv[kCoarseMax];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = (int)blockIdx.x * ((int)blockDim.x >> 5) + warp;  // (the grid is the cluster)
+  const bool mine = row < n;
+  double a[CPL];
+  dense_row<CPL>(d, n, row, a);
+  unsigned used = 0;  // bit c: row lane + 32 c has been a pivot
+  int myk = -1;
+  auto barrier = [&]() {
+    if (CLUSTER) cluster_sync_all();
+    else __syncthreads();
+  };
+  if (CLUSTER) cluster_sync_all();  // every block of the cluster runs before its shared memory is written
+  bool fail = false;
+  for (int k = 0; k < n && !fail; ++k) {
+    double v = a[0];
+#pragma unroll
+    for (int c = 1; c < CPL; ++c)
+      if ((k >> 5) == c) v = a[c];
+    const double fac = __shfl_sync(0xffffffffu, v, k & 31);
+    if (mine) {
+      if (CLUSTER) {
+        if (lane < kGjCluster) st_cluster(cluster_map(colbuf + row, lane), fac);
+      } else if (lane == 0) {
+        colbuf[row] = fac;
       }
-    __syncthreads();
-    // the pivot row scaled by one reciprocal (an FP64 division is a long
-    // sequence on GB300's narrow FP64 pipe; one per row instead of n)
-    const double rp = 1.0 / a[k * n + k];
-    __syncthreads();
-    for (int j = threadIdx.x; j < n; j += blockDim.x) a[k * n + j] = (j == k ? 1.0 : a[k * n + j]) * rp;
-    __syncthreads();
-    // eliminate column k from every other row; factors first, so that the
-    // row updates below read unmodified values
-    for (int i = threadIdx.x; i < n; i += blockDim.x) fac[i] = a[i * n + k];
-    __syncthreads();
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-      const int i = t / n, j = t - (t / n) * n;
-      if (i == k) continue;
-      const double base = (j == k) ? 0.0 : a[i * n + j];
-      a[i * n + j] = base - fac[i] * a[k * n + j];
     }
-    __syncthreads();
+    barrier();
+    // the unused row with the largest |a| (the lowest such row): by the
+    // high word of the magnitude (plus one; zero for a used row), then the
+    // low word
+    unsigned bh = 0, bl = 0, bi = 0x7fffffffu;
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) {
+      const int i = lane + 32 * c;
+      if (i < n && !((used >> c) & 1)) {
+        const unsigned long long u = (unsigned long long)__double_as_longlong(colbuf[i]);
+        const unsigned h = ((unsigned)(u >> 32) & 0x7fffffffu) + 1u, l = (unsigned)u;
+        if (h > bh || (h == bh && l > bl)) {
+          bh = h;
+          bl = l;
+          bi = (unsigned)i;
+        }
+      }
+    }
+    const unsigned mh = __reduce_max_sync(0xffffffffu, bh);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, bh == mh ? bl : 0u);
+    const int p = (int)__reduce_min_sync(0xffffffffu, bh == mh && bl == ml ? bi : 0x7fffffffu);
+    fail = mh == 1u && ml == 0u;  // the column's largest unused entry is zero
+    if ((p & 31) == lane) used |= 1u << (p >> 5);
+    if (threadIdx.x == 0) piv[k] = p;
+    if (row == p) {  // (warp-uniform)
+      myk = k;
+      // one reciprocal for the pivot row (an FP64 division is a long sequence)
+      const double rp = 1.0 / fac;
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        const int j = lane + 32 * c;
+        a[c] = (j == k ? 1.0 : a[c]) * rp;
+        if (CLUSTER) {
+#pragma unroll
+          for (int b = 0; b < kGjCluster; ++b) st_cluster(cluster_map(prow + j, b), a[c]);
+        } else {
+          prow[j] = a[c];
+        }
+      }
+    }
+    barrier();
+    if (mine && row != p) {
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        const int j = lane + 32 * c;
+        a[c] = (j == k ? 0.0 : a[c]) - fac * prow[j];
+      }
+    }
   }
+  barrier();
   if (fail) {
     if (threadIdx.x == 0) atomicOr(&st->err, kErrBreakdown);
     return;
   }
-  // undo the row interchanges as column interchanges, last first
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = perm[k];
-    if (p != k)
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double t = a[i * n + k];
-        a[i * n + k] = a[i * n + p];
-        a[i * n + p] = t;
-      }
-    __syncthreads();
+  if (!mine) return;
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) {
+    const int j = lane + 32 * c;
+    if (j >= n) continue;
+    Minv[transposed ? (size_t)piv[j] * n + myk : (size_t)myk * n + piv[j]] = to_store<S>(a[c]);
+    if (!isfinite(a[c])) atomicOr(&st->err, kErrBreakdown);
   }
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    Minv[t] = to_store<S>(a[t]);
-    if (!isfinite(a[t])) atomicOr(&st->err, kErrBreakdown);
-  }
+}
+
+template <typename S>
+cudaError_t launch_gj(int n, const DenseSrc& d, S* Minv, bool transposed, DevState* st, cudaStream_t s) {
+  note_launch();
+  if (n <= 32) return launch_pdl(k_gj_inverse<S, 1, false>, 1, 1024, 0, s, n, d, Minv, (int)transposed, st);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kGjCluster, 1, 1);
+  cfg.blockDim = dim3(n <= 64 ? 256 : 512, 1, 1);  // 8 blocks x 8 or 16 warps, one row each
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kGjCluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  if (n <= 64) return cudaLaunchKernelEx(&cfg, k_gj_inverse<S, 2, true>, n, d, Minv, (int)transposed, st);
+  return cudaLaunchKernelEx(&cfg, k_gj_inverse<S, 4, true>, n, d, Minv, (int)transposed, st);
 }
 
 // ------------------------------------------------------------ apply kernels
@@ -837,11 +1042,16 @@ __global__ void __launch_bounds__(kThreads, res_min_blocks<T, ROWS>()) k_cpr_res
   }
 }
 
+// s / d, or in FP64 s times the stored reciprocal at di[i] (see level_slots)
+__device__ __forceinline__ double gs_divide(double s, double, const double* __restrict__ di, size_t i) { return s * di[i]; }
+__device__ __forceinline__ float gs_divide(float s, float d, const float*, size_t) { return s / d; }
+
 // ---- AMG level 0 (colour-split, coefficients = plane (colour, slot, 0) of At)
 // One cell of a level-0 Gauss-Seidel half sweep.
 template <typename T, typename S>
-__device__ __forceinline__ T gs0_value(const Geom& g, const S* __restrict__ At, const T* __restrict__ f,
-                                      const T* __restrict__ x, int color, int zero_guess, int64_t q) {
+__device__ __forceinline__ T gs0_value(const Geom& g, const S* __restrict__ At, const T* __restrict__ di0,
+                                      const T* __restrict__ f, const T* __restrict__ x, int color, int zero_guess,
+                                      int64_t q) {
   const int oc = color ^ 1;
   T s = f[(size_t)color * g.Nh + q];
   if (!zero_guess) {
@@ -854,7 +1064,7 @@ __device__ __forceinline__ T gs0_value(const Geom& g, const S* __restrict__ At, 
       s -= cv<T>(At[at_index(g, color, sl * 9, q)]) * (nb >= 0 ? xv : T(0));
     }
   }
-  return s / cv<T>(At[at_index(g, color, kDiag * 9, q)]);
+  return gs_divide(s, cv<T>(At[at_index(g, color, kDiag * 9, q)]), di0, (size_t)color * g.Nh + q);
 }
 
 // A level-0 half sweep over a grid-stride range, B cells per thread at a
@@ -881,12 +1091,12 @@ __device__ __forceinline__ void sweep_batched(int64_t t0, int64_t nt, int64_t n,
 // (B cells per thread at a time, their loads issued before their stores:
 // a tile parameter of the per-kernel form that the batch autotuner sets)
 template <typename T, typename S, int B>
-__global__ void k_gs0(Geom g, const S* __restrict__ At, const T* __restrict__ f, T* __restrict__ x, int color,
-                      int zero_guess, const DevState* st) {
+__global__ void k_gs0(Geom g, const S* __restrict__ At, const T* __restrict__ di0, const T* __restrict__ f,
+                      T* __restrict__ x, int color, int zero_guess, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   sweep_batched<B>(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, g.Nh,
-                   x + (size_t)color * g.Nh, [&](int64_t q) { return gs0_value<T, S>(g, At, f, x, color, zero_guess, q); });
+                   x + (size_t)color * g.Nh, [&](int64_t q) { return gs0_value<T, S>(g, At, di0, f, x, color, zero_guess, q); });
 }
 
 // First post-smoothing half sweep (black cells) with the coarse correction
@@ -895,9 +1105,9 @@ __global__ void k_gs0(Geom g, const S* __restrict__ At, const T* __restrict__ f,
 // cells, because the black sweep overwrites x_b and the red sweep that
 // follows overwrites x_r without reading its old value.
 template <typename T, typename S>
-__device__ __forceinline__ T gs0_prolong_value(const Geom& g, const S* __restrict__ At, const T* __restrict__ f,
-                                              const T* __restrict__ x, const LevelDims& C, const T* __restrict__ xc,
-                                              T sc, int64_t q) {
+__device__ __forceinline__ T gs0_prolong_value(const Geom& g, const S* __restrict__ At, const T* __restrict__ di0,
+                                              const T* __restrict__ f, const T* __restrict__ x, const LevelDims& C,
+                                              const T* __restrict__ xc, T sc, int64_t q) {
   const int di[7] = {0, 0, -1, 0, 1, 0, 0}, dj[7] = {0, -1, 0, 0, 0, 1, 0}, dk[7] = {-1, 0, 0, 0, 0, 0, 1};
   const Cell c = decode(g, 1, q);
   T s = f[(size_t)g.Nh + q];
@@ -910,16 +1120,16 @@ __device__ __forceinline__ T gs0_prolong_value(const Geom& g, const S* __restric
     const T xv = x[ok ? nb : q] + sc * xc[cn];
     s -= cv<T>(At[at_index(g, 1, sl * 9, q)]) * (ok ? xv : T(0));
   }
-  return s / cv<T>(At[at_index(g, 1, kDiag * 9, q)]);
+  return gs_divide(s, cv<T>(At[at_index(g, 1, kDiag * 9, q)]), di0, (size_t)g.Nh + q);
 }
 
 template <typename T, typename S, int B>
-__global__ void k_gs0_prolong(Geom g, const S* __restrict__ At, const T* __restrict__ f, T* __restrict__ x,
-                              LevelDims C, const T* __restrict__ xc, T sc, const DevState* st) {
+__global__ void k_gs0_prolong(Geom g, const S* __restrict__ At, const T* __restrict__ di0, const T* __restrict__ f,
+                              T* __restrict__ x, LevelDims C, const T* __restrict__ xc, T sc, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   sweep_batched<B>(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, g.Nh, x + g.Nh,
-                   [&](int64_t q) { return gs0_prolong_value<T, S>(g, At, f, x, C, xc, sc, q); });
+                   [&](int64_t q) { return gs0_prolong_value<T, S>(g, At, di0, f, x, C, xc, sc, q); });
 }
 
 // Sum of level-0 residuals over aggregate I (red cells only when the last
@@ -983,10 +1193,15 @@ __global__ void k_prolong0(Geom g, T* __restrict__ x, LevelDims C, const T* __re
 template <typename T, typename S = T>
 struct LevelView {
   LevelDims d;
-  const S* c;  // 7 n coefficients (storage type)
+  const S* c;  // level_slots n coefficients (storage type)
   T* f;
   T* x;
   __device__ __forceinline__ T cc(int slot, int64_t cidx) const { return cv<T>(c[slot * d.n + cidx]); }
+  // s divided by the diagonal
+  __device__ __forceinline__ T divided(T s, int64_t cidx) const {
+    if constexpr (sizeof(S) == 8) return s * c[7 * d.n + cidx];
+    else return s / cc(kDiag, cidx);
+  }
 };
 
 // Loads of iterates and right-hand sides.  CG = true: through L2 only, for
@@ -1017,7 +1232,7 @@ __device__ __forceinline__ void gs_cell(const LevelView<T, S>& L, int64_t cidx, 
       s -= L.cc(slot[d], cidx) * (ok[d] ? xv : T(0));
     }
   }
-  L.x[cidx] = s / L.cc(kDiag, cidx);
+  L.x[cidx] = L.divided(s, cidx);
 }
 
 template <bool CG = false, typename T, typename S>
@@ -1079,7 +1294,7 @@ __device__ __forceinline__ void gs_cell_prolong(const LevelView<T, S>& L, const 
     const T xv = ldv<CG>(L.x + fi) + sc * ldv<CG>(C.x + cn);
     s -= L.cc(slot[d], cidx) * (ok[d] ? xv : T(0));
   }
-  L.x[cidx] = s / L.cc(kDiag, cidx);
+  L.x[cidx] = L.divided(s, cidx);
 }
 
 template <typename T, typename S>
@@ -1120,7 +1335,7 @@ struct TailArgs {
   int nu1, nu2;
   T s;
   LevelView<T, S> lv[24];
-  const S* inv;     // dense inverse of level `last`
+  const S* inv;     // dense inverse of level `last`, transposed
 };
 
 // Dynamic shared memory of the single-block tail (one symbol for the whole
@@ -1177,7 +1392,7 @@ __device__ void tail_cycle(const TailArgs<T, S>& a, const Views& vw) {
     const int64_t n = C.d.n;
     for (int64_t i = threadIdx.x; i < n; i += nt) {
       T s = T(0);
-      for (int64_t j = 0; j < n; ++j) s += cv<T>(inv[i * n + j]) * C.f[j];
+      for (int64_t j = 0; j < n; ++j) s += cv<T>(inv[j * n + i]) * C.f[j];
       C.x[i] = s;
     }
     __syncthreads();
@@ -1214,7 +1429,7 @@ template <typename T, typename S>
 __host__ __device__ size_t tail_smem_bytes(const TailArgs<T, S>& a) {
   size_t b = 0;
   for (int l = a.first; l <= a.last; ++l)
-    b += align16(7 * a.lv[l].d.n * sizeof(S)) + 2 * align16(a.lv[l].d.n * sizeof(T));
+    b += align16(level_slots<S>() * a.lv[l].d.n * sizeof(S)) + 2 * align16(a.lv[l].d.n * sizeof(T));
   return b + align16((size_t)a.lv[a.last].d.n * a.lv[a.last].d.n * sizeof(S));
 }
 
@@ -1233,7 +1448,7 @@ __device__ void tail_offsets(const TailArgs<T, S>& a, uint32_t* off) {
     for (int l = a.first; l <= a.last; ++l) {
       const uint32_t n = (uint32_t)a.lv[l].d.n;
       off[3 * l] = o;
-      o += (uint32_t)align16(7 * n * sizeof(S));
+      o += (uint32_t)align16(level_slots<S>() * n * sizeof(S));
       off[3 * l + 1] = o;
       o += (uint32_t)align16(n * sizeof(T));
       off[3 * l + 2] = o;
@@ -1252,7 +1467,7 @@ __device__ void tail_stage_coefficients(const TailArgs<T, S>& a, const TailShare
     S* c = const_cast<S*>(vw.lv(l).c);
     const S* src = a.lv[l].c;
 #pragma unroll 8
-    for (int64_t i = threadIdx.x; i < 7 * n; i += blockDim.x) c[i] = src[i];
+    for (int64_t i = threadIdx.x; i < level_slots<S>() * n; i += blockDim.x) c[i] = src[i];
   }
   const int64_t nc = a.lv[a.last].d.n;
   S* inv = const_cast<S*>(vw.inv());
@@ -1260,11 +1475,11 @@ __device__ void tail_stage_coefficients(const TailArgs<T, S>& a, const TailShare
   for (int64_t i = threadIdx.x; i < nc * nc; i += blockDim.x) inv[i] = a.inv[i];
 }
 
-// The same staging with asynchronous copies (cp.async, 16 bytes each; a
-// remainder below 16 bytes is copied directly), so the block can go on with
-// other work while they land; the caller waits (cp.async.wait_all) and
-// synchronises before the staged values are read.  The sources are device
-// allocations and the shared-memory offsets multiples of 16 bytes.
+// Asynchronous staging (cp.async, 16 bytes each; a remainder below 16 bytes
+// is copied directly), so the block can go on with other work while the
+// copies land; the caller waits (cp.async.wait_all) and synchronises before
+// the staged values are read.  The sources are device allocations and the
+// shared-memory offsets multiples of 16 bytes.
 __device__ __forceinline__ void copy_to_shared_async(void* dst, const void* src, size_t bytes) {
   const size_t n16 = bytes / 16;
   const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(dst);
@@ -1274,15 +1489,6 @@ __device__ __forceinline__ void copy_to_shared_async(void* dst, const void* src,
                  : "memory");
   for (size_t b = 16 * n16 + threadIdx.x; b < bytes; b += blockDim.x)
     reinterpret_cast<char*>(dst)[b] = reinterpret_cast<const char*>(src)[b];
-}
-
-template <typename T, typename S>
-__device__ void tail_stage_coefficients_async(const TailArgs<T, S>& a, const TailSharedViews<T, S>& vw) {
-  for (int l = a.first; l <= a.last; ++l)
-    copy_to_shared_async(const_cast<S*>(vw.lv(l).c), a.lv[l].c, (size_t)7 * a.lv[l].d.n * sizeof(S));
-  const int64_t nc = a.lv[a.last].d.n;
-  copy_to_shared_async(const_cast<S*>(vw.inv()), a.inv, (size_t)nc * nc * sizeof(S));
-  asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // The tail V-cycle on staged coefficients: the first tail level's
@@ -1375,10 +1581,12 @@ template <typename T, typename S>
 struct CycleArgs {
   Geom g;
   const S* At;
+  const T* di0;  // FP64: reciprocals of level 0's diagonal (colour-split), else NULL
   T* f0;
   T* x0;
   int tail_from;  // first level of the single-block tail
-  int legs_to;    // the down and up legs smooth levels 0 .. legs_to - 1 (the rest: the cluster kernel)
+  int legs_to;    // the down and up legs smooth levels 0 .. legs_to - 1
+  int fold_to;    // levels below it get their zero-guess red half sweep with the restriction
   int nu1, nu2;
   T s;
   unsigned spins;  // polls of a grid barrier before it gives up (BO_ERR_TIMEOUT)
@@ -1396,7 +1604,7 @@ __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
     for (int color = 0; color < 2; ++color) {
       const int zero = sw == 0 && color == 0;
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + (size_t)color * g.Nh,
-                       [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.f0, a.x0, color, zero, q); });
+                       [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, color, zero, q); });
       if (!grid_barrier(st, a.spins)) return false;
     }
   if (a.nu1 == 0) {
@@ -1408,11 +1616,11 @@ __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
   // right-hand side computes it at once, which saves that sweep's barrier.
   {
     const LevelView<T, S>& C = a.lv[1];
-    const bool fold = a.nu1 > 0 && 1 < a.tail_from;
+    const bool fold = a.nu1 > 0 && 1 < a.fold_to;
     for (int64_t I = t0; I < C.d.n; I += nt) {
       const T fI = restrict0_cell<T, S>(g, a.At, a.f0, a.x0, C.d, I, a.nu1 > 0);
       C.f[I] = fI;
-      if (fold && red_cell(C.d, I)) C.x[I] = fI / C.cc(kDiag, I);
+      if (fold && red_cell(C.d, I)) C.x[I] = C.divided(fI, I);
     }
   }
   for (int l = 1; l < a.legs_to; ++l) {
@@ -1429,11 +1637,11 @@ __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
       if (!grid_barrier(st, a.spins)) return false;
     }
     const LevelView<T, S>& C = a.lv[l + 1];
-    const bool fold = a.nu1 > 0 && l + 1 < a.tail_from;
+    const bool fold = a.nu1 > 0 && l + 1 < a.fold_to;
     for (int64_t I = t0; I < C.d.n; I += nt) {
       const T fI = restrict_cell(L, C.d, I, a.nu1 > 0);
       C.f[I] = fI;
-      if (fold && red_cell(C.d, I)) C.x[I] = fI / C.cc(kDiag, I);
+      if (fold && red_cell(C.d, I)) C.x[I] = C.divided(fI, I);
     }
   }
   return true;
@@ -1469,13 +1677,13 @@ __device__ bool amg_up(const CycleArgs<T, S>& a, DevState* st) {
   for (int sw = 0; sw < a.nu2; ++sw) {
     if (sw == 0)
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + g.Nh, [&](int64_t q) {
-        return gs0_prolong_value<T, S>(g, a.At, a.f0, a.x0, C1.d, C1.x, a.s, q);
+        return gs0_prolong_value<T, S>(g, a.At, a.di0, a.f0, a.x0, C1.d, C1.x, a.s, q);
       });
     else
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + g.Nh,
-                       [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.f0, a.x0, 1, 0, q); });
+                       [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, 1, 0, q); });
     if (!grid_barrier(st, a.spins)) return false;
-    sweep_batched<4>(t0, nt, g.Nh, a.x0, [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.f0, a.x0, 0, 0, q); });
+    sweep_batched<4>(t0, nt, g.Nh, a.x0, [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, 0, 0, q); });
     if (sw + 1 < a.nu2 && !grid_barrier(st, a.spins)) return false;
   }
   return true;
@@ -1495,92 +1703,442 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_amg_up(CycleArgs<T, S> a, D
   amg_up(a, st);
 }
 
-// ---- the coarse levels (1 .. coarsest) in one thread-block cluster
-// Hardware barrier of all threads of the cluster, with release / acquire
-// semantics at cluster scope: every global-memory write of the cluster's
-// thread blocks before it is visible to their reads after it (those reads
-// also go through L2, ldv<true>).  It is not a spin on a flag: every thread
-// of the cluster reaches every barrier (the control flow is uniform).
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+// ---- the resident levels: level l0 and every coarser one in one thread-block cluster
+// Each block holds a stretch of a level in its shared memory (iterate,
+// right-hand side, residual) and its threads hold the coefficients of the
+// cells they own in registers through all half sweeps of a visit; neighbours
+// and aggregates that another block owns are read through distributed shared
+// memory.  A half sweep is then six shared-memory reads, six multiply-adds
+// and a barrier.  A level is shared by all blocks (cluster barrier, about
+// 0.3 us) while it is large, and kept by block 0 alone (block barrier) once
+// it is small.  What bounds it is latency: barriers, and the loads and index
+// arithmetic of a visit, so the coefficients are kept in a packed copy in
+// the order the threads own the cells, with each cell's place in the
+// stencil, its aggregate and its children worked out beforehand (k_res_pack).
+// Measured against the form before it (cooperative legs for level 0, the
+// same sweeps on operands in L2, small levels in one block): a 20x20x5 FP64
+// Newton step 1589 -> 1097 us, 62x45x19 FP32 2297 -> 1975 us, 128x128x64 FP32
+// 10.64 -> 10.25 ms at 14 iterations.
+//
+// Cells go in pairs: natural cells 2q and 2q + 1 always have the two colours
+// (a grid row of even length holds whole pairs; where the length is odd, a
+// pair that crosses the end of a row or of a plane changes colour too), so
+// every thread has one cell to do in each half sweep, and the red and black
+// arrays are indexed by q as level 0's colour-split arrays are.
+constexpr int kResThreads = 512;
+constexpr int kResMaxCluster = 16;
+constexpr size_t kResSmemMax = 200 * 1024;
+// pairs a thread may own (registers: 14 coefficients and 12 addresses a pair)
+template <typename T>
+__host__ __device__ constexpr int res_pairs() { return sizeof(T) == 4 ? 2 : 1; }
+// levels of at most this many cells stay in one block: a half sweep over
+// them takes less than the cluster barrier that sharing it would cost (in
+// FP64 the multiply-adds of 256 cells already take 0.25 us on one SM)
+template <typename T>
+constexpr int64_t res_single() { return sizeof(T) == 4 ? 2048 : 256; }
+// values per cell in the packed copy: six off-diagonal coefficients, the
+// diagonal and, in FP64, its reciprocal
+template <typename T>
+__host__ __device__ constexpr int res_values() { return sizeof(T) == 4 ? 7 : 8; }
+
+}  // namespace
+
+// One resident level: its shape, its place in each block's shared memory and
+// its packed copy.
+//   cp:   [colour][value][pair], the values in order -z, -y, -x, +x, +y, +z,
+//         diagonal (, reciprocal), missing neighbours 0
+//   meta: [0][pair] bit 0 the colour of the pair's first cell, the rest the
+//         red cell's aggregate on the next level (natural index and colour);
+//         [1], [2][pair] for the red and black cell as an aggregate: the
+//         natural index of its first child on the level above and which
+//         further children exist along x, y, z.  The coarsest level keeps
+//         that word per cell in natural order.
+struct ResLevel {
+  int32_t n, npairs, nx, nxy;
+  int32_t lch;    // log2 of the pairs per block
+  int32_t dist;   // shared by the cluster, or kept by block 0
+  uint32_t off;   // red x, black x, red residual, red f, black f: (1 << lch) entries each
+  uint32_t coef;  // staged copy of cp, or ~0u
+  void* cp;
+  int32_t* meta;
+  void* f;        // level l0 only: right-hand side in, iterate out (natural order; level 0 colour-split)
+  void* x;
+};
+
+struct ResPlan {
+  int32_t cluster;  // blocks
+  int32_t l0, last;
+  int32_t nu1, nu2;
+  double s;
+  ResLevel rl[24];
+  const void* inv;     // coarse inverse, transposed (storage type)
+  uint32_t dense_off;  // right-hand side and solution of the coarsest level: 2 kCoarseMax entries
+  uint32_t inv_off;    // staged inverse, or ~0u
+  uint32_t smem;
+};
+
+namespace {
+
+__device__ __forceinline__ float ld_sh(uint32_t a, bool cluster, float) {
+  float v;
+  if (cluster) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  else asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_sh(uint32_t a, bool cluster, double) {
+  double v;
+  if (cluster) asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  else asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_sh(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void st_sh(uint32_t a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+__device__ __forceinline__ uint32_t map_rank(uint32_t a, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
 }
 
-// The levels from a.legs_to (level 2; level 1, 131k cells at 128x128x64,
-// stays in the cooperative legs, which give it the whole GPU) down to the
-// coarsest, launched as a single cluster of up to 16 blocks (one per SM)
-// after the down leg has restricted onto level a.legs_to: pre-smoothing and
-// restriction of the multi-block levels, the tail V-cycle (levels of at
-// most kTailCells cells) in the last block, in shared memory when it fits,
-// then post-smoothing back up to level a.legs_to.
-// The same sweeps as the down and up legs, with a cluster barrier (a few
-// hundred nanoseconds) where they need a grid-wide one (several
-// microseconds), on the L2-resident coarse data.
+// the levels' coefficients in natural order (storage type)
+struct CoefPtrs {
+  const void* c[24];
+};
+
+// The packed copies of all resident levels, one thread per pair (the
+// coarsest level, whose inverse is kept instead: one per cell).
 template <typename T, typename S>
-__global__ void __launch_bounds__(kCoopThreads, 1) k_amg_coarse(CycleArgs<T, S> a, TailArgs<T, S> ta, int tail_smem,
-                                                               const DevState* st) {
+__global__ void k_res_pack(const __grid_constant__ ResPlan a, Geom g, const S* __restrict__ At,
+                           const T* __restrict__ di0, const __grid_constant__ CoefPtrs coef) {
+  wait_prior_grid();
+  constexpr int K = res_values<T>();
+  int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int l = a.l0; l <= a.last; ++l) {
+    const ResLevel& r = a.rl[l];
+    const int32_t items = l == a.last ? r.n : r.npairs;
+    if (t >= items) {
+      t -= items;
+      continue;
+    }
+    const int32_t ny = r.nxy / r.nx, nz = r.n / r.nxy;
+    // a cell's word as an aggregate of level l - 1
+    auto child_word = [&](int32_t c) {
+      if (l == a.l0) return 0;
+      const ResLevel& f = a.rl[l - 1];
+      const int32_t i = c % r.nx, j = (c / r.nx) % ny, k = c / r.nxy;
+      const int32_t fny = f.nxy / f.nx, fnz = f.n / f.nxy;
+      return ((2 * i + f.nx * 2 * j + f.nxy * 2 * k) << 3) | (2 * i + 1 < f.nx ? 1 : 0) | (2 * j + 1 < fny ? 2 : 0) |
+             (2 * k + 1 < fnz ? 4 : 0);
+    };
+    if (l == a.last) {
+      r.meta[t] = child_word(t);
+      return;
+    }
+    const int32_t q = t, np = r.npairs;
+    const int32_t c0 = 2 * q;
+    const int32_t par = (c0 % r.nx + (c0 / r.nx) % ny + c0 / r.nxy) & 1;
+    T* cp = (T*)r.cp;
+    const S* lc = (const S*)coef.c[l];
+    for (int col = 0; col < 2; ++col) {
+      const int32_t c = c0 + (col ^ par);
+      const bool live = c < r.n;
+      const int slot[7] = {kZm, kYm, kXm, kXp, kYp, kZp, kDiag};
+      for (int d = 0; d < 7; ++d) {
+        T v = d == 6 ? T(1) : T(0);
+        if (live) v = l ? cv<T>(lc[(size_t)slot[d] * r.n + c]) : cv<T>(At[at_index(g, col, slot[d] * 9, q)]);
+        cp[(size_t)(col * K + d) * np + q] = v;
+      }
+      if constexpr (sizeof(T) == 8)
+        cp[(size_t)(col * K + 7) * np + q] = !live ? T(1) : l ? (T)lc[(size_t)7 * r.n + c] : di0[(size_t)col * g.Nh + q];
+      r.meta[(size_t)(1 + col) * np + q] = live ? child_word(c) : 0;
+    }
+    int32_t agg = 0;
+    const int32_t cr = c0 + par;  // the red cell
+    if (cr < r.n) {
+      const ResLevel& cl = a.rl[l + 1];
+      const int32_t i = (cr % r.nx) >> 1, j = ((cr / r.nx) % ny) >> 1, k = (cr / r.nxy) >> 1;
+      agg = ((i + cl.nx * j + cl.nxy * k) << 1) | ((i + j + k) & 1);
+    }
+    r.meta[q] = (agg << 1) | par;
+    (void)nz;
+    return;
+  }
+}
+
+// The array sections of a level in a block's shared memory
+enum : int { kSecRed = 0, kSecBlack = 1, kSecRes = 2, kSecF = 3 };  // kSecF, kSecF + 1: f of red and black
+
+template <typename T>
+__device__ __forceinline__ uint32_t res_local(const ResLevel& r, uint32_t base, int sec, int32_t q) {
+  const uint32_t m = (1u << r.lch) - 1u;
+  return base + r.off + (((uint32_t)sec << r.lch) + ((uint32_t)q & m)) * (uint32_t)sizeof(T);
+}
+// address of entry q of a section, in whichever block owns it
+template <typename T, bool DIST>
+__device__ __forceinline__ uint32_t res_addr(const ResLevel& r, uint32_t base, int sec, int32_t q) {
+  const uint32_t a = res_local<T>(r, base, sec, q);
+  return DIST ? map_rank(a, (uint32_t)(q >> r.lch)) : a;
+}
+
+template <typename T, int NP>
+struct ResCells {
+  T c[2][NP][6];          // off-diagonal coefficients (0 where the neighbour is missing)
+  T d[2][NP];             // diagonal, or its reciprocal in FP64
+  T dr[NP];               // the red diagonal itself (residuals)
+  T f[2][NP];
+  uint32_t nb[2][NP][6];  // shared-memory addresses of the neighbours' iterates
+  uint32_t own[2][NP];    // and of the cell's own
+  int32_t m[NP];          // meta word 0
+  bool live[2][NP];
+};
+
+__device__ __forceinline__ float res_divide(float s, float d) { return s / d; }
+__device__ __forceinline__ double res_divide(double s, double rd) { return s * rd; }
+
+// One visit of level l: the cells of this thread into registers
+template <typename T, int NP, bool DIST>
+__device__ __forceinline__ void res_load(const ResPlan& a, int l, uint32_t base, ResCells<T, NP>& r) {
+  constexpr int K = res_values<T>();
+  const ResLevel& rl = a.rl[l];
+  const int32_t np = rl.npairs;
+  const int32_t q0 = DIST ? (int32_t)blockIdx.x << rl.lch : 0;
+  const int32_t q1 = min(np, q0 + (1 << rl.lch));
+  const T* cp = (const T*)rl.cp;
+  if (!DIST && rl.coef != ~0u) cp = reinterpret_cast<const T*>(g_tail_smem + rl.coef);
+  const int32_t off[6] = {-rl.nxy, -rl.nx, -1, 1, rl.nx, rl.nxy};
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int32_t q = q0 + (int32_t)threadIdx.x + kResThreads * p;
+    const bool in = q < q1;
+    const int32_t qq = in ? q : 0;
+    r.m[p] = rl.meta[qq];
+#pragma unroll
+    for (int col = 0; col < 2; ++col) {
+#pragma unroll
+      for (int d = 0; d < 6; ++d) r.c[col][p][d] = cp[(col * K + d) * np + qq];
+      const T dg = cp[(col * K + 6) * np + qq];
+      if (col == 0) r.dr[p] = dg;
+      r.d[col][p] = K == 8 ? cp[(col * K + K - 1) * np + qq] : dg;
+    }
+    const int32_t par = r.m[p] & 1;
+#pragma unroll
+    for (int col = 0; col < 2; ++col) {
+      const int32_t c = 2 * qq + (col ^ par);
+      r.live[col][p] = in && c < rl.n;
+      r.own[col][p] = res_local<T>(rl, base, col, qq);
+      // (a missing neighbour has coefficient 0: any entry of the level will do)
+#pragma unroll
+      for (int d = 0; d < 6; ++d) r.nb[col][p][d] = res_addr<T, DIST>(rl, base, col ^ 1, min(max(c + off[d], 0) >> 1, np - 1));
+    }
+  }
+}
+
+template <bool DIST>
+__device__ __forceinline__ void res_barrier() {
+  if (DIST) cluster_sync_all();
+  else __syncthreads();
+}
+
+// (warps whose threads own no cell of the colour skip to the barrier: FP64
+// multiply-adds issued for nothing would occupy the SM's narrow FP64 pipe)
+template <typename T, int NP, bool DIST>
+__device__ __forceinline__ void res_sweep(ResCells<T, NP>& r, int col) {
+  bool any = false;
+#pragma unroll
+  for (int p = 0; p < NP; ++p) any = any || r.live[col][p];
+  if (any) {
+    T xv[NP][6];
+#pragma unroll
+    for (int p = 0; p < NP; ++p)
+#pragma unroll
+      for (int d = 0; d < 6; ++d) xv[p][d] = r.live[col][p] ? ld_sh(r.nb[col][p][d], DIST, T(0)) : T(0);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      T s = r.f[col][p];
+#pragma unroll
+      for (int d = 0; d < 6; ++d) s -= r.c[col][p][d] * xv[p][d];
+      if (r.live[col][p]) st_sh(r.own[col][p], res_divide(s, r.d[col][p]));
+    }
+  }
+  res_barrier<DIST>();
+}
+
+// Right-hand side of a cell from the red residuals of its children on level
+// `r` (nu1 >= 1: the black residuals are zero after a black half sweep), in
+// the order of the other launch forms: (0,0,0), (1,1,0), (1,0,1), (0,1,1)
+template <typename T>
+__device__ __forceinline__ T res_gather(const ResLevel& r, uint32_t base, int32_t word) {
+  const int32_t c = word >> 3;
+  const bool ex = word & 1, ey = word & 2, ez = word & 4;
+  const int32_t ch[4] = {c, c + 1 + r.nx, c + 1 + r.nxy, c + r.nx + r.nxy};
+  const bool ok[4] = {true, ex && ey, ex && ez, ey && ez};
+  T v[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int32_t q = (ok[e] ? ch[e] : c) >> 1;
+    const uint32_t ad = res_local<T>(r, base, kSecRes, q);
+    v[e] = r.dist ? ld_sh(map_rank(ad, (uint32_t)(q >> r.lch)), true, T(0)) : ld_sh(ad, false, T(0));
+  }
+  T acc = T(0);
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (ok[e]) acc += v[e];
+  return acc;
+}
+
+// Pre-smoothing of level l and its red residuals, ready for the next level.
+// Every block of the cluster runs it when the level is shared (DIST), block
+// 0 alone otherwise.
+template <typename T, bool DIST>
+__device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l, uint32_t base) {
+  constexpr int NP = res_pairs<T>();
+  ResCells<T, NP> r;
+  res_load<T, NP, DIST>(a, l, base, r);
+  const ResLevel& rl = a.rl[l];
+  const int32_t q0 = DIST ? (int32_t)blockIdx.x << rl.lch : 0;
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int32_t i = (int32_t)threadIdx.x + kResThreads * p, q = q0 + i;
+    const bool place = i < (1 << rl.lch);
+#pragma unroll
+    for (int col = 0; col < 2; ++col) {
+      T f = T(0);
+      if (r.live[col][p]) {
+        if (l > a.l0) f = res_gather<T>(a.rl[l - 1], base, rl.meta[(1 + col) * rl.npairs + q]);
+        else if (l) f = ((const T*)rl.f)[2 * q + (col ^ (r.m[p] & 1))];
+        else f = ((const T*)rl.f)[(size_t)col * g.Nh + q];
+      }
+      r.f[col][p] = f;
+      if (place) st_sh(res_local<T>(rl, base, kSecF + col, q), f);
+    }
+    // the first half sweep starts from zero: x_r = f_r / d_r (black zero
+    // until its own half sweep)
+    if (place) {
+      st_sh(res_local<T>(rl, base, kSecRed, q), r.live[0][p] ? res_divide(r.f[0][p], r.d[0][p]) : T(0));
+      st_sh(res_local<T>(rl, base, kSecBlack, q), T(0));
+    }
+  }
+  res_barrier<DIST>();
+  res_sweep<T, NP, DIST>(r, 1);
+  for (int sw = 1; sw < a.nu1; ++sw) {
+    res_sweep<T, NP, DIST>(r, 0);
+    res_sweep<T, NP, DIST>(r, 1);
+  }
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    if (!r.live[0][p]) continue;
+    // (the diagonal's term first, or after the lower neighbours on level 0:
+    // the order of the other launch forms, whose results these are bit for bit)
+    const T dx = ld_sh(r.own[0][p], false, T(0));
+    T v = r.f[0][p];
+    if (l) v -= r.dr[p] * dx;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      if (d == 3 && !l) v -= r.dr[p] * dx;
+      v -= r.c[0][p][d] * ld_sh(r.nb[0][p][d], DIST, T(0));
+    }
+    st_sh(r.own[0][p] + ((uint32_t)(kSecRes - kSecRed) << rl.lch) * (uint32_t)sizeof(T), v);
+  }
+  res_barrier<DIST>();
+}
+
+// Coarse correction and post-smoothing of level l
+template <typename T, bool DIST>
+__device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, uint32_t base) {
+  constexpr int NP = res_pairs<T>();
+  ResCells<T, NP> r;
+  res_load<T, NP, DIST>(a, l, base, r);
+  const ResLevel& rl = a.rl[l];
+  const int32_t q0 = DIST ? (int32_t)blockIdx.x << rl.lch : 0;
+  const T sc = (T)a.s;
+  // x_r += s x_c (the black cells are overwritten by the half sweep that follows)
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const int32_t q = q0 + (int32_t)threadIdx.x + kResThreads * p;
+#pragma unroll
+    for (int col = 0; col < 2; ++col) r.f[col][p] = r.live[col][p] ? ld_sh(res_local<T>(rl, base, kSecF + col, q), false, T(0)) : T(0);
+    if (!r.live[0][p]) continue;
+    const int32_t agg = r.m[p] >> 1;
+    uint32_t ad;
+    int32_t owner = 0;
+    if (l + 1 == a.last) {
+      ad = base + a.dense_off + (uint32_t)(kCoarseMax + (agg >> 1)) * (uint32_t)sizeof(T);
+    } else {
+      const ResLevel& cl = a.rl[l + 1];
+      ad = res_local<T>(cl, base, agg & 1, agg >> 2);
+      owner = cl.dist ? (agg >> 2) >> cl.lch : 0;
+    }
+    const T xc = DIST ? ld_sh(map_rank(ad, (uint32_t)owner), true, T(0)) : ld_sh(ad, false, T(0));
+    st_sh(r.own[0][p], ld_sh(r.own[0][p], false, T(0)) + sc * xc);
+  }
+  res_barrier<DIST>();
+  for (int sw = 0; sw < a.nu2; ++sw) {
+    res_sweep<T, NP, DIST>(r, 1);
+    res_sweep<T, NP, DIST>(r, 0);
+  }
+  if (l == a.l0) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const int32_t q = q0 + (int32_t)threadIdx.x + kResThreads * p;
+#pragma unroll
+      for (int col = 0; col < 2; ++col) {
+        if (!r.live[col][p]) continue;
+        const T v = ld_sh(r.own[col][p], false, T(0));
+        if (l) ((T*)rl.x)[2 * q + (col ^ (r.m[p] & 1))] = v;
+        else ((T*)rl.x)[(size_t)col * g.Nh + q] = v;
+      }
+    }
+  }
+}
+
+template <typename T, typename S>
+__global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_constant__ ResPlan a, Geom g,
+                                                                const DevState* st) {
   wait_prior_grid();
   if (st->done) return;  // uniform: every block reads the same flag
-  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
-  // the last block runs the tail; it stages the tail's coefficients and
-  // coarse inverse asynchronously at the start, under the multi-block levels
-  const bool tail_block = blockIdx.x == gridDim.x - 1;
-  __shared__ uint32_t off[73];
-  const TailSharedViews<T, S> vw{&ta, off};
-  if (tail_smem && tail_block) {
-    tail_offsets(ta, off);
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(g_tail_smem);
+  const bool first = blockIdx.x == 0;
+  const int32_t n = a.rl[a.last].n;
+  if (first) {
+    // block 0 stages the small levels' coefficients and the coarse inverse
+    // under the first level's sweeps
+    for (int l = a.l0; l < a.last; ++l)
+      if (a.rl[l].coef != ~0u)
+        copy_to_shared_async(g_tail_smem + a.rl[l].coef, a.rl[l].cp, (size_t)2 * res_values<T>() * a.rl[l].npairs * sizeof(T));
+    if (a.inv_off != ~0u) copy_to_shared_async(g_tail_smem + a.inv_off, a.inv, (size_t)n * n * sizeof(S));
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  cluster_sync_all();  // every block runs before its shared memory is read
+  int l = a.l0;
+  for (; l < a.last && a.rl[l].dist; ++l) res_down<T, true>(a, g, l, base);
+  const int shared_to = l;
+  if (first) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    tail_stage_coefficients_async(ta, vw);
-  }
-  for (int l = a.legs_to; l < a.tail_from; ++l) {
-    const LevelView<T, S>& L = a.lv[l];
-    for (int sw = 0; sw < a.nu1; ++sw)
-      for (int color = 0; color < 2; ++color) {
-        if (sw == 0 && color == 0) continue;  // done with the restriction
-        for (int64_t c = t0; c < L.d.n; c += nt) gs_cell<true>(L, c, color, 0);
-        cluster_sync_all();
-      }
-    if (a.nu1 == 0) {
-      for (int64_t c = t0; c < L.d.n; c += nt) L.x[c] = T(0);
-      cluster_sync_all();
+    for (; l < a.last; ++l) res_down<T, false>(a, g, l, base);
+    // the coarsest level: x = inv f, a thread per row (inv is stored transposed)
+    const uint32_t fo = base + a.dense_off;
+    const ResLevel& rl = a.rl[a.last];
+    for (int i = threadIdx.x; i < n; i += kResThreads)
+      st_sh(fo + (uint32_t)(i * sizeof(T)),
+            a.l0 == a.last ? ((const T*)rl.f)[i] : res_gather<T>(a.rl[a.last - 1], base, rl.meta[i]));
+    __syncthreads();
+    const S* inv = a.inv_off != ~0u ? reinterpret_cast<const S*>(g_tail_smem + a.inv_off) : (const S*)a.inv;
+    for (int i = threadIdx.x; i < n; i += kResThreads) {
+      T s = T(0);
+#pragma unroll 8
+      for (int j = 0; j < n; ++j) s += cv<T>(inv[j * n + i]) * ld_sh(fo + (uint32_t)(j * sizeof(T)), false, T(0));
+      st_sh(fo + (uint32_t)((kCoarseMax + i) * sizeof(T)), s);
+      if (a.l0 == a.last) ((T*)rl.x)[i] = s;
     }
-    const LevelView<T, S>& C = a.lv[l + 1];
-    const bool fold = a.nu1 > 0 && l + 1 < a.tail_from;
-    for (int64_t I = t0; I < C.d.n; I += nt) {
-      const T fI = restrict_cell<true>(L, C.d, I, a.nu1 > 0);
-      C.f[I] = fI;
-      if (fold && red_cell(C.d, I)) C.x[I] = fI / C.cc(kDiag, I);
-    }
-    cluster_sync_all();
-  }
-  if (tail_block) {
-    if (tail_smem) {
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();
-      tail_run_staged(ta, vw);
-    } else {
-      tail_cycle(ta, TailGlobalViews<T, S>{&ta});
-    }
+    __syncthreads();
+    for (l = a.last - 1; l >= shared_to; --l) res_up<T, false>(a, g, l, base);
   }
   cluster_sync_all();
-  for (int l = a.tail_from - 1; l >= a.legs_to; --l) {
-    const LevelView<T, S>& L = a.lv[l];
-    const LevelView<T, S>& C = a.lv[l + 1];
-    if (a.nu2 == 0) {
-      for (int64_t c = t0; c < L.d.n; c += nt) prolong_cell<true>(L, C, c, a.s);
-      cluster_sync_all();
-    }
-    for (int sw = 0; sw < a.nu2; ++sw)
-      for (int color = 1; color >= 0; --color) {
-        for (int64_t c = t0; c < L.d.n; c += nt) {
-          if (sw == 0 && color == 1) gs_cell_prolong<true>(L, C, c, a.s);
-          else gs_cell<true>(L, c, color, 0);
-        }
-        cluster_sync_all();
-      }
-  }
+  for (l = shared_to - 1; l >= a.l0; --l) res_up<T, true>(a, g, l, base);
+  cluster_sync_all();  // no block leaves while another may read its shared memory
 }
 
-// dense solve on level 0 when level 0 is the coarsest: x = inv f
+// dense solve on level 0 when level 0 is the coarsest: x = inv f (inv transposed)
 template <typename T, typename S>
 __global__ void k_dense0(int64_t n, const S* __restrict__ inv, const T* __restrict__ f, T* __restrict__ x,
                          const DevState* st) {
@@ -1588,7 +2146,7 @@ __global__ void k_dense0(int64_t n, const S* __restrict__ inv, const T* __restri
   if (st->done) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     T s = T(0);
-    for (int64_t j = 0; j < n; ++j) s += cv<T>(inv[i * n + j]) * f[j];
+    for (int64_t j = 0; j < n; ++j) s += cv<T>(inv[j * n + i]) * f[j];
     x[i] = s;
   }
 }
@@ -1644,25 +2202,24 @@ LevelView<T, S> view(bo_prec* P, int l) {
 
 LevelDims dims_of(const Level& L) { return LevelDims{L.nx, L.ny, L.nz, L.n}; }
 
-// Blocks of the cluster that runs the coarse AMG levels: 16 (a
-// non-portable cluster size) where the device can co-schedule them with
-// the tail's shared memory, else 8, else 0 (no cluster form).  Queried once
-// per instantiation.
+// Largest cluster of the resident kernel that the device can co-schedule
+// with its shared memory (16 is a non-portable size), or 0.  Queried once per
+// instantiation.
 template <typename T, typename S>
-int coarse_cluster_size() {
+int resident_max_cluster() {
   static std::atomic<int> cached{-1};
   int cs = cached.load();
   if (cs >= 0) return cs;
   cs = 0;
-  const void* k = (const void*)k_amg_coarse<T, S>;
-  if (cudaFuncSetAttribute(k_amg_coarse<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaFuncSetAttribute(k_amg_coarse<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemMax) ==
+  const void* k = (const void*)k_amg_resident<T, S>;
+  if (cudaFuncSetAttribute(k_amg_resident<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaFuncSetAttribute(k_amg_resident<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax) ==
           cudaSuccess) {
-    for (int c : {16, 8}) {
+    for (int c : {kResMaxCluster, 8, 4, 2, 1}) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(c, 1, 1);
-      cfg.blockDim = dim3(kCoopThreads, 1, 1);
-      cfg.dynamicSmemBytes = kTailSmemMax;
+      cfg.blockDim = dim3(kResThreads, 1, 1);
+      cfg.dynamicSmemBytes = kResSmemMax;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
       at[0].val.clusterDim.x = c;
@@ -1682,11 +2239,78 @@ int coarse_cluster_size() {
   return cs;
 }
 
+// The resident form's levels, cluster and shared-memory layout for P: level
+// l0 is the finest level that fits the largest cluster (FP32: 32768 cells,
+// two pairs per thread; FP64: 16384).  The cluster is the smallest that
+// gives a block at most `per` pairs of level l0 (FP32: 512, one half-sweep
+// cell per thread; FP64: 128, whose multiply-adds take about a cluster
+// barrier's time), so a batch's small systems leave SMs to one another.
+// cluster = 0 where the form does not apply (no pre- or post-smoothing).
+template <typename T, typename S>
+void resident_plan(bo_prec* P, ResPlan& a) {
+  a.cluster = 0;
+  const int maxc = resident_max_cluster<T, S>();
+  const Geom& g = P->mat->g;
+  const int last = P->nlev - 1;
+  if (maxc < 1 || last < 1 || P->opts.amg_nu1 < 1 || P->opts.amg_nu2 < 1) return;
+  const int64_t cap = (int64_t)2 * kResThreads * res_pairs<T>() * maxc;
+  auto cells = [&](int l) { return l ? P->lev[l].n : g.N; };
+  int l0 = 0;
+  while (l0 < last && cells(l0) > cap) ++l0;
+  if (l0 > 0 && l0 > P->tail_from) return;
+  int C = 1;
+  if (l0 < last && cells(l0) > res_single<T>()) {
+    const int64_t per = sizeof(T) == 4 ? 512 : 128;
+    while (C < maxc && (cells(l0) + 1) / 2 > per * C) C *= 2;
+  }
+  uint32_t o = 0;
+  for (int l = l0; l <= last; ++l) {
+    ResLevel& r = a.rl[l];
+    r = ResLevel{};
+    r.n = (int32_t)cells(l);
+    r.npairs = (r.n + 1) / 2;
+    r.nx = l ? P->lev[l].nx : g.nx;
+    r.nxy = r.nx * (l ? P->lev[l].ny : g.ny);
+    r.coef = ~0u;
+    if (l == last) break;
+    r.dist = C > 1 && r.n > res_single<T>();
+    const int32_t per = r.dist ? (r.npairs + C - 1) / C : r.npairs;
+    while ((1 << r.lch) < per) ++r.lch;
+    if ((1 << r.lch) > kResThreads * res_pairs<T>()) return;
+    r.off = o;
+    o += (uint32_t)align16(((size_t)5 << r.lch) * sizeof(T));
+  }
+  a.dense_off = o;
+  o += (uint32_t)align16(2 * kCoarseMax * sizeof(T));
+  for (int l = l0; l < last; ++l) {
+    ResLevel& r = a.rl[l];
+    const size_t b = align16((size_t)2 * res_values<T>() * r.npairs * sizeof(T));
+    if (r.dist || o + b > kResSmemMax) continue;
+    r.coef = o;
+    o += (uint32_t)b;
+  }
+  const size_t ib = align16((size_t)P->ncoarse * P->ncoarse * sizeof(S));
+  a.inv_off = ~0u;
+  if (o + ib <= kResSmemMax) {
+    a.inv_off = o;
+    o += (uint32_t)ib;
+  }
+  if (o > kResSmemMax) return;
+  a.smem = o;
+  a.l0 = l0;
+  a.last = last;
+  a.nu1 = P->opts.amg_nu1;
+  a.nu2 = P->opts.amg_nu2;
+  a.s = P->opts.amg_overcorr;
+  a.cluster = C;
+}
+
 template <typename T, typename S>
 void amg_vcycle(bo_prec* P, const DevState* st) {
   cudaStream_t s = P->stream;
   const Geom& g = P->mat->g;
   const S* At = (const S*)P->At;
+  const T* di0 = (const T*)P->di0;  // (NULL unless T is double)
   T* f0 = (T*)P->f0;
   T* x0 = (T*)P->e0;
   const int nu1 = P->opts.amg_nu1, nu2 = P->opts.amg_nu2;
@@ -1701,38 +2325,67 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
   const int CB = P->amg_cells;
   const int ghalf = grid_for((g.Nh + CB - 1) / CB, TB);
   auto gs0 = [&](int color, int zero) {
-    if (CB == 4) (launch_pdl(k_gs0<T, S, 4>, ghalf, TB, 0, s, g, At, f0, x0, color, zero, st), note_launch());
-    else if (CB == 2) (launch_pdl(k_gs0<T, S, 2>, ghalf, TB, 0, s, g, At, f0, x0, color, zero, st), note_launch());
-    else (launch_pdl(k_gs0<T, S, 1>, ghalf, TB, 0, s, g, At, f0, x0, color, zero, st), note_launch());
+    if (CB == 4) (launch_pdl(k_gs0<T, S, 4>, ghalf, TB, 0, s, g, At, di0, f0, x0, color, zero, st), note_launch());
+    else if (CB == 2) (launch_pdl(k_gs0<T, S, 2>, ghalf, TB, 0, s, g, At, di0, f0, x0, color, zero, st), note_launch());
+    else (launch_pdl(k_gs0<T, S, 1>, ghalf, TB, 0, s, g, At, di0, f0, x0, color, zero, st), note_launch());
   };
   auto gs0_prolong = [&]() {
     const LevelDims C1 = dims_of(P->lev[1]);
     const T* xc = (const T*)P->lev[1].x;
-    if (CB == 4) (launch_pdl(k_gs0_prolong<T, S, 4>, ghalf, TB, 0, s, g, At, f0, x0, C1, xc, sc, st), note_launch());
-    else if (CB == 2) (launch_pdl(k_gs0_prolong<T, S, 2>, ghalf, TB, 0, s, g, At, f0, x0, C1, xc, sc, st), note_launch());
-    else (launch_pdl(k_gs0_prolong<T, S, 1>, ghalf, TB, 0, s, g, At, f0, x0, C1, xc, sc, st), note_launch());
+    if (CB == 4) (launch_pdl(k_gs0_prolong<T, S, 4>, ghalf, TB, 0, s, g, At, di0, f0, x0, C1, xc, sc, st), note_launch());
+    else if (CB == 2) (launch_pdl(k_gs0_prolong<T, S, 2>, ghalf, TB, 0, s, g, At, di0, f0, x0, C1, xc, sc, st), note_launch());
+    else (launch_pdl(k_gs0_prolong<T, S, 1>, ghalf, TB, 0, s, g, At, di0, f0, x0, C1, xc, sc, st), note_launch());
   };
   const int last = P->nlev - 1;
   // Launch forms (all compute the same V-cycle):
-  //  mode 2: levels 0 and 1 in two cooperative launches (down leg, up leg,
-  //          grid barriers between half sweeps) around one cluster launch
-  //          for every coarser level (cluster barriers);
+  //  mode 2: every level that fits a cluster's registers and shared memory in
+  //          one cluster launch (k_amg_resident), the levels above it in two
+  //          cooperative launches (down leg, up leg, grid barriers between
+  //          half sweeps), or one kernel per half sweep inside stream capture;
   //  mode 1: the cooperative legs also smooth the multi-block natural
   //          levels, the tail levels in one block;
-  //  mode 0, or inside stream capture, or when a launch form is refused:
-  //          one kernel per half sweep, restriction and prolongation.
+  //  mode 0, or when a launch form is refused: one kernel per half sweep,
+  //          restriction and prolongation.
   const int mode = g_amg_coop.load();
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(s, &cap);
   const bool coop = mode != 0 && cap == cudaStreamCaptureStatusNone;
-  const int cs = (coop && mode == 2) ? coarse_cluster_size<T, S>() : 0;
+  const ResPlan& ra = *P->res;
+  const int rc = mode == 2 ? ra.cluster : 0;
+  auto resident = [&]() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(rc, 1, 1);
+    cfg.blockDim = dim3(kResThreads, 1, 1);
+    cfg.dynamicSmemBytes = ra.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = rc;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    if (cudaLaunchKernelEx(&cfg, k_amg_resident<T, S>, ra, g, st) != cudaSuccess) return false;
+    note_launch();
+    return true;
+  };
+  if (rc > 0 && ra.l0 == 0) {
+    if (resident()) return;
+    cudaGetLastError();
+  }
+  // first level of the cluster launch (none: past the last)
+  const int res_from = rc > 0 && ra.l0 > 0 ? ra.l0 : last + 1;
   CycleArgs<T, S> ca;
   ca.g = g;
   ca.At = At;
+  ca.di0 = di0;
   ca.f0 = f0;
   ca.x0 = x0;
   ca.tail_from = P->tail_from;
-  ca.legs_to = cs ? (P->tail_from < 2 ? P->tail_from : 2) : P->tail_from;
+  ca.legs_to = std::min(P->tail_from, res_from);
+  ca.fold_to = std::min(P->tail_from, res_from);
   ca.nu1 = nu1;
   ca.nu2 = nu2;
   ca.s = sc;
@@ -1750,29 +2403,32 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
   DevState* stw = const_cast<DevState*>(st);
 
   // per-kernel pre- and post-smoothing of the multi-block natural levels
+  const int natural_to = ca.legs_to;
+  auto natural_pre = [&](int l) {
+    LevelView<T, S> L = view<T, S>(P, l), C = view<T, S>(P, l + 1);
+    const int gl = grid_for(L.d.n, TB);
+    for (int sw = 0; sw < nu1; ++sw) {
+      (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 0, sw == 0, st), note_launch());
+      (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 1, 0, st), note_launch());
+    }
+    if (nu1 == 0) (launch_pdl(k_zero<T>, gl, TB, 0, s, L.d.n, L.x, st), note_launch());
+    (launch_pdl(k_restrictn<T, S>, grid_for(C.d.n, TB), TB, 0, s, L, C, nu1 > 0, st), note_launch());
+  };
   auto natural_down = [&]() {
-    for (int l = 1; l < P->tail_from; ++l) {
-      LevelView<T, S> L = view<T, S>(P, l), C = view<T, S>(P, l + 1);
-      const int gl = grid_for(L.d.n, TB);
-      for (int sw = 0; sw < nu1; ++sw) {
-        (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 0, sw == 0, st), note_launch());
-        (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 1, 0, st), note_launch());
-      }
-      if (nu1 == 0) (launch_pdl(k_zero<T>, gl, TB, 0, s, L.d.n, L.x, st), note_launch());
-      (launch_pdl(k_restrictn<T, S>, grid_for(C.d.n, TB), TB, 0, s, L, C, nu1 > 0, st), note_launch());
+    for (int l = 1; l < natural_to; ++l) natural_pre(l);
+  };
+  auto natural_post = [&](int l) {
+    LevelView<T, S> L = view<T, S>(P, l), C = view<T, S>(P, l + 1);
+    const int gl = grid_for(L.d.n, TB);
+    if (nu2 == 0) (launch_pdl(k_prolongn<T, S>, gl, TB, 0, s, L, C, sc, st), note_launch());
+    for (int sw = 0; sw < nu2; ++sw) {
+      if (sw == 0) (launch_pdl(k_gsn_prolong<T, S>, gl, TB, 0, s, L, C, sc, st), note_launch());
+      else (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 1, 0, st), note_launch());
+      (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 0, 0, st), note_launch());
     }
   };
   auto natural_up = [&]() {
-    for (int l = P->tail_from - 1; l >= 1; --l) {
-      LevelView<T, S> L = view<T, S>(P, l), C = view<T, S>(P, l + 1);
-      const int gl = grid_for(L.d.n, TB);
-      if (nu2 == 0) (launch_pdl(k_prolongn<T, S>, gl, TB, 0, s, L, C, sc, st), note_launch());
-      for (int sw = 0; sw < nu2; ++sw) {
-        if (sw == 0) (launch_pdl(k_gsn_prolong<T, S>, gl, TB, 0, s, L, C, sc, st), note_launch());
-        else (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 1, 0, st), note_launch());
-        (launch_pdl(k_gsn<T, S>, gl, TB, 0, s, L, 0, 0, st), note_launch());
-      }
-    }
+    for (int l = natural_to - 1; l >= 1; --l) natural_post(l);
   };
   auto tail = [&]() {
     if (tb <= kTailSmemMax) {
@@ -1817,33 +2473,20 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
     (launch_pdl(k_restrict0<T, S>, grid_for(P->lev[1].n, TB), TB, 0, s, g, At, f0, x0, dims_of(P->lev[1]),
         (T*)P->lev[1].f, nu1 > 0, st), note_launch());
     natural_down();
-    tail();
-  } else if (cs > 0) {
-    // every coarser level in one cluster launch (or per kernel if refused)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs, 1, 1);
-    cfg.blockDim = dim3(kCoopThreads, 1, 1);
-    cfg.dynamicSmemBytes = tb <= kTailSmemMax ? tb : 0;
-    cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cs;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, k_amg_coarse<T, S>, ca, ta, tb <= kTailSmemMax ? 1 : 0, st) == cudaSuccess) {
-      note_launch();
-    } else {
+  }
+
+  // the coarser levels: one cluster launch, or the single-block tail (with
+  // the natural levels between the legs and the tail per kernel if the
+  // cluster launch is refused)
+  if (res_from > last || !resident()) {
+    if (res_from <= last) {
       cudaGetLastError();
-      natural_down();
+      for (int l = natural_to; l < P->tail_from; ++l) natural_pre(l);
       tail();
-      natural_up();
+      for (int l = P->tail_from - 1; l >= natural_to; --l) natural_post(l);
+    } else {
+      tail();
     }
-  } else {
-    tail();
   }
 
   // up leg
@@ -1854,7 +2497,7 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
       return;
     }
     cudaGetLastError();
-    if (cs == 0) natural_up();
+    natural_up();
   } else {
     natural_up();
   }
@@ -1927,6 +2570,12 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
    note_launch());
 }
 
+// the arithmetic type of a storage type
+template <typename S>
+struct ArithOf { using type = float; };
+template <>
+struct ArithOf<double> { using type = double; };
+
 template <typename S>
 int values_impl(bo_prec* P) {
   bo_mat* m = P->mat;
@@ -1934,7 +2583,7 @@ int values_impl(bo_prec* P) {
   const Geom& g = m->g;
   const int gN = grid_for(g.N), gh = grid_for(g.Nh);
   (launch_pdl(k_decouple<S>, gN, kThreads, 0, s, g, m->A, m->a2_valid ? m->A2 : nullptr, m->a2_range, (S*)P->At, P->w, P->wf,
-      P->opts.decoupling == BO_DECOUPLE_ABF, P->st), note_launch());
+      P->di0, P->opts.decoupling == BO_DECOUPLE_ABF, P->st), note_launch());
   // FP64 red inverses for the black pass: the Krylov basis is idle during setup
   double* red64 = P->V;
   if (sizeof(S) < sizeof(double) && m->a2_valid) {
@@ -1948,24 +2597,34 @@ int values_impl(bo_prec* P) {
     (launch_pdl(k_ilu_red<S, false>, gh, kThreads, 0, s, g, m->A, P->w, (S*)P->Dinv, red64, P->st), note_launch());
     (launch_pdl(k_ilu_black<S>, gh, kThreads, 0, s, g, m->A, P->w, red64, (S*)P->Dinv, P->st), note_launch());
   }
-  // AMG hierarchy values
+  // AMG hierarchy values (eight lanes per coarse cell)
   for (int l = 1; l < P->nlev; ++l) {
     Level& C = P->lev[l];
-    if (l == 1)
-      (launch_pdl(k_galerkin0, grid_for(C.n), kThreads, 0, s, g, m->A, P->w, dims_of(C), C.c64, P->st), note_launch());
+    if (l == 1 && C.n >= kGalerkinWide)
+      (launch_pdl(k_galerkin0_wide<S>, grid_for(2 * C.n), kThreads, 0, s, g, m->A, P->w, dims_of(C), C.c64, (S*)C.c,
+           P->st), note_launch());
+    else if (l == 1)
+      (launch_pdl(k_galerkin0<S>, grid_for(8 * C.n), kThreads, 0, s, g, m->A, P->w, dims_of(C), C.c64, (S*)C.c, P->st),
+       note_launch());
     else
-      (launch_pdl(k_galerkinn, grid_for(C.n), kThreads, 0, s, dims_of(P->lev[l - 1]), P->lev[l - 1].c64, dims_of(C), C.c64,
-          P->st), note_launch());
-    (launch_pdl(k_convert<S>, grid_for(7 * C.n), kThreads, 0, s, C.c64, (S*)C.c, (size_t)7 * C.n), note_launch());
+      (launch_pdl(k_galerkinn<S>, grid_for(8 * C.n), kThreads, 0, s, dims_of(P->lev[l - 1]), P->lev[l - 1].c64,
+           dims_of(C), C.c64, (S*)C.c, P->st), note_launch());
   }
   const int last = P->nlev - 1;
-  LevelDims cd = last == 0 ? LevelDims{g.nx, g.ny, g.nz, g.N} : dims_of(P->lev[last]);
-  (launch_pdl(k_dense_from_level, 1, kThreads, 0, s, cd, last == 0 ? nullptr : P->lev[last].c64, g, m->A, P->w, last == 0,
-      P->coarse64), note_launch());
-  const int n = (int)P->ncoarse;
-  const size_t smem = (size_t)n * n * sizeof(double) + (size_t)n * sizeof(int);
-  cudaFuncSetAttribute(k_gj_inverse<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  (launch_pdl(k_gj_inverse<S>, 1, 1024, smem, s, n, P->coarse64, (S*)P->coarse_inv, P->st), note_launch());
+  const LevelDims cd = last == 0 ? LevelDims{g.nx, g.ny, g.nz, g.N} : dims_of(P->lev[last]);
+  if (P->res->cluster > 0) {  // the resident levels' packed copies
+    using T = typename ArithOf<S>::type;
+    CoefPtrs cf = {};
+    int64_t items = 0;
+    for (int l = P->res->l0; l <= last; ++l) {
+      if (l) cf.c[l] = P->lev[l].c;
+      items += l == last ? P->res->rl[l].n : P->res->rl[l].npairs;
+    }
+    (launch_pdl(k_res_pack<T, S>, (int)((items + kThreads - 1) / kThreads), kThreads, 0, s, *P->res, g, (const S*)P->At,
+         (const T*)P->di0, cf), note_launch());
+  }
+  const DenseSrc src{nullptr, last == 0 ? nullptr : P->lev[last].c64, cd, g, m->A, P->w};
+  if (launch_gj<S>((int)P->ncoarse, src, (S*)P->coarse_inv, true, P->st, s) != cudaSuccess) return BO_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return BO_ERR_CUDA;
   return learned_coarse_values(P);
 }
@@ -1986,6 +2645,7 @@ int prec_alloc(bo_prec* P) {
   P->w = (double*)al((size_t)3 * g.N * sizeof(double));
   P->wf = ts == sizeof(float) ? (float*)al((size_t)3 * g.N * sizeof(float)) : nullptr;
   P->Dinv = al((size_t)9 * g.N * ss);
+  P->di0 = ss == sizeof(double) ? (double*)al((size_t)g.N * sizeof(double)) : nullptr;
   P->f = al((size_t)3 * g.N * ts);
   P->t = al((size_t)3 * g.N * ts);
   P->r = al((size_t)3 * g.N * ts);
@@ -2004,7 +2664,7 @@ int prec_alloc(bo_prec* P) {
     Level& L = P->lev[P->nlev];
     L.nx = nx; L.ny = ny; L.nz = nz; L.n = n;
     L.c64 = (double*)al((size_t)7 * n * sizeof(double));
-    L.c = al((size_t)7 * n * ss);
+    L.c = al((size_t)(ss == 8 ? 8 : 7) * n * ss);  // level_slots
     L.f = al((size_t)n * ts);
     L.x = al((size_t)n * ts);
     P->nlev++;
@@ -2015,8 +2675,25 @@ int prec_alloc(bo_prec* P) {
   for (int l = 1; l < P->nlev; ++l)
     if (P->lev[l].n <= kTailCells) { P->tail_from = l; break; }
   if (P->tail_from < 1) P->tail_from = 1;
-  P->coarse64 = (double*)al((size_t)n * n * sizeof(double));
   P->coarse_inv = al((size_t)n * n * ss);
+  // the resident AMG levels
+  P->res = new (std::nothrow) ResPlan();
+  if (!P->res) return BO_ERR_OOM;
+  if (P->bf16) resident_plan<float, __nv_bfloat16>(P, *P->res);
+  else if (P->fp32) resident_plan<float, float>(P, *P->res);
+  else resident_plan<double, double>(P, *P->res);
+  if (P->res->cluster > 0) {
+    ResPlan& a = *P->res;
+    const size_t K = ts == sizeof(double) ? res_values<double>() : res_values<float>();
+    for (int l = a.l0; l <= a.last; ++l) {
+      ResLevel& r = a.rl[l];
+      if (l < a.last) r.cp = al(2 * K * r.npairs * ts);
+      r.meta = (int32_t*)al((size_t)(l < a.last ? 3 * r.npairs : r.n) * sizeof(int32_t));
+      r.f = l ? P->lev[l].f : P->f0;
+      r.x = l ? P->lev[l].x : P->e0;
+    }
+    a.inv = P->coarse_inv;
+  }
   if (ok && cudaMalloc(&P->st, sizeof(DevState)) != cudaSuccess) ok = false;
   if (ok) cudaMemsetAsync(P->st, 0, sizeof(DevState), P->stream);
   return ok ? BO_OK : BO_ERR_OOM;
@@ -2024,10 +2701,15 @@ int prec_alloc(bo_prec* P) {
 
 void prec_free(bo_prec* P) {
   auto fr = [](void* p) { if (p) cudaFree(p); };
-  fr(P->At); fr(P->w); fr(P->wf); fr(P->Dinv);
+  fr(P->At); fr(P->w); fr(P->wf); fr(P->Dinv); fr(P->di0);
   fr(P->f); fr(P->t); fr(P->r); fr(P->z1); fr(P->e0); fr(P->f0);
   for (int l = 1; l < P->nlev; ++l) { fr(P->lev[l].c64); fr(P->lev[l].c); fr(P->lev[l].f); fr(P->lev[l].x); }
-  fr(P->coarse64); fr(P->coarse_inv); fr(P->st);
+  fr(P->coarse_inv); fr(P->st);
+  if (P->res) {
+    for (int l = 0; l < 24; ++l) { fr(P->res->rl[l].cp); fr(P->res->rl[l].meta); }
+    delete P->res;
+    P->res = nullptr;
+  }
   learned_coarse_free(P);
   graphs_reset(P);
   if (P->cap_stream) cudaStreamDestroy(P->cap_stream);
@@ -2041,9 +2723,8 @@ int prec_values(bo_prec* P) {
 
 int launch_dense_inverse64(int n, const double* M, double* Minv, DevState* st, cudaStream_t s) {
   if (n < 1 || n > kCoarseMax) return BO_ERR_ARG;
-  const size_t smem = (size_t)n * n * sizeof(double) + (size_t)n * sizeof(int);
-  cudaFuncSetAttribute(k_gj_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  (launch_pdl(k_gj_inverse<double>, 1, 1024, smem, s, n, M, Minv, st), note_launch());
+  const DenseSrc src{M, nullptr, LevelDims{n, 1, 1, n}, Geom{}, nullptr, nullptr};
+  if (launch_gj<double>(n, src, Minv, false, st, s) != cudaSuccess) return BO_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
 }
 
