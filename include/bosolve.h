@@ -676,8 +676,9 @@ int bo_cnn_adam_step(bo_cnn* net, float lr);
  * backward_weights: dw[t][co][ci] = sum_v dy[v][co] x[v + off(t)][ci] and
  *   db[co] = sum_v dy[v][co] (FP32); dy FP32 [batch][V][cout] is rounded to
  *   BF16 for the products.
- * backward_data and backward_weights allocate and free scratch and
- * synchronise.  BO_ERR_ARG on an unsupported (cin, cout) or mode. */
+ * backward_data and backward_weights synchronise; their scratch (at most 34
+ * MB) stays with the context on the tcgen05 engine and is allocated and freed
+ * in the call on the mma.sync engine.  BO_ERR_ARG on an unsupported (cin, cout) or mode. */
 int bo_conv3d_forward(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* x,
                       const uint16_t* w, const float* bias, const uint16_t* residual, int relu, uint16_t* y,
                       float* yf);
@@ -685,9 +686,9 @@ int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int 
                             const uint16_t* w, float* dx);
 int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* x,
                                const float* dy, float* dw, float* db);
-/* Convolution engine for the 32 -> 32 layers (forward and data gradient;
- * process-wide): 0 = mma.sync kernel, 1 = tcgen05 kernel (tensor memory
- * accumulator, TMA-fetched tiles; the default).  The other layers always use
+/* Convolution engine (process-wide): 0 = mma.sync kernels, 1 = tcgen05
+ * kernels (tensor memory accumulators; the default) for every layer's
+ * forward pass and gradients; operands off a 16-byte boundary always take
  * mma.sync. */
 int bo_set_conv_engine(int engine);
 /* How the AMG V-cycle is launched (process-wide); every form computes the

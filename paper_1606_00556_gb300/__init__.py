@@ -847,7 +847,7 @@ def bo_set_amg_barrier_spins(spins: int):
 
 
 def bo_set_conv_engine(engine: int):
-    """0: mma.sync, 1: tcgen05 for the 32 -> 32 convolutions."""
+    """Convolutions on 0: mma.sync, 1 (default): tcgen05."""
     _check(lib().bo_set_conv_engine(int(engine)), "bo_set_conv_engine")
 
 

@@ -332,7 +332,7 @@ extern std::atomic<long long> g_launches;
 // streams of the batched solve's pool in use (1..kMaxPoolStreams)
 constexpr int kMaxPoolStreams = 16;
 extern std::atomic<int> g_pool_width;
-// convolution engine of the 32 -> 32 layers: 0 mma.sync, 1 tcgen05 (conv_tc.cu)
+// convolution engine: 0 mma.sync (cnn.cu), 1 tcgen05 (conv_tc.cu)
 extern std::atomic<int> g_conv_engine;
 // AMG launch form: 2 (default) one cluster launch for the levels that fit it,
 // cooperative legs for the levels above, 1 cooperative legs for every
@@ -398,6 +398,8 @@ struct bo_ctx {
   cudaStream_t stream;
   bool own_stream;
   int refs;
+  void* scratch;         // workspace of the single-layer gradient calls (ordered on the stream like them), or NULL
+  size_t scratch_bytes;  // at most one layer's partial sums (about 34 MB); freed with the context
 };
 
 struct bo_mat {
@@ -554,6 +556,8 @@ void launch_spmv_decoupled_internal(bo_prec* P, const double* x, double* y);  //
 
 // capi.cu: drop a reference on a context (frees it with the last one)
 void ctx_release_ref(bo_ctx* c);
+// the context's workspace, grown to `bytes` (NULL if that fails)
+void* ctx_scratch(bo_ctx* c, size_t bytes);
 
 // krylov.cu
 int fgmres(bo_prec* P, const double* b_nat, double* x_nat, const bo_solve_opts* o, bo_solve_info* info);
@@ -580,10 +584,18 @@ int krylov_alloc(bo_prec* P, int m);
 // shadow as scratch
 void launch_arnoldi_product(bo_prec* P, const double* v, double* w);
 void graphs_reset(bo_prec* P);
-// tcgen05 convolution for 32 -> 32 layers; mode 0 ReLU, 1 ReLU + residual,
-// 2 linear FP32 output.  BO_ERR_ARG where it does not apply.
-int launch_conv_tc(int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W, const float* bias,
-                   const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, cudaStream_t s);
+// tcgen05 convolution (conv_tc.cu); mode 0 ReLU, 1 ReLU + residual, 2 linear
+// FP32 output, 3 linear BF16 output with channels 0..3 in FP32; transposed:
+// the data gradient.  BO_ERR_ARG where it does not apply.
+int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W,
+                   const float* bias, const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, bool transposed,
+                   cudaStream_t s);
+// tcgen05 weight and bias gradients of a layer (part: room for kWgradTcBlocks
+// partials of 27 cin cout floats, bpart: of cout doubles); BO_ERR_ARG where it
+// does not apply
+constexpr int kWgradTcBlocks = 304;
+int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
+                    double* bpart, float* dW, float* db, cudaStream_t s);
 // dense FP64 inverse of an n x n matrix (n <= 128) by one block; sets
 // st->err on a zero pivot
 int launch_dense_inverse64(int n, const double* M, double* Minv, DevState* st, cudaStream_t s);

@@ -50,6 +50,7 @@ namespace {
 void ctx_release(bo_ctx* c) {
   if (--c->refs > 0) return;
   cudaStreamSynchronize(c->stream);
+  if (c->scratch) cudaFree(c->scratch);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -124,6 +125,21 @@ void mat_release(bo_mat* m) {
 namespace bo {
 void ctx_release_ref(bo_ctx* c) { ctx_release(c); }
 void mat_release_ref(bo_mat* m) { mat_release(m); }
+void* ctx_scratch(bo_ctx* c, size_t bytes) {
+  if (c->scratch_bytes < bytes) {
+    cudaStreamSynchronize(c->stream);  // calls that still use the old one
+    if (c->scratch) cudaFree(c->scratch);
+    c->scratch = nullptr;
+    c->scratch_bytes = 0;
+    if (cudaMalloc(&c->scratch, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      c->scratch = nullptr;
+      return nullptr;
+    }
+    c->scratch_bytes = bytes;
+  }
+  return c->scratch;
+}
 }  // namespace bo
 
 namespace {

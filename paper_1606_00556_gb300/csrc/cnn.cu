@@ -387,10 +387,9 @@ enum FwdMode { kReluBf16, kReluResBf16, kLinearOut, kLinearF32All };
 
 int launch_fwd(int cin, int cout, FwdMode mode, int nx, int ny, int nz, int B, const bf16* X, const bf16* W,
                const float* bias, const bf16* R, bf16* Y, float* Yf, cudaStream_t s) {
-  if (g_conv_engine.load() == 1 && cin == 32 && cout == 32 &&
-      (mode == kReluBf16 || mode == kReluResBf16 || mode == kLinearF32All)) {
-    const int tm = mode == kReluBf16 ? 0 : mode == kReluResBf16 ? 1 : 2;
-    const int rc = launch_conv_tc(nx, ny, nz, B, X, W, bias, R, Y, Yf, tm, s);
+  if (g_conv_engine.load() == 1) {
+    const int tm = mode == kReluBf16 ? 0 : mode == kReluResBf16 ? 1 : mode == kLinearF32All ? 2 : 3;
+    const int rc = launch_conv_tc(cin, cout, nx, ny, nz, B, X, W, bias, R, Y, Yf, tm, false, s);
     if (rc != BO_ERR_ARG) return rc;  // else: the mma.sync kernel below
   }
   if (mode == kReluBf16 && cin == 16 && cout == 32)
@@ -436,17 +435,35 @@ int launch_wgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* X
 }
 
 // Data gradient of a layer: dX (FP32, cin channels) from dY (BF16, cout
-// channels): the forward kernel on dY with the flipped, transposed weights.
+// channels): the forward kernel on dY with the flipped, transposed weights
+// (the tcgen05 kernel transposes them itself; wd and zero_bias are the
+// mma.sync kernel's).
 int launch_dgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* dY, const bf16* W, bf16* wd,
                  const float* zero_bias, float* dX, cudaStream_t s) {
+  if (g_conv_engine.load() == 1) {
+    const int rc = launch_conv_tc(cout, cin, nx, ny, nz, B, dY, W, nullptr, nullptr, nullptr, dX, 2, true, s);
+    if (rc != BO_ERR_ARG) return rc;
+  }
   (k_flip_transpose<<<grid_for(27 * cin * cout), kThreads, 0, s>>>(W, wd, cin, cout), note_launch());
   return launch_fwd(cout, cin, kLinearF32All, nx, ny, nz, B, dY, wd, zero_bias, nullptr, nullptr, dX, s);
 }
 
 // Weight and bias gradients of a layer from its input X (BF16) and dY
-// (FP32; its BF16 copy dY16 is made here unless have16)
+// (FP32; its BF16 copy dY16 is made here unless have16).  dY16 = NULL: the
+// tcgen05 kernel only, which needs no copy (BO_ERR_ARG where it does not apply).
 int launch_layer_wgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* X, const float* dY, bf16* dY16,
                        bool have16, float* part, double* bpart, float* dW, float* db, cudaStream_t s) {
+  if (g_conv_engine.load() == 1) {
+    const int rc = launch_wgrad_tc(cin, cout, nx, ny, nz, B, X, dY, part, bpart, dW, db, s);
+    if (rc != BO_ERR_ARG) {
+      // (the data gradient that may follow reads dY16)
+      if (rc == BO_OK && dY16 && !have16)
+        (k_f32_to_bf16<<<grid_for((int64_t)B * nx * ny * nz * cout), kThreads, 0, s>>>(dY, dY16, (int64_t)B * nx * ny * nz * cout),
+         note_launch());
+      return rc;
+    }
+    if (!dY16) return BO_ERR_ARG;
+  }
   const int64_t V = (int64_t)nx * ny * nz, BV = B * V;
   if (!have16) (k_f32_to_bf16<<<grid_for(BV * cout), kThreads, 0, s>>>(dY, dY16, BV * cout), note_launch());
   const int rc = launch_wgrad(cin, cout, nx, ny, nz, B, X, dY16, part, dW, s);
@@ -765,6 +782,14 @@ int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int 
   if (!ctx || !dy || !w || !dx || batch < 1 || nx < 1 || ny < 1 || nz < 1 ||
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
+  if (bo::g_conv_engine.load() == 1) {  // no workspace
+    const int rc = bo::launch_conv_tc(cout, cin, nx, ny, nz, batch, reinterpret_cast<const bf16*>(dy),
+                                      reinterpret_cast<const bf16*>(w), nullptr, nullptr, nullptr, dx, 2, true, ctx->stream);
+    if (rc != BO_ERR_ARG) {
+      cudaStreamSynchronize(ctx->stream);
+      return rc;
+    }
+  }
   bf16* wd = nullptr;
   float* zb = nullptr;
   if (cudaMalloc(&wd, (size_t)27 * cin * cout * 2) != cudaSuccess) return BO_ERR_OOM;
@@ -784,6 +809,17 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
   if (!((cin == 16 && cout == 32) || (cin == 32 && cout == 32) || (cin == 32 && cout == 16))) return BO_ERR_ARG;
+  if (bo::g_conv_engine.load() == 1) {  // the partial sums in the context's workspace
+    const size_t pb = (size_t)bo::kWgradTcBlocks * 27 * cin * cout * 4;
+    void* ws = bo::ctx_scratch(ctx, pb + (size_t)bo::kWgradTcBlocks * 32 * sizeof(double));
+    if (!ws) return BO_ERR_OOM;
+    const int rc = bo::launch_wgrad_tc(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x), dy, (float*)ws,
+                                       (double*)((char*)ws + pb), dw, db, ctx->stream);
+    if (rc != BO_ERR_ARG) {
+      cudaStreamSynchronize(ctx->stream);
+      return rc;
+    }
+  }
   const int64_t BV = (int64_t)batch * nx * ny * nz;
   bf16* d16 = nullptr;
   float* part = nullptr;

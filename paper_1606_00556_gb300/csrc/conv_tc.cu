@@ -1,42 +1,47 @@
-// 3x3x3 convolution, 32 -> 32 channels, on the fifth-generation tensor
-// cores: tcgen05.mma with the accumulator in tensor memory, operands in
-// shared memory, input tiles fetched by TMA.  Computes the same as the
-// mma.sync forward kernel in cnn.cu for the network's 32 -> 32 layers
-// (BF16 in, FP32 accumulate):
+// 3x3x3 convolutions on the fifth-generation tensor cores: tcgen05.mma with
+// the accumulator in tensor memory.  Computes the same as the mma.sync
+// kernels in cnn.cu (BF16 in, FP32 accumulate), for every layer of the
+// network (16 -> 32, 32 -> 32 and 32 -> 16 channels):
 //   Y[v][co] = act(bias[co] + sum_t,ci X[v + off(t)][ci] W[t][co][ci] (+ R[v][co]))
-// with 'same' zero padding.
+// with 'same' zero padding; the data gradient is the same convolution of dY
+// with W[26 - t] transposed, read that way when the weights are staged.
 //
-// Tile = 8 x 16 voxels of one z plane (M = 128 rows of the MMA, row
-// m = x + 8 y).  Its input with a one-voxel halo, 10 x 18 x 3 voxels, comes
-// in as four TMA boxes of 8 channels each (box {8, 10, 18, 3, 1} over the
-// tensor {C, X, Y, Z, batch}; coordinates outside the volume read as zero),
-// so shared memory holds it channel-chunk-major: chunk kc is a plane of
-// 540 rows of 16 bytes.  In that layout the 128 rows a tap needs are, for
-// each 8-voxel run along x, 8 consecutive 16-byte rows: exactly a core
-// matrix of the no-swizzle K-major operand layout, with the next run
-// (y + 1) 10 rows further on.  So every tap is a shared-memory descriptor
-// on the same halo (start address moved by the tap's offset; K-direction
-// core-matrix stride = one chunk plane, M-direction stride = 160 bytes),
-// and a tile is 27 taps x 2 K-steps = 54 MMAs of 128 x 32 x 16 into one
-// 32-column TMEM accumulator.  The weights (N = 32 rows, K = 27 x 32) sit
-// in shared memory for the whole persistent CTA.
+// The x taps go into the N dimension of the MMA.  A tile is 128 voxels (the
+// MMA's M) of one z plane, TY runs of TX along x; for each of the nine (dz,
+// dy) the MMAs multiply the tile's voxels moved by (dz, dy) with the weights
+// of all three dx at once, N = 3 Cout:
+//   D[x][dx][co] = sum_{dz,dy,ci} X[x, y + dy, z + dz][ci] W[dz,dy,dx][co][ci],
+// and the epilogue adds out[x] = D[x - 1][0] + D[x][1] + D[x + 1][2] across
+// TMEM lanes.  With one tap per MMA (N = 32) an MMA reads 5 KB of operands
+// from shared memory for 16 cycles of tensor work; with three it reads 7 KB
+// for 48, and a tile takes 18 MMAs instead of 54.  Runs shorter than the
+// row give up their two end voxels (TX - 2 outputs a run); a row that fits
+// one run loses nothing, its neighbours outside the grid being zero.
+// TX in {16, 32, 64, 128} is the one with the fewest tiles for the grid.
 //
-// One CTA of 288 threads (nine warps) per SM, persistent over tiles.  Warp
-// 0 issues the TMA copies and the MMAs (one elected thread); three halo
-// buffers let the copies of the next tiles overlap the MMAs of the current
-// one, and two 32-column TMEM accumulators let the MMAs of one tile overlap
-// the epilogue of the previous one.  Warps 1-8 form the epilogue: warp w
-// reads TMEM lane quarter w % 4 (the 32 lanes its warp may access) for
-// output channels 16 ((w - 1) / 4) .. + 15 with tcgen05.ld, then applies
-// bias, residual and ReLU and stores BF16 or FP32.  Every wait on an
-// mbarrier is bounded: on expiry the CTA records an error, waits (bounded)
-// for its copies in flight, frees its TMEM and returns.
-#include <cuda.h>
-#include <cudaTypedefs.h>
+// Shared memory holds planes of (TY + 2) x TX voxels, one 16-byte row of 8
+// channels per voxel, chunk by chunk ([channel / 8][voxel][8 channels]): eight
+// consecutive voxels are a core matrix of the no-swizzle K-major operand
+// layout, and a (dz, dy) tap is a descriptor on plane z + dz that starts (dy
+// + 1) runs in.  A CTA marches along z through a column of tiles, so each
+// plane is loaded once per column and serves three tiles; the tiles of all
+// columns are dealt to the CTAs in contiguous ranges of equal length.  The
+// planes are fetched with cp.async by four producer warps (128 contiguous
+// bytes per pair of voxels, out-of-grid voxels zero-filled): TMA boxes for
+// this chunked layout have 16-byte inner rows, and the form before this one,
+// which fetched a 10 x 18 x 3 halo per tile that way, was bound by them
+// (2160 rows, about 3.5 us a tile whose MMAs need 1.1 us).
+//
+// One CTA of 13 warps per SM: warp 0 issues the MMAs (one elected thread),
+// warps 1-8 form the epilogue, warps 9-12 produce; six plane buffers and two
+// TMEM accumulators let all three overlap.  Every wait on an mbarrier is
+// bounded: on expiry the CTA records an error, finishes its copies and MMAs
+// in flight (again bounded), frees its TMEM and returns.
+// Measured, 64x64x32 voxels x 4 samples, 32 -> 32 channels: forward with
+// residual FWD0 -> FWD1 us, data gradient DG0 -> DG1 us (kernel time).
 #include <cuda_bf16.h>
 
 #include <cstring>
-#include <mutex>
 
 #include "bo_internal.cuh"
 
@@ -45,34 +50,38 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int kTcThreads = 288;  // warp 0: TMA + MMA issue; warps 1-8: epilogue
-constexpr int kTileX = 8, kTileY = 16;
-constexpr int kHX = 10, kHY = 18, kHZ = 3;
-constexpr int kHaloRows = kHX * kHY * kHZ;                       // 540
-constexpr int kChunkStride = ((kHaloRows * 16 + 127) / 128) * 128;  // 8704: one 8-channel plane, 128-B aligned
-constexpr int kChunkBytes = kHaloRows * 16;                       // 8640 written by one TMA box
-constexpr int kHaloBuf = 4 * kChunkStride;                        // 34816
-constexpr int kWBytes = 27 * 2048;                                // weights, 27 taps x (32 x 32 bf16)
-constexpr int kOffW = 0;
-constexpr int kOffHalo = kWBytes;                                 // 55296 (128-B aligned)
-constexpr int kStages = 3;                                        // halo buffers
-constexpr int kOffBar = kOffHalo + kStages * kHaloBuf;            // 159744
-constexpr int kSmemBytes = kOffBar + 256 + 1024;                  // barriers, TMEM slot, flag, bias; base-alignment slack
+constexpr int kTcThreads = 416;      // warp 0: MMA issue; 1-8: epilogue; 9-12: producers
+constexpr int kProducers = 128;
+constexpr int kPlanes = 6;           // plane buffers: three of a tile, three on their way
+constexpr int kAhead = 2;            // planes a producer leaves in flight before it signals the oldest
 constexpr long kSpinLimit = 1l << 26;
-constexpr uint32_t kTxBytes = 4 * kChunkBytes;
+constexpr int kTileM = 128;
 
 __device__ int g_tc_err;  // set by a CTA whose wait expired (read and cleared by bo_tc_status)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// shared-memory matrix descriptor: no swizzle, K-major, version 1
+// shared-memory matrix descriptor, no swizzle, version 1: the strides between
+// core matrices (8 rows of 16 bytes) along K (lbo) and along M or N (sbo)
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
 }
 
-// instruction descriptor, kind::f16: D FP32, A and B BF16, both K-major, M = 128, N = 32
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((32u >> 3) << 17) | ((128u >> 4) << 24);
+// instruction descriptor, kind::f16: D FP32, A and B BF16, M = 128; MN: both
+// operands with M (N) contiguous in memory instead of K
+__host__ __device__ constexpr uint32_t idesc(int n, bool mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(n >> 3) << 17) |
+         ((128u >> 4) << 24);
+}
+
+__device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, bool acc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"((uint32_t)acc)
+      : "memory");
+}
 
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   uint32_t done = 0;
@@ -86,317 +95,843 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   }
   return false;
 }
-
-__device__ __forceinline__ void tma_halo(const CUtensorMap* map, uint32_t dst, uint32_t bar, int x0, int y0, int z,
-                                         int b) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kTxBytes) : "memory");
-#pragma unroll
-  for (int kc = 0; kc < 4; ++kc) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
-        "%6}], [%7];\n" ::"r"(dst + kc * kChunkStride),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(8 * kc), "r"(x0 - 1), "r"(y0 - 1), "r"(z - 1), "r"(b), "r"(bar)
-        : "memory");
-  }
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count));
 }
-
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
-
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
 }
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
+// 16 bytes from global to shared memory, or zeros
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
 }
 
-// OUT 0: Y = ReLU(conv + bias (+ R)) in BF16;  OUT 1: Yf = conv + bias in FP32.
-// Warp 0 (one elected thread) feeds TMA and issues the MMAs of tile k into
-// TMEM accumulator k & 1 while warps 1-8 drain the other accumulator
-// (warp w reads TMEM lanes 32 (w % 4) .. and output channels 16 ((w - 1) / 4) ..).  Tile k's halo sits in buffer
-// k % 3: the TMA for tile k + 2 goes out right after tile k's MMAs are
-// queued, once tile k - 1's MMAs (queued earlier) have released its buffer,
-// so the tensor pipe never drains while waiting for a copy.  mbarriers:
-//   full[b]     TMA bytes of halo buffer b landed          (TMA -> MMA)
-//   empty[b]    the MMAs reading halo buffer b finished     (MMA -> TMA)
-//   accfull[a]  the MMAs into accumulator a finished        (MMA -> epilogue)
-//   accempty[a] the epilogue finished reading accumulator a (epilogue -> MMA, 8 arrivals)
-// The n-th completion of a barrier has parity n & 1; each side counts the
-// completions it has waited for.
-template <bool RES, int OUT>
-__global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_constant__ CUtensorMap xmap, int nx, int ny,
-                                                           int nz, int B, const bf16* __restrict__ W,
+// N consecutive TMEM columns at each of three addresses
+#define BO_R8(o) "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), "=r"(r[o + 6]), "=r"(r[o + 7])
+__device__ __forceinline__ void tmem_ld3(uint32_t a0, uint32_t a1, uint32_t a2, float (&v)[3][16]) {
+  uint32_t r[48];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%48];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%49];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47}, [%50];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : BO_R8(0), BO_R8(8), BO_R8(16), BO_R8(24), BO_R8(32), BO_R8(40)
+      : "r"(a0), "r"(a1), "r"(a2)
+      : "memory");
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[k][i] = __uint_as_float(r[16 * k + i]);
+}
+__device__ __forceinline__ void tmem_ld3(uint32_t a0, uint32_t a1, uint32_t a2, float (&v)[3][8]) {
+  uint32_t r[24];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%24];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%25];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%26];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : BO_R8(0), BO_R8(8), BO_R8(16)
+      : "r"(a0), "r"(a1), "r"(a2)
+      : "memory");
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[k][i] = __uint_as_float(r[8 * k + i]);
+}
+
+// The tiles: nz tiles of a column (z fastest), columns by x tile, y tile, sample
+struct ConvGrid {
+  int nx, ny, nz, B;
+  int ltx;              // log2 TX
+  int ntx, nty;
+  int64_t tiles;
+};
+struct Column {
+  int x0, y0, b;
+};
+__device__ __forceinline__ Column column_of(const ConvGrid& g, int64_t t) {
+  const int c = (int)(t / g.nz);
+  const int tx = c % g.ntx, r = c / g.ntx;
+  const int TX = 1 << g.ltx;
+  return Column{tx * (TX - 2), (r % g.nty) * (kTileM >> g.ltx), r / g.nty};
+}
+__host__ __device__ __forceinline__ int plane_rows(int ltx) { return kTileM + (2 << ltx); }
+// bytes of one channel chunk of a plane; the padding puts the chunks of a
+// voxel, which one quarter warp writes together, in different banks
+__host__ __device__ __forceinline__ int chunk_stride(int ltx, int kc) { return plane_rows(ltx) * 16 + 128 / kc; }
+
+template <int CIN, int COUT>
+struct ConvLayout {
+  static constexpr int KC = CIN / 8;
+  static constexpr int NB = 3 * COUT;
+  static constexpr int kW = 9 * KC * NB * 16;
+  static constexpr int kEdge = 2 * 2 * 2 * 4 * 16 * 4;  // [tile parity][side][channel half][warp][channel]
+  static constexpr int kOffEdge = kW;
+  static constexpr int kOffBias = kOffEdge + kEdge;
+  static constexpr int kOffBar = kOffBias + 128;
+  static constexpr int kOffPlanes = kOffBar + 256;
+};
+
+// OUT 0: Y = ReLU(conv + bias (+ R)) in BF16; 1: Yf = conv + bias in FP32;
+// 2: Y = conv + bias in BF16 and its channels 0..3 in FP32 (Yf[v][4]).
+// TRANSPOSED: the data gradient's weights (see the head of the file).
+// mbarriers: full[p] plane buffer p holds its plane (128 producer arrivals);
+// empty[p] the MMAs that read it are done; accfull[a], accempty[a] (8 warps)
+// as the accumulators pass between the MMAs and the epilogue.  The n-th
+// completion of a barrier has parity n & 1.
+template <int CIN, int COUT, int OUT, bool RES, bool TRANSPOSED>
+__global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_constant__ ConvGrid g,
+                                                           const bf16* __restrict__ X, const bf16* __restrict__ W,
                                                            const float* __restrict__ bias, const bf16* __restrict__ R,
                                                            bf16* __restrict__ Y, float* __restrict__ Yf) {
+  using L = ConvLayout<CIN, COUT>;
+  constexpr int KC = L::KC, NB = L::NB;
+  constexpr int CH = COUT / 2;  // channels of an epilogue thread
   extern __shared__ uint8_t smraw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kOffBar);  // full[3], empty[3], accfull[2], accempty[2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kOffBar + 80);
-  volatile int* sfail = reinterpret_cast<volatile int*>(sm + kOffBar + 84);
-  float* sbias = reinterpret_cast<float*>(sm + kOffBar + 128);
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 127) & ~uintptr_t(127));
+  float* edge = reinterpret_cast<float*>(sm + L::kOffEdge);
+  float* sbias = reinterpret_cast<float*>(sm + L::kOffBias);
+  const uint32_t bars = smem_u32(sm + L::kOffBar);
+  auto full = [&](int p) { return bars + 8 * p; };
+  auto empty = [&](int p) { return bars + 8 * (kPlanes + p); };
+  auto accfull = [&](int a) { return bars + 8 * (2 * kPlanes + a); };
+  auto accempty = [&](int a) { return bars + 8 * (2 * kPlanes + 2 + a); };
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + L::kOffBar + 8 * (2 * kPlanes + 4));
+  volatile int* sfail = reinterpret_cast<volatile int*>(tslot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int V = nx * ny * nz;
-  const int ntx = (nx + kTileX - 1) / kTileX, nty = (ny + kTileY - 1) / kTileY;
-  const int ntiles = ntx * nty * nz * B;
-  // weights -> core-matrix layout: tap t, chunk kc = ci / 8, row co: t*2048 + kc*512 + co*16
-  for (int i = tid; i < 27 * 32 * 4; i += kTcThreads) {
-    const int t = i / 128, rem = i - t * 128, co = rem >> 2, kc = rem & 3;
-    const uint4 w = *reinterpret_cast<const uint4*>(W + ((size_t)(t * 32 + co) * 32 + kc * 8));
-    *reinterpret_cast<uint4*>(sm + kOffW + t * 2048 + kc * 512 + co * 16) = w;
-  }
-  if (tid < 32) sbias[tid] = bias[tid];
-  uint32_t full[kStages], empty[kStages], accfull[2], accempty[2];
-  for (int i = 0; i < kStages; ++i) {
-    full[i] = smem_u32(&bars[i]);
-    empty[i] = smem_u32(&bars[kStages + i]);
-  }
-  for (int i = 0; i < 2; ++i) {
-    accfull[i] = smem_u32(&bars[2 * kStages + i]);
-    accempty[i] = smem_u32(&bars[2 * kStages + 2 + i]);
-  }
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(full[i]));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(empty[i]));
+    for (int p = 0; p < kPlanes; ++p) {
+      mbar_init(full(p), kProducers);
+      mbar_init(empty(p), 1);
     }
-    for (int i = 0; i < 2; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(accfull[i]));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;\n" ::"r"(accempty[i]));
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(accfull(a), 1);
+      mbar_init(accempty(a), 8);
     }
     *sfail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;\n" ::"r"(smem_u32(tslot)));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;\n" ::"r"(smem_u32(tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tslot;
-  const uint32_t wbase = smem_u32(sm + kOffW);
-  const uint32_t hbase = smem_u32(sm + kOffHalo);
-  auto tile_xyzb = [&](int t, int& x0, int& y0, int& z, int& b) {
-    const int tx = t % ntx;
-    t /= ntx;
-    const int ty = t % nty;
-    t /= nty;
-    z = t % nz;
-    b = t / nz;
-    x0 = tx * kTileX;
-    y0 = ty * kTileY;
-  };
-  const int first = blockIdx.x, step = gridDim.x;
-  const int mine = first < ntiles ? (ntiles - 1 - first) / step + 1 : 0;  // tiles of this CTA
-  if (warp == 0) {
-    if (lane == 0) {
-      int fills[kStages] = {0, 0, 0}, uses[kStages] = {0, 0, 0}, commits[kStages] = {0, 0, 0},
-          freed[kStages] = {0, 0, 0};
-      int acc_waits[2] = {0, 0};
-      bool ok = true;
-      for (int s = 0; s < 2 && s < mine; ++s) {
-        int x0, y0, z, b;
-        tile_xyzb(first + s * step, x0, y0, z, b);
-        tma_halo(&xmap, hbase + s * kHaloBuf, full[s], x0, y0, z, b);
-        ++fills[s];
-      }
-      for (int k = 0; k < mine && ok; ++k) {
-        const int bf = k % kStages, a = k & 1;
-        if (*sfail) { ok = false; break; }
-        ok = mbar_wait(full[bf], uses[bf] & 1);
+  const int TX = 1 << g.ltx, rows = plane_rows(g.ltx), cs = chunk_stride(g.ltx, KC);
+  const uint32_t pbase = smem_u32(sm + L::kOffPlanes), pstride = (uint32_t)(KC * cs);
+  const int64_t t0 = g.tiles * blockIdx.x / gridDim.x, t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
+  const int V = g.nx * g.ny * g.nz;
+
+  if (warp >= 9) {
+    // ---- producers
+    const int pt = tid - 9 * 32;
+    const bf16* Xc = X + (size_t)(pt % KC) * 8;
+    int seq = 0, done = 0;
+    bool ok = true;
+    auto signal_to = [&](int n) {  // planes before n have landed (the caller's cp_wait)
+      fence_async_proxy();
+      for (; done < n; ++done) mbar_arrive(full(done % kPlanes));
+    };
+    for (int64_t t = t0; t < t1 && ok; ++t) {
+      const int z = (int)(t % g.nz);
+      const bool start = t == t0 || z == 0;
+      const Column c = column_of(g, t);
+      for (int pz = start ? max(z - 1, 0) : z + 1; pz <= min(z + 1, g.nz - 1) && ok; ++pz) {
+        if (seq >= kPlanes) ok = !*sfail && mbar_wait(empty(seq % kPlanes), (seq / kPlanes - 1) & 1);
         if (!ok) break;
-        ++uses[bf];
-        if (k >= 2) {  // tile k - 2's epilogue is done with accumulator a
-          ok = mbar_wait(accempty[a], acc_waits[a] & 1);
-          if (!ok) break;
-          ++acc_waits[a];
+        const uint32_t dst = pbase + (uint32_t)(seq % kPlanes) * pstride + (uint32_t)(pt % KC) * cs;
+        const size_t zb = (size_t)c.b * V + (size_t)pz * g.nx * g.ny;
+        for (int r = pt / KC; r < rows; r += kProducers / KC) {
+          const int x = c.x0 + (r & (TX - 1)), y = c.y0 - 1 + (r >> g.ltx);
+          const bool in = x < g.nx && y >= 0 && y < g.ny;
+          cp16(dst + (uint32_t)r * 16, Xc + (in ? (zb + (size_t)y * g.nx + x) * CIN : 0), in);
         }
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const uint32_t hb = hbase + bf * kHaloBuf;
-        const uint32_t dacc = tmem + (uint32_t)(a * 32);
-        // The 54 descriptors differ from the buffer's first ones only in
-        // their start-address field (address / 16 in the low 14 bits), by
-        // offsets that are compile-time constants once the loops are
-        // unrolled: one add per MMA instead of building each descriptor
-        // (the single issuing thread otherwise spent most of a tile on it).
-        const uint64_t da0 = smem_desc(hb, kChunkStride, kHX * 16);
-        const uint64_t db0 = smem_desc(wbase, 512, 128);
-#pragma unroll
-        for (int tap = 0; tap < 27; ++tap) {
-          const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-          const uint32_t rowoff = ((1 + dz) * kHY + (1 + dy)) * kHX + (1 + dx);
-#pragma unroll
-          for (int ks = 0; ks < 2; ++ks) {
-            const uint64_t da = da0 + (uint64_t)((2 * ks * kChunkStride + rowoff * 16) >> 4);
-            const uint64_t db = db0 + (uint64_t)((tap * 2048 + 2 * ks * 512) >> 4);
-            const uint32_t acc = (tap | ks) ? 1u : 0u;
-            asm volatile(
-                "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dacc),
-                "l"(da), "l"(db), "r"(kIdesc), "r"(acc)
-                : "memory");
-          }
-        }
-        umma_commit(empty[bf]);
-        umma_commit(accfull[a]);
-        ++commits[bf];
-        // tile k + 2 goes into the buffer tile k - 1 used, once its MMAs are done
-        if (k + 2 < mine) {
-          const int nb = (k + 2) % kStages;
-          if (commits[nb] > freed[nb]) {
-            ok = mbar_wait(empty[nb], freed[nb] & 1);
-            if (!ok) break;
-            ++freed[nb];
-          }
-          int x0, y0, z, b;
-          tile_xyzb(first + (k + 2) * step, x0, y0, z, b);
-          tma_halo(&xmap, hbase + nb * kHaloBuf, full[nb], x0, y0, z, b);
-          ++fills[nb];
-        }
-      }
-      if (!ok) {
-        *sfail = 1;
-        atomicExch(&g_tc_err, 1);
-        // copies and MMAs in flight finish before shared and tensor memory go away
-        for (int i = 0; i < kStages; ++i) {
-          if (fills[i] > uses[i]) mbar_wait(full[i], uses[i] & 1);
-          while (commits[i] > freed[i] && mbar_wait(empty[i], freed[i] & 1)) ++freed[i];
-        }
+        cp_commit();
+        ++seq;
+        cp_wait<kAhead>();
+        if (seq > kAhead) signal_to(seq - kAhead);
       }
     }
-    __syncwarp();
+    cp_wait<0>();
+    if (ok) {
+      signal_to(seq);
+    } else {
+      *sfail = 1;
+      atomicExch(&g_tc_err, 1);
+    }
   } else {
-    // epilogue warps: TMEM lane quarter w % 4, output channels 16 ((w - 1) / 4) .. + 15
-    const int quarter = warp & 3, ch0 = 16 * ((warp - 1) >> 2);
-    for (int k = 0; k < mine; ++k) {
-      const int a = k & 1;
-      if (!mbar_wait(accfull[a], (k >> 1) & 1)) {
-        *sfail = 1;
-        atomicExch(&g_tc_err, 1);
-        break;
+    // ---- weights into shared memory (warps 0-8): [dz, dy][channel chunk][dx, co][8 channels]
+    if (!TRANSPOSED) {
+      for (int i = tid; i < 27 * COUT * KC; i += 288) {
+        const int kc = i % KC, r = i / KC, co = r % COUT, t = r / COUT;
+        const uint4 w = *reinterpret_cast<const uint4*>(W + ((size_t)(t * COUT + co) * CIN + kc * 8));
+        *reinterpret_cast<uint4*>(sm + (((t / 3) * KC + kc) * NB + (t % 3) * COUT + co) * 16) = w;
       }
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      float acc[16];
-      tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 32 + ch0), acc);
-      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(accempty[a]);
-      int x0, y0, z, b;
-      tile_xyzb(first + k * step, x0, y0, z, b);
-      const int m = quarter * 32 + lane;
-      const int x = x0 + (m & 7), y = y0 + (m >> 3);
-      if (x < nx && y < ny) {
-        const size_t o = ((size_t)b * V + x + (size_t)nx * (y + (size_t)ny * z)) * 32 + ch0;
-        if (OUT == 0) {
-          float rr[16];
-          if (RES) {
+    } else {
+      // W is [27][CIN][COUT] here (the layer's own output channels are this convolution's inputs)
+      for (int i = tid; i < 27 * CIN * (COUT / 8); i += 288) {
+        const int cg = i % (COUT / 8), r = i / (COUT / 8), ci = r % CIN, t = 26 - r / CIN;
+        const uint4 w = *reinterpret_cast<const uint4*>(W + ((size_t)r * COUT + cg * 8));
+        const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
+        uint8_t* d = sm + (((t / 3) * KC + ci / 8) * NB + (t % 3) * COUT + cg * 8) * 16 + (ci % 8) * 2;
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const uint4 u = *reinterpret_cast<const uint4*>(R + o + 8 * q);
-              const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
+        for (int e = 0; e < 8; ++e)
+          *reinterpret_cast<unsigned short*>(d + 16 * e) = (unsigned short)(wv[e / 2] >> (16 * (e & 1)));
+      }
+    }
+    if (tid < COUT) sbias[tid] = bias ? bias[tid] : 0.f;
+    fence_async_proxy();
+    named_barrier(1, 288);
+    if (warp == 0) {
+      // ---- MMA issue
+      if (lane == 0 && t0 < t1) {
+        const uint32_t wbase = smem_u32(sm);
+        bool ok = true;
+        int waited = 0, next = 0, issued = 0;  // planes waited for; sequence number of the next tile's plane z
+        for (int64_t t = t0; t < t1 && ok; ++t) {
+          const int k = (int)(t - t0), a = k & 1;
+          const int z = (int)(t % g.nz);
+          const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
+          if (start) next = waited + (z > 0 ? 1 : 0);
+          const int need = next + (z < g.nz - 1 ? 1 : 0);
+          for (; waited <= need && ok; ++waited) ok = !*sfail && mbar_wait(full(waited % kPlanes), (waited / kPlanes) & 1);
+          if (ok && k >= 2) ok = mbar_wait(accempty(a), ((k >> 1) - 1) & 1);
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          const uint32_t dacc = tmem + (uint32_t)(a * 128);
+          const uint64_t db0 = smem_desc(wbase, NB * 16, 128);
+          bool acc = false;
+          for (int dz = -1; dz <= 1; ++dz) {
+            if (z + dz < 0 || z + dz >= g.nz) continue;
+            const uint64_t da0 = smem_desc(pbase + (uint32_t)((next + dz) % kPlanes) * pstride, (uint32_t)cs, 128);
+            const uint64_t dbz = db0 + (uint64_t)(((dz + 1) * 3 * KC * NB * 16) >> 4);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                rr[8 * q + 2 * e] = __bfloat162float(__ushort_as_bfloat16((unsigned short)(wv[e] & 0xffffu)));
-                rr[8 * q + 2 * e + 1] = __bfloat162float(__ushort_as_bfloat16((unsigned short)(wv[e] >> 16)));
+            for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+              for (int ks = 0; ks < KC / 2; ++ks) {
+                umma(dacc, da0 + (uint64_t)((2 * ks * cs + dy * TX * 16) >> 4),
+                     dbz + (uint64_t)(((dy * KC + 2 * ks) * NB * 16) >> 4), idesc(NB, false), acc);
+                acc = true;
               }
-            }
           }
+          if (z > 0) umma_commit(empty((next - 1) % kPlanes));
+          if (end) {
+            umma_commit(empty(next % kPlanes));
+            if (z < g.nz - 1) umma_commit(empty((next + 1) % kPlanes));
+          }
+          umma_commit(accfull(a));
+          ++issued;
+          ++next;
+        }
+        if (!ok) {
+          *sfail = 1;
+          atomicExch(&g_tc_err, 1);
+          // the MMAs in flight finish before shared and tensor memory go away
+          for (int k = max(0, issued - 2); k < issued; ++k) mbar_wait(accfull(k & 1), (k >> 1) & 1);
+        }
+      }
+      __syncwarp();
+    } else {
+      // ---- epilogue: TMEM lane quarter warp % 4, channels CH ((warp - 1) / 4) ..
+      const int quarter = warp & 3, half = (warp - 1) >> 2, ch0 = CH * half;
+      const int m = quarter * 32 + lane, xl = m & (TX - 1), yl = m >> g.ltx;
+      const bool cross = TX > 32;  // runs that span warps
+      bool ok = true;
+      for (int64_t t = t0; t < t1; ++t) {
+        const int k = (int)(t - t0), a = k & 1;
+        const int z = (int)(t % g.nz);
+        const Column c = column_of(g, t);
+        const int x = c.x0 + xl, y = c.y0 + yl;
+        const bool mine = x < g.nx && y < g.ny && (xl > 0 || x == 0) && (xl < TX - 1 || x == g.nx - 1);
+        const size_t o = ((size_t)c.b * V + x + (size_t)g.nx * (y + (size_t)g.ny * z)) * COUT + ch0;
+        uint4 res[CH / 8];
+        if (RES && mine) {
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
+          for (int q = 0; q < CH / 8; ++q) res[q] = *reinterpret_cast<const uint4*>(R + o + 8 * q);
+        }
+        // (after an expired wait the warp still meets the barriers, and stores nothing)
+        if (ok && (*sfail || !mbar_wait(accfull(a), (k >> 1) & 1))) {
+          ok = false;
+          *sfail = 1;
+          atomicExch(&g_tc_err, 1);
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        float d[3][CH];
+        if (ok) {
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 128 + ch0);
+          tmem_ld3(ta, ta + COUT, ta + 2 * COUT, d);
+          asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(accempty(a));
+        } else {
+#pragma unroll
+          for (int i = 0; i < CH; ++i) d[0][i] = d[1][i] = d[2][i] = 0.f;
+        }
+        float* eb = edge + ((a * 2) * 2 + half) * 4 * 16;  // side 0; side 1 is 2 x 4 x 16 floats on
+        if (cross) {
+          if (lane == 31)
+#pragma unroll
+            for (int i = 0; i < CH; ++i) eb[quarter * 16 + i] = d[0][i];
+          if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < CH; ++i) eb[2 * 4 * 16 + quarter * 16 + i] = d[2][i];
+          named_barrier(2 + half, 128);
+        }
+        float out[CH];
+#pragma unroll
+        for (int i = 0; i < CH; ++i) {
+          float l = __shfl_up_sync(0xffffffffu, d[0][i], 1), r = __shfl_down_sync(0xffffffffu, d[2][i], 1);
+          if (cross && lane == 0) l = eb[((quarter + 3) & 3) * 16 + i];
+          if (cross && lane == 31) r = eb[2 * 4 * 16 + ((quarter + 1) & 3) * 16 + i];
+          if (xl == 0) l = 0.f;
+          if (xl == TX - 1) r = 0.f;
+          out[i] = l + d[1][i] + r + sbias[ch0 + i];
+        }
+        if (!mine || !ok) continue;
+        if (OUT == 1) {
+#pragma unroll
+          for (int q = 0; q < CH / 4; ++q)
+            *reinterpret_cast<float4*>(Yf + o + 4 * q) = make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
+        } else {
+          if (OUT == 2 && half == 0)
+            *reinterpret_cast<float4*>(Yf + (o / COUT) * 4) = make_float4(out[0], out[1], out[2], out[3]);
+#pragma unroll
+          for (int q = 0; q < CH / 8; ++q) {
+            const uint32_t rw[4] = {RES ? res[q].x : 0u, RES ? res[q].y : 0u, RES ? res[q].z : 0u, RES ? res[q].w : 0u};
             uint32_t pk[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              const int c0 = 8 * q + 2 * e;
-              float y0v = acc[c0] + sbias[ch0 + c0], y1v = acc[c0 + 1] + sbias[ch0 + c0 + 1];
+              float v0 = out[8 * q + 2 * e], v1 = out[8 * q + 2 * e + 1];
               if (RES) {
-                y0v += rr[c0];
-                y1v += rr[c0 + 1];
+                v0 += __uint_as_float(rw[e] << 16);
+                v1 += __uint_as_float(rw[e] & 0xffff0000u);
               }
-              y0v = fmaxf(y0v, 0.f);
-              y1v = fmaxf(y1v, 0.f);
-              pk[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(y0v)) |
-                      ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(y1v)) << 16);
+              if (OUT == 0) {
+                v0 = fmaxf(v0, 0.f);
+                v1 = fmaxf(v1, 0.f);
+              }
+              pk[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v0)) |
+                      ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v1)) << 16);
             }
             *reinterpret_cast<uint4*>(Y + o + 8 * q) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<float4*>(Yf + o + 4 * q) =
-                make_float4(acc[4 * q] + sbias[ch0 + 4 * q], acc[4 * q + 1] + sbias[ch0 + 4 * q + 1],
-                            acc[4 * q + 2] + sbias[ch0 + 4 * q + 2], acc[4 * q + 3] + sbias[ch0 + 4 * q + 3]);
         }
       }
-      if (*sfail) break;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;\n" ::"r"(tmem));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem));
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  });
-  return fn;
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
+}
+
+template <int CIN, int COUT, int OUT, bool RES, bool TRANSPOSED>
+int run_conv(const ConvGrid& g, const bf16* X, const bf16* W, const float* bias, const bf16* R, bf16* Y, float* Yf,
+             cudaStream_t s) {
+  using L = ConvLayout<CIN, COUT>;
+  auto kern = k_conv3d_tc<CIN, COUT, OUT, RES, TRANSPOSED>;
+  const int smem = L::kOffPlanes + kPlanes * L::KC * chunk_stride(g.ltx, L::KC) + 128;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return BO_ERR_CUDA;
+  const int sms = sm_count();
+  const int grid = g.tiles < sms ? (int)g.tiles : sms;
+  (kern<<<grid, kTcThreads, smem, s>>>(g, X, W, bias, R, Y, Yf), note_launch());
+  return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
 }
 
 }  // namespace
 
-// The tensor-core path for a 32 -> 32 layer; BO_ERR_ARG where it does not
-// apply (the caller then uses the mma.sync kernel).
-//   relu_res: 0 ReLU, 1 ReLU with residual, 2 linear FP32 output (Yf)
-int launch_conv_tc(int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W, const float* bias,
-                   const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, cudaStream_t s) {
-  if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(W) & 15) ||
-      (Y && (reinterpret_cast<uintptr_t>(Y) & 15)) || (R && (reinterpret_cast<uintptr_t>(R) & 15)) ||
-      (Yf && (reinterpret_cast<uintptr_t>(Yf) & 15)))
+// The tensor-core path of a layer; BO_ERR_ARG where it does not apply (an
+// operand off a 16-byte boundary: the caller then uses the mma.sync kernel).
+//   mode: 0 ReLU, 1 ReLU with residual, 2 linear FP32 output (Yf), 3 linear
+//   with BF16 output and channels 0..3 in FP32; transposed: the data
+//   gradient, X = dY and W the layer's own weights [27][cin][cout] (mode 2).
+//   bias may be NULL (zero).
+int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W,
+                   const float* bias, const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, bool transposed,
+                   cudaStream_t s) {
+  for (const void* p : {(const void*)X, (const void*)W, (const void*)R, (const void*)Y, (const void*)Yf})
+    if (reinterpret_cast<uintptr_t>(p) & 15) return BO_ERR_ARG;
+  ConvGrid g{nx, ny, nz, B, 0, 0, 0, 0};
+  int64_t best = -1;
+  for (int ltx = 4; ltx <= 7; ++ltx) {
+    const int TX = 1 << ltx, TY = kTileM >> ltx;
+    const int ntx = nx <= TX ? 1 : (nx - TX + TX - 3) / (TX - 2) + 1, nty = (ny + TY - 1) / TY;
+    if (best < 0 || (int64_t)ntx * nty < best) {
+      best = (int64_t)ntx * nty;
+      g.ltx = ltx;
+      g.ntx = ntx;
+      g.nty = nty;
+    }
+  }
+  g.tiles = best * B * nz;
+  if (best * B > INT32_MAX) return BO_ERR_ARG;
+  if (transposed) {
+    if (mode != 2) return BO_ERR_ARG;
+    if (cin == 32 && cout == 32) return run_conv<32, 32, 1, false, true>(g, X, W, bias, R, Y, Yf, s);
+    if (cin == 32 && cout == 16) return run_conv<32, 16, 1, false, true>(g, X, W, bias, R, Y, Yf, s);
+    if (cin == 16 && cout == 32) return run_conv<16, 32, 1, false, true>(g, X, W, bias, R, Y, Yf, s);
     return BO_ERR_ARG;
-  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
-  if (!enc) return BO_ERR_ARG;
-  CUtensorMap map;
-  const cuuint64_t dims[5] = {32, (cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz, (cuuint64_t)B};
-  const cuuint64_t strides[4] = {64, 64ull * nx, 64ull * nx * ny, 64ull * nx * ny * nz};
-  const cuuint32_t box[5] = {8, kHX, kHY, kHZ, 1};
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16*>(X), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return BO_ERR_ARG;
-  const int ntiles = ((nx + kTileX - 1) / kTileX) * ((ny + kTileY - 1) / kTileY) * nz * B;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = ntiles < sms ? ntiles : sms;
-  auto run = [&](auto kern) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
-      return BO_ERR_CUDA;
-    (kern<<<grid, kTcThreads, kSmemBytes, s>>>(map, nx, ny, nz, B, W, bias, R, Y, Yf), note_launch());
-    return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
+  }
+  if (cin == 32 && cout == 32) {
+    if (mode == 0) return run_conv<32, 32, 0, false, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 1) return run_conv<32, 32, 0, true, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 2) return run_conv<32, 32, 1, false, false>(g, X, W, bias, R, Y, Yf, s);
+  }
+  if (cin == 16 && cout == 32) {
+    if (mode == 0) return run_conv<16, 32, 0, false, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 2) return run_conv<16, 32, 1, false, false>(g, X, W, bias, R, Y, Yf, s);
+  }
+  if (cin == 32 && cout == 16) {
+    if (mode == 2) return run_conv<32, 16, 1, false, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 3) return run_conv<32, 16, 2, false, false>(g, X, W, bias, R, Y, Yf, s);
+  }
+  return BO_ERR_ARG;
+}
+
+namespace {
+
+// ---- weight gradient
+// dW[t][co][ci] = sum_v dY[v][co] X[v + off(t)][ci] and db[co] = sum_v dY[v][co].
+//
+// Two tensors meet over voxels: the "halo" tensor (32 channels) at v + off
+// and the "core" tensor at v.  The halo tensor is X, or dY for the 16 -> 32
+// layer (X then is the core and the taps are mirrored), so that it always
+// fills the MMA's M.  An MMA takes 16 consecutive voxels of a grid row as K,
+// both operands with their channels contiguous (MN-major): A is four rows of
+// the halo plane, y - 1 .. y + 2, times 32 channels (M = 128), B two rows of
+// the core plane, y and y + 1, times its channels (N = 64 or 32).  The eight
+// (halo row, core row) pairs hold every dy tap of the two core rows and two
+// pairs that are not taps and are dropped at the end.  dz picks the halo plane
+// and the x tap moves A's start by one voxel, so nine accumulators hold all
+// 27 taps; the pairs need 9 x 64 TMEM columns of the 512, so for 32 core
+// channels the last two accumulators take one core row per MMA (32 columns;
+// A's rows move with it).  A row of a plane is [channel / 8][voxel][8
+// channels] with equal strides from chunk to chunk and row to row, which is
+// what lets one descriptor span four rows of four chunks.
+// The accumulators stay in TMEM over all tiles of a CTA (TX x 4 voxels, a
+// march along z as in the convolution above); each CTA writes one partial
+// sum, k_wgrad_sum adds them in a fixed order in FP64.  dY is read in FP32
+// by four warps that round it to BF16 on its way to shared memory and sum
+// the bias gradient in split FP32 pairs, so it is read once; X comes by
+// cp.async.  What bounds it: the shared-memory operand reads of the MMAs, 48
+// cycles for 2 x 16 voxels and a ninth of the taps.
+// Measured, 64x64x32 x 4 samples, 32 -> 32: WG0 us in five launches (mma.sync
+// gradient 144, FP64 bias sums 95, reduction 30, conversion 18) -> WG1 us.
+constexpr int kWgThreads = 288;   // warp 0: MMAs; 1-4: halo producers; 5-8: core producers; 1-8: the end
+constexpr int kWgHalo = 5, kWgCore = 3;  // plane buffers
+constexpr int kWgTY = 4, kWgHY = kWgTY + 3;
+
+struct WgradGrid {
+  int nx, ny, nz, B;
+  int tx;  // TX: 16, 32 or 64
+  int ntx, nty;
+  int64_t tiles;
+};
+
+__host__ __device__ __forceinline__ int wg_halo_row(int tx) { return (tx + 2) * 16; }          // one chunk of a row
+__host__ __device__ __forceinline__ int wg_core_row(int tx, int kc) { return tx * 16 + 128 / kc; }
+__host__ __device__ __forceinline__ int wg_halo_plane(int tx) { return kWgHY * 4 * wg_halo_row(tx); }
+__host__ __device__ __forceinline__ int wg_core_plane(int tx, int kc) { return kWgTY * kc * wg_core_row(tx, kc); }
+constexpr int kWgOffBar = 0, kWgOffBias = 256, kWgOffPlanes = kWgOffBias + 128 * 8 * 8;
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
+}
+
+// One plane of a tensor into shared memory: NR rows from y0, NX voxels from
+// x0, rows [chunk][voxel].  BF16 by cp.async (the caller commits); FP32 by
+// loads, rounded to BF16, `wait` called between the loads and the first store
+// and the voxels of `own` added to the thread's bias sums.
+template <int KC, int NR>
+__device__ __forceinline__ void wg_plane_bf16(const bf16* T, size_t zb, int nx, int ny, int x0, int y0, int NX, uint32_t dst,
+                                              int row_bytes, int pt) {
+  const int kc = pt % KC;
+  for (int yl = 0; yl < NR; ++yl) {
+    const int y = y0 + yl;
+    for (int xl = pt / KC; xl < NX; xl += 128 / KC) {
+      const int x = x0 + xl;
+      const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+      cp16(dst + (uint32_t)((yl * KC + kc) * row_bytes + xl * 16), T + (in ? (zb + (size_t)y * nx + x) * (KC * 8) : 0) + kc * 8,
+           in);
+    }
+  }
+}
+template <int KC, int NR, typename Wait>
+__device__ __forceinline__ bool wg_plane_f32(const float* T, size_t zb, int nx, int ny, int x0, int y0, int NX, uint32_t dst,
+                                             int row_bytes, int pt, bool own, int own_x0, int own_y0, int own_nx,
+                                             df (&bias)[8], Wait wait) {
+  constexpr int U = 6;  // voxels in flight per thread
+  const int kc = pt % KC;
+  const int n = NR * NX;
+  bool waited = false;
+  for (int i0 = pt / KC; i0 < n; i0 += U * (128 / KC)) {
+    float4 v[U][2];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * (128 / KC);
+      const int yl = i / NX, xl = i - yl * NX;
+      const int x = x0 + xl, y = y0 + yl;
+      const bool in = i < n && x >= 0 && x < nx && y >= 0 && y < ny;
+      const float4* src = reinterpret_cast<const float4*>(T + (in ? (zb + (size_t)y * nx + x) * (KC * 8) : 0) + kc * 8);
+      v[u][0] = in ? __ldcs(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[u][1] = in ? __ldcs(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (!waited) {
+      waited = true;
+      if (!wait()) return false;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * (128 / KC);
+      if (i >= n) continue;
+      const int yl = i / NX, xl = i - yl * NX;
+      const float e[8] = {v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w, v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w};
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)((yl * KC + kc) * row_bytes + xl * 16)),
+                   "r"(pack_bf16(e[0], e[1])), "r"(pack_bf16(e[2], e[3])), "r"(pack_bf16(e[4], e[5])),
+                   "r"(pack_bf16(e[6], e[7]))
+                   : "memory");
+      if (own && yl >= own_y0 && yl < own_y0 + kWgTY && xl >= own_x0 && xl < own_x0 + own_nx) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const df t = df_two_sum(bias[q].hi, e[q]);
+          bias[q] = df{t.hi, __fadd_rn(bias[q].lo, t.lo)};
+        }
+      }
+    }
+  }
+  return true;
+}
+
+template <bool HALO_DY, int CB>
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ WgradGrid g, const bf16* __restrict__ X,
+                                                          const float* __restrict__ dY, float* __restrict__ part,
+                                                          double* __restrict__ bpart) {
+  constexpr int KC = CB / 8;          // chunks of the core tensor (the halo tensor has 4)
+  constexpr int kPair = CB == 32 ? 7 : 9;  // accumulators that take two core rows per MMA
+  constexpr int CY = HALO_DY ? 32 : CB;    // channels of dY
+  extern __shared__ uint8_t smraw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 127) & ~uintptr_t(127));
+  const uint32_t bars = smem_u32(sm + kWgOffBar);
+  auto hfull = [&](int p) { return bars + 8 * p; };
+  auto hempty = [&](int p) { return bars + 8 * (kWgHalo + p); };
+  auto cfull = [&](int p) { return bars + 8 * (2 * kWgHalo + p); };
+  auto cempty = [&](int p) { return bars + 8 * (2 * kWgHalo + kWgCore + p); };
+  const uint32_t alldone = bars + 8 * (2 * kWgHalo + 2 * kWgCore);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kWgOffBar + 8 * (2 * kWgHalo + 2 * kWgCore + 1));
+  volatile int* sfail = reinterpret_cast<volatile int*>(tslot + 1);
+  volatile uint32_t* sstarted = reinterpret_cast<volatile uint32_t*>(tslot + 2);  // accumulators with a sum in them
+  double* sbias = reinterpret_cast<double*>(sm + kWgOffBias);  // [producer][8]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int p = 0; p < kWgHalo; ++p) {
+      mbar_init(hfull(p), 128);
+      mbar_init(hempty(p), 1);
+    }
+    for (int p = 0; p < kWgCore; ++p) {
+      mbar_init(cfull(p), 128);
+      mbar_init(cempty(p), 1);
+    }
+    mbar_init(alldone, 1);
+    *sfail = 0;
+    *sstarted = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_u32(tslot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  const uint32_t tmem = *tslot;
+  const int TX = g.tx, hrow = wg_halo_row(TX), crow = wg_core_row(TX, KC);
+  const uint32_t hbase = smem_u32(sm + kWgOffPlanes), hplane = (uint32_t)wg_halo_plane(TX);
+  const uint32_t cbase = hbase + kWgHalo * hplane, cplane = (uint32_t)wg_core_plane(TX, KC);
+  const int64_t t0 = g.tiles * blockIdx.x / gridDim.x, t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
+  const int V = g.nx * g.ny * g.nz;
+  auto tile = [&](int64_t t, int& x0, int& y0, int& z, int& b) {
+    z = (int)(t % g.nz);
+    const int c = (int)(t / g.nz), r = c / g.ntx;
+    x0 = (c % g.ntx) * TX;
+    y0 = (r % g.nty) * kWgTY;
+    b = r / g.nty;
   };
-  if (mode == 0) return run(k_conv3d_tc<false, 0>);
-  if (mode == 1) return run(k_conv3d_tc<true, 0>);
-  if (mode == 2) return run(k_conv3d_tc<false, 1>);
+  df bias[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) bias[q] = df{0.f, 0.f};
+  bool ok = true;
+  if (warp >= 5) {
+    // ---- core planes
+    const int pt = tid - 5 * 32;
+    for (int64_t t = t0; t < t1 && ok; ++t) {
+      const int k = (int)(t - t0);
+      int x0, y0, z, b;
+      tile(t, x0, y0, z, b);
+      const size_t zb = (size_t)b * V + (size_t)z * g.nx * g.ny;
+      const uint32_t dst = cbase + (uint32_t)(k % kWgCore) * cplane;
+      auto wait = [&]() { return k < kWgCore || (!*sfail && mbar_wait(cempty(k % kWgCore), (k / kWgCore - 1) & 1)); };
+      if constexpr (HALO_DY) {
+        ok = wait();
+        if (!ok) break;
+        wg_plane_bf16<KC, kWgTY>(X, zb, g.nx, g.ny, x0, y0, TX, dst, crow, pt);
+        cp_commit();
+        cp_wait<0>();
+      } else {
+        ok = wg_plane_f32<KC, kWgTY>(dY, zb, g.nx, g.ny, x0, y0, TX, dst, crow, pt, true, 0, 0, TX, bias, wait);
+        if (!ok) break;
+      }
+      fence_async_proxy();
+      mbar_arrive(cfull(k % kWgCore));
+    }
+  } else if (warp >= 1) {
+    // ---- halo planes
+    const int pt = tid - 32;
+    int seq = 0, done = 0;
+    for (int64_t t = t0; t < t1 && ok; ++t) {
+      int x0, y0, z, b;
+      tile(t, x0, y0, z, b);
+      const bool start = t == t0 || z == 0;
+      const int zend = (int)min((int64_t)g.nz, z + (t1 - t));  // the column's tiles of this CTA end there
+      for (int pz = start ? max(z - 1, 0) : z + 1; pz <= min(z + 1, g.nz - 1) && ok; ++pz) {
+        const size_t zb = (size_t)b * V + (size_t)pz * g.nx * g.ny;
+        const uint32_t dst = hbase + (uint32_t)(seq % kWgHalo) * hplane;
+        auto wait = [&]() { return seq < kWgHalo || (!*sfail && mbar_wait(hempty(seq % kWgHalo), (seq / kWgHalo - 1) & 1)); };
+        if constexpr (HALO_DY) {
+          // a plane counts towards the bias where it is one of this CTA's tiles
+          const bool own = pz >= z && pz < zend;
+          ok = wg_plane_f32<4, kWgHY>(dY, zb, g.nx, g.ny, x0 - 1, y0 - 1, TX + 2, dst, hrow, pt, own, 1, 1, TX, bias, wait);
+          if (!ok) break;
+          fence_async_proxy();
+          mbar_arrive(hfull(seq % kWgHalo));
+          ++seq;
+        } else {
+          ok = wait();
+          if (!ok) break;
+          wg_plane_bf16<4, kWgHY>(X, zb, g.nx, g.ny, x0 - 1, y0 - 1, TX + 2, dst, hrow, pt);
+          cp_commit();
+          ++seq;
+          cp_wait<1>();
+          if (seq > 1) {
+            fence_async_proxy();
+            for (; done < seq - 1; ++done) mbar_arrive(hfull(done % kWgHalo));
+          }
+        }
+      }
+    }
+    cp_wait<0>();
+    if constexpr (!HALO_DY) {
+      if (ok) {
+        fence_async_proxy();
+        for (; done < seq; ++done) mbar_arrive(hfull(done % kWgHalo));
+      }
+    }
+  } else if (lane == 0 && t0 < t1) {
+    // ---- MMA issue
+    uint32_t started = 0;
+    int waited = 0, next = 0;
+    for (int64_t t = t0; t < t1 && ok; ++t) {
+      const int k = (int)(t - t0);
+      int x0, y0, z, b;
+      tile(t, x0, y0, z, b);
+      const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
+      if (start) next = waited + (z > 0 ? 1 : 0);
+      const int need = next + (z < g.nz - 1 ? 1 : 0);
+      for (; waited <= need && ok; ++waited) ok = !*sfail && mbar_wait(hfull(waited % kWgHalo), (waited / kWgHalo) & 1);
+      ok = ok && mbar_wait(cfull(k % kWgCore), (k / kWgCore) & 1);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      const uint64_t db0 = smem_desc(cbase + (uint32_t)(k % kWgCore) * cplane, 128, (uint32_t)crow);
+      for (int dz = 0; dz < 3; ++dz) {
+        if (z + dz - 1 < 0 || z + dz - 1 >= g.nz) continue;
+        const uint64_t da0 = smem_desc(hbase + (uint32_t)((next + dz - 1) % kWgHalo) * hplane, 128, (uint32_t)hrow);
+        for (int yp = 0; yp < kWgTY; yp += 2)
+          for (int kx = 0; kx < TX; kx += 16) {
+            const uint64_t da = da0 + (uint64_t)((yp * 4 * hrow + kx * 16) >> 4);
+            const uint64_t db = db0 + (uint64_t)((yp * KC * crow + kx * 16) >> 4);
+#pragma unroll
+            for (int sx = 0; sx < 3; ++sx) {
+              const int i = 3 * dz + sx;
+              const bool acc = (started >> i) & 1u;
+              if (i < kPair) {
+                umma(tmem + (uint32_t)(2 * CB * i), da + (uint64_t)sx, db, idesc(2 * CB, true), acc);
+              } else {
+                const uint32_t d = tmem + (uint32_t)(2 * CB * kPair + CB * (i - kPair));
+                umma(d, da + (uint64_t)sx, db, idesc(CB, true), acc);
+                umma(d, da + (uint64_t)sx + (uint64_t)((4 * hrow) >> 4), db + (uint64_t)((KC * crow) >> 4), idesc(CB, true), true);
+              }
+              started |= 1u << i;
+            }
+          }
+      }
+      umma_commit(cempty(k % kWgCore));
+      if (z > 0) umma_commit(hempty((next - 1) % kWgHalo));
+      if (end) {
+        umma_commit(hempty(next % kWgHalo));
+        if (z < g.nz - 1) umma_commit(hempty((next + 1) % kWgHalo));
+      }
+      ++next;
+    }
+    *sstarted = started;
+    umma_commit(alldone);
+    if (!mbar_wait(alldone, 0)) ok = false;  // every MMA is done before the buffers are used again
+  }
+  if (!ok) {
+    *sfail = 1;
+    atomicExch(&g_tc_err, 1);
+  }
+  if (warp >= 1) {
+    const bool dyside = HALO_DY ? warp < 5 : warp >= 5;
+    if (dyside) {
+      const int pt = HALO_DY ? tid - 32 : tid - 5 * 32;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sbias[pt * 8 + q] = df_to_double(df_renorm(bias[q]));
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  // ---- sums out: accumulator i, halo row a (lane quarter), core row r holds
+  // tap (dz, a - r, sx) of halo channel `lane`
+  float* red = reinterpret_cast<float*>(sm + kWgOffPlanes);
+  const uint32_t started = *sstarted;
+  const bool fine = !*sfail;
+  for (int r = 0; r < 2; ++r) {
+    if (warp >= 1) {
+      const int a = warp & 3, part2 = (warp - 1) >> 2;  // the two warps of a quarter take alternate accumulators
+      for (int i = part2; i < 9; i += 2) {
+        const bool pair = i < kPair;
+        if (!pair && r == 1) continue;
+        const int dy = pair ? a - r : a;
+        if (dy < 0 || dy > 2) continue;  // (warp-uniform)
+        const uint32_t col = pair ? (uint32_t)(2 * CB * i + CB * r) : (uint32_t)(2 * CB * kPair + CB * (i - kPair));
+        const int t = 9 * (i / 3) + 3 * dy + i % 3;
+        const int tap = HALO_DY ? 26 - t : t;
+        const bool have = fine && ((started >> i) & 1u);
+#pragma unroll
+        for (int c0 = 0; c0 < CB; c0 += 16) {
+          uint32_t v[16];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+              "tcgen05.wait::ld.sync.aligned;\n"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+                "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+              : "r"(tmem + ((uint32_t)(a * 32) << 16) + col + (uint32_t)c0)
+              : "memory");
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int o = HALO_DY ? (tap * 32 + lane) * CB + c0 + e : (tap * CB + c0 + e) * 32 + lane;
+            const float f = have ? __uint_as_float(v[e]) : 0.f;
+            red[o] = r == 0 ? f : red[o] + f;
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const int n = 27 * 32 * CB;
+  float* P = part + (size_t)blockIdx.x * n;
+  for (int i = tid; i < n; i += kWgThreads) P[i] = red[i];
+  if (tid < CY) {
+    constexpr int YC = CY / 8;
+    double sum = 0.0;
+    for (int p = tid / 8; p < 128; p += YC) sum += sbias[p * 8 + tid % 8];
+    bpart[(size_t)blockIdx.x * CY + tid] = sum;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+}
+
+// dW[i] = sum over the chunks' partials in a fixed order (FP64); 32 outputs by
+// 8 slices of the chunks per block.  The last block takes the bias gradient.
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, const double* __restrict__ bpart,
+                                                   float* __restrict__ dW, float* __restrict__ db, int n, int chunks, int cy) {
+  __shared__ double sh[8][32];
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double s = 0.0;
+  if (blockIdx.x == gridDim.x - 1) {
+    if (l < cy)
+      for (int k = w; k < chunks; k += 8) s += bpart[(size_t)k * cy + l];
+  } else {
+    const int i = blockIdx.x * 32 + l;
+#pragma unroll 4
+    for (int k = w; k < chunks; k += 8) s += part[(size_t)k * n + i];  // (n is a multiple of 32)
+  }
+  sh[w][l] = s;
+  __syncthreads();
+  if (w == 0) {
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += sh[k][l];
+    if (blockIdx.x == gridDim.x - 1) {
+      if (l < cy) db[l] = (float)t;
+    } else {
+      dW[blockIdx.x * 32 + l] = (float)t;
+    }
+  }
+}
+
+template <bool HALO_DY, int CB>
+int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, double* bpart, float* dW, float* db,
+              cudaStream_t s) {
+  auto kern = k_wgrad_tc<HALO_DY, CB>;
+  const int planes = kWgHalo * wg_halo_plane(g.tx) + kWgCore * wg_core_plane(g.tx, CB / 8);
+  const int red = 27 * 32 * CB * 4;
+  const int smem = kWgOffPlanes + (planes > red ? planes : red) + 128;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return BO_ERR_CUDA;
+  int grid = sm_count();
+  if (grid > kWgradTcBlocks) grid = kWgradTcBlocks;
+  if (g.tiles < grid) grid = (int)g.tiles;
+  (kern<<<grid, kWgThreads, smem, s>>>(g, X, dY, part, bpart), note_launch());
+  const int n = 27 * 32 * CB;
+  (k_wgrad_sum<<<n / 32 + 1, 256, 0, s>>>(part, bpart, dW, db, n, grid, HALO_DY ? 32 : CB), note_launch());
+  return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
+}
+
+}  // namespace
+
+// The tensor-core weight and bias gradients of a layer (part: room for
+// kWgradTcBlocks partials of 27 cin cout floats, bpart: of cout doubles);
+// BO_ERR_ARG where it does not apply.
+int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
+                    double* bpart, float* dW, float* db, cudaStream_t s) {
+  if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(dY) & 15)) return BO_ERR_ARG;
+  WgradGrid g{nx, ny, nz, B, 0, 0, 0, 0};
+  int best = 0;
+  for (int tx : {64, 32, 16}) {  // the fewest padded voxels along x; of equals the longest run
+    const int w = (nx + tx - 1) / tx * tx;
+    if (!best || w < best) {
+      best = w;
+      g.tx = tx;
+    }
+  }
+  g.ntx = (nx + g.tx - 1) / g.tx;
+  g.nty = (ny + kWgTY - 1) / kWgTY;
+  if ((int64_t)g.ntx * g.nty * B > INT32_MAX) return BO_ERR_ARG;
+  g.tiles = (int64_t)g.ntx * g.nty * B * nz;
+  if (cin == 32 && cout == 32) return run_wgrad<false, 32>(g, X, dY, part, bpart, dW, db, s);
+  if (cin == 32 && cout == 16) return run_wgrad<false, 16>(g, X, dY, part, bpart, dW, db, s);
+  if (cin == 16 && cout == 32) return run_wgrad<true, 16>(g, X, dY, part, bpart, dW, db, s);
   return BO_ERR_ARG;
 }
 
