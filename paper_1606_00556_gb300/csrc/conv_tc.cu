@@ -38,7 +38,8 @@
 // bounded: on expiry the CTA records an error, finishes its copies and MMAs
 // in flight (again bounded), frees its TMEM and returns.
 // Measured, 64x64x32 voxels x 4 samples, 32 -> 32 channels: forward with
-// residual FWD0 -> FWD1 us, data gradient DG0 -> DG1 us (kernel time).
+// residual 103 -> 63 us a call, data gradient 150 -> 86 us a call (61 us of
+// it the kernel, the rest the call's synchronisation).
 #include <cuda_bf16.h>
 
 #include <cstring>
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
   const int TX = 1 << g.ltx, rows = plane_rows(g.ltx), cs = chunk_stride(g.ltx, KC);
   const uint32_t pbase = smem_u32(sm + L::kOffPlanes), pstride = (uint32_t)(KC * cs);
   const int64_t t0 = g.tiles * blockIdx.x / gridDim.x, t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
-  const int V = g.nx * g.ny * g.nz;
+  const int64_t V = (int64_t)g.nx * g.ny * g.nz;
 
   if (warp >= 9) {
     // ---- producers
@@ -535,8 +536,10 @@ namespace {
 // the bias gradient in split FP32 pairs, so it is read once; X comes by
 // cp.async.  What bounds it: the shared-memory operand reads of the MMAs, 48
 // cycles for 2 x 16 voxels and a ninth of the taps.
-// Measured, 64x64x32 x 4 samples, 32 -> 32: WG0 us in five launches (mma.sync
-// gradient 144, FP64 bias sums 95, reduction 30, conversion 18) -> WG1 us.
+// Measured, 64x64x32 x 4 samples, 32 -> 32: 587 us a call, with scratch
+// allocated in it and five launches (mma.sync gradient 144, FP64 bias sums
+// 95, reduction 30, conversion 18) -> 164 us (this kernel 118, k_wgrad_sum
+// 21).
 constexpr int kWgThreads = 288;   // warp 0: MMAs; 1-4: halo producers; 5-8: core producers; 1-8: the end
 constexpr int kWgHalo = 5, kWgCore = 3;  // plane buffers
 constexpr int kWgTY = 4, kWgHY = kWgTY + 3;
@@ -668,7 +671,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   const uint32_t hbase = smem_u32(sm + kWgOffPlanes), hplane = (uint32_t)wg_halo_plane(TX);
   const uint32_t cbase = hbase + kWgHalo * hplane, cplane = (uint32_t)wg_core_plane(TX, KC);
   const int64_t t0 = g.tiles * blockIdx.x / gridDim.x, t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
-  const int V = g.nx * g.ny * g.nz;
+  const int64_t V = (int64_t)g.nx * g.ny * g.nz;
   auto tile = [&](int64_t t, int& x0, int& y0, int& z, int& b) {
     z = (int)(t % g.nz);
     const int c = (int)(t / g.nz), r = c / g.ntx;
@@ -804,7 +807,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     if (dyside) {
       const int pt = HALO_DY ? tid - 32 : tid - 5 * 32;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) sbias[pt * 8 + q] = df_to_double(df_renorm(bias[q]));
+      for (int q = 0; q < 8; ++q)  // (a sum that met an infinity has NaN in its low part)
+        sbias[pt * 8 + q] = isfinite(bias[q].hi) ? df_to_double(df_renorm(bias[q])) : (double)bias[q].hi;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
