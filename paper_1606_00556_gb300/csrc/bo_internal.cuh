@@ -464,7 +464,6 @@ struct bo_prec {
   // CPR work vectors (precision T, internal order)
   void* f;                 // 3N decoupled input
   void* t;                 // 3N ILU intermediates
-  void* r;                 // 3N residual
   void* z1;                // 3N first local solve x1 = R^{-1} f
   void* e0;                // N level-0 AMG correction
   void* f0;                // N level-0 AMG right-hand side

@@ -913,131 +913,61 @@ __device__ __forceinline__ void offdiag_sum(const Geom& g, const S* __restrict__
   }
 }
 
-// ILU pass 2 (black): u_b = D_b'^{-1} (src_b - sum A_br t_r).
-// OUT = false: z_b = u_b (precision T).
-// OUT = true: t_b = u_b and the preconditioner's result on black cells,
-//   zo_b = z1_b + Pi_p e_b + u_b, in FP64.
+// ILU pass 2 (black): z_b = D_b'^{-1} (f_b - sum A_br t_r), t_r = D_r^{-1} f_r
+// (pass 1).  Pass 3 (red): x_r = D_r^{-1} (f_r - sum A_rb x_b).
 // blocks per SM the register budget is tuned for: the FP32 passes are
 // memory-latency bound and want more warps; the FP64 ones are FP64-bound
 template <typename T>
 constexpr int ilu_min_blocks() { return sizeof(T) == 4 ? 4 : 3; }
-template <typename T, int ROWS>
-constexpr int res_min_blocks() { return (sizeof(T) == 4 && ROWS == 1) ? 5 : 4; }
 
-template <typename T, typename S, bool OUT>
-__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_b(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* __restrict__ src,
-                        T* __restrict__ tv, T* __restrict__ z, const T* __restrict__ e, OutV zo,
-                        const DevState* st) {
+template <typename T, typename S>
+__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_b(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* __restrict__ f,
+                        const T* __restrict__ tv, T* __restrict__ z, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
     const Cell c = decode(g, 1, q);
     T s[3];
     offdiag_sum(g, At, 1, q, c, tv, s);
-    const T r0 = src[vidx(g, 0, 1, q)] - s[0], r1 = src[vidx(g, 1, 1, q)] - s[1], r2 = src[vidx(g, 2, 1, q)] - s[2];
+    const T r0 = f[vidx(g, 0, 1, q)] - s[0], r1 = f[vidx(g, 1, 1, q)] - s[1], r2 = f[vidx(g, 2, 1, q)] - s[2];
     T d[9];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + g.Nh + q]);
-    const T u0 = d[0] * r0 + d[1] * r1 + d[2] * r2;
-    const T u1 = d[3] * r0 + d[4] * r1 + d[5] * r2;
-    const T u2 = d[6] * r0 + d[7] * r1 + d[8] * r2;
-    if (OUT) {
-      tv[vidx(g, 0, 1, q)] = u0;
-      tv[vidx(g, 1, 1, q)] = u1;
-      tv[vidx(g, 2, 1, q)] = u2;
-      out_put<T>(zo, vidx(g, 0, 1, q), z[vidx(g, 0, 1, q)] + e[g.Nh + q] + u0);
-      out_put<T>(zo, vidx(g, 1, 1, q), z[vidx(g, 1, 1, q)] + u1);
-      out_put<T>(zo, vidx(g, 2, 1, q), z[vidx(g, 2, 1, q)] + u2);
-    } else {
-      z[vidx(g, 0, 1, q)] = u0;
-      z[vidx(g, 1, 1, q)] = u1;
-      z[vidx(g, 2, 1, q)] = u2;
-    }
+    z[vidx(g, 0, 1, q)] = d[0] * r0 + d[1] * r1 + d[2] * r2;
+    z[vidx(g, 1, 1, q)] = d[3] * r0 + d[4] * r1 + d[5] * r2;
+    z[vidx(g, 2, 1, q)] = d[6] * r0 + d[7] * r1 + d[8] * r2;
   }
 }
 
-// ILU pass 3 (red): corr = D_r^{-1} sum A_rb u_b, with u_b in `ub` (black half).
-// OUT = false: z_r = t_r - corr (precision T).
-// OUT = true: zo_r = z1_r + Pi_p e_r + t_r - corr, in FP64.
-template <typename T, typename S, bool OUT>
-__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* __restrict__ tv,
-                         const T* __restrict__ ub, T* __restrict__ z, const T* __restrict__ e, OutV zo,
-                         const DevState* st) {
+// (the black half of xb is read.)  OUT = false: z_r = x_r; OUT = true: the
+// preconditioner's result, from f_r as in the first solve or, with DELTA, as
+// the correction w_r - D_r^{-1} sum A_rb u_b (w_r and u_b the halves of xb)
+template <typename T, typename S, bool OUT, bool DELTA>
+__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* __restrict__ f,
+                         const T* xb, T* z, OutV zo, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
     const Cell c = decode(g, 0, q);
     T s[3];
-    offdiag_sum(g, At, 0, q, c, ub, s);
+    offdiag_sum(g, At, 0, q, c, xb, s);
+    T r0 = -s[0], r1 = -s[1], r2 = -s[2];
+    if (!DELTA) r0 += f[vidx(g, 0, 0, q)], r1 += f[vidx(g, 1, 0, q)], r2 += f[vidx(g, 2, 0, q)];
     T d[9];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
-    const T c0 = d[0] * s[0] + d[1] * s[1] + d[2] * s[2];
-    const T c1 = d[3] * s[0] + d[4] * s[1] + d[5] * s[2];
-    const T c2 = d[6] * s[0] + d[7] * s[1] + d[8] * s[2];
-    const T t0 = tv[vidx(g, 0, 0, q)] - c0, t1 = tv[vidx(g, 1, 0, q)] - c1, t2 = tv[vidx(g, 2, 0, q)] - c2;
+    T x0 = d[0] * r0 + d[1] * r1 + d[2] * r2;
+    T x1 = d[3] * r0 + d[4] * r1 + d[5] * r2;
+    T x2 = d[6] * r0 + d[7] * r1 + d[8] * r2;
+    if (DELTA) x0 += xb[vidx(g, 0, 0, q)], x1 += xb[vidx(g, 1, 0, q)], x2 += xb[vidx(g, 2, 0, q)];
     if (OUT) {
-      out_put<T>(zo, vidx(g, 0, 0, q), z[vidx(g, 0, 0, q)] + e[q] + t0);
-      out_put<T>(zo, vidx(g, 1, 0, q), z[vidx(g, 1, 0, q)] + t1);
-      out_put<T>(zo, vidx(g, 2, 0, q), z[vidx(g, 2, 0, q)] + t2);
+      out_put<T>(zo, vidx(g, 0, 0, q), x0);
+      out_put<T>(zo, vidx(g, 1, 0, q), x1);
+      out_put<T>(zo, vidx(g, 2, 0, q), x2);
     } else {
-      z[vidx(g, 0, 0, q)] = t0;
-      z[vidx(g, 1, 0, q)] = t1;
-      z[vidx(g, 2, 0, q)] = t2;
-    }
-  }
-}
-
-// Residuals of the decoupled system in precision T.
-// ROWS = 1: out[t] = f_p - (At z)_p for all cells (the AMG right-hand side).
-// ROWS = 3: out = f - At (z + Pi_p e), all components, fused with the first
-//   ILU pass of the second local solve on red cells: tv_r = D_r^{-1} out_r.
-template <typename T, typename S, int ROWS>
-__global__ void __launch_bounds__(kThreads, res_min_blocks<T, ROWS>()) k_cpr_residual(Geom g, const S* __restrict__ At, const T* __restrict__ f, const T* __restrict__ z,
-                               const T* __restrict__ e, T* __restrict__ out, const S* __restrict__ Dinv,
-                               T* __restrict__ tv, const DevState* st) {
-  wait_prior_grid();
-  if (st->done) return;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.N; t += (int64_t)gridDim.x * blockDim.x) {
-    const int color = (int)(t / g.Nh);
-    const int64_t q = t - color * g.Nh;
-    const Cell c = decode(g, color, q);
-    T acc[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) acc[r] = T(0);
-    // every slot's loads are issued whether or not its neighbour exists
-    // (a missing one reads the cell's own entries and is masked to zero),
-    // so all of a cell's loads can be in flight at once
-#pragma unroll
-    for (int sl = 0; sl < 7; ++sl) {
-      const int64_t nb = nbr(g, c, q, sl);
-      const bool ok = nb >= 0;
-      const int64_t nq = ok ? nb : q;
-      const int xc = (sl == kDiag || !ok) ? color : (color ^ 1);
-      T x0 = z[vidx(g, 0, xc, nq)];
-      if (ROWS == 3) x0 += e[(size_t)xc * g.Nh + nq];
-      T x1 = z[vidx(g, 1, xc, nq)], x2 = z[vidx(g, 2, xc, nq)];
-      if (!ok) x0 = x1 = x2 = T(0);
-      const S* a = At + at_index(g, color, sl * 9, q);
-      constexpr size_t P = 32;  // entries (rc) of a block lie 32 apart in a tile
-#pragma unroll
-      for (int r = 0; r < ROWS; ++r)
-        acc[r] = fma3(acc[r], cv<T>(ld_stream(a + 3 * r * P)), x0, cv<T>(ld_stream(a + (3 * r + 1) * P)), x1,
-                      cv<T>(ld_stream(a + (3 * r + 2) * P)), x2);
-    }
-    T res[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-      res[r] = f[(size_t)r * g.N + t] - acc[r];
-      out[(size_t)r * g.N + t] = res[r];
-    }
-    if (ROWS == 3 && color == 0) {
-      T d[9];
-#pragma unroll
-      for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
-      tv[t] = d[0] * res[0] + d[1] * res[1 % ROWS] + d[2] * res[2 % ROWS];
-      tv[g.N + t] = d[3] * res[0] + d[4] * res[1 % ROWS] + d[5] * res[2 % ROWS];
-      tv[2 * g.N + t] = d[6] * res[0] + d[7] * res[1 % ROWS] + d[8] * res[2 % ROWS];
+      z[vidx(g, 0, 0, q)] = x0;
+      z[vidx(g, 1, 0, q)] = x1;
+      z[vidx(g, 2, 0, q)] = x2;
     }
   }
 }
@@ -1045,6 +975,165 @@ __global__ void __launch_bounds__(kThreads, res_min_blocks<T, ROWS>()) k_cpr_res
 // s / d, or in FP64 s times the stored reciprocal at di[i] (see level_slots)
 __device__ __forceinline__ double gs_divide(double s, double, const double* __restrict__ di, size_t i) { return s * di[i]; }
 __device__ __forceinline__ float gs_divide(float s, float d, const float*, size_t) { return s / d; }
+
+// ---- the rest of the CPR after its first local solve z = R^{-1} f
+// A red row of the red-black ILU(0)'s product is the row of the decoupled
+// matrix itself (red pivots are the diagonal blocks, and red rows have no
+// fill), so R^{-1} leaves no residual on red cells:
+//   A_rr z_r + A_rb z_b = f_r.
+// Three passes get shorter by it.  (1) The AMG right-hand side f_p - (A z)_p
+// is zero on red cells and needs the pressure rows of the black ones only.
+// (2) With x2 = z + Pi_p e the red pass of the second local solve needs only
+// the pressure columns of the red rows:
+//   w_r := x2_r + D_r^{-1} (f - A x2)_r = z_r - D_r^{-1} sum_b A_rb Pi_p e_b
+// (the diagonal block's term cancels e_r, which is therefore never read).
+// (3) The black pass then is
+//   x3_b = x2_b + D_b'^{-1} (f_b - A_bb x2_b - A_br w_r),
+// which reads A_br once where a residual of all rows followed by a black ILU
+// pass read it twice, and the red rows of x3 again have no residual:
+//   x3_r = D_r^{-1} (f_r - A_rb x3_b).
+// All of it holds where the stored pivots invert the stored diagonal blocks
+// to working precision.  BF16 storage rounds both to 8 bits, and (1), (2) and
+// the last line would change the preconditioner (measured: the solution moved
+// by 2e-9 at a tolerance of 1e-8, 2 of 24 systems took an iteration more), so
+// it keeps the residuals of the red cells and the correction form
+//   w_r = x2_r + D_r^{-1} (f - A x2)_r,  u_b = x3_b - x2_b,
+//   x3_r = w_r - D_r^{-1} A_rb u_b,
+// and gains by the fused black pass alone.  Newton step, 128x128x64 FP32 at 19
+// iterations 11.96 -> 10.59 ms, FP64 19.4 -> 16.8 ms; 256x256x128 BF16 80.7 ->
+// 77.1 ms; 62x45x19 FP32 1853 -> 1714 us.  Iterations are those of the form
+// before this one: 307 over 24 systems of 20x20x5 to 150x149x40 in FP64 and
+// in FP32.
+template <typename S>
+constexpr bool kExactRed = sizeof(S) >= 4;
+
+
+// AMG right-hand side: f0_b = f_p - (A z)_p, f0_r = 0, and with it the first
+// pre-smoothing sweep from zero, x_r = 0 and x_b = f0_b / a_bb; in BF16 f0
+// alone, on all cells
+template <typename T, typename S>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cpr_rhs(Geom g, const S* __restrict__ At,
+                         const T* __restrict__ di0, const T* __restrict__ f, const T* __restrict__ z,
+                         T* __restrict__ f0, T* __restrict__ x0, const DevState* st) {
+  wait_prior_grid();
+  if (st->done) return;
+  const int64_t n = kExactRed<S> ? g.Nh : g.N;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+    const int color = kExactRed<S> || t >= g.Nh;
+    const int64_t q = kExactRed<S> ? t : t - color * g.Nh;
+    const Cell c = decode(g, color, q);
+    T acc = T(0), diag = T(0);
+    // (every slot's loads are issued; a missing neighbour reads this cell's
+    // own entries and is masked to zero)
+#pragma unroll
+    for (int sl = 0; sl < 7; ++sl) {
+      const int64_t nb = nbr(g, c, q, sl);
+      const bool ok = nb >= 0;
+      const int64_t nq = ok ? nb : q;
+      const int xc = (sl == kDiag || !ok) ? color : (color ^ 1);
+      T z0 = z[vidx(g, 0, xc, nq)], z1 = z[vidx(g, 1, xc, nq)], z2 = z[vidx(g, 2, xc, nq)];
+      if (!ok) z0 = z1 = z2 = T(0);
+      const S* a = At + at_index(g, color, sl * 9, q);
+      constexpr size_t P = 32;  // entries (rc) of a block lie 32 apart in a tile
+      const T a0 = cv<T>(ld_stream(a));
+      if (sl == kDiag) diag = a0;
+      acc = fma3(acc, a0, z0, cv<T>(ld_stream(a + P)), z1, cv<T>(ld_stream(a + 2 * P)), z2);
+    }
+    const size_t o = (size_t)color * g.Nh + q;
+    const T r = f[o] - acc;
+    f0[o] = r;
+    if (kExactRed<S>) {
+      f0[q] = T(0);
+      x0[q] = T(0);
+      x0[o] = gs_divide(r, diag, di0, o);
+    }
+  }
+}
+
+// w_r = z_r - D_r^{-1} sum_b A_rb Pi_p e_b, or w_r = x2_r + D_r^{-1} (f - A x2)_r
+template <typename T, typename S>
+__global__ void __launch_bounds__(kThreads, kExactRed<S> && sizeof(T) == 4 ? 5 : 4) k_cpr_red(Geom g, const S* __restrict__ At,
+                         const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ z,
+                         const T* __restrict__ e, T* __restrict__ w, const DevState* st) {
+  wait_prior_grid();
+  if (st->done) return;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
+    const Cell c = decode(g, 0, q);
+    T x[3], s[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[k] = z[vidx(g, k, 0, q)];
+    if (!kExactRed<S>) x[0] += e[q];
+#pragma unroll
+    for (int sl = 0; sl < 7; ++sl) {
+      const S* a = At + at_index(g, 0, sl * 9, q);
+      constexpr size_t P = 32;  // entries (rc) of a block lie 32 apart in a tile
+      if (kExactRed<S>) {
+        if (sl == kDiag) continue;
+        const int64_t nb = nbr(g, c, q, sl);
+        const T en = e[g.Nh + (nb >= 0 ? nb : q)];
+        const T xn = nb >= 0 ? -en : T(0);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k] = fma(cv<T>(ld_stream(a + 3 * k * P)), xn, s[k]);
+      } else {
+        const int64_t nb = nbr(g, c, q, sl);
+        const bool ok = nb >= 0;
+        const int64_t nq = ok ? nb : q;
+        T x0 = x[0], x1 = x[1], x2 = x[2];
+        if (sl != kDiag) {
+          x0 = z[vidx(g, 0, 1, nq)] + e[g.Nh + nq], x1 = z[vidx(g, 1, 1, nq)], x2 = z[vidx(g, 2, 1, nq)];
+          if (!ok) x0 = x1 = x2 = T(0);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          s[k] = fma3(s[k], cv<T>(ld_stream(a + 3 * k * P)), x0, cv<T>(ld_stream(a + (3 * k + 1) * P)), x1,
+                      cv<T>(ld_stream(a + (3 * k + 2) * P)), x2);
+      }
+    }
+    if (!kExactRed<S>) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) s[k] = f[vidx(g, k, 0, q)] - s[k];
+    }
+    T d[9];
+#pragma unroll
+    for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      w[vidx(g, k, 0, q)] = x[k] + (d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2]);
+  }
+}
+
+// x3_b = x2_b + D_b'^{-1} (f_b - A_bb x2_b - A_br w_r), x2_b = z_b + Pi_p e_b:
+// the preconditioner's result, and x3_b (BF16: u_b) into xb for the red pass
+template <typename T, typename S>
+__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_cpr_black(Geom g, const S* __restrict__ At,
+                         const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ w,
+                         const T* __restrict__ z, const T* __restrict__ e, T* __restrict__ xb, OutV zo,
+                         const DevState* st) {
+  wait_prior_grid();
+  if (st->done) return;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
+    const Cell c = decode(g, 1, q);
+    T s[3];
+    offdiag_sum(g, At, 1, q, c, w, s);
+    const T x0 = z[vidx(g, 0, 1, q)] + e[g.Nh + q], x1 = z[vidx(g, 1, 1, q)], x2 = z[vidx(g, 2, 1, q)];
+    const S* a = At + at_index(g, 1, kDiag * 9, q);
+    T r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      r[k] = f[vidx(g, k, 1, q)] - fma3(s[k], cv<T>(ld_stream(a + 96 * k)), x0, cv<T>(ld_stream(a + 96 * k + 32)), x1,
+                                        cv<T>(ld_stream(a + 96 * k + 64)), x2);
+    T d[9];
+#pragma unroll
+    for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + g.Nh + q]);
+    const T x[3] = {x0, x1, x2};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T u = d[3 * k] * r[0] + d[3 * k + 1] * r[1] + d[3 * k + 2] * r[2];
+      xb[vidx(g, k, 1, q)] = kExactRed<S> ? x[k] + u : u;
+      out_put<T>(zo, vidx(g, k, 1, q), x[k] + u);
+    }
+  }
+}
 
 // ---- AMG level 0 (colour-split, coefficients = plane (colour, slot, 0) of At)
 // One cell of a level-0 Gauss-Seidel half sweep.
@@ -1588,6 +1677,7 @@ struct CycleArgs {
   int legs_to;    // the down and up legs smooth levels 0 .. legs_to - 1
   int fold_to;    // levels below it get their zero-guess red half sweep with the restriction
   int nu1, nu2;
+  int cpr;  // see amg_vcycle
   T s;
   unsigned spins;  // polls of a grid barrier before it gives up (BO_ERR_TIMEOUT)
   LevelView<T, S> lv[24];
@@ -1600,7 +1690,7 @@ template <typename T, typename S>
 __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
   const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
   const Geom& g = a.g;
-  for (int sw = 0; sw < a.nu1; ++sw)
+  for (int sw = a.cpr; sw < a.nu1; ++sw)
     for (int color = 0; color < 2; ++color) {
       const int zero = sw == 0 && color == 0;
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + (size_t)color * g.Nh,
@@ -1682,6 +1772,7 @@ __device__ bool amg_up(const CycleArgs<T, S>& a, DevState* st) {
     else
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + g.Nh,
                        [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, 1, 0, q); });
+    if (a.cpr && sw + 1 == a.nu2) break;  // (the red cells are not read any more)
     if (!grid_barrier(st, a.spins)) return false;
     sweep_batched<4>(t0, nt, g.Nh, a.x0, [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, 0, 0, q); });
     if (sw + 1 < a.nu2 && !grid_barrier(st, a.spins)) return false;
@@ -1989,12 +2080,13 @@ __device__ __forceinline__ T res_gather(const ResLevel& r, uint32_t base, int32_
 // Every block of the cluster runs it when the level is shared (DIST), block
 // 0 alone otherwise.
 template <typename T, bool DIST>
-__device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l, uint32_t base) {
+__device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l, uint32_t base, int cpr) {
   constexpr int NP = res_pairs<T>();
   ResCells<T, NP> r;
   res_load<T, NP, DIST>(a, l, base, r);
   const ResLevel& rl = a.rl[l];
   const int32_t q0 = DIST ? (int32_t)blockIdx.x << rl.lch : 0;
+  const bool whole = cpr && l == 0;
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     const int32_t i = (int32_t)threadIdx.x + kResThreads * p, q = q0 + i;
@@ -2011,14 +2103,15 @@ __device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l,
       if (place) st_sh(res_local<T>(rl, base, kSecF + col, q), f);
     }
     // the first half sweep starts from zero: x_r = f_r / d_r (black zero
-    // until its own half sweep)
+    // until its own half sweep; within the CPR level 0's f_r is zero, which
+    // makes that x_b = f_b / d_b)
     if (place) {
       st_sh(res_local<T>(rl, base, kSecRed, q), r.live[0][p] ? res_divide(r.f[0][p], r.d[0][p]) : T(0));
-      st_sh(res_local<T>(rl, base, kSecBlack, q), T(0));
+      st_sh(res_local<T>(rl, base, kSecBlack, q), whole && r.live[1][p] ? res_divide(r.f[1][p], r.d[1][p]) : T(0));
     }
   }
   res_barrier<DIST>();
-  res_sweep<T, NP, DIST>(r, 1);
+  if (!whole) res_sweep<T, NP, DIST>(r, 1);
   for (int sw = 1; sw < a.nu1; ++sw) {
     res_sweep<T, NP, DIST>(r, 0);
     res_sweep<T, NP, DIST>(r, 1);
@@ -2043,7 +2136,7 @@ __device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l,
 
 // Coarse correction and post-smoothing of level l
 template <typename T, bool DIST>
-__device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, uint32_t base) {
+__device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, uint32_t base, int cpr) {
   constexpr int NP = res_pairs<T>();
   ResCells<T, NP> r;
   res_load<T, NP, DIST>(a, l, base, r);
@@ -2073,6 +2166,7 @@ __device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, u
   res_barrier<DIST>();
   for (int sw = 0; sw < a.nu2; ++sw) {
     res_sweep<T, NP, DIST>(r, 1);
+    if (cpr && l == 0 && sw + 1 == a.nu2) break;
     res_sweep<T, NP, DIST>(r, 0);
   }
   if (l == a.l0) {
@@ -2092,7 +2186,7 @@ __device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, u
 
 template <typename T, typename S>
 __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_constant__ ResPlan a, Geom g,
-                                                                const DevState* st) {
+                                                                int cpr, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;  // uniform: every block reads the same flag
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(g_tail_smem);
@@ -2109,12 +2203,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_co
   }
   cluster_sync_all();  // every block runs before its shared memory is read
   int l = a.l0;
-  for (; l < a.last && a.rl[l].dist; ++l) res_down<T, true>(a, g, l, base);
+  for (; l < a.last && a.rl[l].dist; ++l) res_down<T, true>(a, g, l, base, cpr);
   const int shared_to = l;
   if (first) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    for (; l < a.last; ++l) res_down<T, false>(a, g, l, base);
+    for (; l < a.last; ++l) res_down<T, false>(a, g, l, base, cpr);
     // the coarsest level: x = inv f, a thread per row (inv is stored transposed)
     const uint32_t fo = base + a.dense_off;
     const ResLevel& rl = a.rl[a.last];
@@ -2131,10 +2225,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_co
       if (a.l0 == a.last) ((T*)rl.x)[i] = s;
     }
     __syncthreads();
-    for (l = a.last - 1; l >= shared_to; --l) res_up<T, false>(a, g, l, base);
+    for (l = a.last - 1; l >= shared_to; --l) res_up<T, false>(a, g, l, base, cpr);
   }
   cluster_sync_all();
-  for (l = shared_to - 1; l >= a.l0; --l) res_up<T, true>(a, g, l, base);
+  for (l = shared_to - 1; l >= a.l0; --l) res_up<T, true>(a, g, l, base, cpr);
   cluster_sync_all();  // no block leaves while another may read its shared memory
 }
 
@@ -2305,8 +2399,11 @@ void resident_plan(bo_prec* P, ResPlan& a) {
   a.cluster = C;
 }
 
+// cpr: within the CPR of an FP64 or FP32 preconditioner, whose k_cpr_rhs has done the first pre-smoothing sweep
+// (if nu1 > 0) and which never reads the red cells of level 0 afterwards, so
+// the last post-smoothing half sweep is left out too.
 template <typename T, typename S>
-void amg_vcycle(bo_prec* P, const DevState* st) {
+void amg_vcycle(bo_prec* P, const DevState* st, bool cpr) {
   cudaStream_t s = P->stream;
   const Geom& g = P->mat->g;
   const S* At = (const S*)P->At;
@@ -2367,7 +2464,7 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, k_amg_resident<T, S>, ra, g, st) != cudaSuccess) return false;
+    if (cudaLaunchKernelEx(&cfg, k_amg_resident<T, S>, ra, g, (int)cpr, st) != cudaSuccess) return false;
     note_launch();
     return true;
   };
@@ -2388,6 +2485,7 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
   ca.fold_to = std::min(P->tail_from, res_from);
   ca.nu1 = nu1;
   ca.nu2 = nu2;
+  ca.cpr = cpr;
   ca.s = sc;
   ca.spins = g_amg_spins.load();
   for (int l = 1; l <= last; ++l) ca.lv[l] = view<T, S>(P, l);
@@ -2465,7 +2563,7 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
     else cudaGetLastError();
   }
   if (!down_done) {
-    for (int sw = 0; sw < nu1; ++sw) {
+    for (int sw = cpr; sw < nu1; ++sw) {
       gs0(0, sw == 0);
       gs0(1, 0);
     }
@@ -2507,7 +2605,7 @@ void amg_vcycle(bo_prec* P, const DevState* st) {
   for (int sw = 0; sw < nu2; ++sw) {
     if (sw == 0) gs0_prolong();
     else gs0(1, 0);
-    gs0(0, 0);
+    if (!cpr || sw + 1 < nu2) gs0(0, 0);
   }
 }
 
@@ -2521,13 +2619,12 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
   const S* D = (const S*)P->Dinv;
   T* f = (T*)P->f;
   T* tv = (T*)P->t;
-  T* r = (T*)P->r;
   T* e0 = (T*)P->e0;
   T* f0 = (T*)P->f0;
   T* z1 = (T*)P->z1;
   if (stage == BO_STAGE_AMG) {  // (v is a caller's FP64 vector here: vs is NULL)
     (launch_pdl(k_copy_vec<T>, gN, kThreads, 0, s, g.N, v.d, f0, st), note_launch());
-    amg_vcycle<T, S>(P, st);
+    amg_vcycle<T, S>(P, st, false);
     learned_coarse_apply(P, st);
     (launch_pdl(k_place_p<T>, gN, kThreads, 0, s, g, e0, zo.d, st), note_launch());
     return;
@@ -2541,31 +2638,30 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
     (launch_pdl(k_cpr_entry<T, S, false>, occ_grid((const void*)k_cpr_entry<T, S, false>, g.N), kThreads, 0, s, g, v, vs, P->w, P->wf,
         D, f, tv, st),
      note_launch());
-  (launch_pdl(k_ilu_b<T, S, false>, occ_grid((const void*)k_ilu_b<T, S, false>, g.Nh), kThreads, 0, s, g, At, D, f, tv, z1, nullptr,
-      OutV{}, st),
+  (launch_pdl(k_ilu_b<T, S>, occ_grid((const void*)k_ilu_b<T, S>, g.Nh), kThreads, 0, s, g, At, D, f, tv, z1, st),
    note_launch());
-  // (ub and z are both z1: the pass reads its black half and writes its red half)
-  (launch_pdl(k_ilu_r2<T, S, false>, occ_grid((const void*)k_ilu_r2<T, S, false>, g.Nh), kThreads, 0, s, g, At, D, tv, z1, z1,
-      nullptr, OutV{}, st),
+  // (the pass reads z1's black half and writes its red half)
+  (launch_pdl(k_ilu_r2<T, S, false, false>, occ_grid((const void*)k_ilu_r2<T, S, false, false>, g.Nh), kThreads, 0, s, g, At, D, f, z1, z1,
+      OutV{}, st),
    note_launch());
   if (stage == BO_STAGE_ILU) {
     (launch_pdl(k_widen_t<T>, grid_for(3 * g.N), kThreads, 0, s, 3 * g.N, z1, zo.d, st), note_launch());
     return;
   }
   // x2 = x1 + Pi_p AMG(A_pp)^{-1} Pi_r (f - At x1)
-  (launch_pdl(k_cpr_residual<T, S, 1>, occ_grid((const void*)k_cpr_residual<T, S, 1>, g.N), kThreads, 0, s, 
-       g, At, f, z1, nullptr, f0, nullptr, nullptr, st),
+  (launch_pdl(k_cpr_rhs<T, S>, occ_grid((const void*)k_cpr_rhs<T, S>, kExactRed<S> ? g.Nh : g.N), kThreads, 0, s, g, At, (const T*)P->di0, f, z1,
+      f0, e0, st),
    note_launch());
-  amg_vcycle<T, S>(P, st);
+  amg_vcycle<T, S>(P, st, kExactRed<S>);
   learned_coarse_apply(P, st);
-  // r = f - At x2 (with the red pass of R^{-1} r fused);  x3 = x2 + R^{-1} r
-  (launch_pdl(k_cpr_residual<T, S, 3>, occ_grid((const void*)k_cpr_residual<T, S, 3>, g.N), kThreads, 0, s, g, At, f, z1, e0, r,
-      D, tv, st),
-   note_launch());
-  (launch_pdl(k_ilu_b<T, S, true>, occ_grid((const void*)k_ilu_b<T, S, true>, g.Nh), kThreads, 0, s, g, At, D, r, tv, z1, e0, zo,
+  // x3 = x2 + R^{-1} (f - At x2)
+  (launch_pdl(k_cpr_red<T, S>, occ_grid((const void*)k_cpr_red<T, S>, g.Nh), kThreads, 0, s, g, At, D, f, z1, e0, tv,
       st),
    note_launch());
-  (launch_pdl(k_ilu_r2<T, S, true>, occ_grid((const void*)k_ilu_r2<T, S, true>, g.Nh), kThreads, 0, s, g, At, D, tv, tv, z1, e0,
+  (launch_pdl(k_cpr_black<T, S>, occ_grid((const void*)k_cpr_black<T, S>, g.Nh), kThreads, 0, s, g, At, D, f, tv, z1, e0, tv,
+      zo, st),
+   note_launch());
+  (launch_pdl(k_ilu_r2<T, S, true, !kExactRed<S>>, occ_grid((const void*)k_ilu_r2<T, S, true, !kExactRed<S>>, g.Nh), kThreads, 0, s, g, At, D, f, tv, nullptr,
       zo, st),
    note_launch());
 }
@@ -2648,7 +2744,6 @@ int prec_alloc(bo_prec* P) {
   P->di0 = ss == sizeof(double) ? (double*)al((size_t)g.N * sizeof(double)) : nullptr;
   P->f = al((size_t)3 * g.N * ts);
   P->t = al((size_t)3 * g.N * ts);
-  P->r = al((size_t)3 * g.N * ts);
   P->z1 = al((size_t)3 * g.N * ts);
   P->e0 = al((size_t)g.N * ts);
   P->f0 = al((size_t)g.N * ts);
@@ -2702,7 +2797,7 @@ int prec_alloc(bo_prec* P) {
 void prec_free(bo_prec* P) {
   auto fr = [](void* p) { if (p) cudaFree(p); };
   fr(P->At); fr(P->w); fr(P->wf); fr(P->Dinv); fr(P->di0);
-  fr(P->f); fr(P->t); fr(P->r); fr(P->z1); fr(P->e0); fr(P->f0);
+  fr(P->f); fr(P->t); fr(P->z1); fr(P->e0); fr(P->f0);
   for (int l = 1; l < P->nlev; ++l) { fr(P->lev[l].c64); fr(P->lev[l].c); fr(P->lev[l].f); fr(P->lev[l].x); }
   fr(P->coarse_inv); fr(P->st);
   if (P->res) {
