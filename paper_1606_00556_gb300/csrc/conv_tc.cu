@@ -19,30 +19,34 @@
 // one run loses nothing, its neighbours outside the grid being zero.
 // TX in {16, 32, 64, 128} is the one with the fewest tiles for the grid.
 //
-// Shared memory holds planes of (TY + 2) x TX voxels, one 16-byte row of 8
-// channels per voxel, chunk by chunk ([channel / 8][voxel][8 channels]): eight
-// consecutive voxels are a core matrix of the no-swizzle K-major operand
-// layout, and a (dz, dy) tap is a descriptor on plane z + dz that starts (dy
-// + 1) runs in.  A CTA marches along z through a column of tiles, so each
-// plane is loaded once per column and serves three tiles; the tiles of all
-// columns are dealt to the CTAs in contiguous ranges of equal length.  The
-// planes are fetched with cp.async by four producer warps (128 contiguous
-// bytes per pair of voxels, out-of-grid voxels zero-filled): TMA boxes for
-// this chunked layout have 16-byte inner rows, and the form before this one,
-// which fetched a 10 x 18 x 3 halo per tile that way, was bound by them
-// (2160 rows, about 3.5 us a tile whose MMAs need 1.1 us).
+// Shared memory holds planes of (TY + 2) x TX voxels, a row of channels (64
+// or 32 bytes, swizzled over its length) per voxel: one TMA box a plane, which
+// is a K-major operand as it lies, and a (dz, dy) tap is a descriptor on plane
+// z + dz that starts (dy + 1) runs in (a multiple of the swizzle's period).
+// The weights are 9 boxes of 3 Cout rows, or for the data gradient 27 boxes
+// in reversed order that are used with N contiguous, so that nothing is
+// transposed.  A CTA marches along z through a column of tiles, so each plane
+// is loaded once per column and serves three tiles; the tiles of all columns
+// are dealt to the CTAs in contiguous ranges of equal length.
 //
-// One CTA of 13 warps per SM: warp 0 issues the MMAs (one elected thread),
-// warps 1-8 form the epilogue, warps 9-12 produce; six plane buffers and two
-// TMEM accumulators let all three overlap.  Every wait on an mbarrier is
-// bounded: on expiry the CTA records an error, finishes its copies and MMAs
-// in flight (again bounded), frees its TMEM and returns.
+// One CTA of 18 warps per SM: warp 0 issues the MMAs, warp 1 the TMA copies,
+// four groups of four warps form the epilogue, each group of every fourth
+// tile; up to ten plane buffers and four TMEM accumulators let all three
+// overlap.  Every wait on an mbarrier is bounded: on expiry the CTA records an
+// error, finishes its copies and MMAs in flight (again bounded), frees its
+// TMEM and returns.
 // Measured, 64x64x32 voxels x 4 samples, 32 -> 32 channels: forward with
-// residual 103 -> 63 us a call, data gradient 150 -> 86 us a call (61 us of
-// it the kernel, the rest the call's synchronisation).
+// residual 103 us a call on the first tcgen05 form (a tap per MMA, a 10 x 18 x
+// 3 halo a tile in 16-byte TMA rows), 63 with the x taps in N and planes copied
+// by cp.async in 16-byte chunks, 40 in this form; data gradient 150, 82 and 57
+// (about 20 of it the call's synchronisation).  Per tile of 2250 cycles the
+// MMAs take 900 to issue and execute, their commits and waits 900, and the
+// epilogue, two shuffles per output, 1150 of its four groups.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
-#include <cstring>
+#include <mutex>
 
 #include "bo_internal.cuh"
 
@@ -51,31 +55,45 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int kTcThreads = 416;      // warp 0: MMA issue; 1-8: epilogue; 9-12: producers
-constexpr int kProducers = 128;
-constexpr int kPlanes = 6;           // plane buffers: three of a tile, three on their way
-constexpr int kAhead = 2;            // planes a producer leaves in flight before it signals the oldest
-constexpr long kSpinLimit = 1l << 26;
+constexpr int kGroups = 4;           // groups of four epilogue warps
+constexpr int kTcThreads = 64 + 128 * kGroups;  // warp 0: MMA issue; 1: TMA; the others: epilogue
+constexpr int kMaxPlanes = 10;       // plane buffers: three of a tile, the others on their way or signalled
+constexpr int kAccs = 4;             // accumulators (128 TMEM columns each)
+constexpr int kSpinLimit = 1 << 26;
 constexpr int kTileM = 128;
+constexpr int kTcSmem = 227 * 1024;  // shared memory of a block
 
 __device__ int g_tc_err;  // set by a CTA whose wait expired (read and cleared by bo_tc_status)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// shared-memory matrix descriptor, no swizzle, version 1: the strides between
-// core matrices (8 rows of 16 bytes) along K (lbo) and along M or N (sbo)
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+// shared-memory matrix descriptor, version 1.  No swizzle (span 16): lbo and
+// sbo are the strides between core matrices (8 rows of 16 bytes) along K and
+// along M or N.  Rows of 32 or 64 bytes swizzled over that span, as TMA writes
+// them: sbo is the stride between groups of 8 rows; with M or N contiguous lbo
+// is the stride between spans along it (else not used).
+__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo, int span = 16) {
   return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
+         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)(span == 64 ? 4 : span == 32 ? 6 : 0) << 61);
 }
 
-// instruction descriptor, kind::f16: D FP32, A and B BF16, M = 128; MN: both
-// operands with M (N) contiguous in memory instead of K
-__host__ __device__ constexpr uint32_t idesc(int n, bool mn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(n >> 3) << 17) |
+// instruction descriptor, kind::f16: D FP32, A and B BF16, M = 128; am, bn:
+// A (B) with M (N) contiguous in memory instead of K
+__host__ __device__ constexpr uint32_t idesc(int n, bool am, bool bn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (am ? 1u << 15 : 0u) | (bn ? 1u << 16 : 0u) | ((uint32_t)(n >> 3) << 17) |
          ((128u >> 4) << 24);
 }
 
+// one thread of a converged warp (always the same)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
+}
+// (issued by the thread that elect_one picks, for a whole tile in one branch:
+// 45 cycles an MMA.  An elect.sync per MMA took 60, and a branch on lane == 0,
+// which the compiler does not know to be one thread, 92.)
 __device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, bool acc) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
@@ -84,15 +102,17 @@ __device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_
       : "memory");
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// (stop: where not NULL, the flag of another role's failure, which ends the wait)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const volatile int* stop = nullptr) {
   uint32_t done = 0;
-  for (long it = 0; it < kSpinLimit; ++it) {
+  for (int it = 0; it < kSpinLimit; ++it) {
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
+    if (stop && (it & 255) == 255 && *stop) return false;
   }
   return false;
 }
@@ -109,6 +129,22 @@ __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.
 // 16 bytes from global to shared memory, or zeros
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
+}
+// 32 bytes to global memory: one store where the address allows it (wide),
+// which fills a sector, or two of 16 bytes
+__device__ __forceinline__ void st32(void* p, bool wide, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f,
+                                     uint32_t g, uint32_t h) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f),
+                 "r"(g), "r"(h)
+                 : "memory");
+  } else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(a, b, c, d);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(e, f, g, h);
+  }
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -154,289 +190,352 @@ __device__ __forceinline__ void tmem_ld3(uint32_t a0, uint32_t a1, uint32_t a2, 
 struct ConvGrid {
   int nx, ny, nz, B;
   int ltx;              // log2 TX
+  int planes;           // plane buffers
   int ntx, nty;
   int64_t tiles;
 };
-struct Column {
-  int x0, y0, b;
+// A tile's place, stepped from tile to tile (a division once per CTA)
+struct March {
+  int z, tx, ty, b;
+  __device__ __forceinline__ March(const ConvGrid& g, int64_t t) {
+    const int c = (int)(t / g.nz);
+    z = (int)(t - (int64_t)c * g.nz);
+    tx = c % g.ntx;
+    ty = c / g.ntx % g.nty;
+    b = c / g.ntx / g.nty;
+  }
+  __device__ __forceinline__ void next(const ConvGrid& g) {
+    if (++z < g.nz) return;
+    z = 0;
+    if (++tx < g.ntx) return;
+    tx = 0;
+    if (++ty < g.nty) return;
+    ty = 0;
+    ++b;
+  }
+  __device__ __forceinline__ int x0(const ConvGrid& g) const { return tx * ((1 << g.ltx) - 2); }
+  __device__ __forceinline__ int y0(const ConvGrid& g) const { return ty * (kTileM >> g.ltx); }
 };
-__device__ __forceinline__ Column column_of(const ConvGrid& g, int64_t t) {
-  const int c = (int)(t / g.nz);
-  const int tx = c % g.ntx, r = c / g.ntx;
-  const int TX = 1 << g.ltx;
-  return Column{tx * (TX - 2), (r % g.nty) * (kTileM >> g.ltx), r / g.nty};
-}
 __host__ __device__ __forceinline__ int plane_rows(int ltx) { return kTileM + (2 << ltx); }
-// bytes of one channel chunk of a plane; the padding puts the chunks of a
-// voxel, which one quarter warp writes together, in different banks
-__host__ __device__ __forceinline__ int chunk_stride(int ltx, int kc) { return plane_rows(ltx) * 16 + 128 / kc; }
 
 template <int CIN, int COUT>
 struct ConvLayout {
-  static constexpr int KC = CIN / 8;
   static constexpr int NB = 3 * COUT;
-  static constexpr int kW = 9 * KC * NB * 16;
-  static constexpr int kEdge = 2 * 2 * 2 * 4 * 16 * 4;  // [tile parity][side][channel half][warp][channel]
+  static constexpr int kW = 9 * CIN * NB * 2;
+  static constexpr int kEdge = kGroups * 2 * 2 * 4 * 16 * 4;  // [warp group][buffer][side][warp][channel]
   static constexpr int kOffEdge = kW;
   static constexpr int kOffBias = kOffEdge + kEdge;
   static constexpr int kOffBar = kOffBias + 128;
-  static constexpr int kOffPlanes = kOffBar + 256;
+  static constexpr int kOffPlanes = (kOffBar + 256 + 1023) / 1024 * 1024;  // (29 barriers and the TMEM address)
 };
+
+__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_rows(const CUtensorMap* map, uint32_t dst, uint32_t bar, int row) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_plane(const CUtensorMap* map, uint32_t dst, uint32_t bar, int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(
+          dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
 
 // OUT 0: Y = ReLU(conv + bias (+ R)) in BF16; 1: Yf = conv + bias in FP32;
 // 2: Y = conv + bias in BF16 and its channels 0..3 in FP32 (Yf[v][4]).
-// TRANSPOSED: the data gradient's weights (see the head of the file).
-// mbarriers: full[p] plane buffer p holds its plane (128 producer arrivals);
-// empty[p] the MMAs that read it are done; accfull[a], accempty[a] (8 warps)
-// as the accumulators pass between the MMAs and the epilogue.  The n-th
+// TRANSPOSED: the data gradient, W [27][CIN][COUT] (the layer's own output
+// channels are this convolution's inputs).
+// mbarriers: full[p] plane buffer p holds its plane; empty[p] the MMAs that
+// read it are done; accfull[a], accempty[a] (4 warps) as the accumulators pass
+// between the MMAs and the epilogue; wfull the weights are there.  The n-th
 // completion of a barrier has parity n & 1.
 template <int CIN, int COUT, int OUT, bool RES, bool TRANSPOSED>
 __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_constant__ ConvGrid g,
-                                                           const bf16* __restrict__ X, const bf16* __restrict__ W,
+                                                           const __grid_constant__ CUtensorMap xmap,
+                                                           const __grid_constant__ CUtensorMap wmap,
                                                            const float* __restrict__ bias, const bf16* __restrict__ R,
                                                            bf16* __restrict__ Y, float* __restrict__ Yf) {
   using L = ConvLayout<CIN, COUT>;
-  constexpr int KC = L::KC, NB = L::NB;
-  constexpr int CH = COUT / 2;  // channels of an epilogue thread
+  constexpr int NB = L::NB;
+  constexpr int CH = RES || COUT == 16 ? 8 : 16;  // channels an epilogue thread takes at a time (registers)
   extern __shared__ uint8_t smraw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 127) & ~uintptr_t(127));
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   float* edge = reinterpret_cast<float*>(sm + L::kOffEdge);
   float* sbias = reinterpret_cast<float*>(sm + L::kOffBias);
   const uint32_t bars = smem_u32(sm + L::kOffBar);
   auto full = [&](int p) { return bars + 8 * p; };
-  auto empty = [&](int p) { return bars + 8 * (kPlanes + p); };
-  auto accfull = [&](int a) { return bars + 8 * (2 * kPlanes + a); };
-  auto accempty = [&](int a) { return bars + 8 * (2 * kPlanes + 2 + a); };
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + L::kOffBar + 8 * (2 * kPlanes + 4));
+  auto empty = [&](int p) { return bars + 8 * (kMaxPlanes + p); };
+  auto accfull = [&](int a) { return bars + 8 * (2 * kMaxPlanes + a); };
+  auto accempty = [&](int a) { return bars + 8 * (2 * kMaxPlanes + kAccs + a); };
+  const uint32_t wfull = bars + 8 * (2 * kMaxPlanes + 2 * kAccs);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + L::kOffBar + 8 * (2 * kMaxPlanes + 2 * kAccs + 1));
   volatile int* sfail = reinterpret_cast<volatile int*>(tslot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int p = 0; p < kPlanes; ++p) {
-      mbar_init(full(p), kProducers);
+    for (int p = 0; p < kMaxPlanes; ++p) {
+      mbar_init(full(p), 1);
       mbar_init(empty(p), 1);
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < kAccs; ++a) {
       mbar_init(accfull(a), 1);
-      mbar_init(accempty(a), 8);
+      mbar_init(accempty(a), 4);
     }
+    mbar_init(wfull, 1);
     *sfail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;\n" ::"r"(smem_u32(tslot)));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_u32(tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
+  if (tid >= 64 && tid < 64 + COUT) sbias[tid - 64] = bias ? bias[tid - 64] : 0.f;
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tslot;
-  const int TX = 1 << g.ltx, rows = plane_rows(g.ltx), cs = chunk_stride(g.ltx, KC);
-  const uint32_t pbase = smem_u32(sm + L::kOffPlanes), pstride = (uint32_t)(KC * cs);
+  const int TX = 1 << g.ltx;
+  const uint32_t wbase = smem_u32(sm);
+  const uint32_t pbase = smem_u32(sm + L::kOffPlanes), pbytes = (uint32_t)(plane_rows(g.ltx) * CIN * 2);
   const int64_t t0 = g.tiles * blockIdx.x / gridDim.x, t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
   const int64_t V = (int64_t)g.nx * g.ny * g.nz;
+  const bool wide = ((reinterpret_cast<uintptr_t>(Y) | reinterpret_cast<uintptr_t>(Yf)) & 31) == 0;
 
-  if (warp >= 9) {
-    // ---- producers
-    const int pt = tid - 9 * 32;
-    const bf16* Xc = X + (size_t)(pt % KC) * 8;
-    int seq = 0, done = 0;
-    bool ok = true;
-    auto signal_to = [&](int n) {  // planes before n have landed (the caller's cp_wait)
-      fence_async_proxy();
-      for (; done < n; ++done) mbar_arrive(full(done % kPlanes));
-    };
-    for (int64_t t = t0; t < t1 && ok; ++t) {
-      const int z = (int)(t % g.nz);
-      const bool start = t == t0 || z == 0;
-      const Column c = column_of(g, t);
-      for (int pz = start ? max(z - 1, 0) : z + 1; pz <= min(z + 1, g.nz - 1) && ok; ++pz) {
-        if (seq >= kPlanes) ok = !*sfail && mbar_wait(empty(seq % kPlanes), (seq / kPlanes - 1) & 1);
-        if (!ok) break;
-        const uint32_t dst = pbase + (uint32_t)(seq % kPlanes) * pstride + (uint32_t)(pt % KC) * cs;
-        const size_t zb = (size_t)c.b * V + (size_t)pz * g.nx * g.ny;
-        for (int r = pt / KC; r < rows; r += kProducers / KC) {
-          const int x = c.x0 + (r & (TX - 1)), y = c.y0 - 1 + (r >> g.ltx);
-          const bool in = x < g.nx && y >= 0 && y < g.ny;
-          cp16(dst + (uint32_t)r * 16, Xc + (in ? (zb + (size_t)y * g.nx + x) * CIN : 0), in);
-        }
-        cp_commit();
-        ++seq;
-        cp_wait<kAhead>();
-        if (seq > kAhead) signal_to(seq - kAhead);
+  if (warp == 1) {
+    // ---- TMA: the weights and the planes
+    if (elect_one() && t0 < t1) {
+      expect_tx(wfull, (uint32_t)L::kW);
+      if (!TRANSPOSED) {
+        for (int i = 0; i < 9; ++i) tma_rows(&wmap, wbase + (uint32_t)(i * CIN * NB * 2), wfull, i * NB);
+      } else {
+        for (int i = 0; i < 27; ++i) tma_rows(&wmap, wbase + (uint32_t)(i * CIN * COUT * 2), wfull, (26 - i) * CIN);
       }
-    }
-    cp_wait<0>();
-    if (ok) {
-      signal_to(seq);
-    } else {
-      *sfail = 1;
-      atomicExch(&g_tc_err, 1);
-    }
-  } else {
-    // ---- weights into shared memory (warps 0-8): [dz, dy][channel chunk][dx, co][8 channels]
-    if (!TRANSPOSED) {
-      for (int i = tid; i < 27 * COUT * KC; i += 288) {
-        const int kc = i % KC, r = i / KC, co = r % COUT, t = r / COUT;
-        const uint4 w = *reinterpret_cast<const uint4*>(W + ((size_t)(t * COUT + co) * CIN + kc * 8));
-        *reinterpret_cast<uint4*>(sm + (((t / 3) * KC + kc) * NB + (t % 3) * COUT + co) * 16) = w;
-      }
-    } else {
-      // W is [27][CIN][COUT] here (the layer's own output channels are this convolution's inputs)
-      for (int i = tid; i < 27 * CIN * (COUT / 8); i += 288) {
-        const int cg = i % (COUT / 8), r = i / (COUT / 8), ci = r % CIN, t = 26 - r / CIN;
-        const uint4 w = *reinterpret_cast<const uint4*>(W + ((size_t)r * COUT + cg * 8));
-        const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
-        uint8_t* d = sm + (((t / 3) * KC + ci / 8) * NB + (t % 3) * COUT + cg * 8) * 16 + (ci % 8) * 2;
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          *reinterpret_cast<unsigned short*>(d + 16 * e) = (unsigned short)(wv[e / 2] >> (16 * (e & 1)));
-      }
-    }
-    if (tid < COUT) sbias[tid] = bias ? bias[tid] : 0.f;
-    fence_async_proxy();
-    named_barrier(1, 288);
-    if (warp == 0) {
-      // ---- MMA issue
-      if (lane == 0 && t0 < t1) {
-        const uint32_t wbase = smem_u32(sm);
-        bool ok = true;
-        int waited = 0, next = 0, issued = 0;  // planes waited for; sequence number of the next tile's plane z
-        for (int64_t t = t0; t < t1 && ok; ++t) {
-          const int k = (int)(t - t0), a = k & 1;
-          const int z = (int)(t % g.nz);
-          const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
-          if (start) next = waited + (z > 0 ? 1 : 0);
-          const int need = next + (z < g.nz - 1 ? 1 : 0);
-          for (; waited <= need && ok; ++waited) ok = !*sfail && mbar_wait(full(waited % kPlanes), (waited / kPlanes) & 1);
-          if (ok && k >= 2) ok = mbar_wait(accempty(a), ((k >> 1) - 1) & 1);
+      int buf = 0, round = 0, seq = 0;  // the buffer and the round of the next plane; planes issued
+      bool ok = true;
+      March m(g, t0);
+      for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
+        const bool start = t == t0 || m.z == 0;
+        for (int pz = start ? max(m.z - 1, 0) : m.z + 1; pz <= min(m.z + 1, g.nz - 1); ++pz) {
+          if (round > 0) ok = mbar_wait(empty(buf), (round - 1) & 1, sfail);
           if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+          expect_tx(full(buf), pbytes);
+          tma_plane(&xmap, pbase + (uint32_t)buf * pbytes, full(buf), m.x0(g), m.y0(g) - 1, m.b * g.nz + pz);
+          ++seq;
+          if (++buf == g.planes) {
+            buf = 0;
+            ++round;
+          }
+        }
+      }
+      if (!ok) {
+        *sfail = 1;
+        atomicExch(&g_tc_err, 1);
+      }
+      // no copy is in flight when the block ends
+      mbar_wait(wfull, 0);
+      for (int k = max(0, seq - g.planes); k < seq; ++k) mbar_wait(full(k % g.planes), (k / g.planes) & 1);
+    }
+    __syncwarp();
+  } else if (warp == 0) {
+    // ---- MMA issue (the whole warp waits, one thread issues)
+    if (t0 < t1) {
+      bool ok = __all_sync(0xffffffffu, mbar_wait(wfull, 0));
+      // planes waited for, and the buffer and round of the next one; the
+      // buffer of the tile's plane z
+      int waited = 0, wbuf = 0, wround = 0, next = 0, cur = 0, issued = 0;
+      auto around = [&](int p) { return p < 0 ? p + g.planes : p >= g.planes ? p - g.planes : p; };
+      March m(g, t0);
+      for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
+        const int k = (int)(t - t0), a = k % kAccs, z = m.z;
+        const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
+        if (start) {
+          next = waited + (z > 0 ? 1 : 0);
+          cur = around(wbuf + (z > 0 ? 1 : 0));
+        }
+        const int need = next + (z < g.nz - 1 ? 1 : 0);
+        for (; waited <= need && ok; ++waited) {
+          ok = __all_sync(0xffffffffu, mbar_wait(full(wbuf), wround & 1, sfail));
+          if (++wbuf == g.planes) {
+            wbuf = 0;
+            ++wround;
+          }
+        }
+        if (ok && k >= kAccs) ok = __all_sync(0xffffffffu, mbar_wait(accempty(a), (k / kAccs - 1) & 1, sfail));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        if (elect_one()) {
           const uint32_t dacc = tmem + (uint32_t)(a * 128);
-          const uint64_t db0 = smem_desc(wbase, NB * 16, 128);
+          // weights: N rows of CIN channels, or for the data gradient CIN rows
+          // of COUT channels per x tap
+          const uint64_t db0 = TRANSPOSED ? smem_desc(wbase, CIN * COUT * 2, 16 * COUT, COUT * 2)
+                                          : smem_desc(wbase, 16, 16 * CIN, CIN * 2);
           bool acc = false;
           for (int dz = -1; dz <= 1; ++dz) {
             if (z + dz < 0 || z + dz >= g.nz) continue;
-            const uint64_t da0 = smem_desc(pbase + (uint32_t)((next + dz) % kPlanes) * pstride, (uint32_t)cs, 128);
-            const uint64_t dbz = db0 + (uint64_t)(((dz + 1) * 3 * KC * NB * 16) >> 4);
+            const uint64_t da0 = smem_desc(pbase + (uint32_t)around(cur + dz) * pbytes, 16, 16 * CIN, CIN * 2);
+            const uint64_t dbz = db0 + (uint64_t)(((dz + 1) * 3 * CIN * NB * 2) >> 4);
 #pragma unroll
             for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
-              for (int ks = 0; ks < KC / 2; ++ks) {
-                umma(dacc, da0 + (uint64_t)((2 * ks * cs + dy * TX * 16) >> 4),
-                     dbz + (uint64_t)(((dy * KC + 2 * ks) * NB * 16) >> 4), idesc(NB, false), acc);
+              for (int ks = 0; ks < CIN / 16; ++ks) {
+                umma(dacc, da0 + (uint64_t)((dy * TX * CIN * 2 + ks * 32) >> 4),
+                     dbz + (uint64_t)((dy * CIN * NB * 2 + (TRANSPOSED ? ks * 32 * COUT : ks * 32)) >> 4),
+                     idesc(NB, false, TRANSPOSED), acc);
                 acc = true;
               }
           }
-          if (z > 0) umma_commit(empty((next - 1) % kPlanes));
+          if (z > 0) umma_commit(empty(around(cur - 1)));
           if (end) {
-            umma_commit(empty(next % kPlanes));
-            if (z < g.nz - 1) umma_commit(empty((next + 1) % kPlanes));
+            umma_commit(empty(cur));
+            if (z < g.nz - 1) umma_commit(empty(around(cur + 1)));
           }
           umma_commit(accfull(a));
-          ++issued;
-          ++next;
         }
-        if (!ok) {
-          *sfail = 1;
-          atomicExch(&g_tc_err, 1);
-          // the MMAs in flight finish before shared and tensor memory go away
-          for (int k = max(0, issued - 2); k < issued; ++k) mbar_wait(accfull(k & 1), (k >> 1) & 1);
-        }
+        __syncwarp();
+        ++issued;
+        ++next;
+        cur = around(cur + 1);
       }
-      __syncwarp();
-    } else {
-      // ---- epilogue: TMEM lane quarter warp % 4, channels CH ((warp - 1) / 4) ..
-      const int quarter = warp & 3, half = (warp - 1) >> 2, ch0 = CH * half;
-      const int m = quarter * 32 + lane, xl = m & (TX - 1), yl = m >> g.ltx;
+      if (!ok) {
+        *sfail = 1;
+        atomicExch(&g_tc_err, 1);
+        // the MMAs in flight finish before shared and tensor memory go away
+        for (int k = max(0, issued - kAccs); k < issued; ++k) mbar_wait(accfull(k % kAccs), (k / kAccs) & 1);
+      }
+    }
+    __syncwarp();
+  } else {
+    {
+      // ---- epilogue: the four warps of a group take every fourth tile, each
+      // warp the TMEM lane quarter warp % 4, CH channels at a time
+      const int quarter = warp & 3, group = (warp - 2) >> 2;
+      const int row = quarter * 32 + lane, xl = row & (TX - 1), yl = row >> g.ltx;
       const bool cross = TX > 32;  // runs that span warps
+      const bool inner = xl > 0, innerr = xl < TX - 1;
       bool ok = true;
-      for (int64_t t = t0; t < t1; ++t) {
-        const int k = (int)(t - t0), a = k & 1;
-        const int z = (int)(t % g.nz);
-        const Column c = column_of(g, t);
-        const int x = c.x0 + xl, y = c.y0 + yl;
-        const bool mine = x < g.nx && y < g.ny && (xl > 0 || x == 0) && (xl < TX - 1 || x == g.nx - 1);
-        const size_t o = ((size_t)c.b * V + x + (size_t)g.nx * (y + (size_t)g.ny * z)) * COUT + ch0;
-        uint4 res[CH / 8];
+      March at(g, t0);
+      bool mine = false;
+      size_t o = 0;  // the thread's output in this tile
+      uint4 res[RES ? COUT / 8 : 1];
+      // the place of tile t, and its residuals (loaded while the tile before is worked on)
+      auto place = [&](int64_t t) {
+        if (t >= t1) return;
+        const int x = at.x0(g) + xl, y = at.y0(g) + yl;
+        mine = x < g.nx && y < g.ny && (inner || x == 0) && (innerr || x == g.nx - 1);
+        o = ((size_t)at.b * V + x + (size_t)g.nx * (y + (size_t)g.ny * at.z)) * COUT;
         if (RES && mine) {
 #pragma unroll
-          for (int q = 0; q < CH / 8; ++q) res[q] = *reinterpret_cast<const uint4*>(R + o + 8 * q);
+          for (int q = 0; q < COUT / 8; ++q) res[q] = __ldcs(reinterpret_cast<const uint4*>(R + o + 8 * q));
         }
+      };
+      for (int i = 0; i < group; ++i) at.next(g);
+      place(t0 + group);
+      for (int64_t t = t0 + group; t < t1; t += kGroups) {
+        const int k = (int)(t - t0), a = k % kAccs;
         // (after an expired wait the warp still meets the barriers, and stores nothing)
-        if (ok && (*sfail || !mbar_wait(accfull(a), (k >> 1) & 1))) {
+        if (ok && !mbar_wait(accfull(a), (k / kAccs) & 1, sfail)) {
           ok = false;
           *sfail = 1;
           atomicExch(&g_tc_err, 1);
         }
         ok = __all_sync(0xffffffffu, ok);
-        float d[3][CH];
-        if (ok) {
-          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-          const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 128 + ch0);
-          tmem_ld3(ta, ta + COUT, ta + 2 * COUT, d);
-          asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(accempty(a));
-        } else {
+        uint32_t pk[8];  // 16 channels in BF16
 #pragma unroll
-          for (int i = 0; i < CH; ++i) d[0][i] = d[1][i] = d[2][i] = 0.f;
-        }
-        float* eb = edge + ((a * 2) * 2 + half) * 4 * 16;  // side 0; side 1 is 2 x 4 x 16 floats on
-        if (cross) {
-          if (lane == 31)
-#pragma unroll
-            for (int i = 0; i < CH; ++i) eb[quarter * 16 + i] = d[0][i];
-          if (lane == 0)
-#pragma unroll
-            for (int i = 0; i < CH; ++i) eb[2 * 4 * 16 + quarter * 16 + i] = d[2][i];
-          named_barrier(2 + half, 128);
-        }
-        float out[CH];
-#pragma unroll
-        for (int i = 0; i < CH; ++i) {
-          float l = __shfl_up_sync(0xffffffffu, d[0][i], 1), r = __shfl_down_sync(0xffffffffu, d[2][i], 1);
-          if (cross && lane == 0) l = eb[((quarter + 3) & 3) * 16 + i];
-          if (cross && lane == 31) r = eb[2 * 4 * 16 + ((quarter + 1) & 3) * 16 + i];
-          if (xl == 0) l = 0.f;
-          if (xl == TX - 1) r = 0.f;
-          out[i] = l + d[1][i] + r + sbias[ch0 + i];
-        }
-        if (!mine || !ok) continue;
-        if (OUT == 1) {
-#pragma unroll
-          for (int q = 0; q < CH / 4; ++q)
-            *reinterpret_cast<float4*>(Yf + o + 4 * q) = make_float4(out[4 * q], out[4 * q + 1], out[4 * q + 2], out[4 * q + 3]);
-        } else {
-          if (OUT == 2 && half == 0)
-            *reinterpret_cast<float4*>(Yf + (o / COUT) * 4) = make_float4(out[0], out[1], out[2], out[3]);
-#pragma unroll
-          for (int q = 0; q < CH / 8; ++q) {
-            const uint32_t rw[4] = {RES ? res[q].x : 0u, RES ? res[q].y : 0u, RES ? res[q].z : 0u, RES ? res[q].w : 0u};
-            uint32_t pk[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              float v0 = out[8 * q + 2 * e], v1 = out[8 * q + 2 * e + 1];
-              if (RES) {
-                v0 += __uint_as_float(rw[e] << 16);
-                v1 += __uint_as_float(rw[e] & 0xffff0000u);
-              }
-              if (OUT == 0) {
-                v0 = fmaxf(v0, 0.f);
-                v1 = fmaxf(v1, 0.f);
-              }
-              pk[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v0)) |
-                      ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v1)) << 16);
+        for (int part = 0; part < COUT / CH; ++part) {
+          const int ch0 = part * CH;
+          float d[3][CH];
+          if (ok) {
+            if (part == 0) asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 128 + ch0);
+            tmem_ld3(ta, ta + COUT, ta + 2 * COUT, d);
+            if (part == COUT / CH - 1) {
+              asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+              __syncwarp();
+              if (lane == 0) mbar_arrive(accempty(a));
             }
-            *reinterpret_cast<uint4*>(Y + o + 8 * q) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) d[0][i] = d[1][i] = d[2][i] = 0.f;
+          }
+          // the columns beyond the warp's ends, left of lane 0 and right of
+          // lane 31 (two buffers: one is rewritten after the other's barrier)
+          float* eb = edge + (group * 2 + part % 2) * 2 * 4 * 16;
+          if (cross) {
+            if (lane == 31) {
+#pragma unroll
+              for (int i = 0; i < CH; i += 4)
+                *reinterpret_cast<float4*>(eb + quarter * 16 + i) = make_float4(d[0][i], d[0][i + 1], d[0][i + 2], d[0][i + 3]);
+            }
+            if (lane == 0) {
+#pragma unroll
+              for (int i = 0; i < CH; i += 4)
+                *reinterpret_cast<float4*>(eb + 4 * 16 + quarter * 16 + i) =
+                    make_float4(d[2][i], d[2][i + 1], d[2][i + 2], d[2][i + 3]);
+            }
+            named_barrier(2 + group, 128);
+          }
+          // out = D[x - 1][0] + D[x][1] + D[x + 1][2]
+          float out[CH];
+#pragma unroll
+          for (int i = 0; i < CH; ++i) {
+            const float l = __shfl_up_sync(0xffffffffu, d[0][i], 1), r = __shfl_down_sync(0xffffffffu, d[2][i], 1);
+            out[i] = (inner && lane > 0 ? l : 0.f) + d[1][i] + (innerr && lane < 31 ? r : 0.f);
+          }
+          if (cross && ((lane == 0 && inner) || (lane == 31 && innerr))) {
+            const float* ep = eb + (lane == 0 ? ((quarter + 3) & 3) * 16 : 4 * 16 + ((quarter + 1) & 3) * 16);
+#pragma unroll
+            for (int i = 0; i < CH; ++i) out[i] += ep[i];
+          }
+#pragma unroll
+          for (int i = 0; i < CH; i += 4) {
+            const float4 b4 = *reinterpret_cast<const float4*>(sbias + ch0 + i);
+            out[i] += b4.x, out[i + 1] += b4.y, out[i + 2] += b4.z, out[i + 3] += b4.w;
+          }
+          if (mine && ok) {
+            if (OUT == 1) {
+#pragma unroll
+              for (int q = 0; q < CH / 8; ++q) {
+                const float* v = out + 8 * q;
+                st32(Yf + o + ch0 + 8 * q, wide, __float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]),
+                     __float_as_uint(v[3]), __float_as_uint(v[4]), __float_as_uint(v[5]), __float_as_uint(v[6]),
+                     __float_as_uint(v[7]));
+              }
+            } else {
+              if (OUT == 2 && part == 0)
+                *reinterpret_cast<float4*>(Yf + (o / COUT) * 4) = make_float4(out[0], out[1], out[2], out[3]);
+#pragma unroll
+              for (int e = 0; e < CH / 2; ++e) {
+                float v0 = out[2 * e], v1 = out[2 * e + 1];
+                if (RES) {
+                  const uint4 r4 = res[RES ? part * (CH / 8) + e / 4 : 0];
+                  const uint32_t rw = e % 4 == 0 ? r4.x : e % 4 == 1 ? r4.y : e % 4 == 2 ? r4.z : r4.w;
+                  v0 += __uint_as_float(rw << 16);
+                  v1 += __uint_as_float(rw & 0xffff0000u);
+                }
+                if (OUT == 0) {
+                  v0 = fmaxf(v0, 0.f);
+                  v1 = fmaxf(v1, 0.f);
+                }
+                pk[ch0 % 16 / 2 + e] = pack_bf16(v0, v1);
+              }
+              if ((ch0 + CH) % 16 == 0)
+                st32(Y + o + ch0 + CH - 16, wide, pk[0], pk[1], pk[2], pk[3], pk[4], pk[5], pk[6], pk[7]);
+            }
           }
         }
+        for (int i = 0; i < kGroups; ++i) at.next(g);
+        place(t + kGroups);
       }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
 int sm_count() {
@@ -446,16 +545,58 @@ int sm_count() {
   return sms > 0 ? sms : 1;
 }
 
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+  });
+  return fn;
+}
+
+// tensor map over BF16 rows of c channels (16 or 32, swizzled over the row's
+// 32 or 64 bytes), out-of-range coordinates zero
+bool encode(CUtensorMap* map, const bf16* p, int rank, int c, const cuuint64_t* rows, const cuuint32_t* box_rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+  if (!enc) return false;
+  cuuint64_t dims[4] = {(cuuint64_t)c}, strides[3];
+  cuuint32_t box[4] = {(cuuint32_t)c};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  cuuint64_t st = 2 * (cuuint64_t)c;
+  for (int d = 1; d < rank; ++d) {
+    dims[d] = rows[d - 1];
+    box[d] = box_rows[d - 1];
+    strides[d - 1] = st;
+    st *= rows[d - 1];
+  }
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<bf16*>(p), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int CIN, int COUT, int OUT, bool RES, bool TRANSPOSED>
-int run_conv(const ConvGrid& g, const bf16* X, const bf16* W, const float* bias, const bf16* R, bf16* Y, float* Yf,
+int run_conv(ConvGrid g, const bf16* X, const bf16* W, const float* bias, const bf16* R, bf16* Y, float* Yf,
              cudaStream_t s) {
   using L = ConvLayout<CIN, COUT>;
+  CUtensorMap xmap, wmap;
+  const cuuint64_t vox[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz * g.B};
+  const cuuint32_t vbox[3] = {1u << g.ltx, (cuuint32_t)(kTileM >> g.ltx) + 2, 1};
+  const cuuint64_t wrows = 27 * (TRANSPOSED ? CIN : COUT);
+  const cuuint32_t wbox = TRANSPOSED ? CIN : L::NB;
+  if (!encode(&xmap, X, 4, CIN, vox, vbox) || !encode(&wmap, W, 2, TRANSPOSED ? COUT : CIN, &wrows, &wbox)) return BO_ERR_ARG;
   auto kern = k_conv3d_tc<CIN, COUT, OUT, RES, TRANSPOSED>;
-  const int smem = L::kOffPlanes + kPlanes * L::KC * chunk_stride(g.ltx, L::KC) + 128;
+  const int plane = plane_rows(g.ltx) * CIN * 2;
+  g.planes = (kTcSmem - L::kOffPlanes - 1024) / plane;  // (6 at least: TX = 128 with 32 channels)
+  if (g.planes > kMaxPlanes) g.planes = kMaxPlanes;
+  const int smem = L::kOffPlanes + g.planes * plane + 1024;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return BO_ERR_CUDA;
   const int sms = sm_count();
   const int grid = g.tiles < sms ? (int)g.tiles : sms;
-  (kern<<<grid, kTcThreads, smem, s>>>(g, X, W, bias, R, Y, Yf), note_launch());
+  (kern<<<grid, kTcThreads, smem, s>>>(g, xmap, wmap, bias, R, Y, Yf), note_launch());
   return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
 }
 
@@ -472,7 +613,7 @@ int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_
                    cudaStream_t s) {
   for (const void* p : {(const void*)X, (const void*)W, (const void*)R, (const void*)Y, (const void*)Yf})
     if (reinterpret_cast<uintptr_t>(p) & 15) return BO_ERR_ARG;
-  ConvGrid g{nx, ny, nz, B, 0, 0, 0, 0};
+  ConvGrid g{nx, ny, nz, B, 0, 0, 0, 0, 0};
   int64_t best = -1;
   for (int ltx = 4; ltx <= 7; ++ltx) {
     const int TX = 1 << ltx, TY = kTileM >> ltx;
@@ -557,9 +698,6 @@ __host__ __device__ __forceinline__ int wg_halo_plane(int tx) { return kWgHY * 4
 __host__ __device__ __forceinline__ int wg_core_plane(int tx, int kc) { return kWgTY * kc * wg_core_row(tx, kc); }
 constexpr int kWgOffBar = 0, kWgOffBias = 256, kWgOffPlanes = kWgOffBias + 128 * 8 * 8;
 
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) | ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
-}
 
 // One plane of a tensor into shared memory: NR rows from y0, NX voxels from
 // x0, rows [chunk][voxel].  BF16 by cp.async (the caller commits); FP32 by
@@ -692,7 +830,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
       tile(t, x0, y0, z, b);
       const size_t zb = (size_t)b * V + (size_t)z * g.nx * g.ny;
       const uint32_t dst = cbase + (uint32_t)(k % kWgCore) * cplane;
-      auto wait = [&]() { return k < kWgCore || (!*sfail && mbar_wait(cempty(k % kWgCore), (k / kWgCore - 1) & 1)); };
+      auto wait = [&]() { return k < kWgCore || mbar_wait(cempty(k % kWgCore), (k / kWgCore - 1) & 1, sfail); };
       if constexpr (HALO_DY) {
         ok = wait();
         if (!ok) break;
@@ -718,7 +856,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
       for (int pz = start ? max(z - 1, 0) : z + 1; pz <= min(z + 1, g.nz - 1) && ok; ++pz) {
         const size_t zb = (size_t)b * V + (size_t)pz * g.nx * g.ny;
         const uint32_t dst = hbase + (uint32_t)(seq % kWgHalo) * hplane;
-        auto wait = [&]() { return seq < kWgHalo || (!*sfail && mbar_wait(hempty(seq % kWgHalo), (seq / kWgHalo - 1) & 1)); };
+        auto wait = [&]() { return seq < kWgHalo || mbar_wait(hempty(seq % kWgHalo), (seq / kWgHalo - 1) & 1, sfail); };
         if constexpr (HALO_DY) {
           // a plane counts towards the bias where it is one of this CTA's tiles
           const bool own = pz >= z && pz < zend;
@@ -748,8 +886,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
         for (; done < seq; ++done) mbar_arrive(hfull(done % kWgHalo));
       }
     }
-  } else if (lane == 0 && t0 < t1) {
-    // ---- MMA issue
+  } else if (t0 < t1) {
+    // ---- MMA issue (the whole warp waits, one thread issues)
     uint32_t started = 0;
     int waited = 0, next = 0;
     for (int64_t t = t0; t < t1 && ok; ++t) {
@@ -759,43 +897,52 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
       const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
       if (start) next = waited + (z > 0 ? 1 : 0);
       const int need = next + (z < g.nz - 1 ? 1 : 0);
-      for (; waited <= need && ok; ++waited) ok = !*sfail && mbar_wait(hfull(waited % kWgHalo), (waited / kWgHalo) & 1);
-      ok = ok && mbar_wait(cfull(k % kWgCore), (k / kWgCore) & 1);
+      for (; waited <= need && ok; ++waited)
+        ok = __all_sync(0xffffffffu, mbar_wait(hfull(waited % kWgHalo), (waited / kWgHalo) & 1, sfail));
+      ok = ok && __all_sync(0xffffffffu, mbar_wait(cfull(k % kWgCore), (k / kWgCore) & 1, sfail));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const uint64_t db0 = smem_desc(cbase + (uint32_t)(k % kWgCore) * cplane, 128, (uint32_t)crow);
-      for (int dz = 0; dz < 3; ++dz) {
-        if (z + dz - 1 < 0 || z + dz - 1 >= g.nz) continue;
-        const uint64_t da0 = smem_desc(hbase + (uint32_t)((next + dz - 1) % kWgHalo) * hplane, 128, (uint32_t)hrow);
-        for (int yp = 0; yp < kWgTY; yp += 2)
-          for (int kx = 0; kx < TX; kx += 16) {
-            const uint64_t da = da0 + (uint64_t)((yp * 4 * hrow + kx * 16) >> 4);
-            const uint64_t db = db0 + (uint64_t)((yp * KC * crow + kx * 16) >> 4);
+      if (elect_one()) {
+        const uint64_t db0 = smem_desc(cbase + (uint32_t)(k % kWgCore) * cplane, 128, (uint32_t)crow);
 #pragma unroll
-            for (int sx = 0; sx < 3; ++sx) {
-              const int i = 3 * dz + sx;
-              const bool acc = (started >> i) & 1u;
-              if (i < kPair) {
-                umma(tmem + (uint32_t)(2 * CB * i), da + (uint64_t)sx, db, idesc(2 * CB, true), acc);
-              } else {
-                const uint32_t d = tmem + (uint32_t)(2 * CB * kPair + CB * (i - kPair));
-                umma(d, da + (uint64_t)sx, db, idesc(CB, true), acc);
-                umma(d, da + (uint64_t)sx + (uint64_t)((4 * hrow) >> 4), db + (uint64_t)((KC * crow) >> 4), idesc(CB, true), true);
+        for (int dz = 0; dz < 3; ++dz) {
+          if (z + dz - 1 < 0 || z + dz - 1 >= g.nz) continue;
+          const uint64_t da0 = smem_desc(hbase + (uint32_t)((next + dz - 1) % kWgHalo) * hplane, 128, (uint32_t)hrow);
+          bool acc = (started >> (3 * dz)) & 1u;
+          for (int kx = 0; kx < TX; kx += 16)
+#pragma unroll
+            for (int yp = 0; yp < kWgTY; yp += 2) {
+              const uint64_t da = da0 + (uint64_t)((yp * 4 * hrow + kx * 16) >> 4);
+              const uint64_t db = db0 + (uint64_t)((yp * KC * crow + kx * 16) >> 4);
+#pragma unroll
+              for (int sx = 0; sx < 3; ++sx) {
+                const int i = 3 * dz + sx;
+                if (i < kPair) {
+                  umma(tmem + (uint32_t)(2 * CB * i), da + (uint64_t)sx, db, idesc(2 * CB, true, true), acc);
+                } else {
+                  const uint32_t d = tmem + (uint32_t)(2 * CB * kPair + CB * (i - kPair));
+                  umma(d, da + (uint64_t)sx, db, idesc(CB, true, true), acc);
+                  umma(d, da + (uint64_t)sx + (uint64_t)((4 * hrow) >> 4), db + (uint64_t)((KC * crow) >> 4), idesc(CB, true, true),
+                       true);
+                }
               }
-              started |= 1u << i;
+              acc = true;
             }
-          }
+        }
+        umma_commit(cempty(k % kWgCore));
+        if (z > 0) umma_commit(hempty((next - 1) % kWgHalo));
+        if (end) {
+          umma_commit(hempty(next % kWgHalo));
+          if (z < g.nz - 1) umma_commit(hempty((next + 1) % kWgHalo));
+        }
       }
-      umma_commit(cempty(k % kWgCore));
-      if (z > 0) umma_commit(hempty((next - 1) % kWgHalo));
-      if (end) {
-        umma_commit(hempty(next % kWgHalo));
-        if (z < g.nz - 1) umma_commit(hempty((next + 1) % kWgHalo));
-      }
+      __syncwarp();
+      started |= (z > 0 ? 7u : 0u) | 7u << 3 | (z < g.nz - 1 ? 7u << 6 : 0u);
       ++next;
     }
     *sstarted = started;
-    umma_commit(alldone);
+    if (elect_one()) umma_commit(alldone);
+    __syncwarp();
     if (!mbar_wait(alldone, 0)) ok = false;  // every MMA is done before the buffers are used again
   }
   if (!ok) {
