@@ -197,14 +197,16 @@ struct ConvGrid {
 // A tile's place, stepped from tile to tile (a division once per CTA)
 struct March {
   int z, tx, ty, b;
-  __device__ __forceinline__ March(const ConvGrid& g, int64_t t) {
+  template <typename Grid>
+  __device__ __forceinline__ March(const Grid& g, int64_t t) {
     const int c = (int)(t / g.nz);
     z = (int)(t - (int64_t)c * g.nz);
     tx = c % g.ntx;
     ty = c / g.ntx % g.nty;
     b = c / g.ntx / g.nty;
   }
-  __device__ __forceinline__ void next(const ConvGrid& g) {
+  template <typename Grid>
+  __device__ __forceinline__ void next(const Grid& g) {
     if (++z < g.nz) return;
     z = 0;
     if (++tx < g.ntx) return;
@@ -672,16 +674,18 @@ namespace {
 // what lets one descriptor span four rows of four chunks.
 // The accumulators stay in TMEM over all tiles of a CTA (TX x 4 voxels, a
 // march along z as in the convolution above); each CTA writes one partial
-// sum, k_wgrad_sum adds them in a fixed order in FP64.  dY is read in FP32
-// by four warps that round it to BF16 on its way to shared memory and sum
-// the bias gradient in split FP32 pairs, so it is read once; X comes by
-// cp.async.  What bounds it: the shared-memory operand reads of the MMAs, 48
-// cycles for 2 x 16 voxels and a ninth of the taps.
+// sum, k_wgrad_sum adds them in a fixed order.  dY is read in FP32 by eight
+// warps that round it to BF16 on its way to shared memory and sum the bias
+// gradient in split FP32 pairs, so it is read once; X comes by cp.async from
+// eight more (with four of each the dY warps took 5800 cycles a tile, the MMAs
+// 3900).  What bounds it: the shared-memory operand reads of the MMAs, 6 KB in
+// 46 cycles for 2 x 16 voxels and a ninth of the taps.
 // Measured, 64x64x32 x 4 samples, 32 -> 32: 587 us a call, with scratch
 // allocated in it and five launches (mma.sync gradient 144, FP64 bias sums
-// 95, reduction 30, conversion 18) -> 164 us (this kernel 118, k_wgrad_sum
-// 21).
-constexpr int kWgThreads = 288;   // warp 0: MMAs; 1-4: halo producers; 5-8: core producers; 1-8: the end
+// 95, reduction 30, conversion 18) -> 164 with MMAs issued in a loop over
+// lanes -> 103 with four producer warps a side and FP64 sums -> 82.
+constexpr int kWgProd = 256;      // threads that fetch halo planes, and as many core planes
+constexpr int kWgThreads = 32 + 2 * kWgProd;  // warp 0: MMAs; 1-8: halo producers; 9-16: core producers; 1-16: the end
 constexpr int kWgHalo = 5, kWgCore = 3;  // plane buffers
 constexpr int kWgTY = 4, kWgHY = kWgTY + 3;
 
@@ -696,62 +700,65 @@ __host__ __device__ __forceinline__ int wg_halo_row(int tx) { return (tx + 2) * 
 __host__ __device__ __forceinline__ int wg_core_row(int tx, int kc) { return tx * 16 + 128 / kc; }
 __host__ __device__ __forceinline__ int wg_halo_plane(int tx) { return kWgHY * 4 * wg_halo_row(tx); }
 __host__ __device__ __forceinline__ int wg_core_plane(int tx, int kc) { return kWgTY * kc * wg_core_row(tx, kc); }
-constexpr int kWgOffBar = 0, kWgOffBias = 256, kWgOffPlanes = kWgOffBias + 128 * 8 * 8;
+constexpr int kWgOffBar = 0, kWgOffBias = 256, kWgOffPlanes = kWgOffBias + kWgProd * 8 * 8;
 
 
 // One plane of a tensor into shared memory: NR rows from y0, NX voxels from
-// x0, rows [chunk][voxel].  BF16 by cp.async (the caller commits); FP32 by
-// loads, rounded to BF16, `wait` called between the loads and the first store
-// and the voxels of `own` added to the thread's bias sums.
+// x0, rows [chunk][voxel], a thread every kWgProd / KC voxels of a chunk.
+// BF16 by cp.async (the caller commits); FP32 by loads, rounded to BF16,
+// `wait` called between the loads and the first store and the voxels of `own`
+// added to the thread's bias sums.
+struct WgStep {  // voxel index -> (row, place in it), stepped without divisions
+  int yl, xl;
+  __device__ __forceinline__ WgStep(int i, int NX) : yl(i / NX), xl(i - i / NX * NX) {}
+  __device__ __forceinline__ void next(int by, int NX) {
+    for (xl += by; xl >= NX; xl -= NX) ++yl;
+  }
+};
 template <int KC, int NR>
 __device__ __forceinline__ void wg_plane_bf16(const bf16* T, size_t zb, int nx, int ny, int x0, int y0, int NX, uint32_t dst,
                                               int row_bytes, int pt) {
   const int kc = pt % KC;
-  for (int yl = 0; yl < NR; ++yl) {
-    const int y = y0 + yl;
-    for (int xl = pt / KC; xl < NX; xl += 128 / KC) {
-      const int x = x0 + xl;
-      const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
-      cp16(dst + (uint32_t)((yl * KC + kc) * row_bytes + xl * 16), T + (in ? (zb + (size_t)y * nx + x) * (KC * 8) : 0) + kc * 8,
-           in);
-    }
+  for (WgStep a(pt / KC, NX); a.yl < NR; a.next(kWgProd / KC, NX)) {
+    const int x = x0 + a.xl, y = y0 + a.yl;
+    const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+    cp16(dst + (uint32_t)((a.yl * KC + kc) * row_bytes + a.xl * 16), T + (in ? (zb + (size_t)y * nx + x) * (KC * 8) : 0) + kc * 8,
+         in);
   }
 }
 template <int KC, int NR, typename Wait>
 __device__ __forceinline__ bool wg_plane_f32(const float* T, size_t zb, int nx, int ny, int x0, int y0, int NX, uint32_t dst,
                                              int row_bytes, int pt, bool own, int own_x0, int own_y0, int own_nx,
                                              df (&bias)[8], Wait wait) {
-  constexpr int U = 6;  // voxels in flight per thread
+  constexpr int U = 4, kStep = kWgProd / KC;  // U voxels in flight per thread
   const int kc = pt % KC;
   const int n = NR * NX;
+  WgStep ld(pt / KC, NX), a = ld;
   bool waited = false;
-  for (int i0 = pt / KC; i0 < n; i0 += U * (128 / KC)) {
+  for (int base = 0; base < n; base += U * kStep) {  // (the same number of rounds for every thread)
     float4 v[U][2];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * (128 / KC);
-      const int yl = i / NX, xl = i - yl * NX;
-      const int x = x0 + xl, y = y0 + yl;
-      const bool in = i < n && x >= 0 && x < nx && y >= 0 && y < ny;
+      const int x = x0 + ld.xl, y = y0 + ld.yl;
+      const bool in = ld.yl < NR && x >= 0 && x < nx && y >= 0 && y < ny;
       const float4* src = reinterpret_cast<const float4*>(T + (in ? (zb + (size_t)y * nx + x) * (KC * 8) : 0) + kc * 8);
       v[u][0] = in ? __ldcs(src) : make_float4(0.f, 0.f, 0.f, 0.f);
       v[u][1] = in ? __ldcs(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+      ld.next(kStep, NX);
     }
     if (!waited) {
       waited = true;
-      if (!wait()) return false;
+      if (!__all_sync(0xffffffffu, wait())) return false;
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * (128 / KC);
-      if (i >= n) continue;
-      const int yl = i / NX, xl = i - yl * NX;
+    for (int u = 0; u < U; ++u, a.next(kStep, NX)) {
+      if (a.yl >= NR) continue;
       const float e[8] = {v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w, v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w};
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)((yl * KC + kc) * row_bytes + xl * 16)),
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)((a.yl * KC + kc) * row_bytes + a.xl * 16)),
                    "r"(pack_bf16(e[0], e[1])), "r"(pack_bf16(e[2], e[3])), "r"(pack_bf16(e[4], e[5])),
                    "r"(pack_bf16(e[6], e[7]))
                    : "memory");
-      if (own && yl >= own_y0 && yl < own_y0 + kWgTY && xl >= own_x0 && xl < own_x0 + own_nx) {
+      if (own && a.yl >= own_y0 && a.yl < own_y0 + kWgTY && a.xl >= own_x0 && a.xl < own_x0 + own_nx) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const df t = df_two_sum(bias[q].hi, e[q]);
@@ -785,11 +792,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int p = 0; p < kWgHalo; ++p) {
-      mbar_init(hfull(p), 128);
+      mbar_init(hfull(p), kWgProd / 32);  // (an arrival per warp)
       mbar_init(hempty(p), 1);
     }
     for (int p = 0; p < kWgCore; ++p) {
-      mbar_init(cfull(p), 128);
+      mbar_init(cfull(p), kWgProd / 32);
       mbar_init(cempty(p), 1);
     }
     mbar_init(alldone, 1);
@@ -810,90 +817,78 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   const uint32_t cbase = hbase + kWgHalo * hplane, cplane = (uint32_t)wg_core_plane(TX, KC);
   const int64_t t0 = g.tiles * blockIdx.x / gridDim.x, t1 = g.tiles * (blockIdx.x + 1) / gridDim.x;
   const int64_t V = (int64_t)g.nx * g.ny * g.nz;
-  auto tile = [&](int64_t t, int& x0, int& y0, int& z, int& b) {
-    z = (int)(t % g.nz);
-    const int c = (int)(t / g.nz), r = c / g.ntx;
-    x0 = (c % g.ntx) * TX;
-    y0 = (r % g.nty) * kWgTY;
-    b = r / g.nty;
+  // a warp's stores to shared memory are visible to the MMAs: one arrival
+  auto arrive = [&](uint32_t bar) {
+    fence_async_proxy();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
   };
   df bias[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) bias[q] = df{0.f, 0.f};
   bool ok = true;
-  if (warp >= 5) {
+  March m(g, t0);
+  if (warp >= 1 + kWgProd / 32) {
     // ---- core planes
-    const int pt = tid - 5 * 32;
-    for (int64_t t = t0; t < t1 && ok; ++t) {
+    const int pt = tid - 32 - kWgProd;
+    for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
       const int k = (int)(t - t0);
-      int x0, y0, z, b;
-      tile(t, x0, y0, z, b);
-      const size_t zb = (size_t)b * V + (size_t)z * g.nx * g.ny;
+      const size_t zb = (size_t)m.b * V + (size_t)m.z * g.nx * g.ny;
       const uint32_t dst = cbase + (uint32_t)(k % kWgCore) * cplane;
       auto wait = [&]() { return k < kWgCore || mbar_wait(cempty(k % kWgCore), (k / kWgCore - 1) & 1, sfail); };
       if constexpr (HALO_DY) {
-        ok = wait();
+        ok = __all_sync(0xffffffffu, wait());
         if (!ok) break;
-        wg_plane_bf16<KC, kWgTY>(X, zb, g.nx, g.ny, x0, y0, TX, dst, crow, pt);
+        wg_plane_bf16<KC, kWgTY>(X, zb, g.nx, g.ny, m.tx * TX, m.ty * kWgTY, TX, dst, crow, pt);
         cp_commit();
         cp_wait<0>();
       } else {
-        ok = wg_plane_f32<KC, kWgTY>(dY, zb, g.nx, g.ny, x0, y0, TX, dst, crow, pt, true, 0, 0, TX, bias, wait);
+        ok = wg_plane_f32<KC, kWgTY>(dY, zb, g.nx, g.ny, m.tx * TX, m.ty * kWgTY, TX, dst, crow, pt, true, 0, 0, TX, bias, wait);
         if (!ok) break;
       }
-      fence_async_proxy();
-      mbar_arrive(cfull(k % kWgCore));
+      arrive(cfull(k % kWgCore));
     }
   } else if (warp >= 1) {
     // ---- halo planes
     const int pt = tid - 32;
     int seq = 0, done = 0;
-    for (int64_t t = t0; t < t1 && ok; ++t) {
-      int x0, y0, z, b;
-      tile(t, x0, y0, z, b);
+    for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
+      const int z = m.z, x0 = m.tx * TX - 1, y0 = m.ty * kWgTY - 1;
       const bool start = t == t0 || z == 0;
       const int zend = (int)min((int64_t)g.nz, z + (t1 - t));  // the column's tiles of this CTA end there
       for (int pz = start ? max(z - 1, 0) : z + 1; pz <= min(z + 1, g.nz - 1) && ok; ++pz) {
-        const size_t zb = (size_t)b * V + (size_t)pz * g.nx * g.ny;
+        const size_t zb = (size_t)m.b * V + (size_t)pz * g.nx * g.ny;
         const uint32_t dst = hbase + (uint32_t)(seq % kWgHalo) * hplane;
         auto wait = [&]() { return seq < kWgHalo || mbar_wait(hempty(seq % kWgHalo), (seq / kWgHalo - 1) & 1, sfail); };
         if constexpr (HALO_DY) {
           // a plane counts towards the bias where it is one of this CTA's tiles
           const bool own = pz >= z && pz < zend;
-          ok = wg_plane_f32<4, kWgHY>(dY, zb, g.nx, g.ny, x0 - 1, y0 - 1, TX + 2, dst, hrow, pt, own, 1, 1, TX, bias, wait);
+          ok = wg_plane_f32<4, kWgHY>(dY, zb, g.nx, g.ny, x0, y0, TX + 2, dst, hrow, pt, own, 1, 1, TX, bias, wait);
           if (!ok) break;
-          fence_async_proxy();
-          mbar_arrive(hfull(seq % kWgHalo));
+          arrive(hfull(seq % kWgHalo));
           ++seq;
         } else {
-          ok = wait();
+          ok = __all_sync(0xffffffffu, wait());
           if (!ok) break;
-          wg_plane_bf16<4, kWgHY>(X, zb, g.nx, g.ny, x0 - 1, y0 - 1, TX + 2, dst, hrow, pt);
+          wg_plane_bf16<4, kWgHY>(X, zb, g.nx, g.ny, x0, y0, TX + 2, dst, hrow, pt);
           cp_commit();
           ++seq;
           cp_wait<1>();
-          if (seq > 1) {
-            fence_async_proxy();
-            for (; done < seq - 1; ++done) mbar_arrive(hfull(done % kWgHalo));
-          }
+          for (; done < seq - 1; ++done) arrive(hfull(done % kWgHalo));
         }
       }
     }
     cp_wait<0>();
     if constexpr (!HALO_DY) {
-      if (ok) {
-        fence_async_proxy();
-        for (; done < seq; ++done) mbar_arrive(hfull(done % kWgHalo));
-      }
+      if (ok)
+        for (; done < seq; ++done) arrive(hfull(done % kWgHalo));
     }
   } else if (t0 < t1) {
     // ---- MMA issue (the whole warp waits, one thread issues)
     uint32_t started = 0;
     int waited = 0, next = 0;
-    for (int64_t t = t0; t < t1 && ok; ++t) {
-      const int k = (int)(t - t0);
-      int x0, y0, z, b;
-      tile(t, x0, y0, z, b);
+    for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
+      const int k = (int)(t - t0), z = m.z;
       const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
       if (start) next = waited + (z > 0 ? 1 : 0);
       const int need = next + (z < g.nz - 1 ? 1 : 0);
@@ -950,9 +945,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     atomicExch(&g_tc_err, 1);
   }
   if (warp >= 1) {
-    const bool dyside = HALO_DY ? warp < 5 : warp >= 5;
+    const bool dyside = (warp < 1 + kWgProd / 32) == HALO_DY;
     if (dyside) {
-      const int pt = HALO_DY ? tid - 32 : tid - 5 * 32;
+      const int pt = HALO_DY ? tid - 32 : tid - 32 - kWgProd;
 #pragma unroll
       for (int q = 0; q < 8; ++q)  // (a sum that met an infinity has NaN in its low part)
         sbias[pt * 8 + q] = isfinite(bias[q].hi) ? df_to_double(df_renorm(bias[q])) : (double)bias[q].hi;
@@ -968,8 +963,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   const bool fine = !*sfail;
   for (int r = 0; r < 2; ++r) {
     if (warp >= 1) {
-      const int a = warp & 3, part2 = (warp - 1) >> 2;  // the two warps of a quarter take alternate accumulators
-      for (int i = part2; i < 9; i += 2) {
+      const int a = warp & 3, part2 = (warp - 1) >> 2;  // the warps of a quarter share the accumulators
+      for (int i = part2; i < 9; i += kWgProd / 64) {
         const bool pair = i < kPair;
         if (!pair && r == 1) continue;
         const int dy = pair ? a - r : a;
@@ -1001,11 +996,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   }
   const int n = 27 * 32 * CB;
   float* P = part + (size_t)blockIdx.x * n;
-  for (int i = tid; i < n; i += kWgThreads) P[i] = red[i];
+  for (int i = tid; i < n / 4; i += kWgThreads) reinterpret_cast<float4*>(P)[i] = reinterpret_cast<const float4*>(red)[i];
   if (tid < CY) {
     constexpr int YC = CY / 8;
     double sum = 0.0;
-    for (int p = tid / 8; p < 128; p += YC) sum += sbias[p * 8 + tid % 8];
+    for (int p = tid / 8; p < kWgProd; p += YC) sum += sbias[p * 8 + tid % 8];
     bpart[(size_t)blockIdx.x * CY + tid] = sum;
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -1014,8 +1009,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
-// dW[i] = sum over the chunks' partials in a fixed order (FP64); 32 outputs by
-// 8 slices of the chunks per block.  The last block takes the bias gradient.
+// dW[i] = sum over the chunks' partials in a fixed order, in split FP32 pairs
+// (48 bits; 4.2 million FP64 additions took 14 of the 20 us of the form that
+// made them); 32 outputs by 8 slices of the chunks per block.  The last block
+// takes the bias gradient.
 __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, const double* __restrict__ bpart,
                                                    float* __restrict__ dW, float* __restrict__ db, int n, int chunks, int cy) {
   __shared__ double sh[8][32];
@@ -1025,9 +1022,19 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ par
     if (l < cy)
       for (int k = w; k < chunks; k += 8) s += bpart[(size_t)k * cy + l];
   } else {
-    const int i = blockIdx.x * 32 + l;
-#pragma unroll 4
-    for (int k = w; k < chunks; k += 8) s += part[(size_t)k * n + i];  // (n is a multiple of 32)
+    const float* p = part + blockIdx.x * 32 + l;  // (n is a multiple of 32)
+    df a{0.f, 0.f};
+    for (int k0 = w; k0 < chunks; k0 += 80) {
+      float v[10];
+#pragma unroll
+      for (int u = 0; u < 10; ++u) v[u] = k0 + 8 * u < chunks ? p[(size_t)(k0 + 8 * u) * n] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 10; ++u) {
+        const df t = df_two_sum(a.hi, v[u]);
+        a = df{t.hi, __fadd_rn(a.lo, t.lo)};
+      }
+    }
+    s = isfinite(a.hi) ? df_to_double(a) : (double)a.hi;  // (past an infinity the low part is NaN)
   }
   sh[w][l] = s;
   __syncthreads();
