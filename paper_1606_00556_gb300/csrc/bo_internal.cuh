@@ -387,6 +387,24 @@ inline int grid_for(int64_t n, int threads = kThreads, int max_blocks = 152 * 16
 // (one full wave, no partial last wave), capped by the work available.
 int occ_grid(const void* kernel, int64_t n, int threads = kThreads, size_t smem = 0);
 
+// Threads per block of a kernel with a cell per thread: kThreads, or where
+// that would leave SMs without a block, 32 to 128.  A cell takes some 75 FP64
+// multiply-adds of the SM's two a clock, or a chain of split FP32 ones, so
+// the cells of a small system have to be spread: at 20x20x5 in FP64 the four
+// blocks of 256 threads of an ILU pass took 8-10 us (that Newton step 1015 ->
+// 935 us).
+inline int cell_threads(int64_t n) {
+  int threads = kThreads;
+  while (threads > 32 && n < (int64_t)threads * 2 * 152) threads >>= 1;
+  return threads;
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cells(void (*kernel)(KArgs...), int64_t n, cudaStream_t s, Args&&... args) {
+  const int threads = cell_threads(n);
+  const int grid = threads == kThreads ? occ_grid((const void*)kernel, n) : grid_for(n, threads);
+  return launch_pdl(kernel, grid, threads, 0, s, args...);
+}
+
 }  // namespace bo
 
 // ----------------------------------------------------------------- objects

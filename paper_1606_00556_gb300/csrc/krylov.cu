@@ -293,36 +293,46 @@ __global__ void k_scale_beta(int64_t n, const double* __restrict__ src, float* _
 
 // Hessenberg column j from the coefficients col[0..j] and h_{j+1,j} = hn:
 // previous rotations, a new one, the residual estimate and the stop flag.
-// Runs in one thread.
-__device__ void givens_step(DevState* st, double* col, double hn, double* H, double* cs, double* sn, double* gv, int j,
-                            int m, int ldh, double* hist) {
+// Called by one warp with the column, and the previous rotations, in shared
+// memory (loaded by as many threads: a thread that fetched each value as it
+// came to it waited for memory at every step).
+__device__ void givens_step(DevState* st, double* col, double hn, double* H, const double* scs, const double* ssn, double* cs,
+                            double* sn, double* gv, int j, int m, int ldh, double* hist) {
+  const int lane = threadIdx.x & 31;
   double nrm2 = 0.0;
-  for (int i = 0; i <= j; ++i) nrm2 += col[i] * col[i];
-  const double wn0 = sqrt(nrm2 + hn * hn);
-  for (int i = 0; i < j; ++i) {
-    const double a = col[i], b = col[i + 1];
-    col[i] = cs[i] * a + sn[i] * b;
-    col[i + 1] = -sn[i] * a + cs[i] * b;
+  for (int i = lane; i <= j; i += 32) nrm2 += col[i] * col[i];
+  nrm2 = warp_sum(nrm2);
+  if (lane == 0) {
+    const double wn0 = sqrt(nrm2 + hn * hn);
+    const double gj = gv[j], target = st->target;
+    const int hist_at = st->hist_base + j, err = st->err;
+    double a = col[0];
+    for (int i = 0; i < j; ++i) {
+      const double b = col[i + 1];
+      col[i] = scs[i] * a + ssn[i] * b;
+      a = -ssn[i] * a + scs[i] * b;
+    }
+    const double d = hypot(a, hn);
+    const double c = d > 0.0 ? a / d : 1.0, s = d > 0.0 ? hn / d : 0.0;
+    cs[j] = c;
+    sn[j] = s;
+    col[j] = d;
+    const double est = fabs(-s * gj);
+    gv[j + 1] = -s * gj;
+    gv[j] = c * gj;
+    st->k = j + 1;
+    st->est = est;
+    const int happy = hn <= 1e-14 * wn0;
+    st->happy = happy;
+    st->hn = hn;
+    st->scale = hn > 0.0 ? 1.0 / hn : 0.0;
+    if (hist && hist_at < kHistCap) hist[hist_at] = est;
+    const bool bad = !isfinite(est) || !isfinite(d) || d == 0.0;
+    if (bad) atomicOr(&st->err, kErrNonfinite);
+    if (bad || (err & kErrTimeout) || est <= target || happy || j + 1 == m) st->done = 1;
   }
-  const double a = col[j];
-  const double d = hypot(a, hn);
-  const double c = d > 0.0 ? a / d : 1.0, s = d > 0.0 ? hn / d : 0.0;
-  cs[j] = c;
-  sn[j] = s;
-  col[j] = d;
-  for (int i = 0; i <= j; ++i) H[(size_t)i * ldh + j] = col[i];
-  gv[j + 1] = -s * gv[j];
-  gv[j] = c * gv[j];
-  st->k = j + 1;
-  st->est = fabs(gv[j + 1]);
-  st->happy = hn <= 1e-14 * wn0;
-  st->hn = hn;
-  st->scale = hn > 0.0 ? 1.0 / hn : 0.0;
-  const int hist_at = st->hist_base + j;
-  if (hist && hist_at < kHistCap) hist[hist_at] = st->est;
-  const bool bad = !isfinite(st->est) || !isfinite(d) || d == 0.0;
-  if (bad) atomicOr(&st->err, kErrNonfinite);
-  if (bad || (st->err & kErrTimeout) || st->est <= st->target || st->happy || j + 1 == m) st->done = 1;
+  __syncwarp();
+  for (int i = lane; i <= j; i += 32) H[(size_t)i * ldh + j] = col[i];
 }
 
 struct ArnoldiArgs {
@@ -332,6 +342,7 @@ struct ArnoldiArgs {
   double* gv;
   int j, m, ldh;
   double* hist;
+  int* host_done;  // the host's copy of st->done for this column (mapped memory), or NULL
 };
 
 // Gram-Schmidt coefficient passes: h[off + u] = vscale[u] <V_u, w> for
@@ -670,7 +681,13 @@ __global__ void __launch_bounds__(kThreads) k_gs_update(int64_t n, const float* 
   constexpr int B = kGsBatch;
   __shared__ df c[kMaxM + 1];
   __shared__ double sh[32];
-  if (st->done) return;
+  if (st->done) {
+    if (LAST && aa.host_done && blockIdx.x == 0 && threadIdx.x == 0) {
+      *aa.host_done = 1;
+      __threadfence_system();
+    }
+    return;
+  }
   const int nv = aa.j + 1;
   const int off = LAST ? kMaxM : 0;
   const int64_t np = split_pad(n);
@@ -743,14 +760,23 @@ __global__ void __launch_bounds__(kThreads) k_gs_update(int64_t n, const float* 
   acc = block_sum(acc + df_to_double(df_renorm(accs)), sh);
   if (threadIdx.x == 0) partials[blockIdx.x] = acc;
   if (!last_block(&st->counter[3], gridDim.x)) return;
+  __shared__ double col[kMaxM + 1], scs[kMaxM + 1], ssn[kMaxM + 1];
+  for (int u = threadIdx.x; u < nv; u += blockDim.x) {
+    col[u] = st->h[u] + st->h[kMaxM + u];
+    scs[u] = aa.cs[u];  // (entry nv - 1 is not used)
+    ssn[u] = aa.sn[u];
+  }
   const double hn2 = reduce_partials(partials, gridDim.x, sh);
+  if (threadIdx.x >= 32) return;
+  const double hn = sqrt(hn2);
+  givens_step(st, col, hn, aa.H, scs, ssn, aa.cs, aa.sn, aa.gv, aa.j, aa.m, aa.ldh, aa.hist);
   if (threadIdx.x != 0) return;
   st->counter[3] = 0;
-  double col[kMaxM + 1];
-  for (int u = 0; u < nv; ++u) col[u] = st->h[u] + st->h[kMaxM + u];
-  const double hn = sqrt(hn2);
-  givens_step(st, col, hn, aa.H, aa.cs, aa.sn, aa.gv, aa.j, aa.m, aa.ldh, aa.hist);
   st->vscale[aa.j + 1] = hn > 0.0 ? 1.0 / hn : 0.0;
+  if (aa.host_done) {
+    *aa.host_done = st->done;
+    __threadfence_system();
+  }
 }
 
 // chunks per column of a coefficient pass over nv columns: about one wave of
@@ -1009,7 +1035,7 @@ struct Job {
       e1 = P->prof_ev[2 * prof.size() + 1];
       cudaEventRecord(e0, s);
     }
-    (launch_pdl(k_arnoldi_spmv<float>, occ_grid((const void*)k_arnoldi_spmv<float>, g.N), kThreads, 0, s, 
+    (launch_cells(k_arnoldi_spmv<float>, g.N, s, 
          g, P->mat->A2, P->mat->A, P->mat->a2_range, zj, w, st),
      note_launch());
     if (e1) {
@@ -1017,9 +1043,11 @@ struct Job {
       prof.push_back({e0, e1});
     }
     if (P->wl) wells_after_product(P, w, split_pad(nn));
-    const ArnoldiArgs aa{P->H, P->cs, P->sn, P->gvec, j, m, m, dhist};
+    // (the last kernel tells the host whether to go on: a kernel of its own for
+    // that cost each column about 2 us)
+    const ArnoldiArgs aa{P->H, P->cs, P->sn, P->gvec, j, m, m, dhist, P->h_st_dev ? &P->h_st_dev[j % kRing].done : nullptr};
     const int nv = j + 1;
-    const int gu = occ_grid((const void*)k_gs_update<true>, nn);
+    const int gu = occ_grid((const void*)k_gs_update<true>, (nn + 3) / 4);
     if (g_gs_fused.load()) {
       // CGS2 in three passes over the basis: the first coefficients, the
       // first update fused with the second coefficients, the final update
@@ -1086,7 +1114,8 @@ struct Job {
     } else {
       enqueue_column_kernels(j, profile);
     }
-    mark(j % kRing);
+    if (!P->h_st_dev) publish_state(P, P->st, j % kRing, stream());
+    cudaEventRecord(P->ev[j % kRing], stream());
   }
 
   void end_cycle() {
@@ -1257,7 +1286,7 @@ void launch_arnoldi_product(bo_prec* P, const double* v, double* w) {
   float* z = (float*)P->Z;  // the first preconditioned vector's split planes as scratch
   float* ws = (float*)P->V;  // the first basis vector's split planes as scratch
   (launch_pdl(k_split_vec, grid_for(n), kThreads, 0, s, n, v, z), note_launch());
-  (launch_pdl(k_arnoldi_spmv<float>, occ_grid((const void*)k_arnoldi_spmv<float>, g.N), kThreads, 0, s, 
+  (launch_cells(k_arnoldi_spmv<float>, g.N, s, 
        g, m->A2, m->A, m->a2_range, z, ws, P->st),
    note_launch());
   (launch_pdl(k_join_vec, grid_for(n), kThreads, 0, s, n, ws, w), note_launch());
@@ -1670,7 +1699,7 @@ bool capture_batch_column(BatchGraphs& c, const std::vector<Job*>& act, int j) {
     cudaStream_t saved = jb->P->stream;
     jb->P->stream = g_bg_cap[r % W];
     jb->enqueue_column_kernels(j, false);
-    publish_state(jb->P, jb->P->st, j % kRing, jb->P->stream);
+    if (!jb->P->h_st_dev) publish_state(jb->P, jb->P->st, j % kRing, jb->P->stream);
     jb->P->stream = saved;
   }
   for (int w = 0; w < W; ++w) {

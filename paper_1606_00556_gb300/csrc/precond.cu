@@ -2631,17 +2631,17 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
   }
   // x1 = R^{-1} f with f = D_QI^{-1} v (stage CPR) or f = v
   if (stage == BO_STAGE_CPR)
-    (launch_pdl(k_cpr_entry<T, S, true>, occ_grid((const void*)k_cpr_entry<T, S, true>, g.N), kThreads, 0, s, g, v, vs, P->w, P->wf,
+    (launch_cells(k_cpr_entry<T, S, true>, g.N, s, g, v, vs, P->w, P->wf,
         D, f, tv, st),
      note_launch());
   else
-    (launch_pdl(k_cpr_entry<T, S, false>, occ_grid((const void*)k_cpr_entry<T, S, false>, g.N), kThreads, 0, s, g, v, vs, P->w, P->wf,
+    (launch_cells(k_cpr_entry<T, S, false>, g.N, s, g, v, vs, P->w, P->wf,
         D, f, tv, st),
      note_launch());
-  (launch_pdl(k_ilu_b<T, S>, occ_grid((const void*)k_ilu_b<T, S>, g.Nh), kThreads, 0, s, g, At, D, f, tv, z1, st),
+  (launch_cells(k_ilu_b<T, S>, g.Nh, s, g, At, D, f, tv, z1, st),
    note_launch());
   // (the pass reads z1's black half and writes its red half)
-  (launch_pdl(k_ilu_r2<T, S, false, false>, occ_grid((const void*)k_ilu_r2<T, S, false, false>, g.Nh), kThreads, 0, s, g, At, D, f, z1, z1,
+  (launch_cells(k_ilu_r2<T, S, false, false>, g.Nh, s, g, At, D, f, z1, z1,
       OutV{}, st),
    note_launch());
   if (stage == BO_STAGE_ILU) {
@@ -2649,19 +2649,19 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
     return;
   }
   // x2 = x1 + Pi_p AMG(A_pp)^{-1} Pi_r (f - At x1)
-  (launch_pdl(k_cpr_rhs<T, S>, occ_grid((const void*)k_cpr_rhs<T, S>, kExactRed<S> ? g.Nh : g.N), kThreads, 0, s, g, At, (const T*)P->di0, f, z1,
+  (launch_cells(k_cpr_rhs<T, S>, kExactRed<S> ? g.Nh : g.N, s, g, At, (const T*)P->di0, f, z1,
       f0, e0, st),
    note_launch());
   amg_vcycle<T, S>(P, st, kExactRed<S>);
   learned_coarse_apply(P, st);
   // x3 = x2 + R^{-1} (f - At x2)
-  (launch_pdl(k_cpr_red<T, S>, occ_grid((const void*)k_cpr_red<T, S>, g.Nh), kThreads, 0, s, g, At, D, f, z1, e0, tv,
+  (launch_cells(k_cpr_red<T, S>, g.Nh, s, g, At, D, f, z1, e0, tv,
       st),
    note_launch());
-  (launch_pdl(k_cpr_black<T, S>, occ_grid((const void*)k_cpr_black<T, S>, g.Nh), kThreads, 0, s, g, At, D, f, tv, z1, e0, tv,
+  (launch_cells(k_cpr_black<T, S>, g.Nh, s, g, At, D, f, tv, z1, e0, tv,
       zo, st),
    note_launch());
-  (launch_pdl(k_ilu_r2<T, S, true, !kExactRed<S>>, occ_grid((const void*)k_ilu_r2<T, S, true, !kExactRed<S>>, g.Nh), kThreads, 0, s, g, At, D, f, tv, nullptr,
+  (launch_cells(k_ilu_r2<T, S, true, !kExactRed<S>>, g.Nh, s, g, At, D, f, tv, nullptr,
       zo, st),
    note_launch());
 }
@@ -2677,21 +2677,22 @@ int values_impl(bo_prec* P) {
   bo_mat* m = P->mat;
   cudaStream_t s = P->stream;
   const Geom& g = m->g;
-  const int gN = grid_for(g.N), gh = grid_for(g.Nh);
-  (launch_pdl(k_decouple<S>, gN, kThreads, 0, s, g, m->A, m->a2_valid ? m->A2 : nullptr, m->a2_range, (S*)P->At, P->w, P->wf,
+  const int tN = cell_threads(g.N), th = cell_threads(g.Nh);
+  const int gN = grid_for(g.N, tN), gh = grid_for(g.Nh, th);
+  (launch_pdl(k_decouple<S>, gN, tN, 0, s, g, m->A, m->a2_valid ? m->A2 : nullptr, m->a2_range, (S*)P->At, P->w, P->wf,
       P->di0, P->opts.decoupling == BO_DECOUPLE_ABF, P->st), note_launch());
   // FP64 red inverses for the black pass: the Krylov basis is idle during setup
   double* red64 = P->V;
   if (sizeof(S) < sizeof(double) && m->a2_valid) {
     // black pivots in split arithmetic (the kernel takes the FP64 products
     // itself where the split copy of A could not hold every value)
-    (launch_pdl(k_ilu_red<S, true>, gh, kThreads, 0, s, g, m->A, P->w, (S*)P->Dinv, red64, P->st), note_launch());
-    (launch_pdl(k_ilu_black_split<S>, gh, kThreads, 0, s, g, m->A2, m->A, m->a2_range, P->w,
+    (launch_pdl(k_ilu_red<S, true>, gh, th, 0, s, g, m->A, P->w, (S*)P->Dinv, red64, P->st), note_launch());
+    (launch_pdl(k_ilu_black_split<S>, gh, th, 0, s, g, m->A2, m->A, m->a2_range, P->w,
         reinterpret_cast<const float2*>(red64), (S*)P->Dinv, P->st),
      note_launch());
   } else {
-    (launch_pdl(k_ilu_red<S, false>, gh, kThreads, 0, s, g, m->A, P->w, (S*)P->Dinv, red64, P->st), note_launch());
-    (launch_pdl(k_ilu_black<S>, gh, kThreads, 0, s, g, m->A, P->w, red64, (S*)P->Dinv, P->st), note_launch());
+    (launch_pdl(k_ilu_red<S, false>, gh, th, 0, s, g, m->A, P->w, (S*)P->Dinv, red64, P->st), note_launch());
+    (launch_pdl(k_ilu_black<S>, gh, th, 0, s, g, m->A, P->w, red64, (S*)P->Dinv, P->st), note_launch());
   }
   // AMG hierarchy values (eight lanes per coarse cell)
   for (int l = 1; l < P->nlev; ++l) {
