@@ -913,6 +913,11 @@ __device__ __forceinline__ void offdiag_sum(const Geom& g, const S* __restrict__
   }
 }
 
+// Whether a red row's residual after a local solve counts as zero (the
+// comment on the CPR's passes below): FP64 and FP32 storage.
+template <typename S>
+constexpr bool kExactRed = sizeof(S) >= 4;
+
 // ILU pass 2 (black): z_b = D_b'^{-1} (f_b - sum A_br t_r), t_r = D_r^{-1} f_r
 // (pass 1).  Pass 3 (red): x_r = D_r^{-1} (f_r - sum A_rb x_b).
 // blocks per SM the register budget is tuned for: the FP32 passes are
@@ -940,34 +945,42 @@ __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_b(Geom g,
 }
 
 // (the black half of xb is read.)  OUT = false: z_r = x_r; OUT = true: the
-// preconditioner's result, from f_r as in the first solve or, with DELTA, as
-// the correction w_r - D_r^{-1} sum A_rb u_b (w_r and u_b the halves of xb)
-template <typename T, typename S, bool OUT, bool DELTA>
+// preconditioner's result.  In BF16 storage x_r is t_r - D_r^{-1} sum A_rb x_b
+// with t_r from tv (see kExactRed), OUT = true adds it to z_r + Pi_p e_r.
+template <typename T, typename S, bool OUT>
 __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* __restrict__ f,
-                         const T* xb, T* z, OutV zo, const DevState* st) {
+                         const T* tv, const T* xb, T* z, const T* __restrict__ e, OutV zo, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
     const Cell c = decode(g, 0, q);
     T s[3];
     offdiag_sum(g, At, 0, q, c, xb, s);
-    T r0 = -s[0], r1 = -s[1], r2 = -s[2];
-    if (!DELTA) r0 += f[vidx(g, 0, 0, q)], r1 += f[vidx(g, 1, 0, q)], r2 += f[vidx(g, 2, 0, q)];
-    T d[9];
+    T d[9], x[3];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
-    T x0 = d[0] * r0 + d[1] * r1 + d[2] * r2;
-    T x1 = d[3] * r0 + d[4] * r1 + d[5] * r2;
-    T x2 = d[6] * r0 + d[7] * r1 + d[8] * r2;
-    if (DELTA) x0 += xb[vidx(g, 0, 0, q)], x1 += xb[vidx(g, 1, 0, q)], x2 += xb[vidx(g, 2, 0, q)];
-    if (OUT) {
-      out_put<T>(zo, vidx(g, 0, 0, q), x0);
-      out_put<T>(zo, vidx(g, 1, 0, q), x1);
-      out_put<T>(zo, vidx(g, 2, 0, q), x2);
+    if (kExactRed<S>) {
+      T r[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) r[k] = f[vidx(g, k, 0, q)] - s[k];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) x[k] = d[3 * k] * r[0] + d[3 * k + 1] * r[1] + d[3 * k + 2] * r[2];
     } else {
-      z[vidx(g, 0, 0, q)] = x0;
-      z[vidx(g, 1, 0, q)] = x1;
-      z[vidx(g, 2, 0, q)] = x2;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const T corr = d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2];
+        x[k] = tv[vidx(g, k, 0, q)] - corr;
+      }
+      if (OUT) {
+        x[0] = z[vidx(g, 0, 0, q)] + e[q] + x[0];
+        x[1] = z[vidx(g, 1, 0, q)] + x[1];
+        x[2] = z[vidx(g, 2, 0, q)] + x[2];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (OUT) out_put<T>(zo, vidx(g, k, 0, q), x[k]);
+      else z[vidx(g, k, 0, q)] = x[k];
     }
   }
 }
@@ -993,20 +1006,21 @@ __device__ __forceinline__ float gs_divide(float s, float d, const float*, size_
 // pass read it twice, and the red rows of x3 again have no residual:
 //   x3_r = D_r^{-1} (f_r - A_rb x3_b).
 // All of it holds where the stored pivots invert the stored diagonal blocks
-// to working precision.  BF16 storage rounds both to 8 bits, and (1), (2) and
-// the last line would change the preconditioner (measured: the solution moved
-// by 2e-9 at a tolerance of 1e-8, 2 of 24 systems took an iteration more), so
-// it keeps the residuals of the red cells and the correction form
-//   w_r = x2_r + D_r^{-1} (f - A x2)_r,  u_b = x3_b - x2_b,
-//   x3_r = w_r - D_r^{-1} A_rb u_b,
-// and gains by the fused black pass alone.  Newton step, 128x128x64 FP32 at 19
-// iterations 11.96 -> 10.59 ms, FP64 19.4 -> 16.8 ms; 256x256x128 BF16 80.7 ->
-// 77.1 ms; 62x45x19 FP32 1853 -> 1714 us.  Iterations are those of the form
+// to working precision.  BF16 storage rounds both to 8 bits, where (1), (2)
+// and the last line change the preconditioner, and even another order of its
+// sums moves a solution by more than the solver's tolerance (3.6e-8 at
+// 256x256x128 and 1e-8: FGMRES then stops at another iterate).  So BF16 keeps
+// the residuals of all cells and adds up what the local solve of a whole
+// residual adds up, in that order,
+//   t_r = D_r^{-1} r_r,  u_b = D_b'^{-1} (r_b - A_br t_r),
+//   x3_b = x2_b + u_b,   x3_r = x2_r + (t_r - D_r^{-1} A_rb u_b),
+// and gains by the black pass alone, which forms r_b = (f - A x2)_b and
+// A_br t_r over one read of A_br.  (The solutions are those of separate
+// passes bit for bit; 256x256x128 81.9 -> 75.4 ms.)
+// Newton step, 128x128x64 FP32 at 19 iterations 11.96 -> 10.59 ms, FP64 19.4
+// -> 16.8 ms; 62x45x19 FP32 1853 -> 1714 us.  Iterations are those of the form
 // before this one: 307 over 24 systems of 20x20x5 to 150x149x40 in FP64 and
 // in FP32.
-template <typename S>
-constexpr bool kExactRed = sizeof(S) >= 4;
-
 
 // AMG right-hand side: f0_b = f_p - (A z)_p, f0_r = 0, and with it the first
 // pre-smoothing sweep from zero, x_r = 0 and x_b = f0_b / a_bb; in BF16 f0
@@ -1050,7 +1064,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cpr_rhs(Ge
   }
 }
 
-// w_r = z_r - D_r^{-1} sum_b A_rb Pi_p e_b, or w_r = x2_r + D_r^{-1} (f - A x2)_r
+// w_r = z_r - D_r^{-1} sum_b A_rb Pi_p e_b, in BF16 t_r = D_r^{-1} (f - A x2)_r
 template <typename T, typename S>
 __global__ void __launch_bounds__(kThreads, kExactRed<S> && sizeof(T) == 4 ? 5 : 4) k_cpr_red(Geom g, const S* __restrict__ At,
                          const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ z,
@@ -1059,30 +1073,24 @@ __global__ void __launch_bounds__(kThreads, kExactRed<S> && sizeof(T) == 4 ? 5 :
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
     const Cell c = decode(g, 0, q);
-    T x[3], s[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) x[k] = z[vidx(g, k, 0, q)];
-    if (!kExactRed<S>) x[0] += e[q];
+    T s[3] = {T(0), T(0), T(0)};
 #pragma unroll
     for (int sl = 0; sl < 7; ++sl) {
+      if (kExactRed<S> && sl == kDiag) continue;
       const S* a = At + at_index(g, 0, sl * 9, q);
       constexpr size_t P = 32;  // entries (rc) of a block lie 32 apart in a tile
+      const int64_t nb = nbr(g, c, q, sl);
+      const bool ok = nb >= 0;
+      const int64_t nq = ok ? nb : q;
       if (kExactRed<S>) {
-        if (sl == kDiag) continue;
-        const int64_t nb = nbr(g, c, q, sl);
-        const T en = e[g.Nh + (nb >= 0 ? nb : q)];
-        const T xn = nb >= 0 ? -en : T(0);
+        const T en = e[g.Nh + nq];
+        const T xn = ok ? -en : T(0);
 #pragma unroll
         for (int k = 0; k < 3; ++k) s[k] = fma(cv<T>(ld_stream(a + 3 * k * P)), xn, s[k]);
       } else {
-        const int64_t nb = nbr(g, c, q, sl);
-        const bool ok = nb >= 0;
-        const int64_t nq = ok ? nb : q;
-        T x0 = x[0], x1 = x[1], x2 = x[2];
-        if (sl != kDiag) {
-          x0 = z[vidx(g, 0, 1, nq)] + e[g.Nh + nq], x1 = z[vidx(g, 1, 1, nq)], x2 = z[vidx(g, 2, 1, nq)];
-          if (!ok) x0 = x1 = x2 = T(0);
-        }
+        const int xc = sl == kDiag ? 0 : 1;
+        T x0 = z[vidx(g, 0, xc, nq)] + e[(size_t)xc * g.Nh + nq], x1 = z[vidx(g, 1, xc, nq)], x2 = z[vidx(g, 2, xc, nq)];
+        if (!ok) x0 = x1 = x2 = T(0);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
           s[k] = fma3(s[k], cv<T>(ld_stream(a + 3 * k * P)), x0, cv<T>(ld_stream(a + (3 * k + 1) * P)), x1,
@@ -1097,13 +1105,16 @@ __global__ void __launch_bounds__(kThreads, kExactRed<S> && sizeof(T) == 4 ? 5 :
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-      w[vidx(g, k, 0, q)] = x[k] + (d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2]);
+    for (int k = 0; k < 3; ++k) {
+      const T t = d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2];
+      w[vidx(g, k, 0, q)] = kExactRed<S> ? z[vidx(g, k, 0, q)] + t : t;
+    }
   }
 }
 
 // x3_b = x2_b + D_b'^{-1} (f_b - A_bb x2_b - A_br w_r), x2_b = z_b + Pi_p e_b:
-// the preconditioner's result, and x3_b (BF16: u_b) into xb for the red pass
+// the preconditioner's result, and x3_b into xb for the red pass.  In BF16
+// w is t_r, x3_b = x2_b + D_b'^{-1} ((f - A x2)_b - A_br t_r), xb takes u_b.
 template <typename T, typename S>
 __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_cpr_black(Geom g, const S* __restrict__ At,
                          const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ w,
@@ -1113,19 +1124,44 @@ __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_cpr_black(Geo
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
     const Cell c = decode(g, 1, q);
-    T s[3];
-    offdiag_sum(g, At, 1, q, c, w, s);
-    const T x0 = z[vidx(g, 0, 1, q)] + e[g.Nh + q], x1 = z[vidx(g, 1, 1, q)], x2 = z[vidx(g, 2, 1, q)];
-    const S* a = At + at_index(g, 1, kDiag * 9, q);
+    const T x[3] = {z[vidx(g, 0, 1, q)] + e[g.Nh + q], z[vidx(g, 1, 1, q)], z[vidx(g, 2, 1, q)]};
     T r[3];
+    if (kExactRed<S>) {
+      T s[3];
+      offdiag_sum(g, At, 1, q, c, w, s);
+      const S* a = At + at_index(g, 1, kDiag * 9, q);
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-      r[k] = f[vidx(g, k, 1, q)] - fma3(s[k], cv<T>(ld_stream(a + 96 * k)), x0, cv<T>(ld_stream(a + 96 * k + 32)), x1,
-                                        cv<T>(ld_stream(a + 96 * k + 64)), x2);
+      for (int k = 0; k < 3; ++k)
+        r[k] = f[vidx(g, k, 1, q)] - fma3(s[k], cv<T>(ld_stream(a + 96 * k)), x[0], cv<T>(ld_stream(a + 96 * k + 32)), x[1],
+                                          cv<T>(ld_stream(a + 96 * k + 64)), x[2]);
+    } else {
+      T acc[3] = {T(0), T(0), T(0)}, s[3] = {T(0), T(0), T(0)};
+#pragma unroll
+      for (int sl = 0; sl < 7; ++sl) {
+        const S* a = At + at_index(g, 1, sl * 9, q);
+        T y[3] = {x[0], x[1], x[2]}, t[3];
+        if (sl != kDiag) {
+          const int64_t nb = nbr(g, c, q, sl);
+          const bool ok = nb >= 0;
+          const int64_t nq = ok ? nb : q;
+          y[0] = z[vidx(g, 0, 0, nq)] + e[nq], y[1] = z[vidx(g, 1, 0, nq)], y[2] = z[vidx(g, 2, 0, nq)];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) t[k] = w[vidx(g, k, 0, nq)];
+          if (!ok) y[0] = y[1] = y[2] = t[0] = t[1] = t[2] = T(0);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const T a0 = cv<T>(ld_stream(a + 96 * k)), a1 = cv<T>(ld_stream(a + 96 * k + 32)), a2 = cv<T>(ld_stream(a + 96 * k + 64));
+          acc[k] = fma3(acc[k], a0, y[0], a1, y[1], a2, y[2]);
+          if (sl != kDiag) s[k] = fma3(s[k], a0, t[0], a1, t[1], a2, t[2]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) r[k] = (f[vidx(g, k, 1, q)] - acc[k]) - s[k];
+    }
     T d[9];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + g.Nh + q]);
-    const T x[3] = {x0, x1, x2};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const T u = d[3 * k] * r[0] + d[3 * k + 1] * r[1] + d[3 * k + 2] * r[2];
@@ -2641,8 +2677,7 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
   (launch_cells(k_ilu_b<T, S>, g.Nh, s, g, At, D, f, tv, z1, st),
    note_launch());
   // (the pass reads z1's black half and writes its red half)
-  (launch_cells(k_ilu_r2<T, S, false, false>, g.Nh, s, g, At, D, f, z1, z1,
-      OutV{}, st),
+  (launch_cells(k_ilu_r2<T, S, false>, g.Nh, s, g, At, D, f, tv, z1, z1, nullptr, OutV{}, st),
    note_launch());
   if (stage == BO_STAGE_ILU) {
     (launch_pdl(k_widen_t<T>, grid_for(3 * g.N), kThreads, 0, s, 3 * g.N, z1, zo.d, st), note_launch());
@@ -2661,8 +2696,7 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
   (launch_cells(k_cpr_black<T, S>, g.Nh, s, g, At, D, f, tv, z1, e0, tv,
       zo, st),
    note_launch());
-  (launch_cells(k_ilu_r2<T, S, true, !kExactRed<S>>, g.Nh, s, g, At, D, f, tv, nullptr,
-      zo, st),
+  (launch_cells(k_ilu_r2<T, S, true>, g.Nh, s, g, At, D, f, tv, tv, z1, e0, zo, st),
    note_launch());
 }
 
