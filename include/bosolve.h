@@ -720,9 +720,19 @@ int bo_set_amg_barrier_spins(uint32_t spins);
  * 0 four separate passes.  The same arithmetic; process-wide. */
 int bo_set_gs_fused(int on);
 /* BO_ERR_TIMEOUT if a tcgen05 convolution gave up waiting on one of its
- * barriers since the last call (its output is then incomplete), else BO_OK;
- * clears the flag.  Synchronises the device. */
+ * barriers since the last call (the outputs it did not reach are then NaN),
+ * else BO_OK; clears the flag.  Process-wide; synchronises the device.  The
+ * convolution and network calls that synchronise (bo_conv3d_backward_*,
+ * bo_cnn_backward with a loss, bo_cnn_get_grads) return BO_ERR_TIMEOUT
+ * themselves, once, where that happened to a call on their context since. */
 int bo_tc_status(void);
+/* Makes the tcgen05 convolutions' bounded waits run out (process-wide; read
+ * at each launch): the warp that issues a block's MMAs takes its wait for the
+ * block's tile number `tile` as expired, and the block's other waits then end
+ * as they do after a real expiry.  A negative number restores the default,
+ * never.  No counterpart in the paper: it exists so that error path can be
+ * exercised without hanging a GPU. */
+int bo_set_conv_expire_tile(int tile);
 
 #ifdef __cplusplus
 }

@@ -60,6 +60,7 @@ EXPORTS = (
     "bo_dp_destroy",
     "bo_prec_set_launch_mode", "bo_prec_set_amg_tile", "bo_set_batch_streams", "bo_autotune_batched", "bo_update_batched",
     "bo_set_conv_engine", "bo_tc_status", "bo_set_amg_cooperative", "bo_set_amg_barrier_spins", "bo_set_gs_fused",
+    "bo_set_conv_expire_tile",
     "bo_newton_opts_default", "bo_model_create", "bo_model_destroy", "bo_model_assemble", "bo_newton_solve",
     "bo_wells_create", "bo_wells_update_values", "bo_wells_set_coupling", "bo_wells_spmv", "bo_solve_bordered",
     "bo_wells_destroy",
@@ -225,6 +226,7 @@ def lib():
         L.bo_set_amg_barrier_spins.argtypes = [ctypes.c_uint32]
         L.bo_set_gs_fused.argtypes = [_i]
         L.bo_tc_status.argtypes = []
+        L.bo_set_conv_expire_tile.argtypes = [_i]
         L.bo_update_batched.argtypes = [ctypes.POINTER(_VP), _i, ctypes.POINTER(_VP), _i]
         L.bo_autotune_batched.argtypes = [ctypes.POINTER(_VP), _i, ctypes.POINTER(_VP), ctypes.POINTER(_VP),
                                           ctypes.POINTER(bo_solve_opts), ctypes.c_char_p, ctypes.POINTER(bo_tune_result)]
@@ -849,6 +851,11 @@ def bo_set_amg_barrier_spins(spins: int):
 def bo_set_conv_engine(engine: int):
     """Convolutions on 0: mma.sync, 1 (default): tcgen05."""
     _check(lib().bo_set_conv_engine(int(engine)), "bo_set_conv_engine")
+
+
+def bo_set_conv_expire_tile(tile: int):
+    """The tile of each block of a tcgen05 convolution whose wait is taken as expired (negative: none)."""
+    _check(lib().bo_set_conv_expire_tile(int(tile)), "bo_set_conv_expire_tile")
 
 
 def bo_tc_status() -> int:

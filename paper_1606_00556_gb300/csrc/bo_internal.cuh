@@ -340,6 +340,15 @@ extern std::atomic<int> g_conv_engine;
 extern std::atomic<int> g_amg_coop;
 // polls of an AMG grid barrier before it gives up (default 2^22, about 0.1 s)
 constexpr unsigned kAmgSpinsDefault = 1u << 22;
+// tcgen05 convolutions: the tile of each block whose wait is taken to expire
+// (by default one that no block reaches), and the word that a kernel with an
+// expired wait sets (the context's)
+constexpr int kConvNoTile = INT32_MAX;
+extern std::atomic<int> g_conv_expire_tile;
+struct TcWait {
+  int tiles;
+  int* err;
+};
 extern std::atomic<unsigned> g_amg_spins;
 // Gram-Schmidt form: 1 (default) three passes (first update fused with the
 // second coefficients), 0 four separate passes
@@ -417,6 +426,7 @@ struct bo_ctx {
   bool own_stream;
   int refs;
   void* scratch;         // workspace of the single-layer gradient calls (ordered on the stream like them), or NULL
+  int* tc_err;           // pinned word that a tcgen05 convolution on this context sets when a wait expires
   size_t scratch_bytes;  // at most one layer's partial sums (about 34 MB); freed with the context
 };
 
@@ -573,6 +583,10 @@ void launch_spmv_decoupled_internal(bo_prec* P, const double* x, double* y);  //
 
 // capi.cu: drop a reference on a context (frees it with the last one)
 void ctx_release_ref(bo_ctx* c);
+// the end of the context's stream: BO_ERR_TIMEOUT once after a tcgen05
+// convolution on it gave up a wait
+int ctx_synchronize(bo_ctx* c);
+TcWait tc_wait(const bo_ctx* c);
 // the context's workspace, grown to `bytes` (NULL if that fails)
 void* ctx_scratch(bo_ctx* c, size_t bytes);
 
@@ -606,13 +620,13 @@ void graphs_reset(bo_prec* P);
 // the data gradient.  BO_ERR_ARG where it does not apply.
 int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W,
                    const float* bias, const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, bool transposed,
-                   cudaStream_t s);
+                   const TcWait& lim, cudaStream_t s);
 // tcgen05 weight and bias gradients of a layer (part: room for kWgradTcBlocks
 // partials of 27 cin cout floats, bpart: of cout doubles); BO_ERR_ARG where it
 // does not apply
 constexpr int kWgradTcBlocks = 304;
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
-                    double* bpart, float* dW, float* db, cudaStream_t s);
+                    double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s);
 // dense FP64 inverse of an n x n matrix (n <= 128) by one block; sets
 // st->err on a zero pivot
 int launch_dense_inverse64(int n, const double* M, double* Minv, DevState* st, cudaStream_t s);

@@ -19,6 +19,7 @@ std::atomic<int> g_pool_width{kMaxPoolStreams};
 std::atomic<int> g_conv_engine{1};
 std::atomic<int> g_amg_coop{2};
 std::atomic<unsigned> g_amg_spins{kAmgSpinsDefault};
+std::atomic<int> g_conv_expire_tile{kConvNoTile};
 std::atomic<int> g_gs_fused{1};
 
 int occ_grid(const void* kernel, int64_t n, int threads, size_t smem) {
@@ -51,6 +52,7 @@ void ctx_release(bo_ctx* c) {
   if (--c->refs > 0) return;
   cudaStreamSynchronize(c->stream);
   if (c->scratch) cudaFree(c->scratch);
+  cudaFreeHost(c->tc_err);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -125,6 +127,15 @@ void mat_release(bo_mat* m) {
 namespace bo {
 void ctx_release_ref(bo_ctx* c) { ctx_release(c); }
 void mat_release_ref(bo_mat* m) { mat_release(m); }
+// (the word is pinned, so the device reaches it at its host address)
+TcWait tc_wait(const bo_ctx* c) { return TcWait{g_conv_expire_tile.load(), c->tc_err}; }
+int ctx_synchronize(bo_ctx* c) {
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return BO_ERR_CUDA;
+  volatile int* err = c->tc_err;
+  if (!*err) return BO_OK;
+  *err = 0;
+  return BO_ERR_TIMEOUT;
+}
 void* ctx_scratch(bo_ctx* c, size_t bytes) {
   if (c->scratch_bytes < bytes) {
     cudaStreamSynchronize(c->stream);  // calls that still use the old one
@@ -317,11 +328,18 @@ int bo_ctx_create(int device, void* cuda_stream, bo_ctx** out) {
   if (!c) return BO_ERR_OOM;
   c->device = device;
   c->refs = 1;
+  if (cudaHostAlloc((void**)&c->tc_err, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    delete c;
+    return BO_ERR_OOM;
+  }
+  *c->tc_err = 0;
   if (cuda_stream) {
     c->stream = (cudaStream_t)cuda_stream;
     c->own_stream = false;
   } else {
     if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaFreeHost(c->tc_err);
       delete c;
       return BO_ERR_CUDA;
     }
@@ -595,6 +613,11 @@ int bo_set_amg_cooperative(int on) {
 
 int bo_set_amg_barrier_spins(uint32_t spins) {
   g_amg_spins.store(spins == 0 ? kAmgSpinsDefault : spins);
+  return BO_OK;
+}
+
+int bo_set_conv_expire_tile(int tile) {
+  g_conv_expire_tile.store(tile < 0 ? kConvNoTile : tile);
   return BO_OK;
 }
 

@@ -386,10 +386,10 @@ int launch_fwd_t(int nx, int ny, int nz, int B, const bf16* X, const bf16* W, co
 enum FwdMode { kReluBf16, kReluResBf16, kLinearOut, kLinearF32All };
 
 int launch_fwd(int cin, int cout, FwdMode mode, int nx, int ny, int nz, int B, const bf16* X, const bf16* W,
-               const float* bias, const bf16* R, bf16* Y, float* Yf, cudaStream_t s) {
+               const float* bias, const bf16* R, bf16* Y, float* Yf, const TcWait& lim, cudaStream_t s) {
   if (g_conv_engine.load() == 1) {
     const int tm = mode == kReluBf16 ? 0 : mode == kReluResBf16 ? 1 : mode == kLinearF32All ? 2 : 3;
-    const int rc = launch_conv_tc(cin, cout, nx, ny, nz, B, X, W, bias, R, Y, Yf, tm, false, s);
+    const int rc = launch_conv_tc(cin, cout, nx, ny, nz, B, X, W, bias, R, Y, Yf, tm, false, lim, s);
     if (rc != BO_ERR_ARG) return rc;  // else: the mma.sync kernel below
   }
   if (mode == kReluBf16 && cin == 16 && cout == 32)
@@ -439,22 +439,22 @@ int launch_wgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* X
 // (the tcgen05 kernel transposes them itself; wd and zero_bias are the
 // mma.sync kernel's).
 int launch_dgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* dY, const bf16* W, bf16* wd,
-                 const float* zero_bias, float* dX, cudaStream_t s) {
+                 const float* zero_bias, float* dX, const TcWait& lim, cudaStream_t s) {
   if (g_conv_engine.load() == 1) {
-    const int rc = launch_conv_tc(cout, cin, nx, ny, nz, B, dY, W, nullptr, nullptr, nullptr, dX, 2, true, s);
+    const int rc = launch_conv_tc(cout, cin, nx, ny, nz, B, dY, W, nullptr, nullptr, nullptr, dX, 2, true, lim, s);
     if (rc != BO_ERR_ARG) return rc;
   }
   (k_flip_transpose<<<grid_for(27 * cin * cout), kThreads, 0, s>>>(W, wd, cin, cout), note_launch());
-  return launch_fwd(cout, cin, kLinearF32All, nx, ny, nz, B, dY, wd, zero_bias, nullptr, nullptr, dX, s);
+  return launch_fwd(cout, cin, kLinearF32All, nx, ny, nz, B, dY, wd, zero_bias, nullptr, nullptr, dX, lim, s);
 }
 
 // Weight and bias gradients of a layer from its input X (BF16) and dY
 // (FP32; its BF16 copy dY16 is made here unless have16).  dY16 = NULL: the
 // tcgen05 kernel only, which needs no copy (BO_ERR_ARG where it does not apply).
 int launch_layer_wgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* X, const float* dY, bf16* dY16,
-                       bool have16, float* part, double* bpart, float* dW, float* db, cudaStream_t s) {
+                       bool have16, float* part, double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s) {
   if (g_conv_engine.load() == 1) {
-    const int rc = launch_wgrad_tc(cin, cout, nx, ny, nz, B, X, dY, part, bpart, dW, db, s);
+    const int rc = launch_wgrad_tc(cin, cout, nx, ny, nz, B, X, dY, part, bpart, dW, db, lim, s);
     if (rc != BO_ERR_ARG) {
       // (the data gradient that may follow reads dY16)
       if (rc == BO_OK && dY16 && !have16)
@@ -573,13 +573,14 @@ void sync_p16(bo_cnn* n) {
 
 int cnn_forward(bo_cnn* n, const bf16* x, int B) {
   cudaStream_t s = n->ctx->stream;
+  const bo::TcWait lim = bo::tc_wait(n->ctx);
   if (cudaMemcpyAsync(n->act[0], x, (size_t)B * n->V * 16 * 2, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return BO_ERR_CUDA;
   for (size_t l = 0; l < n->layers.size(); ++l) {
     const Layer& L = n->layers[l];
     const bf16* R = L.mode == bo::kReluResBf16 ? n->act[l - 1] : nullptr;  // the block's input
     const int rc = bo::launch_fwd(L.cin, L.cout, L.mode, n->nx, n->ny, n->nz, B, n->act[l], n->p16 + L.woff,
-                                  n->p + L.boff, R, n->act[l + 1], L.mode == bo::kLinearOut ? n->outf : nullptr, s);
+                                  n->p + L.boff, R, n->act[l + 1], L.mode == bo::kLinearOut ? n->outf : nullptr, lim, s);
     if (rc != BO_OK) return rc;
   }
   return BO_OK;
@@ -590,6 +591,7 @@ int cnn_backward(bo_cnn* n, const bf16* x, const float* target, const float* mas
   int rc = cnn_forward(n, x, B);
   if (rc != BO_OK) return rc;
   cudaStream_t s = n->ctx->stream;
+  const bo::TcWait lim = bo::tc_wait(n->ctx);
   const int64_t BV = (int64_t)B * n->V;
   const int nl = (int)n->layers.size();
   const int lgrid = bo::grid_for(BV, bo::kThreads, 1024);
@@ -600,10 +602,10 @@ int cnn_backward(bo_cnn* n, const bf16* x, const float* target, const float* mas
   // output layer (linear)
   const Layer& Lo = n->layers[nl - 1];
   rc = bo::launch_layer_wgrad(Lo.cin, Lo.cout, n->nx, n->ny, n->nz, B, n->act[nl - 1], n->gA, n->g16, false,
-                              n->part, n->bpart, n->gr + Lo.woff, n->gr + Lo.boff, s);
+                              n->part, n->bpart, n->gr + Lo.woff, n->gr + Lo.boff, lim, s);
   if (rc != BO_OK) return rc;
   rc = bo::launch_dgrad(Lo.cin, Lo.cout, n->nx, n->ny, n->nz, B, n->g16, n->p16 + Lo.woff, n->wd, n->zero_bias,
-                        n->gB, s);  // gB = d act[nl-1] (output of the last block)
+                        n->gB, lim, s);  // gB = d act[nl-1] (output of the last block)
   if (rc != BO_OK) return rc;
   // residual blocks, last to first: layer a = l - 1, layer b = l
   for (int l = nl - 2; l >= 2; l -= 2) {
@@ -614,20 +616,20 @@ int cnn_backward(bo_cnn* n, const bf16* x, const float* target, const float* mas
     (bo::k_relu_bwd<<<bo::grid_for(cnt), bo::kThreads, 0, s>>>(n->gB, n->act[l + 1], n->gA, n->g16, cnt),
      bo::note_launch());
     rc = bo::launch_layer_wgrad(Lb.cin, Lb.cout, n->nx, n->ny, n->nz, B, n->act[l], n->gA, n->g16, true,
-                                n->part, n->bpart, n->gr + Lb.woff, n->gr + Lb.boff, s);
+                                n->part, n->bpart, n->gr + Lb.woff, n->gr + Lb.boff, lim, s);
     if (rc != BO_OK) return rc;
     rc = bo::launch_dgrad(Lb.cin, Lb.cout, n->nx, n->ny, n->nz, B, n->g16, n->p16 + Lb.woff, n->wd, n->zero_bias,
-                          n->gC, s);  // gC = d act[l] (output of conv a)
+                          n->gC, lim, s);  // gC = d act[l] (output of conv a)
     if (rc != BO_OK) return rc;
     // the residual path: d block input starts as dpre_b (gA); keep it in gB
     cudaMemcpyAsync(n->gB, n->gA, cnt * 4, cudaMemcpyDeviceToDevice, s);
     (bo::k_relu_bwd<<<bo::grid_for(cnt), bo::kThreads, 0, s>>>(n->gC, n->act[l], n->gA, n->g16, cnt),
      bo::note_launch());
     rc = bo::launch_layer_wgrad(La.cin, La.cout, n->nx, n->ny, n->nz, B, n->act[l - 1], n->gA, n->g16, true,
-                                n->part, n->bpart, n->gr + La.woff, n->gr + La.boff, s);
+                                n->part, n->bpart, n->gr + La.woff, n->gr + La.boff, lim, s);
     if (rc != BO_OK) return rc;
     rc = bo::launch_dgrad(La.cin, La.cout, n->nx, n->ny, n->nz, B, n->g16, n->p16 + La.woff, n->wd, n->zero_bias,
-                          n->gC, s);
+                          n->gC, lim, s);
     if (rc != BO_OK) return rc;
     (bo::k_add_f32<<<bo::grid_for(cnt), bo::kThreads, 0, s>>>(n->gB, n->gC, cnt), bo::note_launch());
   }
@@ -636,15 +638,17 @@ int cnn_backward(bo_cnn* n, const bf16* x, const float* target, const float* mas
   (bo::k_relu_bwd<<<bo::grid_for(BV * 32), bo::kThreads, 0, s>>>(n->gB, n->act[1], n->gA, n->g16, BV * 32),
    bo::note_launch());
   rc = bo::launch_layer_wgrad(Li.cin, Li.cout, n->nx, n->ny, n->nz, B, n->act[0], n->gA, n->g16, true,
-                              n->part, n->bpart, n->gr + Li.woff, n->gr + Li.boff, s);
+                              n->part, n->bpart, n->gr + Li.woff, n->gr + Li.boff, lim, s);
   if (rc != BO_OK) return rc;
   if (loss) {
     std::vector<double> lp(lgrid);
     cudaMemcpyAsync(lp.data(), n->loss_part, lgrid * sizeof(double), cudaMemcpyDeviceToHost, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) return BO_ERR_CUDA;
+    rc = bo::ctx_synchronize(n->ctx);
+    if (rc == BO_ERR_CUDA) return rc;
     double t = 0.0;
     for (double q : lp) t += q;
     *loss = t;
+    if (rc != BO_OK) return rc;
   }
   return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
 }
@@ -731,7 +735,7 @@ int bo_cnn_set_params(bo_cnn* n, const float* host, int64_t count) {
 int bo_cnn_get_grads(bo_cnn* n, float* host, int64_t cap) {
   if (!n || !host || cap < n->nparam) return BO_ERR_ARG;
   cudaMemcpyAsync(host, n->gr, n->nparam * 4, cudaMemcpyDeviceToHost, n->ctx->stream);
-  return cudaStreamSynchronize(n->ctx->stream) == cudaSuccess ? BO_OK : BO_ERR_CUDA;
+  return bo::ctx_synchronize(n->ctx);
 }
 
 int bo_cnn_forward(bo_cnn* n, const uint16_t* x, int batch, float* pred) {
@@ -774,7 +778,7 @@ int bo_conv3d_forward(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, i
   else return BO_ERR_ARG;
   return bo::launch_fwd(cin, cout, mode, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x),
                         reinterpret_cast<const bf16*>(w), bias, reinterpret_cast<const bf16*>(residual),
-                        reinterpret_cast<bf16*>(y), yf, ctx->stream);
+                        reinterpret_cast<bf16*>(y), yf, bo::tc_wait(ctx), ctx->stream);
 }
 
 int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* dy,
@@ -784,10 +788,11 @@ int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int 
     return BO_ERR_ARG;
   if (bo::g_conv_engine.load() == 1) {  // no workspace
     const int rc = bo::launch_conv_tc(cout, cin, nx, ny, nz, batch, reinterpret_cast<const bf16*>(dy),
-                                      reinterpret_cast<const bf16*>(w), nullptr, nullptr, nullptr, dx, 2, true, ctx->stream);
+                                      reinterpret_cast<const bf16*>(w), nullptr, nullptr, nullptr, dx, 2, true,
+                                      bo::tc_wait(ctx), ctx->stream);
     if (rc != BO_ERR_ARG) {
-      cudaStreamSynchronize(ctx->stream);
-      return rc;
+      const int rs = bo::ctx_synchronize(ctx);
+      return rc != BO_OK ? rc : rs;
     }
   }
   bf16* wd = nullptr;
@@ -796,11 +801,11 @@ int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int 
   if (cudaMalloc(&zb, 64 * 4) != cudaSuccess) { cudaFree(wd); return BO_ERR_OOM; }
   cudaMemsetAsync(zb, 0, 64 * 4, ctx->stream);
   const int rc = bo::launch_dgrad(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(dy),
-                                  reinterpret_cast<const bf16*>(w), wd, zb, dx, ctx->stream);
-  cudaStreamSynchronize(ctx->stream);
+                                  reinterpret_cast<const bf16*>(w), wd, zb, dx, bo::tc_wait(ctx), ctx->stream);
+  const int rs = bo::ctx_synchronize(ctx);
   cudaFree(wd);
   cudaFree(zb);
-  return rc;
+  return rc != BO_OK ? rc : rs;
 }
 
 int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* x,
@@ -814,10 +819,10 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
     void* ws = bo::ctx_scratch(ctx, pb + (size_t)bo::kWgradTcBlocks * 32 * sizeof(double));
     if (!ws) return BO_ERR_OOM;
     const int rc = bo::launch_wgrad_tc(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x), dy, (float*)ws,
-                                       (double*)((char*)ws + pb), dw, db, ctx->stream);
+                                       (double*)((char*)ws + pb), dw, db, bo::tc_wait(ctx), ctx->stream);
     if (rc != BO_ERR_ARG) {
-      cudaStreamSynchronize(ctx->stream);
-      return rc;
+      const int rs = bo::ctx_synchronize(ctx);
+      return rc != BO_OK ? rc : rs;
     }
   }
   const int64_t BV = (int64_t)batch * nx * ny * nz;
@@ -828,11 +833,11 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
             cudaMalloc(&part, (size_t)bo::kWgMaxBlocks * 27 * cin * cout * 4) == cudaSuccess &&
             cudaMalloc(&bpart, (size_t)bo::kWgMaxBlocks * cout * sizeof(double)) == cudaSuccess;
   int rc = ok ? bo::launch_layer_wgrad(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x), dy, d16, false,
-                                       part, bpart, dw, db, ctx->stream)
+                                       part, bpart, dw, db, bo::tc_wait(ctx), ctx->stream)
               : BO_ERR_OOM;
-  cudaStreamSynchronize(ctx->stream);
+  const int rs = bo::ctx_synchronize(ctx);
   cudaFree(d16); cudaFree(part); cudaFree(bpart);
-  return rc;
+  return rc != BO_OK ? rc : rs;
 }
 
 }  // extern "C"

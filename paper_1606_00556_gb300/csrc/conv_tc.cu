@@ -34,7 +34,8 @@
 // tile; up to ten plane buffers and four TMEM accumulators let all three
 // overlap.  Every wait on an mbarrier is bounded: on expiry the CTA records an
 // error, finishes its copies and MMAs in flight (again bounded), frees its
-// TMEM and returns.
+// TMEM and returns; the outputs it did not reach are NaN, and the context's
+// next call that synchronises returns BO_ERR_TIMEOUT.
 // Measured, 64x64x32 voxels x 4 samples, 32 -> 32 channels: forward with
 // residual 103 us a call on the first tcgen05 form (a tap per MMA, a 10 x 18 x
 // 3 halo a tile in 16-byte TMA rows), 63 with the x taps in N and planes copied
@@ -115,6 +116,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const v
     if (stop && (it & 255) == 255 && *stop) return false;
   }
   return false;
+}
+// a wait of this block expired: the block's flag, the process's and the context's
+__device__ __forceinline__ void report_timeout(volatile int* sfail, const TcWait& lim) {
+  *sfail = 1;
+  atomicExch(&g_tc_err, 1);
+  if (lim.err) {
+    *lim.err = 1;
+    __threadfence_system();
+  }
 }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count));
@@ -261,7 +271,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
                                                            const __grid_constant__ CUtensorMap xmap,
                                                            const __grid_constant__ CUtensorMap wmap,
                                                            const float* __restrict__ bias, const bf16* __restrict__ R,
-                                                           bf16* __restrict__ Y, float* __restrict__ Yf) {
+                                                           bf16* __restrict__ Y, float* __restrict__ Yf, const TcWait lim) {
   using L = ConvLayout<CIN, COUT>;
   constexpr int NB = L::NB;
   constexpr int CH = RES || COUT == 16 ? 8 : 16;  // channels an epilogue thread takes at a time (registers)
@@ -333,10 +343,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
           }
         }
       }
-      if (!ok) {
-        *sfail = 1;
-        atomicExch(&g_tc_err, 1);
-      }
+      if (!ok) report_timeout(sfail, lim);
       // no copy is in flight when the block ends
       mbar_wait(wfull, 0);
       for (int k = max(0, seq - g.planes); k < seq; ++k) mbar_wait(full(k % g.planes), (k / g.planes) & 1);
@@ -345,13 +352,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
   } else if (warp == 0) {
     // ---- MMA issue (the whole warp waits, one thread issues)
     if (t0 < t1) {
-      bool ok = __all_sync(0xffffffffu, mbar_wait(wfull, 0));
+      bool ok = __all_sync(0xffffffffu, mbar_wait(wfull, 0, sfail));
       // planes waited for, and the buffer and round of the next one; the
       // buffer of the tile's plane z
       int waited = 0, wbuf = 0, wround = 0, next = 0, cur = 0, issued = 0;
       auto around = [&](int p) { return p < 0 ? p + g.planes : p >= g.planes ? p - g.planes : p; };
       March m(g, t0);
-      for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
+      const int64_t ts = min(t1, t0 + lim.tiles);
+      for (int64_t t = t0; t < ts && ok; ++t, m.next(g)) {
         const int k = (int)(t - t0), a = k % kAccs, z = m.z;
         const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
         if (start) {
@@ -402,12 +410,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
         ++next;
         cur = around(cur + 1);
       }
-      if (!ok) {
-        *sfail = 1;
-        atomicExch(&g_tc_err, 1);
-        // the MMAs in flight finish before shared and tensor memory go away
-        for (int k = max(0, issued - kAccs); k < issued; ++k) mbar_wait(accfull(k % kAccs), (k / kAccs) & 1);
-      }
+      if (!ok || ts < t1) report_timeout(sfail, lim);
+      // the MMAs in flight finish before shared and tensor memory go away (an
+      // epilogue group that gave up has not waited for them)
+      for (int k = max(0, issued - kAccs); k < issued; ++k) mbar_wait(accfull(k % kAccs), (k / kAccs) & 1);
     }
     __syncwarp();
   } else {
@@ -441,8 +447,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
         // (after an expired wait the warp still meets the barriers, and stores nothing)
         if (ok && !mbar_wait(accfull(a), (k / kAccs) & 1, sfail)) {
           ok = false;
-          *sfail = 1;
-          atomicExch(&g_tc_err, 1);
+          report_timeout(sfail, lim);
         }
         ok = __all_sync(0xffffffffu, ok);
         uint32_t pk[8];  // 16 channels in BF16
@@ -532,6 +537,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv3d_tc(const __grid_consta
         for (int i = 0; i < kGroups; ++i) at.next(g);
         place(t + kGroups);
       }
+      // a wait of the block expired: NaN on all tiles of the group (a warp that
+      // did not give up may have added a column of one that did)
+      if (*sfail) {
+        at = March(g, t0);
+        for (int64_t t = t0; t < t1; ++t, at.next(g)) {
+          if ((t - t0) % kGroups != group) continue;
+          place(t);
+          if (!mine) continue;
+          for (int i = 0; i < COUT; ++i) {
+            if (OUT != 1) Y[o + i] = __ushort_as_bfloat16(0x7fff);
+            if (OUT == 1) Yf[o + i] = __int_as_float(0x7fffffff);
+            if (OUT == 2 && i < 4) Yf[(o / COUT) * 4 + i] = __int_as_float(0x7fffffff);
+          }
+        }
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -582,7 +602,7 @@ bool encode(CUtensorMap* map, const bf16* p, int rank, int c, const cuuint64_t* 
 
 template <int CIN, int COUT, int OUT, bool RES, bool TRANSPOSED>
 int run_conv(ConvGrid g, const bf16* X, const bf16* W, const float* bias, const bf16* R, bf16* Y, float* Yf,
-             cudaStream_t s) {
+             const TcWait& lim, cudaStream_t s) {
   using L = ConvLayout<CIN, COUT>;
   CUtensorMap xmap, wmap;
   const cuuint64_t vox[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz * g.B};
@@ -598,7 +618,7 @@ int run_conv(ConvGrid g, const bf16* X, const bf16* W, const float* bias, const 
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return BO_ERR_CUDA;
   const int sms = sm_count();
   const int grid = g.tiles < sms ? (int)g.tiles : sms;
-  (kern<<<grid, kTcThreads, smem, s>>>(g, xmap, wmap, bias, R, Y, Yf), note_launch());
+  (kern<<<grid, kTcThreads, smem, s>>>(g, xmap, wmap, bias, R, Y, Yf, lim), note_launch());
   return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
 }
 
@@ -612,7 +632,7 @@ int run_conv(ConvGrid g, const bf16* X, const bf16* W, const float* bias, const 
 //   bias may be NULL (zero).
 int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W,
                    const float* bias, const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, bool transposed,
-                   cudaStream_t s) {
+                   const TcWait& lim, cudaStream_t s) {
   for (const void* p : {(const void*)X, (const void*)W, (const void*)R, (const void*)Y, (const void*)Yf})
     if (reinterpret_cast<uintptr_t>(p) & 15) return BO_ERR_ARG;
   ConvGrid g{nx, ny, nz, B, 0, 0, 0, 0, 0};
@@ -631,23 +651,23 @@ int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_
   if (best * B > INT32_MAX) return BO_ERR_ARG;
   if (transposed) {
     if (mode != 2) return BO_ERR_ARG;
-    if (cin == 32 && cout == 32) return run_conv<32, 32, 1, false, true>(g, X, W, bias, R, Y, Yf, s);
-    if (cin == 32 && cout == 16) return run_conv<32, 16, 1, false, true>(g, X, W, bias, R, Y, Yf, s);
-    if (cin == 16 && cout == 32) return run_conv<16, 32, 1, false, true>(g, X, W, bias, R, Y, Yf, s);
+    if (cin == 32 && cout == 32) return run_conv<32, 32, 1, false, true>(g, X, W, bias, R, Y, Yf, lim, s);
+    if (cin == 32 && cout == 16) return run_conv<32, 16, 1, false, true>(g, X, W, bias, R, Y, Yf, lim, s);
+    if (cin == 16 && cout == 32) return run_conv<16, 32, 1, false, true>(g, X, W, bias, R, Y, Yf, lim, s);
     return BO_ERR_ARG;
   }
   if (cin == 32 && cout == 32) {
-    if (mode == 0) return run_conv<32, 32, 0, false, false>(g, X, W, bias, R, Y, Yf, s);
-    if (mode == 1) return run_conv<32, 32, 0, true, false>(g, X, W, bias, R, Y, Yf, s);
-    if (mode == 2) return run_conv<32, 32, 1, false, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 0) return run_conv<32, 32, 0, false, false>(g, X, W, bias, R, Y, Yf, lim, s);
+    if (mode == 1) return run_conv<32, 32, 0, true, false>(g, X, W, bias, R, Y, Yf, lim, s);
+    if (mode == 2) return run_conv<32, 32, 1, false, false>(g, X, W, bias, R, Y, Yf, lim, s);
   }
   if (cin == 16 && cout == 32) {
-    if (mode == 0) return run_conv<16, 32, 0, false, false>(g, X, W, bias, R, Y, Yf, s);
-    if (mode == 2) return run_conv<16, 32, 1, false, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 0) return run_conv<16, 32, 0, false, false>(g, X, W, bias, R, Y, Yf, lim, s);
+    if (mode == 2) return run_conv<16, 32, 1, false, false>(g, X, W, bias, R, Y, Yf, lim, s);
   }
   if (cin == 32 && cout == 16) {
-    if (mode == 2) return run_conv<32, 16, 1, false, false>(g, X, W, bias, R, Y, Yf, s);
-    if (mode == 3) return run_conv<32, 16, 2, false, false>(g, X, W, bias, R, Y, Yf, s);
+    if (mode == 2) return run_conv<32, 16, 1, false, false>(g, X, W, bias, R, Y, Yf, lim, s);
+    if (mode == 3) return run_conv<32, 16, 2, false, false>(g, X, W, bias, R, Y, Yf, lim, s);
   }
   return BO_ERR_ARG;
 }
@@ -773,7 +793,7 @@ __device__ __forceinline__ bool wg_plane_f32(const float* T, size_t zb, int nx, 
 template <bool HALO_DY, int CB>
 __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ WgradGrid g, const bf16* __restrict__ X,
                                                           const float* __restrict__ dY, float* __restrict__ part,
-                                                          double* __restrict__ bpart) {
+                                                          double* __restrict__ bpart, const TcWait lim) {
   constexpr int KC = CB / 8;          // chunks of the core tensor (the halo tensor has 4)
   constexpr int kPair = CB == 32 ? 7 : 9;  // accumulators that take two core rows per MMA
   constexpr int CY = HALO_DY ? 32 : CB;    // channels of dY
@@ -887,7 +907,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     // ---- MMA issue (the whole warp waits, one thread issues)
     uint32_t started = 0;
     int waited = 0, next = 0;
-    for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
+    const int64_t ts = min(t1, t0 + lim.tiles);
+    for (int64_t t = t0; t < ts && ok; ++t, m.next(g)) {
       const int k = (int)(t - t0), z = m.z;
       const bool start = t == t0 || z == 0, end = t + 1 == t1 || z == g.nz - 1;
       if (start) next = waited + (z > 0 ? 1 : 0);
@@ -938,12 +959,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     *sstarted = started;
     if (elect_one()) umma_commit(alldone);
     __syncwarp();
-    if (!mbar_wait(alldone, 0)) ok = false;  // every MMA is done before the buffers are used again
+    if (!mbar_wait(alldone, 0) || ts < t1) ok = false;  // every MMA is done before the buffers are used again
   }
-  if (!ok) {
-    *sfail = 1;
-    atomicExch(&g_tc_err, 1);
-  }
+  if (!ok) report_timeout(sfail, lim);
   if (warp >= 1) {
     const bool dyside = (warp < 1 + kWgProd / 32) == HALO_DY;
     if (dyside) {
@@ -957,7 +975,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   // ---- sums out: accumulator i, halo row a (lane quarter), core row r holds
-  // tap (dz, a - r, sx) of halo channel `lane`
+  // tap (dz, a - r, sx) of halo channel `lane`; after an expired wait NaN
   float* red = reinterpret_cast<float*>(sm + kWgOffPlanes);
   const uint32_t started = *sstarted;
   const bool fine = !*sfail;
@@ -972,7 +990,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
         const uint32_t col = pair ? (uint32_t)(2 * CB * i + CB * r) : (uint32_t)(2 * CB * kPair + CB * (i - kPair));
         const int t = 9 * (i / 3) + 3 * dy + i % 3;
         const int tap = HALO_DY ? 26 - t : t;
-        const bool have = fine && ((started >> i) & 1u);
+        const bool have = (started >> i) & 1u;
+        const float none = fine ? 0.f : __int_as_float(0x7fffffff);
 #pragma unroll
         for (int c0 = 0; c0 < CB; c0 += 16) {
           uint32_t v[16];
@@ -986,7 +1005,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             const int o = HALO_DY ? (tap * 32 + lane) * CB + c0 + e : (tap * CB + c0 + e) * 32 + lane;
-            const float f = have ? __uint_as_float(v[e]) : 0.f;
+            const float f = have && fine ? __uint_as_float(v[e]) : none;
             red[o] = r == 0 ? f : red[o] + f;
           }
         }
@@ -1001,7 +1020,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     constexpr int YC = CY / 8;
     double sum = 0.0;
     for (int p = tid / 8; p < kWgProd; p += YC) sum += sbias[p * 8 + tid % 8];
-    bpart[(size_t)blockIdx.x * CY + tid] = sum;
+    bpart[(size_t)blockIdx.x * CY + tid] = fine ? sum : (double)__int_as_float(0x7fffffff);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -1051,7 +1070,7 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ par
 
 template <bool HALO_DY, int CB>
 int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, double* bpart, float* dW, float* db,
-              cudaStream_t s) {
+              const TcWait& lim, cudaStream_t s) {
   auto kern = k_wgrad_tc<HALO_DY, CB>;
   const int planes = kWgHalo * wg_halo_plane(g.tx) + kWgCore * wg_core_plane(g.tx, CB / 8);
   const int red = 27 * 32 * CB * 4;
@@ -1060,7 +1079,7 @@ int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, d
   int grid = sm_count();
   if (grid > kWgradTcBlocks) grid = kWgradTcBlocks;
   if (g.tiles < grid) grid = (int)g.tiles;
-  (kern<<<grid, kWgThreads, smem, s>>>(g, X, dY, part, bpart), note_launch());
+  (kern<<<grid, kWgThreads, smem, s>>>(g, X, dY, part, bpart, lim), note_launch());
   const int n = 27 * 32 * CB;
   (k_wgrad_sum<<<n / 32 + 1, 256, 0, s>>>(part, bpart, dW, db, n, grid, HALO_DY ? 32 : CB), note_launch());
   return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
@@ -1072,7 +1091,7 @@ int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, d
 // kWgradTcBlocks partials of 27 cin cout floats, bpart: of cout doubles);
 // BO_ERR_ARG where it does not apply.
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
-                    double* bpart, float* dW, float* db, cudaStream_t s) {
+                    double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s) {
   if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(dY) & 15)) return BO_ERR_ARG;
   WgradGrid g{nx, ny, nz, B, 0, 0, 0, 0};
   int best = 0;
@@ -1087,9 +1106,9 @@ int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv
   g.nty = (ny + kWgTY - 1) / kWgTY;
   if ((int64_t)g.ntx * g.nty * B > INT32_MAX) return BO_ERR_ARG;
   g.tiles = (int64_t)g.ntx * g.nty * B * nz;
-  if (cin == 32 && cout == 32) return run_wgrad<false, 32>(g, X, dY, part, bpart, dW, db, s);
-  if (cin == 32 && cout == 16) return run_wgrad<false, 16>(g, X, dY, part, bpart, dW, db, s);
-  if (cin == 16 && cout == 32) return run_wgrad<true, 16>(g, X, dY, part, bpart, dW, db, s);
+  if (cin == 32 && cout == 32) return run_wgrad<false, 32>(g, X, dY, part, bpart, dW, db, lim, s);
+  if (cin == 32 && cout == 16) return run_wgrad<false, 16>(g, X, dY, part, bpart, dW, db, lim, s);
+  if (cin == 16 && cout == 32) return run_wgrad<true, 16>(g, X, dY, part, bpart, dW, db, lim, s);
   return BO_ERR_ARG;
 }
 
