@@ -587,7 +587,7 @@ void ctx_release_ref(bo_ctx* c);
 // convolution on it gave up a wait
 int ctx_synchronize(bo_ctx* c);
 TcWait tc_wait(const bo_ctx* c);
-// the context's workspace, grown to `bytes` (NULL if that fails)
+// the context's workspace on its device, grown to `bytes` (NULL if that fails)
 void* ctx_scratch(bo_ctx* c, size_t bytes);
 
 // krylov.cu

@@ -142,6 +142,7 @@ void* ctx_scratch(bo_ctx* c, size_t bytes) {
     if (c->scratch) cudaFree(c->scratch);
     c->scratch = nullptr;
     c->scratch_bytes = 0;
+    if (cudaSetDevice(c->device) != cudaSuccess) return nullptr;
     if (cudaMalloc(&c->scratch, bytes) != cudaSuccess) {
       cudaGetLastError();
       c->scratch = nullptr;

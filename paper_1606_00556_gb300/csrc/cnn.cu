@@ -770,6 +770,7 @@ int bo_conv3d_forward(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, i
   if (!ctx || !x || !w || !bias || batch < 1 || nx < 1 || ny < 1 || nz < 1 ||
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
+  if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   bo::FwdMode mode;
   if (yf && !y && !relu && !residual) mode = bo::kLinearF32All;
   else if (relu && residual && y) mode = bo::kReluResBf16;
@@ -786,6 +787,7 @@ int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int 
   if (!ctx || !dy || !w || !dx || batch < 1 || nx < 1 || ny < 1 || nz < 1 ||
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
+  if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   if (bo::g_conv_engine.load() == 1) {  // no workspace
     const int rc = bo::launch_conv_tc(cout, cin, nx, ny, nz, batch, reinterpret_cast<const bf16*>(dy),
                                       reinterpret_cast<const bf16*>(w), nullptr, nullptr, nullptr, dx, 2, true,
@@ -814,6 +816,7 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
   if (!((cin == 16 && cout == 32) || (cin == 32 && cout == 32) || (cin == 32 && cout == 16))) return BO_ERR_ARG;
+  if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   if (bo::g_conv_engine.load() == 1) {  // the partial sums in the context's workspace
     const size_t pb = (size_t)bo::kWgradTcBlocks * 27 * cin * cout * 4;
     void* ws = bo::ctx_scratch(ctx, pb + (size_t)bo::kWgradTcBlocks * 32 * sizeof(double));

@@ -25,6 +25,7 @@
 #include <new>
 
 #include "bo_internal.cuh"
+#include "per_device.h"
 
 namespace bo {
 namespace {
@@ -2332,41 +2333,36 @@ LevelView<T, S> view(bo_prec* P, int l) {
 
 LevelDims dims_of(const Level& L) { return LevelDims{L.nx, L.ny, L.nz, L.n}; }
 
-// Largest cluster of the resident kernel that the device can co-schedule
-// with its shared memory (16 is a non-portable size), or 0.  Queried once per
-// instantiation.
+// Largest cluster of the resident kernel that the current device can
+// co-schedule with its shared memory (16 is a non-portable size), or 0.
+// Queried, and the kernel's attributes set, once per instantiation and device.
 template <typename T, typename S>
-int resident_max_cluster() {
-  static std::atomic<int> cached{-1};
-  int cs = cached.load();
-  if (cs >= 0) return cs;
-  cs = 0;
-  const void* k = (const void*)k_amg_resident<T, S>;
-  if (cudaFuncSetAttribute(k_amg_resident<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaFuncSetAttribute(k_amg_resident<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax) ==
-          cudaSuccess) {
-    for (int c : {kResMaxCluster, 8, 4, 2, 1}) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(c, 1, 1);
-      cfg.blockDim = dim3(kResThreads, 1, 1);
-      cfg.dynamicSmemBytes = kResSmemMax;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = c;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1) {
-        cs = c;
-        break;
+int resident_max_cluster(int device) {
+  static PerDevice cached;
+  return cached.get(device, [] {
+    const void* k = (const void*)k_amg_resident<T, S>;
+    if (cudaFuncSetAttribute(k_amg_resident<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_amg_resident<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax) ==
+            cudaSuccess) {
+      for (int c : {kResMaxCluster, 8, 4, 2, 1}) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c, 1, 1);
+        cfg.blockDim = dim3(kResThreads, 1, 1);
+        cfg.dynamicSmemBytes = kResSmemMax;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = c;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int nclus = 0;
+        if (cudaOccupancyMaxActiveClusters(&nclus, k, &cfg) == cudaSuccess && nclus >= 1) return c;
       }
     }
-  }
-  cudaGetLastError();
-  cached.store(cs);
-  return cs;
+    cudaGetLastError();
+    return 0;
+  });
 }
 
 // The resident form's levels, cluster and shared-memory layout for P: level
@@ -2379,7 +2375,7 @@ int resident_max_cluster() {
 template <typename T, typename S>
 void resident_plan(bo_prec* P, ResPlan& a) {
   a.cluster = 0;
-  const int maxc = resident_max_cluster<T, S>();
+  const int maxc = resident_max_cluster<T, S>(P->mat->ctx->device);
   const Geom& g = P->mat->g;
   const int last = P->nlev - 1;
   if (maxc < 1 || last < 1 || P->opts.amg_nu1 < 1 || P->opts.amg_nu2 < 1) return;
