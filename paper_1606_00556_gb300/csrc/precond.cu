@@ -1875,8 +1875,11 @@ __host__ __device__ constexpr int res_values() { return sizeof(T) == 4 ? 7 : 8; 
 // its packed copy.
 //   cp:   [colour][value][pair], the values in order -z, -y, -x, +x, +y, +z,
 //         diagonal (, reciprocal), missing neighbours 0
-//   meta: [0][pair] bit 0 the colour of the pair's first cell, the rest the
-//         red cell's aggregate on the next level (natural index and colour);
+//   meta: [0][pair] bit 0 the colour of the pair's first cell, bits 1-6 and
+//         7-12 the neighbours (in that order) that its red and black cell
+//         have, the rest the red cell's aggregate on the next level (natural
+//         index and colour: 16 bits, since no level holds more cells than a
+//         cluster's threads own);
 //         [1], [2][pair] for the red and black cell as an aggregate: the
 //         natural index of its first child on the level above and which
 //         further children exist along x, y, z.  The coarsest level keeps
@@ -1900,6 +1903,7 @@ struct ResPlan {
   double s;
   ResLevel rl[24];
   const void* inv;     // coarse inverse, transposed (storage type)
+  uint32_t zero_off;   // zeros in each block, one a lane: what a missing neighbour's iterate reads as
   uint32_t dense_off;  // right-hand side and solution of the coarsest level: 2 kCoarseMax entries
   uint32_t inv_off;    // staged inverse, or ~0u
   uint32_t smem;
@@ -1948,6 +1952,12 @@ __global__ void k_res_pack(const __grid_constant__ ResPlan a, Geom g, const S* _
       continue;
     }
     const int32_t ny = r.nxy / r.nx, nz = r.n / r.nxy;
+    // the neighbours a cell has, -z, -y, -x, +x, +y, +z
+    auto neighbours = [&](int32_t c) {
+      const int32_t i = c % r.nx, j = (c / r.nx) % ny, k = c / r.nxy;
+      return (k > 0 ? 1 : 0) | (j > 0 ? 2 : 0) | (i > 0 ? 4 : 0) | (i + 1 < r.nx ? 8 : 0) | (j + 1 < ny ? 16 : 0) |
+             (k + 1 < nz ? 32 : 0);
+    };
     // a cell's word as an aggregate of level l - 1
     auto child_word = [&](int32_t c) {
       if (l == a.l0) return 0;
@@ -1966,6 +1976,7 @@ __global__ void k_res_pack(const __grid_constant__ ResPlan a, Geom g, const S* _
     const int32_t par = (c0 % r.nx + (c0 / r.nx) % ny + c0 / r.nxy) & 1;
     T* cp = (T*)r.cp;
     const S* lc = (const S*)coef.c[l];
+    int32_t have = 0;
     for (int col = 0; col < 2; ++col) {
       const int32_t c = c0 + (col ^ par);
       const bool live = c < r.n;
@@ -1978,6 +1989,7 @@ __global__ void k_res_pack(const __grid_constant__ ResPlan a, Geom g, const S* _
       if constexpr (sizeof(T) == 8)
         cp[(size_t)(col * K + 7) * np + q] = !live ? T(1) : l ? (T)lc[(size_t)7 * r.n + c] : di0[(size_t)col * g.Nh + q];
       r.meta[(size_t)(1 + col) * np + q] = live ? child_word(c) : 0;
+      if (live) have |= neighbours(c) << (6 * col);
     }
     int32_t agg = 0;
     const int32_t cr = c0 + par;  // the red cell
@@ -1986,8 +1998,7 @@ __global__ void k_res_pack(const __grid_constant__ ResPlan a, Geom g, const S* _
       const int32_t i = (cr % r.nx) >> 1, j = ((cr / r.nx) % ny) >> 1, k = (cr / r.nxy) >> 1;
       agg = ((i + cl.nx * j + cl.nxy * k) << 1) | ((i + j + k) & 1);
     }
-    r.meta[q] = (agg << 1) | par;
-    (void)nz;
+    r.meta[q] = (agg << 13) | (have << 1) | par;
     return;
   }
 }
@@ -2053,9 +2064,16 @@ __device__ __forceinline__ void res_load(const ResPlan& a, int l, uint32_t base,
       const int32_t c = 2 * qq + (col ^ par);
       r.live[col][p] = in && c < rl.n;
       r.own[col][p] = res_local<T>(rl, base, col, qq);
-      // (a missing neighbour has coefficient 0: any entry of the level will do)
+      // (a missing neighbour reads as zero, whatever the iterates hold: its
+      // coefficient is 0, but 0 times an infinity is not)
+      const uint32_t zl = base + a.zero_off + (threadIdx.x & 31u) * (uint32_t)sizeof(T);
+      const uint32_t zero = DIST ? map_rank(zl, blockIdx.x) : zl;
 #pragma unroll
-      for (int d = 0; d < 6; ++d) r.nb[col][p][d] = res_addr<T, DIST>(rl, base, col ^ 1, min(max(c + off[d], 0) >> 1, np - 1));
+      for (int d = 0; d < 6; ++d) {
+        const bool have = (r.m[p] >> (1 + 6 * col + d)) & 1;
+        const uint32_t ad = res_addr<T, DIST>(rl, base, col ^ 1, have ? (c + off[d]) >> 1 : qq);
+        r.nb[col][p][d] = have ? ad : zero;
+      }
     }
   }
 }
@@ -2187,7 +2205,7 @@ __device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, u
 #pragma unroll
     for (int col = 0; col < 2; ++col) r.f[col][p] = r.live[col][p] ? ld_sh(res_local<T>(rl, base, kSecF + col, q), false, T(0)) : T(0);
     if (!r.live[0][p]) continue;
-    const int32_t agg = r.m[p] >> 1;
+    const int32_t agg = r.m[p] >> 13;
     uint32_t ad;
     int32_t owner = 0;
     if (l + 1 == a.last) {
@@ -2238,6 +2256,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_co
     if (a.inv_off != ~0u) copy_to_shared_async(g_tail_smem + a.inv_off, a.inv, (size_t)n * n * sizeof(S));
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
+  if (threadIdx.x < 32) st_sh(base + a.zero_off + threadIdx.x * (uint32_t)sizeof(T), T(0));
   cluster_sync_all();  // every block runs before its shared memory is read
   int l = a.l0;
   for (; l < a.last && a.rl[l].dist; ++l) res_down<T, true>(a, g, l, base, cpr);
@@ -2406,6 +2425,8 @@ void resident_plan(bo_prec* P, ResPlan& a) {
     r.off = o;
     o += (uint32_t)align16(((size_t)5 << r.lch) * sizeof(T));
   }
+  a.zero_off = o;
+  o += 32 * sizeof(T);
   a.dense_off = o;
   o += (uint32_t)align16(2 * kCoarseMax * sizeof(T));
   for (int l = l0; l < last; ++l) {
