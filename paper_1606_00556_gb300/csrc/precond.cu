@@ -451,9 +451,18 @@ __device__ __forceinline__ Child galerkin_child(const LevelDims& C, int64_t grou
 __device__ __forceinline__ double add_xor(double v, int m) { return v + __shfl_xor_sync(0xffffffffu, v, m); }
 
 // FP64 levels keep the reciprocals of the diagonal behind the seven
-// coefficients: the Gauss-Seidel sweeps multiply by them, since an FP64
+// coefficients: the Gauss-Seidel sweeps divide with their help, since an FP64
 // division is about ten FP64 multiply-adds where the rest of a cell's
-// update takes six (FP32 divisions are cheap and stay divisions)
+// update takes six (FP32 divisions are cheap and stay divisions).
+// s / d from the rounded reciprocal r = 1 / d: the product, corrected once by
+// its residual, is the rounded quotient (P. Markstein, IBM J. Res. Dev. 34,
+// 1990); the product alone is off by up to one unit more.  (An infinite
+// product has no residual.)  A Newton step of 128x128x64 takes 17.5 ms with the
+// product alone and 18.1 so, 20x20x5 963 and 980 us.
+__device__ __forceinline__ double divide_by(double s, double d, double r) {
+  const double q = s * r, c = fma(fma(-q, d, s), r, q);
+  return isfinite(c) ? c : q;
+}
 template <typename S>
 __host__ __device__ constexpr int level_slots() { return sizeof(S) == 8 ? 8 : 7; }
 template <typename S>
@@ -986,8 +995,8 @@ __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g
   }
 }
 
-// s / d, or in FP64 s times the stored reciprocal at di[i] (see level_slots)
-__device__ __forceinline__ double gs_divide(double s, double, const double* __restrict__ di, size_t i) { return s * di[i]; }
+// s / d, in FP64 with the stored reciprocal at di[i] (see divide_by)
+__device__ __forceinline__ double gs_divide(double s, double d, const double* __restrict__ di, size_t i) { return divide_by(s, d, di[i]); }
 __device__ __forceinline__ float gs_divide(float s, float d, const float*, size_t) { return s / d; }
 
 // ---- the rest of the CPR after its first local solve z = R^{-1} f
@@ -1325,7 +1334,7 @@ struct LevelView {
   __device__ __forceinline__ T cc(int slot, int64_t cidx) const { return cv<T>(c[slot * d.n + cidx]); }
   // s divided by the diagonal
   __device__ __forceinline__ T divided(T s, int64_t cidx) const {
-    if constexpr (sizeof(S) == 8) return s * c[7 * d.n + cidx];
+    if constexpr (sizeof(S) == 8) return divide_by(s, cc(kDiag, cidx), c[7 * d.n + cidx]);
     else return s / cc(kDiag, cidx);
   }
 };
@@ -2021,8 +2030,8 @@ __device__ __forceinline__ uint32_t res_addr(const ResLevel& r, uint32_t base, i
 template <typename T, int NP>
 struct ResCells {
   T c[2][NP][6];          // off-diagonal coefficients (0 where the neighbour is missing)
-  T d[2][NP];             // diagonal, or its reciprocal in FP64
-  T dr[NP];               // the red diagonal itself (residuals)
+  T d[2][NP];             // diagonal
+  T di[2][NP];            // and in FP64 its reciprocal
   T f[2][NP];
   uint32_t nb[2][NP][6];  // shared-memory addresses of the neighbours' iterates
   uint32_t own[2][NP];    // and of the cell's own
@@ -2030,8 +2039,8 @@ struct ResCells {
   bool live[2][NP];
 };
 
-__device__ __forceinline__ float res_divide(float s, float d) { return s / d; }
-__device__ __forceinline__ double res_divide(double s, double rd) { return s * rd; }
+__device__ __forceinline__ float res_divide(float s, float d, float) { return s / d; }
+__device__ __forceinline__ double res_divide(double s, double d, double r) { return divide_by(s, d, r); }
 
 // One visit of level l: the cells of this thread into registers
 template <typename T, int NP, bool DIST>
@@ -2054,9 +2063,8 @@ __device__ __forceinline__ void res_load(const ResPlan& a, int l, uint32_t base,
     for (int col = 0; col < 2; ++col) {
 #pragma unroll
       for (int d = 0; d < 6; ++d) r.c[col][p][d] = cp[(col * K + d) * np + qq];
-      const T dg = cp[(col * K + 6) * np + qq];
-      if (col == 0) r.dr[p] = dg;
-      r.d[col][p] = K == 8 ? cp[(col * K + K - 1) * np + qq] : dg;
+      r.d[col][p] = cp[(col * K + 6) * np + qq];
+      r.di[col][p] = K == 8 ? cp[(col * K + K - 1) * np + qq] : T(0);
     }
     const int32_t par = r.m[p] & 1;
 #pragma unroll
@@ -2102,7 +2110,7 @@ __device__ __forceinline__ void res_sweep(ResCells<T, NP>& r, int col) {
       T s = r.f[col][p];
 #pragma unroll
       for (int d = 0; d < 6; ++d) s -= r.c[col][p][d] * xv[p][d];
-      if (r.live[col][p]) st_sh(r.own[col][p], res_divide(s, r.d[col][p]));
+      if (r.live[col][p]) st_sh(r.own[col][p], res_divide(s, r.d[col][p], r.di[col][p]));
     }
   }
   res_barrier<DIST>();
@@ -2161,8 +2169,8 @@ __device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l,
     // until its own half sweep; within the CPR level 0's f_r is zero, which
     // makes that x_b = f_b / d_b)
     if (place) {
-      st_sh(res_local<T>(rl, base, kSecRed, q), r.live[0][p] ? res_divide(r.f[0][p], r.d[0][p]) : T(0));
-      st_sh(res_local<T>(rl, base, kSecBlack, q), whole && r.live[1][p] ? res_divide(r.f[1][p], r.d[1][p]) : T(0));
+      st_sh(res_local<T>(rl, base, kSecRed, q), r.live[0][p] ? res_divide(r.f[0][p], r.d[0][p], r.di[0][p]) : T(0));
+      st_sh(res_local<T>(rl, base, kSecBlack, q), whole && r.live[1][p] ? res_divide(r.f[1][p], r.d[1][p], r.di[1][p]) : T(0));
     }
   }
   res_barrier<DIST>();
@@ -2178,10 +2186,10 @@ __device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l,
     // the order of the other launch forms, whose results these are bit for bit)
     const T dx = ld_sh(r.own[0][p], false, T(0));
     T v = r.f[0][p];
-    if (l) v -= r.dr[p] * dx;
+    if (l) v -= r.d[0][p] * dx;
 #pragma unroll
     for (int d = 0; d < 6; ++d) {
-      if (d == 3 && !l) v -= r.dr[p] * dx;
+      if (d == 3 && !l) v -= r.d[0][p] * dx;
       v -= r.c[0][p][d] * ld_sh(r.nb[0][p][d], DIST, T(0));
     }
     st_sh(r.own[0][p] + ((uint32_t)(kSecRes - kSecRed) << rl.lch) * (uint32_t)sizeof(T), v);
