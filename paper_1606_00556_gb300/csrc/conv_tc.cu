@@ -695,15 +695,32 @@ namespace {
 // The accumulators stay in TMEM over all tiles of a CTA (TX x 4 voxels, a
 // march along z as in the convolution above); each CTA writes one partial
 // sum, k_wgrad_sum adds them in a fixed order.  dY is read in FP32 by eight
-// warps that round it to BF16 on its way to shared memory and sum the bias
-// gradient in split FP32 pairs, so it is read once; X comes by cp.async from
-// eight more (with four of each the dY warps took 5800 cycles a tile, the MMAs
-// 3900).  What bounds it: the shared-memory operand reads of the MMAs, 6 KB in
-// 46 cycles for 2 x 16 voxels and a ninth of the taps.
+// warps that round it to BF16 on its way to shared memory; X comes by cp.async
+// from eight more (with four of each the dY warps took 5800 cycles a tile, the
+// MMAs 3900).
+// The bias gradient is summed in three FP32 parts, 72 bits, so that it keeps
+// what an FP64 sum keeps (two parts took 81 us a call in place of 84, but lose
+// to FP64 where large values cancel): by the dY warps as they read it, and
+// where dY is the halo tensor by the X warps, which read it again from L2 (16
+// -> 32: 103 us a call when the halo warps did it, 85 so).
+// What bounds it: the shared-memory operand reads of the MMAs, 6 KB in 46
+// cycles for 2 x 16 voxels and a ninth of the taps.
 // Measured, 64x64x32 x 4 samples, 32 -> 32: 587 us a call, with scratch
 // allocated in it and five launches (mma.sync gradient 144, FP64 bias sums
 // 95, reduction 30, conversion 18) -> 164 with MMAs issued in a loop over
-// lanes -> 103 with four producer warps a side and FP64 sums -> 82.
+// lanes -> 103 with four producer warps a side and FP64 sums -> 84.
+
+struct Sum3 {  // a running sum of FP32 values in three of them: 72 bits
+  float a, b, c;
+  __device__ __forceinline__ void add(float e) {
+    const df t = df_two_sum(a, e), u = df_two_sum(b, t.lo);
+    a = t.hi;
+    b = u.hi;
+    c = __fadd_rn(c, u.lo);
+  }
+  // (the parts below an infinity are NaN)
+  __device__ __forceinline__ double value() const { return isfinite(a) ? (double)a + ((double)b + (double)c) : (double)a; }
+};
 constexpr int kWgProd = 256;      // threads that fetch halo planes, and as many core planes
 constexpr int kWgThreads = 32 + 2 * kWgProd;  // warp 0: MMAs; 1-8: halo producers; 9-16: core producers; 1-16: the end
 constexpr int kWgHalo = 5, kWgCore = 3;  // plane buffers
@@ -726,7 +743,7 @@ constexpr int kWgOffBar = 0, kWgOffBias = 256, kWgOffPlanes = kWgOffBias + kWgPr
 // One plane of a tensor into shared memory: NR rows from y0, NX voxels from
 // x0, rows [chunk][voxel], a thread every kWgProd / KC voxels of a chunk.
 // BF16 by cp.async (the caller commits); FP32 by loads, rounded to BF16,
-// `wait` called between the loads and the first store and the voxels of `own`
+// `wait` called between the loads and the first store, the values (BIAS)
 // added to the thread's bias sums.
 struct WgStep {  // voxel index -> (row, place in it), stepped without divisions
   int yl, xl;
@@ -746,10 +763,9 @@ __device__ __forceinline__ void wg_plane_bf16(const bf16* T, size_t zb, int nx, 
          in);
   }
 }
-template <int KC, int NR, typename Wait>
+template <int KC, int NR, bool BIAS, typename Wait>
 __device__ __forceinline__ bool wg_plane_f32(const float* T, size_t zb, int nx, int ny, int x0, int y0, int NX, uint32_t dst,
-                                             int row_bytes, int pt, bool own, int own_x0, int own_y0, int own_nx,
-                                             df (&bias)[8], Wait wait) {
+                                             int row_bytes, int pt, Sum3 (&bias)[8], Wait wait) {
   constexpr int U = 4, kStep = kWgProd / KC;  // U voxels in flight per thread
   const int kc = pt % KC;
   const int n = NR * NX;
@@ -778,16 +794,38 @@ __device__ __forceinline__ bool wg_plane_f32(const float* T, size_t zb, int nx, 
                    "r"(pack_bf16(e[0], e[1])), "r"(pack_bf16(e[2], e[3])), "r"(pack_bf16(e[4], e[5])),
                    "r"(pack_bf16(e[6], e[7]))
                    : "memory");
-      if (own && a.yl >= own_y0 && a.yl < own_y0 + kWgTY && a.xl >= own_x0 && a.xl < own_x0 + own_nx) {
+      if (BIAS) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const df t = df_two_sum(bias[q].hi, e[q]);
-          bias[q] = df{t.hi, __fadd_rn(bias[q].lo, t.lo)};
-        }
+        for (int q = 0; q < 8; ++q) bias[q].add(e[q]);
       }
     }
   }
   return true;
+}
+// The bias sums alone: a tile's values, a thread every kWgProd / 4 voxels of a
+// chunk of eight channels.
+__device__ __forceinline__ void wg_bias_f32(const float* T, size_t zb, int nx, int ny, int x0, int y0, int NX, int pt,
+                                            Sum3 (&bias)[8]) {
+  constexpr int U = 2, kStep = kWgProd / 4;
+  const int kc = pt % 4;
+  WgStep a(pt / 4, NX);
+  while (a.yl < kWgTY) {
+    float4 v[U][2];
+#pragma unroll
+    for (int u = 0; u < U; ++u, a.next(kStep, NX)) {
+      const int x = x0 + a.xl, y = y0 + a.yl;
+      const bool in = a.yl < kWgTY && x < nx && y < ny;
+      const float4* src = reinterpret_cast<const float4*>(T + (in ? (zb + (size_t)y * nx + x) * 32 : 0) + kc * 8);
+      v[u][0] = in ? __ldg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[u][1] = in ? __ldg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float e[8] = {v[u][0].x, v[u][0].y, v[u][0].z, v[u][0].w, v[u][1].x, v[u][1].y, v[u][1].z, v[u][1].w};
+#pragma unroll
+      for (int q = 0; q < 8; ++q) bias[q].add(e[q]);
+    }
+  }
 }
 
 template <bool HALO_DY, int CB>
@@ -843,9 +881,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     __syncwarp();
     if (lane == 0) mbar_arrive(bar);
   };
-  df bias[8];
+  Sum3 bias[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) bias[q] = df{0.f, 0.f};
+  for (int q = 0; q < 8; ++q) bias[q] = Sum3{0.f, 0.f, 0.f};
   bool ok = true;
   March m(g, t0);
   if (warp >= 1 + kWgProd / 32) {
@@ -861,9 +899,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
         if (!ok) break;
         wg_plane_bf16<KC, kWgTY>(X, zb, g.nx, g.ny, m.tx * TX, m.ty * kWgTY, TX, dst, crow, pt);
         cp_commit();
+        wg_bias_f32(dY, zb, g.nx, g.ny, m.tx * TX, m.ty * kWgTY, TX, pt, bias);
         cp_wait<0>();
       } else {
-        ok = wg_plane_f32<KC, kWgTY>(dY, zb, g.nx, g.ny, m.tx * TX, m.ty * kWgTY, TX, dst, crow, pt, true, 0, 0, TX, bias, wait);
+        ok = wg_plane_f32<KC, kWgTY, true>(dY, zb, g.nx, g.ny, m.tx * TX, m.ty * kWgTY, TX, dst, crow, pt, bias, wait);
         if (!ok) break;
       }
       arrive(cfull(k % kWgCore));
@@ -875,15 +914,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     for (int64_t t = t0; t < t1 && ok; ++t, m.next(g)) {
       const int z = m.z, x0 = m.tx * TX - 1, y0 = m.ty * kWgTY - 1;
       const bool start = t == t0 || z == 0;
-      const int zend = (int)min((int64_t)g.nz, z + (t1 - t));  // the column's tiles of this CTA end there
       for (int pz = start ? max(z - 1, 0) : z + 1; pz <= min(z + 1, g.nz - 1) && ok; ++pz) {
         const size_t zb = (size_t)m.b * V + (size_t)pz * g.nx * g.ny;
         const uint32_t dst = hbase + (uint32_t)(seq % kWgHalo) * hplane;
         auto wait = [&]() { return seq < kWgHalo || mbar_wait(hempty(seq % kWgHalo), (seq / kWgHalo - 1) & 1, sfail); };
         if constexpr (HALO_DY) {
-          // a plane counts towards the bias where it is one of this CTA's tiles
-          const bool own = pz >= z && pz < zend;
-          ok = wg_plane_f32<4, kWgHY>(dY, zb, g.nx, g.ny, x0, y0, TX + 2, dst, hrow, pt, own, 1, 1, TX, bias, wait);
+          ok = wg_plane_f32<4, kWgHY, false>(dY, zb, g.nx, g.ny, x0, y0, TX + 2, dst, hrow, pt, bias, wait);
           if (!ok) break;
           arrive(hfull(seq % kWgHalo));
           ++seq;
@@ -962,14 +998,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     if (!mbar_wait(alldone, 0) || ts < t1) ok = false;  // every MMA is done before the buffers are used again
   }
   if (!ok) report_timeout(sfail, lim);
-  if (warp >= 1) {
-    const bool dyside = (warp < 1 + kWgProd / 32) == HALO_DY;
-    if (dyside) {
-      const int pt = HALO_DY ? tid - 32 : tid - 32 - kWgProd;
+  if (warp >= 1 + kWgProd / 32) {
+    const int pt = tid - 32 - kWgProd;
 #pragma unroll
-      for (int q = 0; q < 8; ++q)  // (a sum that met an infinity has NaN in its low part)
-        sbias[pt * 8 + q] = isfinite(bias[q].hi) ? df_to_double(df_renorm(bias[q])) : (double)bias[q].hi;
-    }
+    for (int q = 0; q < 8; ++q) sbias[pt * 8 + q] = bias[q].value();
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -1028,9 +1060,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
-// dW[i] = sum over the chunks' partials in a fixed order, in split FP32 pairs
-// (48 bits; 4.2 million FP64 additions took 14 of the 20 us of the form that
-// made them); 32 outputs by 8 slices of the chunks per block.  The last block
+// dW[i] = sum over the chunks' partials in a fixed order, in three FP32 parts
+// (4.2 million FP64 additions took 14 of the 20 us of the form that made them);
+// 32 outputs by 8 slices of the chunks per block.  The last block
 // takes the bias gradient.
 __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, const double* __restrict__ bpart,
                                                    float* __restrict__ dW, float* __restrict__ db, int n, int chunks, int cy) {
@@ -1042,18 +1074,15 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ par
       for (int k = w; k < chunks; k += 8) s += bpart[(size_t)k * cy + l];
   } else {
     const float* p = part + blockIdx.x * 32 + l;  // (n is a multiple of 32)
-    df a{0.f, 0.f};
+    Sum3 a{0.f, 0.f, 0.f};
     for (int k0 = w; k0 < chunks; k0 += 80) {
       float v[10];
 #pragma unroll
       for (int u = 0; u < 10; ++u) v[u] = k0 + 8 * u < chunks ? p[(size_t)(k0 + 8 * u) * n] : 0.f;
 #pragma unroll
-      for (int u = 0; u < 10; ++u) {
-        const df t = df_two_sum(a.hi, v[u]);
-        a = df{t.hi, __fadd_rn(a.lo, t.lo)};
-      }
+      for (int u = 0; u < 10; ++u) a.add(v[u]);
     }
-    s = isfinite(a.hi) ? df_to_double(a) : (double)a.hi;  // (past an infinity the low part is NaN)
+    s = a.value();
   }
   sh[w][l] = s;
   __syncthreads();
