@@ -622,9 +622,10 @@ int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_
                    const float* bias, const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, bool transposed,
                    const TcWait& lim, cudaStream_t s);
 // tcgen05 weight and bias gradients of a layer (part: room for kWgradTcBlocks
-// partials of 27 cin cout floats, bpart: of cout doubles); BO_ERR_ARG where it
-// does not apply
+// partials of 27 cin cout floats, bpart: wgrad_bias_bytes, cout doubles and a
+// flag of each); BO_ERR_ARG where it does not apply
 constexpr int kWgradTcBlocks = 304;
+constexpr size_t wgrad_bias_bytes(int cout) { return kWgradTcBlocks * (cout * sizeof(double) + sizeof(int)); }
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
                     double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s);
 // dense FP64 inverse of an n x n matrix (n <= 128) by one block; sets

@@ -180,7 +180,7 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t r[4], const void* p) {
 // Voxels of a brick outside the grid have dY = 0, so they add nothing.
 constexpr int kBrickX = 8, kBrickY = 8, kBrickZ = 4, kBrick = 256;
 constexpr int kHaloX = 10, kHaloY = 10, kHalo = 600;
-constexpr int kWgMaxBlocks = 304;
+constexpr int kWgMaxBlocks = kWgradTcBlocks;  // (the two engines share the network's buffers)
 
 template <int CIN, int COUT>
 constexpr size_t wgrad_smem() {
@@ -556,7 +556,7 @@ int cnn_alloc(bo_cnn* n) {
   n->gB = (float*)al(BV * 32 * 4);
   n->gC = (float*)al(BV * 32 * 4);
   n->g16 = (bf16*)al(BV * 32 * 2);
-  n->bpart = (double*)al((size_t)bo::kWgMaxBlocks * 32 * sizeof(double));
+  n->bpart = (double*)al(bo::wgrad_bias_bytes(32));
   if (!ok) return BO_ERR_OOM;
   cudaStream_t s = n->ctx->stream;
   cudaMemsetAsync(n->m, 0, n->nparam * 4, s);
@@ -819,7 +819,7 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
   if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   if (bo::g_conv_engine.load() == 1) {  // the partial sums in the context's workspace
     const size_t pb = (size_t)bo::kWgradTcBlocks * 27 * cin * cout * 4;
-    void* ws = bo::ctx_scratch(ctx, pb + (size_t)bo::kWgradTcBlocks * 32 * sizeof(double));
+    void* ws = bo::ctx_scratch(ctx, pb + bo::wgrad_bias_bytes(cout));
     if (!ws) return BO_ERR_OOM;
     const int rc = bo::launch_wgrad_tc(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x), dy, (float*)ws,
                                        (double*)((char*)ws + pb), dw, db, bo::tc_wait(ctx), ctx->stream);

@@ -831,7 +831,8 @@ __device__ __forceinline__ void wg_bias_f32(const float* T, size_t zb, int nx, i
 template <bool HALO_DY, int CB>
 __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ WgradGrid g, const bf16* __restrict__ X,
                                                           const float* __restrict__ dY, float* __restrict__ part,
-                                                          double* __restrict__ bpart, const TcWait lim) {
+                                                          double* __restrict__ bpart, int* __restrict__ odd,
+                                                          const TcWait lim) {
   constexpr int KC = CB / 8;          // chunks of the core tensor (the halo tensor has 4)
   constexpr int kPair = CB == 32 ? 7 : 9;  // accumulators that take two core rows per MMA
   constexpr int CY = HALO_DY ? 32 : CB;    // channels of dY
@@ -1048,32 +1049,84 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
   const int n = 27 * 32 * CB;
   float* P = part + (size_t)blockIdx.x * n;
   for (int i = tid; i < n / 4; i += kWgThreads) reinterpret_cast<float4*>(P)[i] = reinterpret_cast<const float4*>(red)[i];
+  double sum = 0.0;
   if (tid < CY) {
     constexpr int YC = CY / 8;
-    double sum = 0.0;
     for (int p = tid / 8; p < kWgProd; p += YC) sum += sbias[p * 8 + tid % 8];
-    bpart[(size_t)blockIdx.x * CY + tid] = fine ? sum : (double)__int_as_float(0x7fffffff);
+    if (!fine) sum = (double)__int_as_float(0x7fffffff);
+    bpart[(size_t)blockIdx.x * CY + tid] = sum;
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
+  const int infinite = __syncthreads_or(!isfinite(sum));
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+  if (tid == 0) odd[blockIdx.x] = !fine ? 2 : infinite ? 1 : 0;
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+}
+
+// Weight i or (bias) channel i of the gradient straight from its definition, the
+// voxels whose neighbour lies outside the grid with x = 0 as well: the part of
+// slice w of the block's eight, 32 consecutive i side by side.
+__device__ __noinline__ double wgrad_direct(const WgradGrid& g, const bf16* X, const float* dY, int cin, int cout, int i,
+                                            bool bias, int w) {
+  const int64_t rows = (int64_t)g.B * g.nz * g.ny;
+  if (bias) {
+    double s = 0.0;
+    for (int64_t v = w; v < rows * g.nx && !isnan(s); v += 8 * 16) {
+      float e[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) e[u] = v + 8 * u < rows * g.nx ? dY[(v + 8 * u) * cout + i] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) s += e[u];
+    }
+    return s;
+  }
+  const int t = i / (cin * cout), co = i / cin % cout, ci = i % cin;
+  const int dx = t % 3 - 1, dy = t / 3 % 3 - 1, dz = t / 9 - 1;
+  Sum3 s{0.f, 0.f, 0.f};
+  for (int64_t r = w; r < rows; r += 8) {
+    const int y = (int)(r % g.ny), z = (int)(r / g.ny % g.nz);
+    const bool row = y + dy >= 0 && y + dy < g.ny && z + dz >= 0 && z + dz < g.nz;
+    const float* D = dY + r * g.nx * cout + co;
+    const bf16* N = X + ((r + dy + (int64_t)dz * g.ny) * g.nx + dx) * cin + ci;
+    for (int x = 0; x < g.nx; ++x) {
+      const float d = __bfloat162float(__float2bfloat16_rn(D[(int64_t)x * cout]));
+      const bool in = row && x + dx >= 0 && x + dx < g.nx;
+      s.add(d * (in ? __bfloat162float(N[(int64_t)x * cin]) : 0.f));
+    }
+    if (__all_sync(0xffffffffu, isnan(s.a))) break;
+  }
+  return s.value();
 }
 
 // dW[i] = sum over the chunks' partials in a fixed order, in three FP32 parts
 // (4.2 million FP64 additions took 14 of the 20 us of the form that made them);
 // 32 outputs by 8 slices of the chunks per block.  The last block
-// takes the bias gradient.
-__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, const double* __restrict__ bpart,
-                                                   float* __restrict__ dW, float* __restrict__ db, int n, int chunks, int cy) {
+// takes the bias gradient.  odd[chunk]: 1 where one of its bias sums is not
+// finite, 2 where it gave up a wait.
+// Infinite values: a tile's voxels beyond the grid are zeros, and their
+// products with an infinite neighbour that lies in it NaN; conversely planes
+// beyond the grid are left out, and the zeros that an infinite dY meets there.
+// So a sum that came out as NaN, and all of a channel whose bias is not finite,
+// are taken again from the definition (at 64x64x32 x 4, 32 -> 32, 0 to 11 ms,
+// the more the later the NaN that ends a sum; finite values: 9.8 -> 10.9 us for
+// looking).  Six blocks per SM: the 865 of 32 x 32 channels in one wave.
+__global__ void __launch_bounds__(256, 6) k_wgrad_sum(const float* __restrict__ part, const double* __restrict__ bpart,
+                                                   const int* __restrict__ odd, const __grid_constant__ WgradGrid g, const bf16* __restrict__ X,
+                                                   const float* __restrict__ dY, float* __restrict__ dW,
+                                                   float* __restrict__ db, int cin, int cout, int chunks) {
   __shared__ double sh[8][32];
-  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5, n = 27 * cin * cout;
+  const bool last = blockIdx.x == gridDim.x - 1;
+  const int i = last ? l : (int)blockIdx.x * 32 + l;  // (n is a multiple of 32)
   double s = 0.0;
-  if (blockIdx.x == gridDim.x - 1) {
-    if (l < cy)
-      for (int k = w; k < chunks; k += 8) s += bpart[(size_t)k * cy + l];
+  int flag = 0;  // (chunks <= 304)
+  if (threadIdx.x < chunks) flag = odd[threadIdx.x];
+  if (threadIdx.x + 256 < chunks) flag = max(flag, odd[threadIdx.x + 256]);
+  if (last) {
+    if (l < cout)
+      for (int k = w; k < chunks; k += 8) s += bpart[(size_t)k * cout + l];
   } else {
-    const float* p = part + blockIdx.x * 32 + l;  // (n is a multiple of 32)
+    const float* p = part + i;
     Sum3 a{0.f, 0.f, 0.f};
     for (int k0 = w; k0 < chunks; k0 += 80) {
       float v[10];
@@ -1083,18 +1136,33 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ par
       for (int u = 0; u < 10; ++u) a.add(v[u]);
     }
     s = a.value();
-  }
-  sh[w][l] = s;
-  __syncthreads();
-  if (w == 0) {
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += sh[k][l];
-    if (blockIdx.x == gridDim.x - 1) {
-      if (l < cy) db[l] = (float)t;
-    } else {
-      dW[blockIdx.x * 32 + l] = (float)t;
+    if (!isfinite(a.a)) {  // (beyond FP32's range on the way, maybe)
+      s = 0.0;
+      for (int k = w; k < chunks; k += 8) s += p[(size_t)k * n];
     }
   }
+  auto total = [&]() {
+    sh[w][l] = s;
+    __syncthreads();
+    double t = 0.0;
+    if (w == 0)  // (FP64 additions are few a clock: one warp's)
+      for (int k = 0; k < 8; ++k) t += sh[k][l];
+    return t;
+  };
+  double t = total();
+  bool again = last ? l < cout && !isfinite(t) : isnan(t);
+  if (__syncthreads_or(again || flag)) {
+    if (!last) {  // the block's output channels, 32 / cin from c0 on
+      const int per = 32 / cin, c0 = (int)blockIdx.x * per % cout;
+      for (int k = threadIdx.x; k < chunks * per; k += 256)
+        again = again || !isfinite(bpart[(size_t)(k / per) * cout + c0 + k % per]);
+    }
+    if (__syncthreads_or(again) && !__syncthreads_or(flag > 1)) {
+      s = i < (last ? cout : n) ? wgrad_direct(g, X, dY, cin, cout, i, last, w) : 0.0;
+      t = total();
+    }
+  }
+  if (w == 0 && i < (last ? cout : n)) (last ? db : dW)[i] = (float)t;
 }
 
 template <bool HALO_DY, int CB>
@@ -1108,16 +1176,17 @@ int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, d
   int grid = sm_count();
   if (grid > kWgradTcBlocks) grid = kWgradTcBlocks;
   if (g.tiles < grid) grid = (int)g.tiles;
-  (kern<<<grid, kWgThreads, smem, s>>>(g, X, dY, part, bpart, lim), note_launch());
-  const int n = 27 * 32 * CB;
-  (k_wgrad_sum<<<n / 32 + 1, 256, 0, s>>>(part, bpart, dW, db, n, grid, HALO_DY ? 32 : CB), note_launch());
+  int* odd = reinterpret_cast<int*>(bpart + kWgradTcBlocks * (HALO_DY ? 32 : CB));
+  (kern<<<grid, kWgThreads, smem, s>>>(g, X, dY, part, bpart, odd, lim), note_launch());
+  (k_wgrad_sum<<<27 * CB + 1, 256, 0, s>>>(part, bpart, odd, g, X, dY, dW, db, HALO_DY ? CB : 32, HALO_DY ? 32 : CB, grid),
+   note_launch());
   return cudaGetLastError() == cudaSuccess ? BO_OK : BO_ERR_CUDA;
 }
 
 }  // namespace
 
 // The tensor-core weight and bias gradients of a layer (part: room for
-// kWgradTcBlocks partials of 27 cin cout floats, bpart: of cout doubles);
+// kWgradTcBlocks partials of 27 cin cout floats, bpart: for wgrad_bias_bytes);
 // BO_ERR_ARG where it does not apply.
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
                     double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s) {
