@@ -676,9 +676,9 @@ int bo_cnn_adam_step(bo_cnn* net, float lr);
  * backward_weights: dw[t][co][ci] = sum_v dy[v][co] x[v + off(t)][ci] and
  *   db[co] = sum_v dy[v][co] (FP32); dy FP32 [batch][V][cout] is rounded to
  *   BF16 for the products.
- * backward_data and backward_weights synchronise; their scratch (at most 34
- * MB) stays with the context on the tcgen05 engine and is allocated and freed
- * in the call on the mma.sync engine.  BO_ERR_ARG on an unsupported (cin, cout) or mode. */
+ * backward_data and backward_weights synchronise; their scratch (at most 17 MB
+ * on 152 SMs) stays with the context on the tcgen05 engine and is allocated
+ * and freed in the call where the mma.sync kernels run.  BO_ERR_ARG on an unsupported (cin, cout) or mode. */
 int bo_conv3d_forward(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* x,
                       const uint16_t* w, const float* bias, const uint16_t* residual, int relu, uint16_t* y,
                       float* yf);

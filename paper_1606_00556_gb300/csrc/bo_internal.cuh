@@ -427,7 +427,7 @@ struct bo_ctx {
   int refs;
   void* scratch;         // workspace of the single-layer gradient calls (ordered on the stream like them), or NULL
   int* tc_err;           // pinned word that a tcgen05 convolution on this context sets when a wait expires
-  size_t scratch_bytes;  // at most one layer's partial sums (about 34 MB); freed with the context
+  size_t scratch_bytes;  // at most one layer's partial sums (17 MB on 152 SMs); freed with the context
 };
 
 struct bo_mat {
@@ -621,11 +621,14 @@ void graphs_reset(bo_prec* P);
 int launch_conv_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const __nv_bfloat16* W,
                    const float* bias, const __nv_bfloat16* R, __nv_bfloat16* Y, float* Yf, int mode, bool transposed,
                    const TcWait& lim, cudaStream_t s);
-// tcgen05 weight and bias gradients of a layer (part: room for kWgradTcBlocks
-// partials of 27 cin cout floats, bpart: wgrad_bias_bytes, cout doubles and a
-// flag of each); BO_ERR_ARG where it does not apply
+// tcgen05 weight and bias gradients of a layer: BO_ERR_ARG where it does not
+// apply.  part: room for the partials of wgrad_tc_blocks() thread blocks (one
+// an SM of the current device, at most kWgradTcBlocks), 27 cin cout floats
+// each; bpart: wgrad_bias_bytes, cout doubles and a flag of each
 constexpr int kWgradTcBlocks = 304;
-constexpr size_t wgrad_bias_bytes(int cout) { return kWgradTcBlocks * (cout * sizeof(double) + sizeof(int)); }
+int wgrad_tc_blocks();
+bool wgrad_tc_applies(const __nv_bfloat16* X, const float* dY);
+constexpr size_t wgrad_bias_bytes(int cout, int blocks) { return blocks * (cout * sizeof(double) + sizeof(int)); }
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
                     double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s);
 // dense FP64 inverse of an n x n matrix (n <= 128) by one block; sets

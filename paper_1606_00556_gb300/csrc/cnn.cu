@@ -449,20 +449,18 @@ int launch_dgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* d
 }
 
 // Weight and bias gradients of a layer from its input X (BF16) and dY
-// (FP32; its BF16 copy dY16 is made here unless have16).  dY16 = NULL: the
-// tcgen05 kernel only, which needs no copy (BO_ERR_ARG where it does not apply).
+// (FP32; its BF16 copy dY16 is made here unless have16).
 int launch_layer_wgrad(int cin, int cout, int nx, int ny, int nz, int B, const bf16* X, const float* dY, bf16* dY16,
                        bool have16, float* part, double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s) {
   if (g_conv_engine.load() == 1) {
     const int rc = launch_wgrad_tc(cin, cout, nx, ny, nz, B, X, dY, part, bpart, dW, db, lim, s);
     if (rc != BO_ERR_ARG) {
       // (the data gradient that may follow reads dY16)
-      if (rc == BO_OK && dY16 && !have16)
+      if (rc == BO_OK && !have16)
         (k_f32_to_bf16<<<grid_for((int64_t)B * nx * ny * nz * cout), kThreads, 0, s>>>(dY, dY16, (int64_t)B * nx * ny * nz * cout),
          note_launch());
       return rc;
     }
-    if (!dY16) return BO_ERR_ARG;
   }
   const int64_t V = (int64_t)nx * ny * nz, BV = B * V;
   if (!have16) (k_f32_to_bf16<<<grid_for(BV * cout), kThreads, 0, s>>>(dY, dY16, BV * cout), note_launch());
@@ -556,7 +554,7 @@ int cnn_alloc(bo_cnn* n) {
   n->gB = (float*)al(BV * 32 * 4);
   n->gC = (float*)al(BV * 32 * 4);
   n->g16 = (bf16*)al(BV * 32 * 2);
-  n->bpart = (double*)al(bo::wgrad_bias_bytes(32));
+  n->bpart = (double*)al(bo::wgrad_bias_bytes(32, bo::kWgMaxBlocks));
   if (!ok) return BO_ERR_OOM;
   cudaStream_t s = n->ctx->stream;
   cudaMemsetAsync(n->m, 0, n->nparam * 4, s);
@@ -817,12 +815,14 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
     return BO_ERR_ARG;
   if (!((cin == 16 && cout == 32) || (cin == 32 && cout == 32) || (cin == 32 && cout == 16))) return BO_ERR_ARG;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
-  if (bo::g_conv_engine.load() == 1) {  // the partial sums in the context's workspace
-    const size_t pb = (size_t)bo::kWgradTcBlocks * 27 * cin * cout * 4;
-    void* ws = bo::ctx_scratch(ctx, pb + bo::wgrad_bias_bytes(cout));
+  const bf16* x16 = reinterpret_cast<const bf16*>(x);
+  if (bo::g_conv_engine.load() == 1 && bo::wgrad_tc_applies(x16, dy)) {  // the partial sums in the context's workspace
+    const int blocks = bo::wgrad_tc_blocks();
+    const size_t pb = (size_t)blocks * 27 * cin * cout * 4;
+    void* ws = bo::ctx_scratch(ctx, pb + bo::wgrad_bias_bytes(cout, blocks));
     if (!ws) return BO_ERR_OOM;
-    const int rc = bo::launch_wgrad_tc(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x), dy, (float*)ws,
-                                       (double*)((char*)ws + pb), dw, db, bo::tc_wait(ctx), ctx->stream);
+    const int rc = bo::launch_wgrad_tc(cin, cout, nx, ny, nz, batch, x16, dy, (float*)ws, (double*)((char*)ws + pb), dw, db,
+                                       bo::tc_wait(ctx), ctx->stream);
     if (rc != BO_ERR_ARG) {
       const int rs = bo::ctx_synchronize(ctx);
       return rc != BO_OK ? rc : rs;
@@ -835,7 +835,7 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
   bool ok = cudaMalloc(&d16, BV * cout * 2) == cudaSuccess &&
             cudaMalloc(&part, (size_t)bo::kWgMaxBlocks * 27 * cin * cout * 4) == cudaSuccess &&
             cudaMalloc(&bpart, (size_t)bo::kWgMaxBlocks * cout * sizeof(double)) == cudaSuccess;
-  int rc = ok ? bo::launch_layer_wgrad(cin, cout, nx, ny, nz, batch, reinterpret_cast<const bf16*>(x), dy, d16, false,
+  int rc = ok ? bo::launch_layer_wgrad(cin, cout, nx, ny, nz, batch, x16, dy, d16, false,
                                        part, bpart, dw, db, bo::tc_wait(ctx), ctx->stream)
               : BO_ERR_OOM;
   const int rs = bo::ctx_synchronize(ctx);

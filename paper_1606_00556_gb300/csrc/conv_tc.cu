@@ -47,6 +47,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "bo_internal.cuh"
@@ -1165,6 +1166,12 @@ __global__ void __launch_bounds__(256, 6) k_wgrad_sum(const float* __restrict__ 
   if (w == 0 && i < (last ? cout : n)) (last ? db : dW)[i] = (float)t;
 }
 
+}  // namespace
+
+int wgrad_tc_blocks() { return std::min(sm_count(), kWgradTcBlocks); }
+
+namespace {
+
 template <bool HALO_DY, int CB>
 int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, double* bpart, float* dW, float* db,
               const TcWait& lim, cudaStream_t s) {
@@ -1173,10 +1180,9 @@ int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, d
   const int red = 27 * 32 * CB * 4;
   const int smem = kWgOffPlanes + (planes > red ? planes : red) + 128;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return BO_ERR_CUDA;
-  int grid = sm_count();
-  if (grid > kWgradTcBlocks) grid = kWgradTcBlocks;
-  if (g.tiles < grid) grid = (int)g.tiles;
-  int* odd = reinterpret_cast<int*>(bpart + kWgradTcBlocks * (HALO_DY ? 32 : CB));
+  const int blocks = wgrad_tc_blocks();
+  const int grid = g.tiles < blocks ? (int)g.tiles : blocks;
+  int* odd = reinterpret_cast<int*>(bpart + grid * (HALO_DY ? 32 : CB));
   (kern<<<grid, kWgThreads, smem, s>>>(g, X, dY, part, bpart, odd, lim), note_launch());
   (k_wgrad_sum<<<27 * CB + 1, 256, 0, s>>>(part, bpart, odd, g, X, dY, dW, db, HALO_DY ? CB : 32, HALO_DY ? 32 : CB, grid),
    note_launch());
@@ -1185,12 +1191,13 @@ int run_wgrad(const WgradGrid& g, const bf16* X, const float* dY, float* part, d
 
 }  // namespace
 
-// The tensor-core weight and bias gradients of a layer (part: room for
-// kWgradTcBlocks partials of 27 cin cout floats, bpart: for wgrad_bias_bytes);
-// BO_ERR_ARG where it does not apply.
+bool wgrad_tc_applies(const __nv_bfloat16* X, const float* dY) {
+  return !(reinterpret_cast<uintptr_t>(X) & 15) && !(reinterpret_cast<uintptr_t>(dY) & 15);
+}
+
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
                     double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s) {
-  if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(dY) & 15)) return BO_ERR_ARG;
+  if (!wgrad_tc_applies(X, dY)) return BO_ERR_ARG;
   WgradGrid g{nx, ny, nz, B, 0, 0, 0, 0};
   int best = 0;
   for (int tx : {64, 32, 16}) {  // the fewest padded voxels along x; of equals the longest run
