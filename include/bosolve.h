@@ -678,7 +678,9 @@ int bo_cnn_adam_step(bo_cnn* net, float lr);
  *   BF16 for the products.
  * backward_data and backward_weights synchronise; their scratch (at most 17 MB
  * on 152 SMs) stays with the context on the tcgen05 engine and is allocated
- * and freed in the call where the mma.sync kernels run.  BO_ERR_ARG on an unsupported (cin, cout) or mode. */
+ * and freed in the call where the mma.sync kernels run.  BO_ERR_ARG on an unsupported (cin, cout) or mode,
+ * and on an x of backward_weights off a 16-byte boundary or any other operand
+ * off a 4-byte one. */
 int bo_conv3d_forward(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* x,
                       const uint16_t* w, const float* bias, const uint16_t* residual, int relu, uint16_t* y,
                       float* yf);
@@ -688,8 +690,8 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
                                const float* dy, float* dw, float* db);
 /* Convolution engine (process-wide): 0 = mma.sync kernels, 1 = tcgen05
  * kernels (tensor memory accumulators; the default) for every layer's
- * forward pass and gradients; operands off a 16-byte boundary always take
- * mma.sync. */
+ * forward pass and gradients; other operands off a 16-byte boundary
+ * always take mma.sync. */
 int bo_set_conv_engine(int engine);
 /* How the AMG V-cycle is launched (process-wide); every form computes the
  * same V-cycle of paper Sec. 3.2's pressure AMG stage:

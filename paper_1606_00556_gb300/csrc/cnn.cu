@@ -23,8 +23,10 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
+#include <initializer_list>
 #include <cstring>
 #include <new>
+#include <initializer_list>
 #include <random>
 #include <vector>
 
@@ -762,12 +764,20 @@ int bo_cnn_adam_step(bo_cnn* n, float lr) {
 }
 
 // ---- single-layer primitives (parity checks and other callers)
+// (BF16 operands are read and written in pairs at least, an X of the weight
+// gradient in 16 bytes: what lies off those boundaries is refused here)
+static bool off_boundary(size_t bytes, std::initializer_list<const void*> p) {
+  for (const void* q : p)
+    if (reinterpret_cast<uintptr_t>(q) % bytes) return true;
+  return false;
+}
 int bo_conv3d_forward(bo_ctx* ctx, int nx, int ny, int nz, int batch, int cin, int cout, const uint16_t* x,
                       const uint16_t* w, const float* bias, const uint16_t* residual, int relu, uint16_t* y,
                       float* yf) {
   if (!ctx || !x || !w || !bias || batch < 1 || nx < 1 || ny < 1 || nz < 1 ||
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
+  if (off_boundary(4, {x, w, residual, y, bias, yf})) return BO_ERR_ARG;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   bo::FwdMode mode;
   if (yf && !y && !relu && !residual) mode = bo::kLinearF32All;
@@ -785,6 +795,7 @@ int bo_conv3d_backward_data(bo_ctx* ctx, int nx, int ny, int nz, int batch, int 
   if (!ctx || !dy || !w || !dx || batch < 1 || nx < 1 || ny < 1 || nz < 1 ||
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
+  if (off_boundary(4, {dy, w, dx})) return BO_ERR_ARG;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   if (bo::g_conv_engine.load() == 1) {  // no workspace
     const int rc = bo::launch_conv_tc(cout, cin, nx, ny, nz, batch, reinterpret_cast<const bf16*>(dy),
@@ -814,6 +825,7 @@ int bo_conv3d_backward_weights(bo_ctx* ctx, int nx, int ny, int nz, int batch, i
       (int64_t)nx * ny * nz * batch > (1ll << 31))
     return BO_ERR_ARG;
   if (!((cin == 16 && cout == 32) || (cin == 32 && cout == 32) || (cin == 32 && cout == 16))) return BO_ERR_ARG;
+  if (off_boundary(16, {x}) || off_boundary(4, {dy, dw, db})) return BO_ERR_ARG;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return BO_ERR_CUDA;
   const bf16* x16 = reinterpret_cast<const bf16*>(x);
   if (bo::g_conv_engine.load() == 1 && bo::wgrad_tc_applies(x16, dy)) {  // the partial sums in the context's workspace
