@@ -250,15 +250,18 @@ typedef struct {
   int32_t amg_cells;     /* chosen tile of the per-kernel AMG form (bo_prec_set_amg_tile) */
   int32_t amg_threads;
   double tile_ms[5];     /* graph forms only: (cells, threads) = (2, 256), (4, 256), (1, 128),
-                            (2, 128), (1, 512) with the chosen form and width; 0 otherwise */
+                            (2, 128), (1, 512) with the chosen form and width (best_ms where no
+                            realisation launches the per-kernel form, so that they are the
+                            same); 0 otherwise */
 } bo_tune_result;
 
 /* Autotuner for bo_solve_batched (no counterpart in the paper).  Times the
  * caller's batch (same arguments as bo_solve_batched; x is overwritten,
  * solves start from zero) under every launch mode (stream, graph, batch
  * graph) and stream-pool width of 4, 8 and 16, then, when a graph form wins,
- * under five more tiles of the per-kernel AMG form with that form and width, two passes each (the first untimed), applies the fastest to
- * all P and to the pool, and records it in the JSON file cache_path (NULL:
+ * under five more tiles of the per-kernel AMG form with that form and width
+ * (if any realisation launches it), two passes each (the first untimed),
+ * applies the fastest to all P and to the pool, and records it in the JSON file cache_path (NULL:
  * no cache) under a key of the batch's shape (count, total and largest cell
  * counts as powers of two, FP32 preconditioners, restart).  With an entry
  * for the key already present it applies that entry without timing.  Returns

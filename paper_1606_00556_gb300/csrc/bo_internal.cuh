@@ -615,6 +615,9 @@ int krylov_alloc(bo_prec* P, int m);
 // shadow as scratch
 void launch_arnoldi_product(bo_prec* P, const double* v, double* w);
 void graphs_reset(bo_prec* P);
+// whether P's V-cycle inside a captured graph has launches of the per-kernel
+// form (and with it a use for amg_cells and amg_threads)
+bool amg_has_tiles(const bo_prec* P);
 // tcgen05 convolution (conv_tc.cu); mode 0 ReLU, 1 ReLU + residual, 2 linear
 // FP32 output, 3 linear BF16 output with channels 0..3 in FP32; transposed:
 // the data gradient.  BO_ERR_ARG where it does not apply.

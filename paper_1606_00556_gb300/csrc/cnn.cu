@@ -23,10 +23,9 @@
 #include <cuda_bf16.h>
 
 #include <cmath>
-#include <initializer_list>
 #include <cstring>
-#include <new>
 #include <initializer_list>
+#include <new>
 #include <random>
 #include <vector>
 

@@ -2876,6 +2876,11 @@ int prec_values(bo_prec* P) {
   return P->fp32 ? values_impl<float>(P) : values_impl<double>(P);
 }
 
+// (not where the cluster launch takes every level, nor where level 0 is the coarsest)
+bool amg_has_tiles(const bo_prec* P) {
+  return P->nlev > 1 && !(g_amg_coop.load() == 2 && P->res->cluster > 0 && P->res->l0 == 0);
+}
+
 int launch_dense_inverse64(int n, const double* M, double* Minv, DevState* st, cudaStream_t s) {
   if (n < 1 || n > kCoarseMax) return BO_ERR_ARG;
   const DenseSrc src{M, nullptr, LevelDims{n, 1, 1, n}, Geom{}, nullptr, nullptr};

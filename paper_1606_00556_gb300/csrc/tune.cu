@@ -134,12 +134,19 @@ int bo_autotune_batched(bo_prec* const* P, int nreal, const double* const* b, do
     }
   // the tile of the per-kernel AMG form, which the graph forms run: level-0
   // cells per thread and threads per block, tried with the best form and
-  // width (the default, 1 cell and 256 threads, was timed above)
+  // width (the default, 1 cell and 256 threads, was timed above).  Where no
+  // realisation has such a launch every tile is the same graph: the default
+  // stays, and its time stands for the others.
   const int tiles[5][2] = {{2, 256}, {4, 256}, {1, 128}, {2, 128}, {1, 512}};
   double tms[5] = {0, 0, 0, 0, 0};
   int best_cells = 1, best_threads = 256;
+  const bool tiled = std::any_of(P, P + nreal, bo::amg_has_tiles);
   if (best_mode != BO_LAUNCH_STREAM) {
     for (int ti = 0; ti < 5; ++ti) {
+      if (!tiled) {
+        tms[ti] = best;
+        continue;
+      }
       apply(P, nreal, best_mode, best_w, tiles[ti][0], tiles[ti][1]);
       for (int pass = 0; pass < 2; ++pass) {
         const auto t0 = std::chrono::steady_clock::now();
