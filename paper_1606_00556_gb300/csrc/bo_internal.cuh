@@ -634,8 +634,8 @@ bool wgrad_tc_applies(const __nv_bfloat16* X, const float* dY);
 constexpr size_t wgrad_bias_bytes(int cout, int blocks) { return blocks * (cout * sizeof(double) + sizeof(int)); }
 int launch_wgrad_tc(int cin, int cout, int nx, int ny, int nz, int B, const __nv_bfloat16* X, const float* dY, float* part,
                     double* bpart, float* dW, float* db, const TcWait& lim, cudaStream_t s);
-// dense FP64 inverse of an n x n matrix (n <= 128) by one block; sets
-// st->err on a zero pivot
+// dense FP64 inverse of an n x n matrix (n <= 128) by one block, above 32 rows
+// a cluster of eight; sets st->err on a zero pivot
 int launch_dense_inverse64(int n, const double* M, double* Minv, DevState* st, cudaStream_t s);
 int learned_coarse_values(bo_prec* P);
 void learned_coarse_apply(bo_prec* P, const DevState* st);

@@ -17,8 +17,10 @@
 // at <= coarse_max cells, whose dense inverse is formed once per setup.
 // V(nu1, nu2) with red-black Gauss-Seidel: red then black before the coarse
 // correction, black then red after it.  After a black half sweep only red
-// cells carry a residual, so restriction sums red residuals.  Levels of at
-// most kTailCells cells run inside one thread block (kernel k_tail).
+// cells carry a residual, so restriction sums red residuals.  The levels that
+// fit one thread-block cluster run in one launch (k_amg_resident); without
+// that form the levels of at most kTailCells cells run inside one thread block
+// (k_tail, k_tail_smem).
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
@@ -454,6 +456,7 @@ __device__ __forceinline__ double add_xor(double v, int m) { return v + __shfl_x
 // coefficients: the Gauss-Seidel sweeps divide with their help, since an FP64
 // division is about ten FP64 multiply-adds where the rest of a cell's
 // update takes six (FP32 divisions are cheap and stay divisions).
+//
 // s / d from the rounded reciprocal r = 1 / d: the product, corrected once by
 // its residual, is the rounded quotient (P. Markstein, IBM J. Res. Dev. 34,
 // 1990); the product alone is off by up to one unit more.  (An infinite
@@ -1339,21 +1342,12 @@ struct LevelView {
   }
 };
 
-// Loads of iterates and right-hand sides.  CG = true: through L2 only, for
-// values that other thread blocks of the same launch wrote before a barrier
-// (the cluster form of the coarse levels); false: ordinary loads.
-template <bool CG, typename T>
-__device__ __forceinline__ T ldv(const T* p) {
-  if (CG) return __ldcg(p);
-  return *p;
-}
-
-template <bool CG = false, typename T, typename S>
+template <typename T, typename S>
 __device__ __forceinline__ void gs_cell(const LevelView<T, S>& L, int64_t cidx, int color, int zero_guess) {
   const Ijk p = ijk_of(L.d, cidx);
   const int i = p.i, j = p.j, k = p.k;
   if (((i + j + k) & 1) != color) return;
-  T s = ldv<CG>(L.f + cidx);
+  T s = L.f[cidx];
   if (!zero_guess) {
     // every neighbour's loads are issued; a missing one reads the cell
     // itself and the value read is replaced by zero
@@ -1363,28 +1357,28 @@ __device__ __forceinline__ void gs_cell(const LevelView<T, S>& L, int64_t cidx, 
     const int64_t off[6] = {-nxy, -(int64_t)L.d.nx, -1, 1, (int64_t)L.d.nx, nxy};
 #pragma unroll
     for (int d = 0; d < 6; ++d) {
-      const T xv = ldv<CG>(L.x + (ok[d] ? cidx + off[d] : cidx));
+      const T xv = L.x[ok[d] ? cidx + off[d] : cidx];
       s -= L.cc(slot[d], cidx) * (ok[d] ? xv : T(0));
     }
   }
   L.x[cidx] = L.divided(s, cidx);
 }
 
-template <bool CG = false, typename T, typename S>
+template <typename T, typename S>
 __device__ __forceinline__ T residual_cell(const LevelView<T, S>& L, int i, int j, int k) {
   const int64_t cidx = nat_index(L.d, i, j, k);
   const int64_t nxy = (int64_t)L.d.nx * L.d.ny;
-  T r = ldv<CG>(L.f + cidx) - L.cc(kDiag, cidx) * ldv<CG>(L.x + cidx);
-  if (k > 0) r -= L.cc(kZm, cidx) * ldv<CG>(L.x + cidx - nxy);
-  if (j > 0) r -= L.cc(kYm, cidx) * ldv<CG>(L.x + cidx - L.d.nx);
-  if (i > 0) r -= L.cc(kXm, cidx) * ldv<CG>(L.x + cidx - 1);
-  if (i < L.d.nx - 1) r -= L.cc(kXp, cidx) * ldv<CG>(L.x + cidx + 1);
-  if (j < L.d.ny - 1) r -= L.cc(kYp, cidx) * ldv<CG>(L.x + cidx + L.d.nx);
-  if (k < L.d.nz - 1) r -= L.cc(kZp, cidx) * ldv<CG>(L.x + cidx + nxy);
+  T r = L.f[cidx] - L.cc(kDiag, cidx) * L.x[cidx];
+  if (k > 0) r -= L.cc(kZm, cidx) * L.x[cidx - nxy];
+  if (j > 0) r -= L.cc(kYm, cidx) * L.x[cidx - L.d.nx];
+  if (i > 0) r -= L.cc(kXm, cidx) * L.x[cidx - 1];
+  if (i < L.d.nx - 1) r -= L.cc(kXp, cidx) * L.x[cidx + 1];
+  if (j < L.d.ny - 1) r -= L.cc(kYp, cidx) * L.x[cidx + L.d.nx];
+  if (k < L.d.nz - 1) r -= L.cc(kZp, cidx) * L.x[cidx + nxy];
   return r;
 }
 
-template <bool CG = false, typename T, typename S>
+template <typename T, typename S>
 __device__ __forceinline__ T restrict_cell(const LevelView<T, S>& F, const LevelDims& C, int64_t I, int red_only) {
   const Ijk cc = ijk_of(C, I);
   const int ci = cc.i, cj = cc.j, ck = cc.k;
@@ -1395,27 +1389,27 @@ __device__ __forceinline__ T restrict_cell(const LevelView<T, S>& F, const Level
         const int i = 2 * ci + di, j = 2 * cj + dj, k = 2 * ck + dk;
         if (i >= F.d.nx || j >= F.d.ny || k >= F.d.nz) continue;
         if (red_only && ((i + j + k) & 1)) continue;
-        acc += residual_cell<CG>(F, i, j, k);
+        acc += residual_cell(F, i, j, k);
       }
   return acc;
 }
 
-template <bool CG = false, typename T, typename S>
+template <typename T, typename S>
 __device__ __forceinline__ void prolong_cell(const LevelView<T, S>& F, const LevelView<T, S>& C, int64_t cidx, T s) {
   const Ijk p = ijk_of(F.d, cidx);
   const int i = p.i, j = p.j, k = p.k;
-  F.x[cidx] = ldv<CG>(F.x + cidx) + s * ldv<CG>(C.x + nat_index(C.d, i / 2, j / 2, k / 2));
+  F.x[cidx] = F.x[cidx] + s * C.x[nat_index(C.d, i / 2, j / 2, k / 2)];
 }
 
 // black half sweep with the coarse correction of the red neighbours folded in
 // (the natural-order counterpart of k_gs0_prolong)
-template <bool CG = false, typename T, typename S>
+template <typename T, typename S>
 __device__ __forceinline__ void gs_cell_prolong(const LevelView<T, S>& L, const LevelView<T, S>& C, int64_t cidx, T sc) {
   const Ijk p = ijk_of(L.d, cidx);
   const int i = p.i, j = p.j, k = p.k;
   if (((i + j + k) & 1) != 1) return;
   const int64_t nxy = (int64_t)L.d.nx * L.d.ny;
-  T s = ldv<CG>(L.f + cidx);
+  T s = L.f[cidx];
   const bool ok[6] = {k > 0, j > 0, i > 0, i < L.d.nx - 1, j < L.d.ny - 1, k < L.d.nz - 1};
   const int slot[6] = {kZm, kYm, kXm, kXp, kYp, kZp};
   const int64_t off[6] = {-nxy, -(int64_t)L.d.nx, -1, 1, (int64_t)L.d.nx, nxy};
@@ -1426,7 +1420,7 @@ __device__ __forceinline__ void gs_cell_prolong(const LevelView<T, S>& L, const 
   for (int d = 0; d < 6; ++d) {
     const int64_t fi = ok[d] ? cidx + off[d] : cidx;
     const int64_t cn = ok[d] ? nat_index(C.d, ci[d], cj[d], ck[d]) : nat_index(C.d, i / 2, j / 2, k / 2);
-    const T xv = ldv<CG>(L.x + fi) + sc * ldv<CG>(C.x + cn);
+    const T xv = L.x[fi] + sc * C.x[cn];
     s -= L.cc(slot[d], cidx) * (ok[d] ? xv : T(0));
   }
   L.x[cidx] = L.divided(s, cidx);
@@ -1720,8 +1714,8 @@ struct CycleArgs {
   T* f0;
   T* x0;
   int tail_from;  // first level of the single-block tail
-  int legs_to;    // the down and up legs smooth levels 0 .. legs_to - 1
-  int fold_to;    // levels below it get their zero-guess red half sweep with the restriction
+  int legs_to;    // the down and up legs smooth levels 0 .. legs_to - 1 (from 1 on their zero-guess red half
+                  // sweep comes with the restriction)
   int nu1, nu2;
   int cpr;  // see amg_vcycle
   T s;
@@ -1752,7 +1746,7 @@ __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
   // right-hand side computes it at once, which saves that sweep's barrier.
   {
     const LevelView<T, S>& C = a.lv[1];
-    const bool fold = a.nu1 > 0 && 1 < a.fold_to;
+    const bool fold = a.nu1 > 0 && 1 < a.legs_to;
     for (int64_t I = t0; I < C.d.n; I += nt) {
       const T fI = restrict0_cell<T, S>(g, a.At, a.f0, a.x0, C.d, I, a.nu1 > 0);
       C.f[I] = fI;
@@ -1773,7 +1767,7 @@ __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
       if (!grid_barrier(st, a.spins)) return false;
     }
     const LevelView<T, S>& C = a.lv[l + 1];
-    const bool fold = a.nu1 > 0 && l + 1 < a.fold_to;
+    const bool fold = a.nu1 > 0 && l + 1 < a.legs_to;
     for (int64_t I = t0; I < C.d.n; I += nt) {
       const T fI = restrict_cell(L, C.d, I, a.nu1 > 0);
       C.f[I] = fI;
@@ -2543,7 +2537,6 @@ void amg_vcycle(bo_prec* P, const DevState* st, bool cpr) {
   ca.x0 = x0;
   ca.tail_from = P->tail_from;
   ca.legs_to = std::min(P->tail_from, res_from);
-  ca.fold_to = std::min(P->tail_from, res_from);
   ca.nu1 = nu1;
   ca.nu2 = nu2;
   ca.cpr = cpr;
@@ -2675,7 +2668,7 @@ template <typename T, typename S>
 void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const double* vs) {
   cudaStream_t s = P->stream;
   const Geom& g = P->mat->g;
-  const int gN = grid_for(g.N), gh = grid_for(g.Nh);
+  const int gN = grid_for(g.N);
   const S* At = (const S*)P->At;
   const S* D = (const S*)P->Dinv;
   T* f = (T*)P->f;

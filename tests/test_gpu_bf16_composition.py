@@ -6,8 +6,8 @@ V-cycles by the library's own stages, the residuals here in FP32 in the
 matrix's slot order (-z, -y, -x, cell, +x, +y, +z), one fused multiply-add a
 product.  Where storage keeps 8 bits, another order of the same sums moves a
 solution by more than the solver's tolerance, so the results are equal bit for
-bit.  Sizes: single cells, rows and planes, odd lengths, several thread
-blocks."""
+bit, in every launch form of the V-cycle.  Sizes: single cells, rows and
+planes, odd lengths, several thread blocks."""
 import numpy as np
 import pytest
 
@@ -84,10 +84,16 @@ def test_bf16_equals_the_whole_residual_composition(bo, dims):
             assert np.isfinite(z).all() and np.array_equal(z, z.astype(np.float32))  # FP32 values
             return z.astype(np.float32)
 
-        x = stage(bo.BO_STAGE_ILU, f)
-        e = stage(bo.BO_STAGE_AMG, _residual(B, nb, f, x))
-        assert not e[:, 1:].any()
-        x = x + e
-        x = x + stage(bo.BO_STAGE_ILU, _residual(B, nb, f, x))
-        assert np.array_equal(stage(bo.BO_STAGE_CPR_DECOUPLED, f), x)
+        x1 = stage(bo.BO_STAGE_ILU, f)
+        r1 = _residual(B, nb, f, x1)
+        for mode in (2, 1, 0):
+            bo.bo_set_amg_cooperative(mode)
+            try:
+                e = stage(bo.BO_STAGE_AMG, r1)
+                z = stage(bo.BO_STAGE_CPR_DECOUPLED, f)
+            finally:
+                bo.bo_set_amg_cooperative(2)
+            assert not e[:, 1:].any()
+            x2 = x1 + e
+            assert np.array_equal(z, x2 + stage(bo.BO_STAGE_ILU, _residual(B, nb, f, x2)))
         P.close()
