@@ -48,11 +48,41 @@ int occ_grid(const void* kernel, int64_t n, int threads, size_t smem) {
 
 namespace {
 
+// The contexts' error words: pinned memory in pages of 1024 words that stay with
+// the process, as many as its contexts have filled at one time (a page of its
+// own cost a context about 40 us, and its release a synchronisation).
+std::mutex g_words_mu;
+std::vector<int*>& error_words() {
+  static std::vector<int*>* w = new std::vector<int*>();  // (outlives every context)
+  return *w;
+}
+int* get_error_word() {
+  std::lock_guard<std::mutex> lk(g_words_mu);
+  std::vector<int*>& w = error_words();
+  if (w.empty()) {
+    constexpr int kPage = 1024;
+    int* p = nullptr;
+    if (cudaHostAlloc((void**)&p, kPage * sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    for (int i = 0; i < kPage; ++i) w.push_back(p + i);
+  }
+  int* p = w.back();
+  w.pop_back();
+  *p = 0;
+  return p;
+}
+void put_error_word(int* p) {
+  std::lock_guard<std::mutex> lk(g_words_mu);
+  error_words().push_back(p);
+}
+
 void ctx_release(bo_ctx* c) {
   if (--c->refs > 0) return;
   cudaStreamSynchronize(c->stream);
   if (c->scratch) cudaFree(c->scratch);
-  cudaFreeHost(c->tc_err);
+  put_error_word(c->tc_err);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -329,18 +359,17 @@ int bo_ctx_create(int device, void* cuda_stream, bo_ctx** out) {
   if (!c) return BO_ERR_OOM;
   c->device = device;
   c->refs = 1;
-  if (cudaHostAlloc((void**)&c->tc_err, sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-    cudaGetLastError();
+  c->tc_err = get_error_word();
+  if (!c->tc_err) {
     delete c;
     return BO_ERR_OOM;
   }
-  *c->tc_err = 0;
   if (cuda_stream) {
     c->stream = (cudaStream_t)cuda_stream;
     c->own_stream = false;
   } else {
     if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaFreeHost(c->tc_err);
+      put_error_word(c->tc_err);
       delete c;
       return BO_ERR_CUDA;
     }
