@@ -926,13 +926,8 @@ __device__ __forceinline__ void offdiag_sum(const Geom& g, const S* __restrict__
   }
 }
 
-// Whether a red row's residual after a local solve counts as zero (the
-// comment on the CPR's passes below): FP64 and FP32 storage.
-template <typename S>
-constexpr bool kExactRed = sizeof(S) >= 4;
-
 // ILU pass 2 (black): z_b = D_b'^{-1} (f_b - sum A_br t_r), t_r = D_r^{-1} f_r
-// (pass 1).  Pass 3 (red): x_r = D_r^{-1} (f_r - sum A_rb x_b).
+// (pass 1).  Pass 3 (red): x_r = t_r - D_r^{-1} sum A_rb x_b.
 // blocks per SM the register budget is tuned for: the FP32 passes are
 // memory-latency bound and want more warps; the FP64 ones are FP64-bound
 template <typename T>
@@ -958,11 +953,10 @@ __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_b(Geom g,
 }
 
 // (the black half of xb is read.)  OUT = false: z_r = x_r; OUT = true: the
-// preconditioner's result.  In BF16 storage x_r is t_r - D_r^{-1} sum A_rb x_b
-// with t_r from tv (see kExactRed), OUT = true adds it to z_r + Pi_p e_r.
+// preconditioner's result, z_r + Pi_p e_r + x_r.
 template <typename T, typename S, bool OUT>
-__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* __restrict__ f,
-                         const T* tv, const T* xb, T* z, const T* __restrict__ e, OutV zo, const DevState* st) {
+__global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g, const S* __restrict__ At, const S* __restrict__ Dinv, const T* tv,
+                         const T* xb, T* z, const T* __restrict__ e, OutV zo, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
@@ -972,28 +966,18 @@ __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_ilu_r2(Geom g
     T d[9], x[3];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
-    if (kExactRed<S>) {
-      T r[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) r[k] = f[vidx(g, k, 0, q)] - s[k];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) x[k] = d[3 * k] * r[0] + d[3 * k + 1] * r[1] + d[3 * k + 2] * r[2];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const T corr = d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2];
-        x[k] = tv[vidx(g, k, 0, q)] - corr;
-      }
-      if (OUT) {
-        x[0] = z[vidx(g, 0, 0, q)] + e[q] + x[0];
-        x[1] = z[vidx(g, 1, 0, q)] + x[1];
-        x[2] = z[vidx(g, 2, 0, q)] + x[2];
-      }
-    }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      if (OUT) out_put<T>(zo, vidx(g, k, 0, q), x[k]);
-      else z[vidx(g, k, 0, q)] = x[k];
+      const T corr = d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2];
+      x[k] = tv[vidx(g, k, 0, q)] - corr;
+    }
+    if (OUT) {
+      out_put<T>(zo, vidx(g, 0, 0, q), z[vidx(g, 0, 0, q)] + e[q] + x[0]);
+      out_put<T>(zo, vidx(g, 1, 0, q), z[vidx(g, 1, 0, q)] + x[1]);
+      out_put<T>(zo, vidx(g, 2, 0, q), z[vidx(g, 2, 0, q)] + x[2]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) z[vidx(g, k, 0, q)] = x[k];
     }
   }
 }
@@ -1003,51 +987,36 @@ __device__ __forceinline__ double gs_divide(double s, double d, const double* __
 __device__ __forceinline__ float gs_divide(float s, float d, const float*, size_t) { return s / d; }
 
 // ---- the rest of the CPR after its first local solve z = R^{-1} f
-// A red row of the red-black ILU(0)'s product is the row of the decoupled
-// matrix itself (red pivots are the diagonal blocks, and red rows have no
-// fill), so R^{-1} leaves no residual on red cells:
-//   A_rr z_r + A_rb z_b = f_r.
-// Three passes get shorter by it.  (1) The AMG right-hand side f_p - (A z)_p
-// is zero on red cells and needs the pressure rows of the black ones only.
-// (2) With x2 = z + Pi_p e the red pass of the second local solve needs only
-// the pressure columns of the red rows:
-//   w_r := x2_r + D_r^{-1} (f - A x2)_r = z_r - D_r^{-1} sum_b A_rb Pi_p e_b
-// (the diagonal block's term cancels e_r, which is therefore never read).
-// (3) The black pass then is
-//   x3_b = x2_b + D_b'^{-1} (f_b - A_bb x2_b - A_br w_r),
-// which reads A_br once where a residual of all rows followed by a black ILU
-// pass read it twice, and the red rows of x3 again have no residual:
-//   x3_r = D_r^{-1} (f_r - A_rb x3_b).
-// All of it holds where the stored pivots invert the stored diagonal blocks
-// to working precision.  BF16 storage rounds both to 8 bits, where (1), (2)
-// and the last line change the preconditioner, and even another order of its
-// sums moves a solution by more than the solver's tolerance (3.6e-8 at
-// 256x256x128 and 1e-8: FGMRES then stops at another iterate).  So BF16 keeps
-// the residuals of all cells and adds up what the local solve of a whole
-// residual adds up, in that order,
+//   x2 = z + Pi_p e,  e = AMG(A_pp)^{-1} Pi_r (f - A z),  x3 = x2 + R^{-1} (f - A x2),
+// the local solve of a residual r = f - A x2 being
 //   t_r = D_r^{-1} r_r,  u_b = D_b'^{-1} (r_b - A_br t_r),
-//   x3_b = x2_b + u_b,   x3_r = x2_r + (t_r - D_r^{-1} A_rb u_b),
-// and gains by the black pass alone, which forms r_b = (f - A x2)_b and
-// A_br t_r over one read of A_br.  (The solutions are those of separate
-// passes bit for bit; 256x256x128 81.9 -> 75.4 ms.)
-// Newton step, 128x128x64 FP32 at 19 iterations 11.96 -> 10.59 ms, FP64 19.4
-// -> 16.8 ms; 62x45x19 FP32 1853 -> 1714 us.  Iterations are those of the form
-// before this one: 307 over 24 systems of 20x20x5 to 150x149x40 in FP64 and
-// in FP32.
+//   x3_b = x2_b + u_b,   x3_r = x2_r + (t_r - D_r^{-1} A_rb u_b).
+// The black pass forms r_b and A_br t_r over one read of A_br, and so reads
+// the off-diagonal blocks of the black rows once where a residual of all rows
+// and a black ILU pass read them twice; every sum is added up in the order of
+// those separate passes, which gives their results bit for bit.  Newton step
+// with separate passes and no cluster form of the AMG -> now: 128x128x64 FP32
+// 13.0 -> 11.9 ms, FP64 24.2 -> 20.8 ms, 256x256x128 BF16 91.5 -> 86.3 ms.
+//
+// Red rows of the red-black ILU(0)'s product are rows of the matrix itself,
+// so in exact arithmetic r_r = 0, the AMG right-hand side is zero on red
+// cells and x3_r = D_r^{-1} (f_r - A_rb x3_b): passes that use it read a third
+// less (128x128x64 FP32 another 7%, FP64 14%).  They are not used.  On some 3%
+// of systems (flooded injector cells) the preconditioner amplifies rounding so
+// far that another order of its sums takes FGMRES to another iterate: solutions
+// moved by 1e-9 to 4e-8 at a tolerance of 1e-8 in all three precisions.
 
-// AMG right-hand side: f0_b = f_p - (A z)_p, f0_r = 0, and with it the first
-// pre-smoothing sweep from zero, x_r = 0 and x_b = f0_b / a_bb; in BF16 f0
-// alone, on all cells
+// AMG right-hand side f0 = f_p - (A z)_p, and with it the V-cycle's first half
+// sweep, x_r = f0_r / a_rr from zero
 template <typename T, typename S>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cpr_rhs(Geom g, const S* __restrict__ At,
                          const T* __restrict__ di0, const T* __restrict__ f, const T* __restrict__ z,
                          T* __restrict__ f0, T* __restrict__ x0, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
-  const int64_t n = kExactRed<S> ? g.Nh : g.N;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int color = kExactRed<S> || t >= g.Nh;
-    const int64_t q = kExactRed<S> ? t : t - color * g.Nh;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < g.N; t += (int64_t)gridDim.x * blockDim.x) {
+    const int color = t >= g.Nh;
+    const int64_t q = t - color * g.Nh;
     const Cell c = decode(g, color, q);
     T acc = T(0), diag = T(0);
     // (every slot's loads are issued; a missing neighbour reads this cell's
@@ -1066,22 +1035,17 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 5 : 4) k_cpr_rhs(Ge
       if (sl == kDiag) diag = a0;
       acc = fma3(acc, a0, z0, cv<T>(ld_stream(a + P)), z1, cv<T>(ld_stream(a + 2 * P)), z2);
     }
-    const size_t o = (size_t)color * g.Nh + q;
-    const T r = f[o] - acc;
-    f0[o] = r;
-    if (kExactRed<S>) {
-      f0[q] = T(0);
-      x0[q] = T(0);
-      x0[o] = gs_divide(r, diag, di0, o);
-    }
+    const T r = f[t] - acc;
+    f0[t] = r;
+    if (color == 0) x0[t] = gs_divide(r, diag, di0, (size_t)t);
   }
 }
 
-// w_r = z_r - D_r^{-1} sum_b A_rb Pi_p e_b, in BF16 t_r = D_r^{-1} (f - A x2)_r
+// t_r = D_r^{-1} (f - A x2)_r
 template <typename T, typename S>
-__global__ void __launch_bounds__(kThreads, kExactRed<S> && sizeof(T) == 4 ? 5 : 4) k_cpr_red(Geom g, const S* __restrict__ At,
+__global__ void __launch_bounds__(kThreads, 4) k_cpr_red(Geom g, const S* __restrict__ At,
                          const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ z,
-                         const T* __restrict__ e, T* __restrict__ w, const DevState* st) {
+                         const T* __restrict__ e, T* __restrict__ tv, const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
@@ -1089,96 +1053,72 @@ __global__ void __launch_bounds__(kThreads, kExactRed<S> && sizeof(T) == 4 ? 5 :
     T s[3] = {T(0), T(0), T(0)};
 #pragma unroll
     for (int sl = 0; sl < 7; ++sl) {
-      if (kExactRed<S> && sl == kDiag) continue;
       const S* a = At + at_index(g, 0, sl * 9, q);
       constexpr size_t P = 32;  // entries (rc) of a block lie 32 apart in a tile
       const int64_t nb = nbr(g, c, q, sl);
       const bool ok = nb >= 0;
       const int64_t nq = ok ? nb : q;
-      if (kExactRed<S>) {
-        const T en = e[g.Nh + nq];
-        const T xn = ok ? -en : T(0);
+      const int xc = sl == kDiag ? 0 : 1;
+      T x0 = z[vidx(g, 0, xc, nq)] + e[(size_t)xc * g.Nh + nq], x1 = z[vidx(g, 1, xc, nq)], x2 = z[vidx(g, 2, xc, nq)];
+      if (!ok) x0 = x1 = x2 = T(0);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) s[k] = fma(cv<T>(ld_stream(a + 3 * k * P)), xn, s[k]);
-      } else {
-        const int xc = sl == kDiag ? 0 : 1;
-        T x0 = z[vidx(g, 0, xc, nq)] + e[(size_t)xc * g.Nh + nq], x1 = z[vidx(g, 1, xc, nq)], x2 = z[vidx(g, 2, xc, nq)];
-        if (!ok) x0 = x1 = x2 = T(0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-          s[k] = fma3(s[k], cv<T>(ld_stream(a + 3 * k * P)), x0, cv<T>(ld_stream(a + (3 * k + 1) * P)), x1,
-                      cv<T>(ld_stream(a + (3 * k + 2) * P)), x2);
-      }
+      for (int k = 0; k < 3; ++k)
+        s[k] = fma3(s[k], cv<T>(ld_stream(a + 3 * k * P)), x0, cv<T>(ld_stream(a + (3 * k + 1) * P)), x1,
+                    cv<T>(ld_stream(a + (3 * k + 2) * P)), x2);
     }
-    if (!kExactRed<S>) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) s[k] = f[vidx(g, k, 0, q)] - s[k];
-    }
+    for (int k = 0; k < 3; ++k) s[k] = f[vidx(g, k, 0, q)] - s[k];
     T d[9];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + q]);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const T t = d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2];
-      w[vidx(g, k, 0, q)] = kExactRed<S> ? z[vidx(g, k, 0, q)] + t : t;
-    }
+    for (int k = 0; k < 3; ++k)
+      tv[vidx(g, k, 0, q)] = d[3 * k] * s[0] + d[3 * k + 1] * s[1] + d[3 * k + 2] * s[2];
   }
 }
 
-// x3_b = x2_b + D_b'^{-1} (f_b - A_bb x2_b - A_br w_r), x2_b = z_b + Pi_p e_b:
-// the preconditioner's result, and x3_b into xb for the red pass.  In BF16
-// w is t_r, x3_b = x2_b + D_b'^{-1} ((f - A x2)_b - A_br t_r), xb takes u_b.
+// u_b = D_b'^{-1} ((f - A x2)_b - A_br t_r) into the black half of ub (tv holds
+// t_r) and the preconditioner's result x2_b + u_b
 template <typename T, typename S>
 __global__ void __launch_bounds__(kThreads, ilu_min_blocks<T>()) k_cpr_black(Geom g, const S* __restrict__ At,
-                         const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ w,
-                         const T* __restrict__ z, const T* __restrict__ e, T* __restrict__ xb, OutV zo,
+                         const S* __restrict__ Dinv, const T* __restrict__ f, const T* __restrict__ tv,
+                         const T* __restrict__ z, const T* __restrict__ e, T* __restrict__ ub, OutV zo,
                          const DevState* st) {
   wait_prior_grid();
   if (st->done) return;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.Nh; q += (int64_t)gridDim.x * blockDim.x) {
     const Cell c = decode(g, 1, q);
     const T x[3] = {z[vidx(g, 0, 1, q)] + e[g.Nh + q], z[vidx(g, 1, 1, q)], z[vidx(g, 2, 1, q)]};
-    T r[3];
-    if (kExactRed<S>) {
-      T s[3];
-      offdiag_sum(g, At, 1, q, c, w, s);
-      const S* a = At + at_index(g, 1, kDiag * 9, q);
+    T acc[3] = {T(0), T(0), T(0)}, s[3] = {T(0), T(0), T(0)};
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-        r[k] = f[vidx(g, k, 1, q)] - fma3(s[k], cv<T>(ld_stream(a + 96 * k)), x[0], cv<T>(ld_stream(a + 96 * k + 32)), x[1],
-                                          cv<T>(ld_stream(a + 96 * k + 64)), x[2]);
-    } else {
-      T acc[3] = {T(0), T(0), T(0)}, s[3] = {T(0), T(0), T(0)};
+    for (int sl = 0; sl < 7; ++sl) {
+      const S* a = At + at_index(g, 1, sl * 9, q);
+      T y[3] = {x[0], x[1], x[2]}, t[3];
+      if (sl != kDiag) {
+        const int64_t nb = nbr(g, c, q, sl);
+        const bool ok = nb >= 0;
+        const int64_t nq = ok ? nb : q;
+        y[0] = z[vidx(g, 0, 0, nq)] + e[nq], y[1] = z[vidx(g, 1, 0, nq)], y[2] = z[vidx(g, 2, 0, nq)];
 #pragma unroll
-      for (int sl = 0; sl < 7; ++sl) {
-        const S* a = At + at_index(g, 1, sl * 9, q);
-        T y[3] = {x[0], x[1], x[2]}, t[3];
-        if (sl != kDiag) {
-          const int64_t nb = nbr(g, c, q, sl);
-          const bool ok = nb >= 0;
-          const int64_t nq = ok ? nb : q;
-          y[0] = z[vidx(g, 0, 0, nq)] + e[nq], y[1] = z[vidx(g, 1, 0, nq)], y[2] = z[vidx(g, 2, 0, nq)];
-#pragma unroll
-          for (int k = 0; k < 3; ++k) t[k] = w[vidx(g, k, 0, nq)];
-          if (!ok) y[0] = y[1] = y[2] = t[0] = t[1] = t[2] = T(0);
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const T a0 = cv<T>(ld_stream(a + 96 * k)), a1 = cv<T>(ld_stream(a + 96 * k + 32)), a2 = cv<T>(ld_stream(a + 96 * k + 64));
-          acc[k] = fma3(acc[k], a0, y[0], a1, y[1], a2, y[2]);
-          if (sl != kDiag) s[k] = fma3(s[k], a0, t[0], a1, t[1], a2, t[2]);
-        }
+        for (int k = 0; k < 3; ++k) t[k] = tv[vidx(g, k, 0, nq)];
+        if (!ok) y[0] = y[1] = y[2] = t[0] = t[1] = t[2] = T(0);
       }
 #pragma unroll
-      for (int k = 0; k < 3; ++k) r[k] = (f[vidx(g, k, 1, q)] - acc[k]) - s[k];
+      for (int k = 0; k < 3; ++k) {
+        const T a0 = cv<T>(ld_stream(a + 96 * k)), a1 = cv<T>(ld_stream(a + 96 * k + 32)), a2 = cv<T>(ld_stream(a + 96 * k + 64));
+        acc[k] = fma3(acc[k], a0, y[0], a1, y[1], a2, y[2]);
+        if (sl != kDiag) s[k] = fma3(s[k], a0, t[0], a1, t[1], a2, t[2]);
+      }
     }
-    T d[9];
+    T r[3], d[9];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r[k] = (f[vidx(g, k, 1, q)] - acc[k]) - s[k];
 #pragma unroll
     for (int rc = 0; rc < 9; ++rc) d[rc] = cv<T>(Dinv[(size_t)rc * g.N + g.Nh + q]);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const T u = d[3 * k] * r[0] + d[3 * k + 1] * r[1] + d[3 * k + 2] * r[2];
-      xb[vidx(g, k, 1, q)] = kExactRed<S> ? x[k] + u : u;
+      ub[vidx(g, k, 1, q)] = u;
       out_put<T>(zo, vidx(g, k, 1, q), x[k] + u);
     }
   }
@@ -1730,8 +1670,8 @@ template <typename T, typename S>
 __device__ bool amg_down(const CycleArgs<T, S>& a, DevState* st) {
   const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
   const Geom& g = a.g;
-  for (int sw = a.cpr; sw < a.nu1; ++sw)
-    for (int color = 0; color < 2; ++color) {
+  for (int sw = 0; sw < a.nu1; ++sw)
+    for (int color = sw == 0 ? a.cpr : 0; color < 2; ++color) {
       const int zero = sw == 0 && color == 0;
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + (size_t)color * g.Nh,
                        [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, color, zero, q); });
@@ -1812,7 +1752,6 @@ __device__ bool amg_up(const CycleArgs<T, S>& a, DevState* st) {
     else
       sweep_batched<4>(t0, nt, g.Nh, a.x0 + g.Nh,
                        [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, 1, 0, q); });
-    if (a.cpr && sw + 1 == a.nu2) break;  // (the red cells are not read any more)
     if (!grid_barrier(st, a.spins)) return false;
     sweep_batched<4>(t0, nt, g.Nh, a.x0, [&](int64_t q) { return gs0_value<T, S>(g, a.At, a.di0, a.f0, a.x0, 0, 0, q); });
     if (sw + 1 < a.nu2 && !grid_barrier(st, a.spins)) return false;
@@ -2137,13 +2076,12 @@ __device__ __forceinline__ T res_gather(const ResLevel& r, uint32_t base, int32_
 // Every block of the cluster runs it when the level is shared (DIST), block
 // 0 alone otherwise.
 template <typename T, bool DIST>
-__device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l, uint32_t base, int cpr) {
+__device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l, uint32_t base) {
   constexpr int NP = res_pairs<T>();
   ResCells<T, NP> r;
   res_load<T, NP, DIST>(a, l, base, r);
   const ResLevel& rl = a.rl[l];
   const int32_t q0 = DIST ? (int32_t)blockIdx.x << rl.lch : 0;
-  const bool whole = cpr && l == 0;
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     const int32_t i = (int32_t)threadIdx.x + kResThreads * p, q = q0 + i;
@@ -2160,15 +2098,14 @@ __device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l,
       if (place) st_sh(res_local<T>(rl, base, kSecF + col, q), f);
     }
     // the first half sweep starts from zero: x_r = f_r / d_r (black zero
-    // until its own half sweep; within the CPR level 0's f_r is zero, which
-    // makes that x_b = f_b / d_b)
+    // until its own half sweep)
     if (place) {
       st_sh(res_local<T>(rl, base, kSecRed, q), r.live[0][p] ? res_divide(r.f[0][p], r.d[0][p], r.di[0][p]) : T(0));
-      st_sh(res_local<T>(rl, base, kSecBlack, q), whole && r.live[1][p] ? res_divide(r.f[1][p], r.d[1][p], r.di[1][p]) : T(0));
+      st_sh(res_local<T>(rl, base, kSecBlack, q), T(0));
     }
   }
   res_barrier<DIST>();
-  if (!whole) res_sweep<T, NP, DIST>(r, 1);
+  res_sweep<T, NP, DIST>(r, 1);
   for (int sw = 1; sw < a.nu1; ++sw) {
     res_sweep<T, NP, DIST>(r, 0);
     res_sweep<T, NP, DIST>(r, 1);
@@ -2193,7 +2130,7 @@ __device__ __forceinline__ void res_down(const ResPlan& a, const Geom& g, int l,
 
 // Coarse correction and post-smoothing of level l
 template <typename T, bool DIST>
-__device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, uint32_t base, int cpr) {
+__device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, uint32_t base) {
   constexpr int NP = res_pairs<T>();
   ResCells<T, NP> r;
   res_load<T, NP, DIST>(a, l, base, r);
@@ -2223,7 +2160,6 @@ __device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, u
   res_barrier<DIST>();
   for (int sw = 0; sw < a.nu2; ++sw) {
     res_sweep<T, NP, DIST>(r, 1);
-    if (cpr && l == 0 && sw + 1 == a.nu2) break;
     res_sweep<T, NP, DIST>(r, 0);
   }
   if (l == a.l0) {
@@ -2243,7 +2179,7 @@ __device__ __forceinline__ void res_up(const ResPlan& a, const Geom& g, int l, u
 
 template <typename T, typename S>
 __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_constant__ ResPlan a, Geom g,
-                                                                int cpr, const DevState* st) {
+                                                                const DevState* st) {
   wait_prior_grid();
   if (st->done) return;  // uniform: every block reads the same flag
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(g_tail_smem);
@@ -2261,12 +2197,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_co
   if (threadIdx.x < 32) st_sh(base + a.zero_off + threadIdx.x * (uint32_t)sizeof(T), T(0));
   cluster_sync_all();  // every block runs before its shared memory is read
   int l = a.l0;
-  for (; l < a.last && a.rl[l].dist; ++l) res_down<T, true>(a, g, l, base, cpr);
+  for (; l < a.last && a.rl[l].dist; ++l) res_down<T, true>(a, g, l, base);
   const int shared_to = l;
   if (first) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    for (; l < a.last; ++l) res_down<T, false>(a, g, l, base, cpr);
+    for (; l < a.last; ++l) res_down<T, false>(a, g, l, base);
     // the coarsest level: x = inv f, a thread per row (inv is stored transposed)
     const uint32_t fo = base + a.dense_off;
     const ResLevel& rl = a.rl[a.last];
@@ -2283,10 +2219,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_amg_resident(const __grid_co
       if (a.l0 == a.last) ((T*)rl.x)[i] = s;
     }
     __syncthreads();
-    for (l = a.last - 1; l >= shared_to; --l) res_up<T, false>(a, g, l, base, cpr);
+    for (l = a.last - 1; l >= shared_to; --l) res_up<T, false>(a, g, l, base);
   }
   cluster_sync_all();
-  for (l = shared_to - 1; l >= a.l0; --l) res_up<T, true>(a, g, l, base, cpr);
+  for (l = shared_to - 1; l >= a.l0; --l) res_up<T, true>(a, g, l, base);
   cluster_sync_all();  // no block leaves while another may read its shared memory
 }
 
@@ -2454,9 +2390,8 @@ void resident_plan(bo_prec* P, ResPlan& a) {
   a.cluster = C;
 }
 
-// cpr: within the CPR of an FP64 or FP32 preconditioner, whose k_cpr_rhs has done the first pre-smoothing sweep
-// (if nu1 > 0) and which never reads the red cells of level 0 afterwards, so
-// the last post-smoothing half sweep is left out too.
+// cpr: within the CPR, whose k_cpr_rhs has done the first half sweep (if nu1 >
+// 0; the cluster form starts from the right-hand side alone).
 template <typename T, typename S>
 void amg_vcycle(bo_prec* P, const DevState* st, bool cpr) {
   cudaStream_t s = P->stream;
@@ -2519,7 +2454,7 @@ void amg_vcycle(bo_prec* P, const DevState* st, bool cpr) {
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, k_amg_resident<T, S>, ra, g, (int)cpr, st) != cudaSuccess) return false;
+    if (cudaLaunchKernelEx(&cfg, k_amg_resident<T, S>, ra, g, st) != cudaSuccess) return false;
     note_launch();
     return true;
   };
@@ -2617,8 +2552,8 @@ void amg_vcycle(bo_prec* P, const DevState* st, bool cpr) {
     else cudaGetLastError();
   }
   if (!down_done) {
-    for (int sw = cpr; sw < nu1; ++sw) {
-      gs0(0, sw == 0);
+    for (int sw = 0; sw < nu1; ++sw) {
+      if (sw > 0 || !cpr) gs0(0, sw == 0);
       gs0(1, 0);
     }
     if (nu1 == 0) (launch_pdl(k_zero<T>, grid_for(g.N, TB), TB, 0, s, g.N, x0, st), note_launch());
@@ -2659,7 +2594,7 @@ void amg_vcycle(bo_prec* P, const DevState* st, bool cpr) {
   for (int sw = 0; sw < nu2; ++sw) {
     if (sw == 0) gs0_prolong();
     else gs0(1, 0);
-    if (!cpr || sw + 1 < nu2) gs0(0, 0);
+    gs0(0, 0);
   }
 }
 
@@ -2695,17 +2630,17 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
   (launch_cells(k_ilu_b<T, S>, g.Nh, s, g, At, D, f, tv, z1, st),
    note_launch());
   // (the pass reads z1's black half and writes its red half)
-  (launch_cells(k_ilu_r2<T, S, false>, g.Nh, s, g, At, D, f, tv, z1, z1, nullptr, OutV{}, st),
+  (launch_cells(k_ilu_r2<T, S, false>, g.Nh, s, g, At, D, tv, z1, z1, nullptr, OutV{}, st),
    note_launch());
   if (stage == BO_STAGE_ILU) {
     (launch_pdl(k_widen_t<T>, grid_for(3 * g.N), kThreads, 0, s, 3 * g.N, z1, zo.d, st), note_launch());
     return;
   }
   // x2 = x1 + Pi_p AMG(A_pp)^{-1} Pi_r (f - At x1)
-  (launch_cells(k_cpr_rhs<T, S>, kExactRed<S> ? g.Nh : g.N, s, g, At, (const T*)P->di0, f, z1,
+  (launch_cells(k_cpr_rhs<T, S>, g.N, s, g, At, (const T*)P->di0, f, z1,
       f0, e0, st),
    note_launch());
-  amg_vcycle<T, S>(P, st, kExactRed<S>);
+  amg_vcycle<T, S>(P, st, true);
   learned_coarse_apply(P, st);
   // x3 = x2 + R^{-1} (f - At x2)
   (launch_cells(k_cpr_red<T, S>, g.Nh, s, g, At, D, f, z1, e0, tv,
@@ -2714,7 +2649,7 @@ void cpr_apply(bo_prec* P, InV v, OutV zo, int stage, const DevState* st, const 
   (launch_cells(k_cpr_black<T, S>, g.Nh, s, g, At, D, f, tv, z1, e0, tv,
       zo, st),
    note_launch());
-  (launch_cells(k_ilu_r2<T, S, true>, g.Nh, s, g, At, D, f, tv, tv, z1, e0, zo, st),
+  (launch_cells(k_ilu_r2<T, S, true>, g.Nh, s, g, At, D, tv, tv, z1, e0, zo, st),
    note_launch());
 }
 

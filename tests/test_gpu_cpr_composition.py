@@ -1,13 +1,13 @@
-"""The CPR in BF16 storage against the composition it stands for,
+"""The CPR in FP32 and BF16 storage against the composition it stands for,
   x1 = R^{-1} f,  x2 = x1 + Pi_p AMG(A_pp)^{-1} Pi_r (f - A x1),
   z  = x2 + R^{-1} (f - A x2),
-with whole residuals of the BF16-rounded decoupled matrix: local solves and
+with whole residuals of the rounded decoupled matrix: local solves and
 V-cycles by the library's own stages, the residuals here in FP32 in the
 matrix's slot order (-z, -y, -x, cell, +x, +y, +z), one fused multiply-add a
-product.  Where storage keeps 8 bits, another order of the same sums moves a
-solution by more than the solver's tolerance, so the results are equal bit for
-bit, in every launch form of the V-cycle.  Sizes: single cells, rows and
-planes, odd lengths, several thread blocks."""
+product.  Some systems amplify rounding so far that another order of the same
+sums moves a solution by more than the solver's tolerance, so the results are
+equal bit for bit, in every launch form of the V-cycle.  Sizes: single cells,
+rows and planes, odd lengths, several thread blocks."""
 import numpy as np
 import pytest
 
@@ -42,12 +42,12 @@ def _fma32(a, x, acc):
     return s.astype(np.float32)
 
 
-def _blocks(Ao, dims):
+def _blocks(Ao, dims, dtype):
     """(7, 3, 3, N) blocks of the decoupled matrix, rounded as the library stores them, and the neighbours (7, N)."""
     At, _ = oracle.qi_decouple(Ao)
     nx, ny, nz = dims
     N = nx * ny * nz
-    val = torch.from_numpy(At.val.reshape(-1, 3, 3).astype(np.float32)).to(torch.bfloat16).float().numpy()
+    val = torch.from_numpy(At.val.reshape(-1, 3, 3).astype(np.float32)).to(dtype).float().numpy()
     rows = np.repeat(np.arange(N), np.diff(At.rowptr))
     i, j, k = rows % nx, rows // nx % ny, rows // (nx * ny)
     ci, cj, ck = At.col % nx, At.col // nx % ny, At.col // (nx * ny)
@@ -69,14 +69,19 @@ def _residual(B, nb, f, x):
 
 
 @pytest.mark.parametrize("dims", DIMS)
-def test_bf16_equals_the_whole_residual_composition(bo, dims):
+@pytest.mark.parametrize("storage", ["fp32", "bf16"])
+def test_cpr_equals_the_whole_residual_composition(bo, dims, storage):
+    precision, dtype = {"fp32": (bo.BO_PREC_FP32, torch.float32), "bf16": (bo.BO_PREC_BF16, torch.bfloat16)}[storage]
     a = bogen.assemble(bogen.tiny_case(5, *dims))
+    val = a["val"].reshape(-1, 3, 3).copy()
+    if storage == "fp32":  # (decoupled rows are formed in 48 bits: FP32 values of them may differ from FP64's)
+        val[:, 0, 1:] = 0.0
     ctx = bo.Context(0)
-    A = bo.Matrix.from_bsr(ctx, bo.grid(*dims), a["rowptr"], a["col"], a["val"])
-    B, nb = _blocks(oracle.BsrMatrix(a["rowptr"], a["col"], a["val"]), dims)
+    A = bo.Matrix.from_bsr(ctx, bo.grid(*dims), a["rowptr"], a["col"], val)
+    B, nb = _blocks(oracle.BsrMatrix(a["rowptr"], a["col"], val), dims, dtype)
     f = np.random.default_rng(3).standard_normal((B.shape[-1], 3)).astype(np.float32)
     for nu1, nu2 in ((2, 2), (1, 0), (0, 1)):
-        P = bo.Preconditioner(A, precision=bo.BO_PREC_BF16, nu1=nu1, nu2=nu2)
+        P = bo.Preconditioner(A, precision=precision, nu1=nu1, nu2=nu2)
 
         def stage(st, v):
             r = torch.from_numpy(v.astype(np.float64).ravel()).cuda()
