@@ -424,8 +424,11 @@ __device__ __forceinline__ int64_t nat_index(const LevelDims& L, int i, int j, i
 // cell walked its children one after the other, 8 dependent rounds of loads,
 // and left small levels with a handful of warps: 43-56 us for level 1 and 17
 // us per coarser level whatever their size).  A child's entries towards its
-// own aggregate join the diagonal, the three others the coarse faces; the
-// children's sums meet by shuffles in a fixed order.  Lane bits: child x
+// own aggregate join the diagonal, the three others the coarse faces.  The
+// children's entries are fetched by shuffles and added one after the other, in
+// the order of a loop over the children (x fastest) and their slots: another
+// order leaves another last bit, which some systems amplify (see the CPR's
+// passes below).  Lane bits: child x
 // offset (1), coarse cell of the four (2, 4), child y (8), child z (16), so
 // the lanes of a row of children read consecutive fine cells.  The value is
 // written in FP64 (the next level's input) and in the storage type.
@@ -450,7 +453,6 @@ __device__ __forceinline__ Child galerkin_child(const LevelDims& C, int64_t grou
   c.ok = c.ok && c.i < fnx && c.j < fny && c.k < fnz;
   return c;
 }
-__device__ __forceinline__ double add_xor(double v, int m) { return v + __shfl_xor_sync(0xffffffffu, v, m); }
 
 // FP64 levels keep the reciprocals of the diagonal behind the seven
 // coefficients: the Gauss-Seidel sweeps divide with their help, since an FP64
@@ -477,17 +479,32 @@ __device__ __forceinline__ void put_reciprocal(S* __restrict__ c, const LevelDim
 template <typename S>
 __device__ __forceinline__ void galerkin_sum(const LevelDims& C, const Child& ch, const double a[7],
                                              double* __restrict__ c64, S* __restrict__ c, DevState* st) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, cell = lane & 6;  // (the lanes of this coarse cell: its bits and the child's)
   const bool di = lane & 1, dj = lane & 8, dk = lane & 16;
-  double diag = a[kDiag];
-  diag += dk ? a[kZm] : a[kZp];
-  diag += dj ? a[kYm] : a[kYp];
-  diag += di ? a[kXm] : a[kXp];
-  double fx = di ? a[kXp] : a[kXm], fy = dj ? a[kYp] : a[kYm], fz = dk ? a[kZp] : a[kZm];
-  diag = add_xor(add_xor(add_xor(diag, 1), 8), 16);
-  fx = add_xor(add_xor(fx, 8), 16);
-  fy = add_xor(add_xor(fy, 1), 16);
-  fz = add_xor(add_xor(fz, 1), 8);
+  auto from = [](double v, int src) { return __shfl_sync(0xffffffffu, v, src); };
+  double diag = 0.0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int src = cell | (q & 1) | ((q & 2) << 2) | ((q & 4) << 2);
+    // (slot order; a child's entries towards its own aggregate)
+    if (q & 4) diag += from(a[kZm], src);
+    if (q & 2) diag += from(a[kYm], src);
+    if (q & 1) diag += from(a[kXm], src);
+    diag += from(a[kDiag], src);
+    if (!(q & 1)) diag += from(a[kXp], src);
+    if (!(q & 2)) diag += from(a[kYp], src);
+    if (!(q & 4)) diag += from(a[kZp], src);
+  }
+  // the entry across the aggregate's face: four children, in their order
+  auto face = [&](double v, int bit0, int bit1) {
+    const int own = lane & ~(bit0 | bit1);
+    double t = from(v, own);
+    t += from(v, own | bit0);
+    t += from(v, own | bit1);
+    return t + from(v, own | bit0 | bit1);
+  };
+  const double fx = face(di ? a[kXp] : a[kXm], 8, 16), fy = face(dj ? a[kYp] : a[kYm], 1, 16),
+               fz = face(dk ? a[kZp] : a[kZm], 1, 8);
   if (ch.I < 0) return;
   auto put = [&](int s, double v) {
     c64[(size_t)s * C.n + ch.I] = v;
@@ -553,24 +570,35 @@ __global__ void k_galerkin0_wide(Geom g, const double* __restrict__ A, const dou
     const Ijk p = ijk_of(C, live ? I : 0);
     const int i = 2 * p.i + di;
     double diag = 0.0, fx = 0.0, y0 = 0.0, y1 = 0.0, z0 = 0.0, z1 = 0.0;
+    // both children of a row: their values by shuffles, in the order of the children
+    const int l0 = threadIdx.x & 30;
+    auto both = [&](double& t, double v) {
+      t += __shfl_sync(0xffffffffu, v, l0);
+      t += __shfl_sync(0xffffffffu, v, l0 | 1);
+    };
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int j = 2 * p.j + (r & 1), k = 2 * p.k + (r >> 1);
-      if (!live || i >= g.nx || j >= g.ny || k >= g.nz) continue;
-      double a[7];
-      galerkin0_row(g, A, w, i, j, k, a);
-      diag += a[kDiag] + (di ? a[kXm] : a[kXp]) + (r & 1 ? a[kYm] : a[kYp]) + (r >> 1 ? a[kZm] : a[kZp]);
+      double a[7] = {0, 0, 0, 0, 0, 0, 0};
+      if (live && i < g.nx && j < g.ny && k < g.nz) galerkin0_row(g, A, w, i, j, k, a);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {  // (the child's entries towards its own aggregate in slot order)
+        const int src = l0 | e;
+        auto own = [&](int s) { diag += __shfl_sync(0xffffffffu, a[s], src); };
+        if (r >> 1) own(kZm);
+        if (r & 1) own(kYm);
+        if (e) own(kXm);
+        own(kDiag);
+        if (!e) own(kXp);
+        if (!(r & 1)) own(kYp);
+        if (!(r >> 1)) own(kZp);
+      }
       fx += di ? a[kXp] : a[kXm];
-      if (r & 1) y1 += a[kYp];
-      else y0 += a[kYm];
-      if (r >> 1) z1 += a[kZp];
-      else z0 += a[kZm];
+      if (r & 1) both(y1, a[kYp]);
+      else both(y0, a[kYm]);
+      if (r >> 1) both(z1, a[kZp]);
+      else both(z0, a[kZm]);
     }
-    diag = add_xor(diag, 1);
-    y0 = add_xor(y0, 1);
-    y1 = add_xor(y1, 1);
-    z0 = add_xor(z0, 1);
-    z1 = add_xor(z1, 1);
     if (!live) continue;
     auto put = [&](int s, double v) {
       c64[(size_t)s * C.n + I] = v;
