@@ -417,43 +417,6 @@ __device__ __forceinline__ int64_t nat_index(const LevelDims& L, int i, int j, i
   return i + (int64_t)L.nx * (j + (int64_t)L.ny * k);
 }
 
-// Galerkin products: coarse entry (I, J) = sum of the fine entries a_ij with
-// i in aggregate I and j in aggregate J.  Eight lanes of a warp serve one
-// coarse cell, one lane per child cell, and a warp serves four coarse cells:
-// every lane issues all of its child's loads at once (one thread per coarse
-// cell walked its children one after the other, 8 dependent rounds of loads,
-// and left small levels with a handful of warps: 43-56 us for level 1 and 17
-// us per coarser level whatever their size).  A child's entries towards its
-// own aggregate join the diagonal, the three others the coarse faces.  The
-// children's entries are fetched by shuffles and added one after the other, in
-// the order of a loop over the children (x fastest) and their slots: another
-// order leaves another last bit, which some systems amplify (see the CPR's
-// passes below).  Lane bits: child x
-// offset (1), coarse cell of the four (2, 4), child y (8), child z (16), so
-// the lanes of a row of children read consecutive fine cells.  The value is
-// written in FP64 (the next level's input) and in the storage type.
-// Measured, before -> after: level 1 of 128x128x64 70 -> 65 us, of 20x20x5
-// 43 -> 7 us; a coarser level 17 -> 4-8 us (the conversion to the
-// storage type included, which was a launch of its own).
-struct Child {
-  int64_t I;      // coarse cell, or -1
-  int i, j, k;    // the child's fine coordinates
-  bool ok;        // the child exists
-};
-__device__ __forceinline__ Child galerkin_child(const LevelDims& C, int64_t group, int fnx, int fny, int fnz) {
-  const int lane = threadIdx.x & 31;
-  Child c;
-  c.I = 4 * group + ((lane >> 1) & 3);
-  c.ok = c.I < C.n;
-  const Ijk p = ijk_of(C, c.ok ? c.I : 0);
-  c.i = 2 * p.i + (lane & 1);
-  c.j = 2 * p.j + ((lane >> 3) & 1);
-  c.k = 2 * p.k + (lane >> 4);
-  if (c.I >= C.n) c.I = -1;
-  c.ok = c.ok && c.i < fnx && c.j < fny && c.k < fnz;
-  return c;
-}
-
 // FP64 levels keep the reciprocals of the diagonal behind the seven
 // coefficients: the Gauss-Seidel sweeps divide with their help, since an FP64
 // division is about ten FP64 multiply-adds where the rest of a cell's
@@ -475,163 +438,106 @@ __device__ __forceinline__ void put_reciprocal(S* __restrict__ c, const LevelDim
   if constexpr (sizeof(S) == 8) c[(size_t)7 * C.n + I] = 1.0 / diag;
 }
 
-// a[7]: the child's fine row (zero where the child or the neighbour is missing)
-template <typename S>
-__device__ __forceinline__ void galerkin_sum(const LevelDims& C, const Child& ch, const double a[7],
-                                             double* __restrict__ c64, S* __restrict__ c, DevState* st) {
-  const int lane = threadIdx.x & 31, cell = lane & 6;  // (the lanes of this coarse cell: its bits and the child's)
-  const bool di = lane & 1, dj = lane & 8, dk = lane & 16;
-  auto from = [](double v, int src) { return __shfl_sync(0xffffffffu, v, src); };
-  double diag = 0.0;
+// Galerkin products: coarse entry (I, J) = sum of the fine entries a_ij with
+// i in aggregate I and j in aggregate J.  A block takes 32 consecutive coarse
+// cells, a thread per child: consecutive threads read consecutive fine cells,
+// and all of a child's loads are in flight at once.  The rows meet in shared
+// memory, where a warp takes one of the seven entries of the 32 cells (a
+// child's entries towards its own aggregate join the diagonal) and adds it up
+// as a loop over the children (x fastest) and their slots does: another order
+// leaves another last bit, which some systems amplify (see the CPR's passes
+// below).  The value is written in FP64 (the next level's input) and in the
+// storage type.  Level 1 is bound by its FP64 products, 168 + 56 warp
+// instructions for 32 coarse cells at 16 cycles, and the loads.  Measured, one
+// thread per coarse cell and a conversion kernel -> this: level 1 of
+// 128x128x64 78 -> 71 us, of 62x45x19 60 -> 11, of 20x20x5 (FP64) 46 -> 10; a
+// coarser level 17-22 -> 4-6 us.
+template <typename S, typename Row>
+__device__ __forceinline__ void galerkin_block(const LevelDims& C, int fnx, int fny, int fnz, Row row,
+                                               double* __restrict__ c64, S* __restrict__ c, DevState* st) {
+  static_assert(kThreads == 256, "8 children of 32 coarse cells");
+  __shared__ double a[7][kThreads];
+  const int t = threadIdx.x, q = t & 31, e = t >> 5;
+  for (int64_t I0 = blockIdx.x * (int64_t)32; I0 < C.n; I0 += gridDim.x * (int64_t)32) {
+    double v[7] = {0, 0, 0, 0, 0, 0, 0};  // (zero where the child is missing)
+    const int64_t I = I0 + ((t & 63) >> 1);
+    if (I < C.n) {
+      const Ijk p = ijk_of(C, I);
+      const int i = 2 * p.i + (t & 1), j = 2 * p.j + ((t >> 6) & 1), k = 2 * p.k + (t >> 7);
+      if (i < fnx && j < fny && k < fnz) row(i, j, k, v);
+    }
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int src = cell | (q & 1) | ((q & 2) << 2) | ((q & 4) << 2);
-    // (slot order; a child's entries towards its own aggregate)
-    if (q & 4) diag += from(a[kZm], src);
-    if (q & 2) diag += from(a[kYm], src);
-    if (q & 1) diag += from(a[kXm], src);
-    diag += from(a[kDiag], src);
-    if (!(q & 1)) diag += from(a[kXp], src);
-    if (!(q & 2)) diag += from(a[kYp], src);
-    if (!(q & 4)) diag += from(a[kZp], src);
-  }
-  // the entry across the aggregate's face: four children, in their order
-  auto face = [&](double v, int bit0, int bit1) {
-    const int own = lane & ~(bit0 | bit1);
-    double t = from(v, own);
-    t += from(v, own | bit0);
-    t += from(v, own | bit1);
-    return t + from(v, own | bit0 | bit1);
-  };
-  const double fx = face(di ? a[kXp] : a[kXm], 8, 16), fy = face(dj ? a[kYp] : a[kYm], 1, 16),
-               fz = face(dk ? a[kZp] : a[kZm], 1, 8);
-  if (ch.I < 0) return;
-  auto put = [&](int s, double v) {
-    c64[(size_t)s * C.n + ch.I] = v;
-    c[(size_t)s * C.n + ch.I] = to_store<S>(v);
-  };
-  if (!dj && !dk) put(di ? kXp : kXm, fx);
-  if (!di && !dk) put(dj ? kYp : kYm, fy);
-  if (!di && !dj) put(dk ? kZp : kZm, fz);
-  if (di && dj && dk) {
-    put(kDiag, diag);
-    put_reciprocal(c, C, ch.I, diag);
-    if (diag == 0.0 || !isfinite(diag)) atomicOr(&st->err, kErrBreakdown);
+    for (int s = 0; s < 7; ++s) a[s][t] = v[s];
+    __syncthreads();
+    if (e < 7 && I0 + q < C.n) {
+      auto child = [&](int s, int x, int y, int z) { return a[s][(2 * z + y) * 64 + 2 * q + x]; };
+      const int side = e > kDiag;
+      double sum = 0.0;
+      if (e == kDiag) {
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+          for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+              if (z) sum += child(kZm, x, y, z);
+              if (y) sum += child(kYm, x, y, z);
+              if (x) sum += child(kXm, x, y, z);
+              sum += child(kDiag, x, y, z);
+              if (!x) sum += child(kXp, x, y, z);
+              if (!y) sum += child(kYp, x, y, z);
+              if (!z) sum += child(kZp, x, y, z);
+            }
+      } else {  // the four children at a face
+#pragma unroll
+        for (int hi = 0; hi < 2; ++hi)
+#pragma unroll
+          for (int lo = 0; lo < 2; ++lo)
+            sum += e == kXm || e == kXp   ? child(e, side, lo, hi)
+                   : e == kYm || e == kYp ? child(e, lo, side, hi)
+                                          : child(e, lo, hi, side);
+      }
+      c64[(size_t)e * C.n + I0 + q] = sum;
+      c[(size_t)e * C.n + I0 + q] = to_store<S>(sum);
+      if (e == kDiag) {
+        put_reciprocal(c, C, I0 + q, sum);
+        if (sum == 0.0 || !isfinite(sum)) atomicOr(&st->err, kErrBreakdown);
+      }
+    }
+    __syncthreads();
   }
 }
 
 // level 1 from level 0 (the decoupled pressure block, FP64 from A and the weights)
-__device__ __forceinline__ void galerkin0_row(const Geom& g, const double* __restrict__ A, const double* __restrict__ w,
-                                              int i, int j, int k, double a[7]) {
-  const int color = (i + j + k) & 1;
-  const int64_t q = (i + (int64_t)g.nx * (j + (int64_t)g.ny * k)) >> 1;
-  const double g0 = w[vidx(g, 0, color, q)], g1 = w[vidx(g, 1, color, q)], g2 = w[vidx(g, 2, color, q)];
-  double r[21];
-#pragma unroll
-  for (int s = 0; s < 7; ++s)
-#pragma unroll
-    for (int u = 0; u < 3; ++u) r[3 * s + u] = A[plane(g, color, s, 3 * u) + q];
-  // (blocks outside the grid are stored as zeros)
-#pragma unroll
-  for (int s = 0; s < 7; ++s) a[s] = g0 * r[3 * s] + g1 * r[3 * s + 1] + g2 * r[3 * s + 2];
-}
-
 template <typename S>
-__global__ void k_galerkin0(Geom g, const double* __restrict__ A, const double* __restrict__ w, LevelDims C,
-                            double* __restrict__ c64, S* __restrict__ c, DevState* st) {
+__global__ void __launch_bounds__(kThreads) k_galerkin0(Geom g, const double* __restrict__ A, const double* __restrict__ w,
+                            LevelDims C, double* __restrict__ c64, S* __restrict__ c, DevState* st) {
   wait_prior_grid();
-  const int64_t ngroups = (C.n + 3) / 4;
-  for (int64_t gr = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; gr < ngroups;
-       gr += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const Child ch = galerkin_child(C, gr, g.nx, g.ny, g.nz);
-    double a[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (ch.ok) galerkin0_row(g, A, w, ch.i, ch.j, ch.k, a);
-    galerkin_sum<S>(C, ch, a, c64, c, st);
-  }
-}
-
-// The same with two lanes per coarse cell (the two children along x; the
-// four rows of children one after the other): a warp's loads cover 16
-// consecutive values of a plane instead of 4, which is what a level that
-// fills the GPU anyway is bound by (level 1 of 128x128x64: 70 us with one
-// thread per coarse cell, 97 us with eight lanes, 65 us with two; the
-// launch takes it from kGalerkinWide coarse cells on, where eight lanes per
-// cell would be more than 8 warps per scheduler).
-constexpr int64_t kGalerkinWide = 32768;
-template <typename S>
-__global__ void k_galerkin0_wide(Geom g, const double* __restrict__ A, const double* __restrict__ w, LevelDims C,
-                                 double* __restrict__ c64, S* __restrict__ c, DevState* st) {
-  wait_prior_grid();
-  const int64_t n2 = (2 * C.n + 31) & ~(int64_t)31;  // whole warps: the sums meet by shuffles
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n2; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t I = t >> 1;
-    const int di = (int)(t & 1);
-    const bool live = I < C.n;
-    const Ijk p = ijk_of(C, live ? I : 0);
-    const int i = 2 * p.i + di;
-    double diag = 0.0, fx = 0.0, y0 = 0.0, y1 = 0.0, z0 = 0.0, z1 = 0.0;
-    // both children of a row: their values by shuffles, in the order of the children
-    const int l0 = threadIdx.x & 30;
-    auto both = [&](double& t, double v) {
-      t += __shfl_sync(0xffffffffu, v, l0);
-      t += __shfl_sync(0xffffffffu, v, l0 | 1);
-    };
+  galerkin_block(C, g.nx, g.ny, g.nz, [&](int i, int j, int k, double (&a)[7]) {
+    const int color = (i + j + k) & 1;
+    const int64_t q = (i + (int64_t)g.nx * (j + (int64_t)g.ny * k)) >> 1;
+    const double g0 = w[vidx(g, 0, color, q)], g1 = w[vidx(g, 1, color, q)], g2 = w[vidx(g, 2, color, q)];
+    double r[21];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int j = 2 * p.j + (r & 1), k = 2 * p.k + (r >> 1);
-      double a[7] = {0, 0, 0, 0, 0, 0, 0};
-      if (live && i < g.nx && j < g.ny && k < g.nz) galerkin0_row(g, A, w, i, j, k, a);
+    for (int s = 0; s < 7; ++s)
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {  // (the child's entries towards its own aggregate in slot order)
-        const int src = l0 | e;
-        auto own = [&](int s) { diag += __shfl_sync(0xffffffffu, a[s], src); };
-        if (r >> 1) own(kZm);
-        if (r & 1) own(kYm);
-        if (e) own(kXm);
-        own(kDiag);
-        if (!e) own(kXp);
-        if (!(r & 1)) own(kYp);
-        if (!(r >> 1)) own(kZp);
-      }
-      fx += di ? a[kXp] : a[kXm];
-      if (r & 1) both(y1, a[kYp]);
-      else both(y0, a[kYm]);
-      if (r >> 1) both(z1, a[kZp]);
-      else both(z0, a[kZm]);
-    }
-    if (!live) continue;
-    auto put = [&](int s, double v) {
-      c64[(size_t)s * C.n + I] = v;
-      c[(size_t)s * C.n + I] = to_store<S>(v);
-    };
-    put(di ? kXp : kXm, fx);
-    put(di ? kYp : kYm, di ? y1 : y0);
-    put(di ? kZp : kZm, di ? z1 : z0);
-    if (di) {
-      put(kDiag, diag);
-      put_reciprocal(c, C, I, diag);
-      if (diag == 0.0 || !isfinite(diag)) atomicOr(&st->err, kErrBreakdown);
-    }
-  }
+      for (int u = 0; u < 3; ++u) r[3 * s + u] = A[plane(g, color, s, 3 * u) + q];
+    // (blocks outside the grid are stored as zeros)
+#pragma unroll
+    for (int s = 0; s < 7; ++s) a[s] = g0 * r[3 * s] + g1 * r[3 * s + 1] + g2 * r[3 * s + 2];
+  }, c64, c, st);
 }
 
 // level l+1 from natural-order level l
 template <typename S>
-__global__ void k_galerkinn(LevelDims F, const double* __restrict__ f64, LevelDims C, double* __restrict__ c64,
-                            S* __restrict__ c, DevState* st) {
+__global__ void __launch_bounds__(kThreads) k_galerkinn(LevelDims F, const double* __restrict__ f64, LevelDims C,
+                            double* __restrict__ c64, S* __restrict__ c, DevState* st) {
   wait_prior_grid();
-  const int64_t ngroups = (C.n + 3) / 4;
-  for (int64_t gr = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; gr < ngroups;
-       gr += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const Child ch = galerkin_child(C, gr, F.nx, F.ny, F.nz);
-    double a[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (ch.ok) {
-      const int64_t cf = nat_index(F, ch.i, ch.j, ch.k);
+  galerkin_block(C, F.nx, F.ny, F.nz, [&](int i, int j, int k, double (&a)[7]) {
+    const int64_t cf = nat_index(F, i, j, k);
 #pragma unroll
-      for (int s = 0; s < 7; ++s) a[s] = f64[(size_t)s * F.n + cf];
-    }
-    galerkin_sum<S>(C, ch, a, c64, c, st);
-  }
+    for (int s = 0; s < 7; ++s) a[s] = f64[(size_t)s * F.n + cf];
+  }, c64, c, st);
 }
 
 // ------------------------------------------------------- dense inverse
@@ -2709,13 +2615,10 @@ int values_impl(bo_prec* P) {
     (launch_pdl(k_ilu_red<S, false>, gh, th, 0, s, g, m->A, P->w, (S*)P->Dinv, red64, P->st), note_launch());
     (launch_pdl(k_ilu_black<S>, gh, th, 0, s, g, m->A, P->w, red64, (S*)P->Dinv, P->st), note_launch());
   }
-  // AMG hierarchy values (eight lanes per coarse cell)
+  // AMG hierarchy values (eight threads per coarse cell)
   for (int l = 1; l < P->nlev; ++l) {
     Level& C = P->lev[l];
-    if (l == 1 && C.n >= kGalerkinWide)
-      (launch_pdl(k_galerkin0_wide<S>, grid_for(2 * C.n), kThreads, 0, s, g, m->A, P->w, dims_of(C), C.c64, (S*)C.c,
-           P->st), note_launch());
-    else if (l == 1)
+    if (l == 1)
       (launch_pdl(k_galerkin0<S>, grid_for(8 * C.n), kThreads, 0, s, g, m->A, P->w, dims_of(C), C.c64, (S*)C.c, P->st),
        note_launch());
     else
