@@ -425,8 +425,8 @@ __device__ __forceinline__ int64_t nat_index(const LevelDims& L, int i, int j, i
 // s / d from the rounded reciprocal r = 1 / d: the product, corrected once by
 // its residual, is the rounded quotient (P. Markstein, IBM J. Res. Dev. 34,
 // 1990); the product alone is off by up to one unit more.  (An infinite
-// product has no residual.)  A Newton step of 128x128x64 takes 17.5 ms with the
-// product alone and 18.1 so, 20x20x5 963 and 980 us.
+// product has no residual.)  The correction costs a Newton step of 128x128x64
+// 0.6 of 18 ms, of 20x20x5 17 of 980 us.
 __device__ __forceinline__ double divide_by(double s, double d, double r) {
   const double q = s * r, c = fma(fma(-q, d, s), r, q);
   return isfinite(c) ? c : q;
