@@ -41,7 +41,7 @@ def test_one_partial_sum_per_sm_is_kept():
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     need = sms * (27 * C * C * 4 + C * 8 + 4)
     kept = start - _free()
-    assert need <= kept <= need + 4 * MB  # (the driver allocates in steps of 2 MB)
+    assert need <= kept <= need + 4 * MB  # (device memory comes in steps of 2 MB)
     for _ in range(3):
         bo.bo_conv3d_backward_weights(ctx, DIMS, x, on, dw, db)
     assert start - _free() == kept
